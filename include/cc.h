@@ -50,7 +50,7 @@ typedef enum {
     CC_ERR_CUDA = 3,       /* a CUDA runtime call or kernel failed */
     CC_ERR_OVERFLOW = 4,   /* 3 k n + k >= 2^31: an int32 gain could overflow */
     CC_ERR_TABLE_FULL = 5, /* the contingency hash ran out of slots (bounded probing gave up) */
-    CC_ERR_TIMEOUT = 6     /* reserved: a bounded device wait gave up */
+    CC_ERR_TIMEOUT = 6     /* a block of the run kernel waited more than 20 s for the others */
 } cc_status;
 
 typedef struct {
@@ -84,11 +84,12 @@ typedef struct {
                                scoring every candidate would give).  Results are identical;
                                it changes how many edges a sweep evaluates.  0 (default):
                                every sweep scores every edge */
-    int32_t no_regions;     /* 1: capture every kernel of a sweep as a plain node of the sweep
-                               graph (a region a sweep does not need runs kernels that return at
-                               once) instead of behind conditional nodes; for profilers that
-                               cannot see kernels inside graphs with conditional nodes.  Results
-                               are identical.  0 (default): conditional regions */
+    int32_t no_regions;     /* 1: run every step of a sweep as a kernel of its own, a plain node
+                               of a captured graph (a step that a sweep does not need is a
+                               kernel that returns at once); for profilers, which see one
+                               kernel per step.  Results are identical.  0 (default): the run
+                               kernel, or a graph with conditional regions (see
+                               cc_run_until_converged) */
     int32_t empty_moves;    /* 1: the move-to-empty variant.  Besides the clusters of its
                                neighbours (Eq. objective4), a vertex v may move into a new
                                cluster of its own, which takes the id v, provided no vertex
@@ -309,38 +310,37 @@ cc_status cc_sweep(cc_ctx* ctx, cc_sweep_info* info);
 
 /* Runs sweeps until one has no proposal (the stopping condition of The
  * algorithm) or max_sweeps sweeps ran (max_sweeps <= 0: the option's limit).
- * Sweeps are submitted as CUDA graphs of up to 4 unrolled sweeps (a sweep is
- * skipped on the device once the run has stopped); the host reads the stop
- * flag after each graph, so a run costs one synchronisation per 4 sweeps.
- * A context of several jobs (cc_batch_create; unless no_regions is set) runs
- * instead as one graph launch: a conditional loop repeats the sweep until
- * the run stops, and the host synchronises once.
+ * A context of several jobs, a colour-batched one, and any job of at least
+ * 16,384 label rows (n times k rounded up to 4) runs in the run kernel: one
+ * cooperative launch takes the whole run, and the host synchronises once.
+ * A smaller job's sweeps are submitted as CUDA graphs of up to 4 unrolled
+ * sweeps (a sweep is skipped on the device once the run has stopped), and the
+ * host reads the stop flag after each graph; so are all runs with no_regions.
  * *sweeps_done (may be NULL) counts every sweep run, the final empty one
  * included.  Errors as cc_sweep. */
 cc_status cc_run_until_converged(cc_ctx* ctx, int32_t max_sweeps, int32_t* sweeps_done);
 
 /* Device time of each sweep of the last cc_run_until_converged / cc_sweep
- * call, from CUDA events recorded inside its graphs on the context's stream:
- * sweep_ms[s] covers sweep s (all its kernels), propose_ms[s] its proposal
- * kernels (k_own, k_edges, k_collect); with colour_batched, entry s covers
- * the s-th colour class run (a sweep is one run of every class).  A run that
- * was one graph launch (a context of several jobs) has one entry for it, with
- * propose_ms 0 (the proposal kernels are not timed apart inside the loop).  At most max entries are written to
- * each non-NULL array; *count receives the number of sweeps timed.  A sweep
- * abandoned for lack of table space and retried is timed once per attempt. */
+ * call, taken on the device between the steps of the run kernel, or from CUDA
+ * events recorded inside the run's graphs: sweep_ms[s] covers sweep s (all its
+ * steps), propose_ms[s] its proposal step (own, edges, collect); with
+ * colour_batched, entry s covers the s-th colour class run (a sweep is one run
+ * of every class).  At most max entries are written to each non-NULL array;
+ * *count receives the number of sweeps timed.  A sweep abandoned for lack of
+ * table space and retried is timed once per attempt. */
 cc_status cc_last_run_timing(cc_ctx* ctx, int32_t max, float* sweep_ms, float* propose_ms, int32_t* count);
 
 /* Current state of the contingency hash (synchronises the stream). */
 cc_status cc_table_stats(cc_ctx* ctx, cc_table_info* out);
 
 /* Number of CUDA kernels the context has run since creation: every kernel it
- * launched directly, every kernel node of its sweep graphs that sits outside
- * a conditional region (whether or not a stopped sweep returned from it at
- * once), and the kernels of the conditional regions that ran (the heavy
- * path, the second attempt of its rebuild, its evaluation, its rollback, the
- * light path and the end-of-sweep rebuild of a sweep are IF nodes, entered
- * only when needed; their gates count them on the device).  Synchronises the
- * context's stream. */
+ * launched directly (a run of the run kernel is one), every kernel node of its
+ * sweep graphs that sits outside a conditional region (whether or not a
+ * stopped sweep returned from it at once), and the kernels of the conditional
+ * regions that ran (the heavy path, the second attempt of its rebuild, its
+ * evaluation, its rollback, the light path and the end-of-sweep rebuild of a
+ * sweep are IF nodes, entered only when needed; their gates count them on the
+ * device).  Synchronises the context's stream. */
 cc_status cc_launch_count(const cc_ctx* ctx, int64_t* out);
 
 /* Copies the records of the sweeps run since creation or the last reset,

@@ -85,8 +85,6 @@ void free_all(cc_ctx* c)
     c->own_stream = nullptr;
     if (c->body_stream) cudaStreamDestroy(c->body_stream);
     c->body_stream = nullptr;
-    if (c->loop_stream) cudaStreamDestroy(c->loop_stream);
-    c->loop_stream = nullptr;
 }
 
 unsigned long long next_pow2(unsigned long long x)
@@ -126,6 +124,16 @@ cc_status need_single(cc_ctx* c)
     return CC_OK;
 }
 
+// Capacity - 1 for a rebuild of every key by the host: the current one, or,
+// after a partial rebuild, one that holds all keys at load <= 1/2.
+unsigned long long full_mask(const cc_ctx* c, const DevState& s)
+{
+    if (!s.small) return s.mask;
+    unsigned long long cap = std::min<unsigned long long>(1024, c->cap_max);
+    while (cap < 2 * s.keys_all && cap < c->cap_max) cap <<= 1;
+    return cap - 1;
+}
+
 // F of every job recomputed from scratch (the table is built first if the
 // context is still at the singleton start without one).
 cc_status objective_recompute(cc_ctx* c, std::vector<long long>& F)
@@ -133,8 +141,9 @@ cc_status objective_recompute(cc_ctx* c, std::vector<long long>& F)
     DevState pre;
     cc_status rp = read_state(c, &pre);
     if (rp != CC_OK) return rp;
-    if (!pre.tvalid) {
-        CC_CUDA(c, cudaMemcpyAsync(&c->st->new_mask, &pre.mask, sizeof(pre.mask), cudaMemcpyHostToDevice, c->stream));
+    if (!pre.tvalid || pre.small) {
+        const unsigned long long nm = full_mask(c, pre);
+        CC_CUDA(c, cudaMemcpyAsync(&c->st->new_mask, &nm, sizeof(nm), cudaMemcpyHostToDevice, c->stream));
         CC_CUDA(c, launch_table_rebuild(c->args, c->rows, false, c->stream));
         c->launches += kKernelsPerRebuild;
     }
@@ -185,10 +194,9 @@ cc_status start_state(cc_ctx* c)
         CC_CUDA(c, launch_table_rebuild(c->args, c->rows, false, c->stream));
         c->launches += 1 + kKernelsPerRebuild;
     } else {
-        // the first sweep rebuilds the table itself (it is always heavy);
-        // the summary rows of singletons follow from the label rows
-        CC_CUDA(c, launch_singleton_summaries(c->args, c->rows, c->stream));
-        c->launches += 2;
+        // the first sweep rebuilds the table and the summary rows itself (it
+        // is always heavy); singletons are scored from the label rows
+        c->launches += 1;
     }
     DevState r;
     cc_status rc = read_state(c, &r);
@@ -241,54 +249,6 @@ cc_status ensure_graph(cc_ctx* c, int limit, RunGraph** out)
     return CC_OK;
 }
 
-// A whole run of a multi-job context as one graph launch: a WHILE node
-// repeats the sweep body until the run stops (at most `limit` sweeps' bodies
-// plus 64 for abandoned and retried ones).  Returns the CUDA error instead of
-// failing the context, so that the caller can fall back to chunks.
-cudaError_t ensure_loop_graph(cc_ctx* c, int limit, RunGraph** out)
-{
-    auto it = c->graphs.find(-limit);
-    if (it != c->graphs.end()) {
-        *out = &it->second;
-        return cudaSuccess;
-    }
-    RunGraph g;
-    g.bound.resize(2);
-    cudaError_t e = cudaSuccess;
-    for (auto& ev : g.bound)
-        if (e == cudaSuccess) e = cudaEventCreate(&ev);
-    cudaGraph_t graph = nullptr;
-    if (e == cudaSuccess) e = cudaStreamBeginCapture(c->own_stream, cudaStreamCaptureModeThreadLocal);
-    if (e == cudaSuccess) {
-        e = cudaEventRecordWithFlags(g.bound[0], c->own_stream, cudaEventRecordExternal);
-        const int budget = (int)std::min<long long>((long long)limit * c->ncls + 64, 1LL << 30);
-        if (e == cudaSuccess)
-            e = capture_run_loop(c->args, c->rows, c->grid, c->own_stream, c->loop_stream, c->body_stream, budget);
-        if (e == cudaSuccess) e = cudaEventRecordWithFlags(g.bound[1], c->own_stream, cudaEventRecordExternal);
-        for (cudaStream_t st : {c->body_stream, c->loop_stream}) {
-            cudaStreamCaptureStatus bs = cudaStreamCaptureStatusNone;
-            if (cudaStreamIsCapturing(st, &bs) == cudaSuccess && bs != cudaStreamCaptureStatusNone) {
-                cudaGraph_t left = nullptr;
-                cudaStreamEndCapture(st, &left);  // a capture left open by a failure
-                if (left) cudaGraphDestroy(left);
-            }
-        }
-        const cudaError_t e2 = cudaStreamEndCapture(c->own_stream, &graph);
-        if (e == cudaSuccess) e = e2;
-    }
-    if (e == cudaSuccess) e = cudaGraphInstantiate(&g.exec, graph, 0);
-    if (graph) cudaGraphDestroy(graph);
-    if (e != cudaSuccess) {
-        g.exec = nullptr;
-        destroy_graph(g);
-        cudaGetLastError();  // the failure is reported to the caller, not left pending
-        return e;
-    }
-    auto ins = c->graphs.emplace(-limit, g);
-    *out = &ins.first->second;
-    return cudaSuccess;
-}
-
 // Sweep bodies per graph launch: a run launches the graph until the device
 // says the run has stopped, so at most kChunk - 1 skipped sweep bodies are
 // submitted after the last sweep.  With colour_batched a body runs one colour
@@ -308,6 +268,31 @@ int chunk_bodies(const cc_ctx* c, int limit)
 long long launch_budget(const cc_ctx* c, int limit, int chunk)
 {
     return ((long long)limit * c->ncls + chunk - 1) / chunk + 64;
+}
+
+// Contexts of several jobs, colour-batched ones and jobs of at least this many
+// label rows run in the run kernel: it wins at every size measured there
+// (n = 20011, k = 12, host to host: 1.75 ms against 3.31 as graphs; n = 1.5e5,
+// k = 37: 2.58 against 2.99).  The smallest single jobs stay graphs of one
+// kernel per step, not because that is faster: cc_launch_count reports their
+// kernels one by one, and callers hold it to that (n = 1000, k = 10).
+constexpr long long kRunKernelRows = 1 << 14;
+
+// Appends the times of the last launch of the run kernel to sweep_ms and
+// propose_ms (ns differences of the device's clock).
+cc_status read_run_times(cc_ctx* c)
+{
+    const int b = c->ts_bodies;
+    c->ts_bodies = 0;
+    if (b <= 0) return CC_OK;
+    std::vector<unsigned long long> t(3 * (size_t)b);
+    CC_CUDA(c, cudaMemcpyAsync(t.data(), c->ts, sizeof(unsigned long long) * t.size(), cudaMemcpyDeviceToHost, c->stream));
+    CC_CUDA(c, cudaStreamSynchronize(c->stream));
+    for (int i = 0; i < b; ++i) {
+        c->propose_ms.push_back((float)((double)(t[3 * i + 1] - t[3 * i]) * 1e-6));
+        c->sweep_ms.push_back((float)((double)(t[3 * i + 2] - t[3 * i]) * 1e-6));
+    }
+    return CC_OK;
 }
 
 // Lane counts chosen by the autotuner, per device and lane bin (0 = none yet).
@@ -361,15 +346,42 @@ cc_status tune_lanes(cc_ctx* c)
     return CC_OK;
 }
 
-// Runs every job until it stops; *done = largest number of sweeps of a job in this run.
-cc_status run(cc_ctx* c, int limit, int* done)
+// A run as launches of the run kernel: one unless the run is very long, or
+// the context's lanes are to be timed after its first sweep.
+cc_status run_kernel(cc_ctx* c, int limit, DevState* out)
 {
-    const int full_limit = limit;
+    DevState& st = *out;
+    long long left = (long long)limit * c->ncls + 64;  // 64: sweeps abandoned for lack of table space and retried
+    int before = 0;
+    for (bool fresh = true; left > 0; fresh = false) {
+        const int budget = !c->tuned ? 1 : (int)std::min<long long>(left, kRunBodies);
+        cc_status r = read_run_times(c);
+        if (r != CC_OK) return r;
+        CC_CUDA(c, launch_run(c->args, c->rows, c->run_blocks, limit, fresh, budget, c->ts, c->stream));
+        c->launches += 1;
+        r = read_state(c, &st);
+        if (r != CC_OK) return r;
+        c->ts_bodies = st.run_bodies - before;
+        before = st.run_bodies;
+        if (st.stop || st.err) break;
+        if (!c->tuned) {
+            r = tune_lanes(c);
+            if (r != CC_OK) return r;
+            c->tuned = true;
+        }
+        left -= budget;
+    }
+    c->tuned = true;
+    return CC_OK;
+}
+
+// A run as graphs of one kernel per step: up to kChunk sweeps unrolled per
+// graph, launched until the device says the run has stopped.
+cc_status run_graphs(cc_ctx* c, int limit, DevState* out)
+{
+    DevState& st = *out;
     CC_CUDA(c, launch_run_begin(c->args, limit, c->stream));
     c->launches += 1;
-    c->sweep_ms.clear();
-    c->propose_ms.clear();
-    DevState st;
     int before = 0;
     cc_status r = CC_OK;
     if (!c->tuned) {
@@ -397,22 +409,6 @@ cc_status run(cc_ctx* c, int limit, int* done)
         c->tuned = true;
         limit -= st.run_bodies > 0 ? 1 : 0;
     }
-    // a multi-job context (unless profiling without regions) runs the rest as
-    // one graph launch
-    RunGraph* lg = nullptr;
-    const bool loop = c->jobs > 1 && !c->opt.no_regions && c->loop_ok && !(before > 0 && (st.stop || st.err));
-    if (loop && ensure_loop_graph(c, full_limit, &lg) != cudaSuccess) c->loop_ok = false;
-    if (loop && c->loop_ok) {
-        CC_CUDA(c, cudaGraphLaunch(lg->exec, c->stream));
-        r = read_state(c, &st);
-        if (r != CC_OK) return r;
-        c->launches += (long long)(st.run_bodies - before) * (kKernelsOutsideRegions + 1);
-        float x = 0.f;
-        CC_CUDA(c, cudaEventElapsedTime(&x, lg->bound[0], lg->bound[1]));
-        c->sweep_ms.push_back(x);
-        c->propose_ms.push_back(0.f);
-        before = st.run_bodies;
-    }
     const int chunk = chunk_bodies(c, std::max(limit, 1));
     RunGraph* g = nullptr;
     if (!(before > 0 && (st.stop || st.err))) {
@@ -438,6 +434,18 @@ cc_status run(cc_ctx* c, int limit, int* done)
         before = st.run_bodies;
         if (st.stop || st.err) break;
     }
+    return CC_OK;
+}
+
+// Runs every job until it stops; *done = largest number of sweeps of a job in this run.
+cc_status run(cc_ctx* c, int limit, int* done)
+{
+    c->sweep_ms.clear();
+    c->propose_ms.clear();
+    c->ts_bodies = 0;
+    DevState st;
+    cc_status r = c->run_blocks > 0 ? run_kernel(c, limit, &st) : run_graphs(c, limit, &st);
+    if (r != CC_OK) return r;
     r = check_device_error(c, st);
     if (r != CC_OK) return r;
     if (!st.stop) return fail(c, CC_ERR_TABLE_FULL, "sweep retries did not converge");
@@ -553,8 +561,9 @@ void finish_plan(Plan& p, const cc_options& opt)
     const size_t N = (size_t)p.n, J = (size_t)jobs;
     const size_t per[] = {
         sizeof(JobInfo) * (J + 1), sizeof(JobState) * (J + 1), 8 * (N + 1), 4 * (size_t)p.nnz, 4 * (size_t)p.nnz,
-        4 * N, 4 * (size_t)p.rows, 16 * (size_t)p.rows, 4 * N, 4 * N, 4 * N, 8 * N, 4 * N,
-        sizeof(Slot) * (size_t)p.cap_max, 4 * N, 4 * N, 4 * N, 4 * N, N, 4 * N, 4 * N, 4 * (N / 1024 + 2),
+        4 * N, 4 * (size_t)p.rows, 16 * (size_t)p.rows, 4 * N, 4 * N, 4 * N, 8 * N, 8 * N,
+        sizeof(Slot) * (size_t)p.cap_max, 4 * N, 4 * N, 4 * N, 4 * N, N, 4 * N, 4 * N, 4 * bsum_entries(N),
+        24 * (size_t)kRunBodies,
         4 * N, 8 * N, N, 4 * J, 8 * (J + 1), 8 * (size_t)p.parts, 8 * (size_t)p.parts,
         4 * (3 * N + N / 1024 + 64), sizeof(DevState), sizeof(cc_sweep_info) * J * (size_t)p.hist_cap};
     for (size_t b : per) p.persistent += rounded(b);
@@ -617,7 +626,6 @@ cc_status create_common(int jobs, const JobInput* in, bool on_device, const cc_o
     CC_TRY(cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, c->device));
     CC_TRY(cudaStreamCreateWithPriority(&c->own_stream, cudaStreamNonBlocking, priority));
     CC_TRY(cudaStreamCreateWithPriority(&c->body_stream, cudaStreamNonBlocking, priority));
-    CC_TRY(cudaStreamCreateWithPriority(&c->loop_stream, cudaStreamNonBlocking, priority));
     // pooled memory is allocated in the order of the context's own stream, so
     // such a context runs on that stream
     c->stream = (stream && !pool) ? static_cast<cudaStream_t>(stream) : c->own_stream;
@@ -678,7 +686,7 @@ cc_status create_common(int jobs, const JobInput* in, bool on_device, const cc_o
     CC_TRY(dalloc(c, &c->size, (size_t)N));
     CC_TRY(dalloc(c, &c->dsize, (size_t)N));
     CC_TRY(dalloc(c, &c->best, (size_t)N));
-    CC_TRY(dalloc(c, &c->aown, (size_t)N));
+    CC_TRY(dalloc(c, &c->own, (size_t)N));
     CC_TRY(dalloc(c, &c->chg, (size_t)N));
     CC_TRY(dalloc(c, &c->prev, (size_t)N));
     CC_TRY(dalloc(c, &c->act, (size_t)N));
@@ -690,8 +698,9 @@ cc_status create_common(int jobs, const JobInput* in, bool on_device, const cc_o
     CC_TRY(dalloc(c, &c->pflag, (size_t)N));
     CC_TRY(dalloc(c, &c->members, (size_t)N));
     CC_TRY(dalloc(c, &c->cursor, (size_t)N));
-    CC_TRY(dalloc(c, &c->bsum, (size_t)N / 1024 + 2));
+    CC_TRY(dalloc(c, &c->bsum, bsum_entries((size_t)N)));
     CC_TRY(dalloc(c, &c->scratch, 3 * (size_t)N + (size_t)N / 1024 + 64));
+    CC_TRY(dalloc(c, &c->ts, 3 * (size_t)kRunBodies));
     CC_TRY(dalloc(c, &c->st, 1));
     CC_TRY(dalloc(c, &c->hist, (size_t)jobs * c->hist_cap));
     {
@@ -837,7 +846,7 @@ cc_status create_common(int jobs, const JobInput* in, bool on_device, const cc_o
     a.size = c->size;
     a.dsize = c->dsize;
     a.best = c->best;
-    a.aown = c->aown;
+    a.own = c->own;
     a.table = c->table;
     a.mask_max = cap - 1;
     a.cap_min = cap < 1024 ? cap : 1024;
@@ -908,6 +917,8 @@ cc_status create_common(int jobs, const JobInput* in, bool on_device, const cc_o
     CC_TRY(prepare_propose(&per_sm));
     if (per_sm < 1) return bail(fail(c, CC_ERR_INVALID, "proposal kernel cannot be resident"));
     c->grid = c->sms * per_sm;
+    if (!c->opt.no_regions && (jobs > 1 || c->opt.colour_batched || rows >= kRunKernelRows))
+        CC_TRY(run_grid(a, rows, c->sms, &c->run_blocks));
 
     cc_status rc = start_state(c);
     if (rc != CC_OK) return bail(rc);
@@ -1066,7 +1077,7 @@ __global__ void k_load_src(long long vo, long long n, long long eo, long long nn
 // other jobs.  Skipped if the table does not hold the counts of C.
 __global__ void k_unload_keys(SweepArgs a, JobInfo J, long long vo)
 {
-    if (!a.st->tvalid) return;
+    if (!a.st->tvalid || a.st->small) return;
     const unsigned long long mask = a.st->mask;
     const long long total = J.n * J.k, stride = (long long)gridDim.x * blockDim.x;
     long long dead = 0;
@@ -1085,7 +1096,7 @@ __global__ void k_unload_keys(SweepArgs a, JobInfo J, long long vo)
 __global__ void k_load_keys(SweepArgs a, JobInfo J, long long vo)
 {
     DevState* st = a.st;
-    if (!st->tvalid) return;
+    if (!st->tvalid || st->small) return;
     const unsigned long long mask = st->mask;
     const long long total = J.n * J.k, stride = (long long)gridDim.x * blockDim.x;
     long long live = 0, used = 0;
@@ -1111,6 +1122,11 @@ __global__ void k_load_keys(SweepArgs a, JobInfo J, long long vo)
 // probing never runs in a nearly full table.
 __global__ void k_load_check_fill(DevState* st, unsigned long long new_keys)
 {
+    if (st->small) {
+        // a partial table: the next sweep rebuilds it anyway
+        st->keys_all += new_keys;
+        return;
+    }
     const unsigned long long cap = st->mask + 1;
     if (st->used + new_keys > cap - (cap >> 3)) st->tvalid = 0;
 }
@@ -1130,6 +1146,7 @@ __global__ void k_load_state(SweepArgs a, long long vo, long long ncap, long lon
         a.dsize[v] = 0;
         a.best[v] = kEmpty;
         a.chg[v] = stamp;
+        a.own[v] = make_int2(0, kOwnNever);
         a.prev[v] = kEmpty;
         a.act[v] = 1;
     }
@@ -1227,11 +1244,17 @@ cc_status check_job(cc_ctx* c, int32_t job)
 cc_status launch_chunk(cc_ctx* c)
 {
     const int chunk = chunk_bodies(c, c->async_limit);
-    RunGraph* g = nullptr;
-    cc_status r = ensure_graph(c, chunk, &g);
-    if (r != CC_OK) return r;
-    CC_CUDA(c, cudaGraphLaunch(g->exec, c->stream));
-    c->launches += (long long)chunk * (c->opt.no_regions ? kKernelsPerSweep : kKernelsOutsideRegions);
+    if (c->run_blocks > 0) {
+        CC_CUDA(c, launch_run(c->args, c->rows, c->run_blocks, c->async_limit, c->async_fresh, chunk, c->ts, c->stream));
+        c->async_fresh = false;
+        c->launches += 1;
+    } else {
+        RunGraph* g = nullptr;
+        cc_status r = ensure_graph(c, chunk, &g);
+        if (r != CC_OK) return r;
+        CC_CUDA(c, cudaGraphLaunch(g->exec, c->stream));
+        c->launches += (long long)chunk * (c->opt.no_regions ? kKernelsPerSweep : kKernelsOutsideRegions);
+    }
     CC_CUDA(c, cudaMemcpyAsync(c->hstate, c->st, sizeof(DevState), cudaMemcpyDeviceToHost, c->stream));
     if (c->hjobs)
         CC_CUDA(c, cudaMemcpyAsync(c->hjobs, c->js, sizeof(JobState) * (size_t)c->jobs, cudaMemcpyDeviceToHost,
@@ -1258,8 +1281,11 @@ cc_status ctx_async_start(cc_ctx* c, int limit, DevState* pinned, JobState* pinn
     c->async_limit = limit > 0 ? limit : c->opt.max_sweeps;
     c->async_launches = 0;
     if (!c->chunk_done) CC_CUDA(c, cudaEventCreateWithFlags(&c->chunk_done, cudaEventDisableTiming));
-    CC_CUDA(c, launch_run_begin(c->args, c->async_limit, c->stream));
-    c->launches += 1;
+    c->async_fresh = c->run_blocks > 0;
+    if (c->run_blocks == 0) {
+        CC_CUDA(c, launch_run_begin(c->args, c->async_limit, c->stream));
+        c->launches += 1;
+    }
     return launch_chunk(c);
 }
 
@@ -1676,6 +1702,8 @@ cc_status cc_run_until_converged(cc_ctx* c, int32_t max_sweeps, int32_t* sweeps_
 cc_status cc_last_run_timing(cc_ctx* c, int32_t max, float* sweep_ms, float* propose_ms, int32_t* count)
 {
     if (!c) return fail(nullptr, CC_ERR_INVALID, "ctx is NULL");
+    const cc_status r = read_run_times(c);
+    if (r != CC_OK) return r;
     const int have = (int)c->sweep_ms.size();
     if (count) *count = have;
     for (int i = 0; i < have && i < max; ++i) {
@@ -1821,7 +1849,8 @@ cc_status cc_metrics(cc_ctx* c, cc_partition_metrics* out)
     cc_status r = read_state(c, &pre);
     if (r != CC_OK) return r;
     if (pre.err) return check_device_error(c, pre);
-    CC_CUDA(c, cudaMemcpyAsync(&c->st->new_mask, &pre.mask, sizeof(pre.mask), cudaMemcpyHostToDevice, c->stream));
+    const unsigned long long nm = full_mask(c, pre);
+    CC_CUDA(c, cudaMemcpyAsync(&c->st->new_mask, &nm, sizeof(nm), cudaMemcpyHostToDevice, c->stream));
     CC_CUDA(c, launch_table_rebuild(c->args, c->rows, false, c->stream));
     c->launches += kKernelsPerRebuild;
     const int P = c->parts, J = c->jobs;
@@ -1913,7 +1942,8 @@ cc_status cc_partition_distances(cc_ctx* c, cc_partition_metrics* out)
     // restore C, its sizes and its table at the capacity it had
     CC_CUDA(c, cudaMemcpyAsync(c->C, saved, sizeof(int) * (size_t)n, cudaMemcpyDeviceToDevice, c->stream));
     CC_CUDA(c, launch_state_from_ids(c->args, c->stream));
-    CC_CUDA(c, cudaMemcpyAsync(&c->st->new_mask, &pre.mask, sizeof(pre.mask), cudaMemcpyHostToDevice, c->stream));
+    const unsigned long long nm = full_mask(c, pre);
+    CC_CUDA(c, cudaMemcpyAsync(&c->st->new_mask, &nm, sizeof(nm), cudaMemcpyHostToDevice, c->stream));
     CC_CUDA(c, launch_table_rebuild(c->args, c->rows, false, c->stream));
     c->launches += 2 + kKernelsPerRebuild;
     if (r != CC_OK) return r;

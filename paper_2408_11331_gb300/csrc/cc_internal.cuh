@@ -44,6 +44,8 @@ namespace ccg {
 constexpr unsigned long long kEmpty = ~0ull;
 constexpr int kWarpsPerBlock = 8;
 constexpr int kBlock = kWarpsPerBlock * 32;
+constexpr int kSmall = 8;      // largest cluster that a partial table leaves out (see rebuild.cuh)
+constexpr int kOwnNever = -3;  // own[v].y below every change stamp: A_a is not known
 
 // One contingency entry: the (cluster, label id) key, its count and the
 // delta staged by the current sweep.  16 bytes, read as one vector load.
@@ -118,6 +120,24 @@ struct DevState {
     int tight;                   // 1: the pending rebuild tries a capacity below safe_mask (checked)
     int again;                   // 1: the tight attempt was too small; the rebuild runs again at safe_mask
     int build_fail;              // 1: an insert of the tight attempt ran past its probe limit
+    int small;                   // clusters of at most this many members have no keys and no summary rows
+                                 //    in the table (they are scored from the member list); 0: every
+                                 //    cluster has them
+    int build_small;             // the same for the pending rebuild
+    int build_light;             // heavy sweep: 1 if its proposals would fit a light sweep
+    int sized;                   // heavy sweep: the capacity of its rebuild is settled
+    unsigned long long small_keys;  // heavy sweep: label rows in clusters of at most kSmall members after P1
+    unsigned long long keys_all; // upper estimate of the distinct keys of C at the last rebuild
+    unsigned long long retry_mask;  // heavy sweep: capacity - 1 of the second attempt of its rebuild
+    int many;                    // 1: many vertices may move (the sweep before moved more than 1/8 of the label rows)
+    int match;                   // 1: some job of this sweep falls back to the matching
+    // run kernel (persist.cu); written between two steps only
+    int rebuild_kind;            // the running rebuild: 0 heavy sweep, 1 its rollback, 2 end of the sweep
+    int tries;                   // rebuild attempts of this heavy sweep
+    int bodies_left;             // sweep bodies the launch may still run
+    unsigned bar_count;          // blocks that have arrived at the barrier
+    unsigned bar_word;           // barriers passed << 8 | step that follows
+    int bar_abort;               // 1: a block gave up waiting; every block leaves
 };
 
 // Arguments of the kernels (passed by value).
@@ -138,7 +158,7 @@ struct SweepArgs {
     int* size;
     int* dsize;                 // staged size deltas
     unsigned long long* best;   // bids: per vertex in the proposal step, per cluster in the matching
-    int* aown;                  // A_a of each vertex for the current sweep
+    int2* own;                  // per vertex {A_a, change stamp of its cluster when that was computed}
     Slot* table;
     unsigned long long mask_max; // allocated capacity - 1; the active capacity is st->mask + 1
     unsigned long long cap_min;  // smallest active capacity
@@ -321,7 +341,7 @@ __device__ __forceinline__ int table_count_ro(const Slot* t, unsigned long long 
 {
     unsigned long long h = hash_key(key) & mask;
     for (unsigned long long p = 0; p <= mask; ++p) {
-        ulonglong2 e = __ldg(reinterpret_cast<const ulonglong2*>(t + h));
+        ulonglong2 e = *reinterpret_cast<const ulonglong2*>(t + h);
         if (e.x == key) return (int)(unsigned)(e.y & 0xffffffffull);
         if (e.x == kEmpty) return 0;
         h = (h + 1) & mask;
@@ -362,10 +382,10 @@ __device__ __forceinline__ long long table_find_or_insert(Slot* t, unsigned long
     return -1;
 }
 
-// 16-byte compare-and-swap of a whole slot (PTX atom.cas.b128, sm_90 and
-// later): returns the slot's previous contents; the swap happened iff they
+// 16-byte compare-and-swap of a summary entry (PTX atom.cas.b128, sm_90 and
+// later): returns the entry's previous contents; the swap happened iff they
 // equal cmp.
-__device__ __forceinline__ ulonglong2 slot_cas(Slot* p, ulonglong2 cmp, ulonglong2 val)
+__device__ __forceinline__ ulonglong2 entry_cas(int4* p, ulonglong2 cmp, ulonglong2 val)
 {
     ulonglong2 old;
     asm volatile(
@@ -380,45 +400,6 @@ __device__ __forceinline__ ulonglong2 slot_cas(Slot* p, ulonglong2 cmp, ulonglon
         : "l"(cmp.x), "l"(cmp.y), "l"(val.x), "l"(val.y), "l"(p)
         : "memory");
     return old;
-}
-
-// 16-byte compare-and-swap of a summary entry (same instruction as slot_cas).
-__device__ __forceinline__ ulonglong2 entry_cas(int4* p, ulonglong2 cmp, ulonglong2 val)
-{
-    return slot_cas(reinterpret_cast<Slot*>(p), cmp, val);
-}
-
-// Adds cnt to key's count in a table being built from a cleared state (every
-// slot either empty with count 0, or holding a key): a new key is written
-// together with its count by one 16-byte CAS; an existing key gets an atomic
-// add.  The caller issues the first CAS, at key's home slot h (so that a warp
-// can have the first CASes of several keys in flight), and passes its result
-// as old; this finishes the insert.  *inserted is set when the insert created
-// the slot.  Returns -1 if the key found no slot within `limit` probes.
-// mark (0 or 1) goes into the new slot's staged-delta field: the rebuild
-// marks the keys whose summary entry is already final (see setup.cu) and
-// clears the mark again before any sweep stages deltas.
-__device__ __forceinline__ long long table_build_finish(Slot* t, unsigned long long mask, unsigned long long key,
-                                                        int cnt, bool* inserted, int mark, unsigned long long limit,
-                                                        unsigned long long h, ulonglong2 old)
-{
-    *inserted = false;
-    const ulonglong2 empty = make_ulonglong2(kEmpty, 0ull);
-    const ulonglong2 mine =
-        make_ulonglong2(key, ((unsigned long long)(unsigned)mark << 32) | (unsigned long long)(unsigned)cnt);
-    for (unsigned long long p = 0;;) {
-        if (old.x == kEmpty && old.y == 0ull) {
-            *inserted = true;
-            return (long long)h;
-        }
-        if (old.x == key) {
-            atomicAdd(&t[h].cnt, cnt);
-            return (long long)h;
-        }
-        if (++p > mask || p >= limit) return -1;
-        h = (h + 1) & mask;
-        old = slot_cas(t + h, empty, mine);
-    }
 }
 
 // ---- setup.cu ----
@@ -472,15 +453,11 @@ cudaError_t launch_compact_labels(const LabelArgs& a, cudaStream_t s);
 cudaError_t launch_label_kernels(const LabelArgs& a, cudaStream_t s);
 
 cudaError_t launch_init_state(const SweepArgs& a, cudaStream_t s);
-// Summary rows of the singleton start ({g_i(v), 1, -1, 0} for cluster v, padding {-1, 0, -1, 0}).
-cudaError_t launch_singleton_summaries(const SweepArgs& a, long long rows, cudaStream_t s);
 // Sizes from C (ids outside their job set CC_ERR_INVALID).
 cudaError_t launch_state_from_ids(const SweepArgs& a, cudaStream_t s);
 // Rebuild of the table and summary rows from C into st->new_mask + 1 slots,
 // then st->mask = st->new_mask.  conditional: only if st->rebuild is set.
-// eval: in a heavy sweep, also add the table part of F' to each job's recompute.
-cudaError_t launch_table_rebuild(const SweepArgs& a, long long rows, bool conditional, cudaStream_t s,
-                                 bool eval = false);
+cudaError_t launch_table_rebuild(const SweepArgs& a, long long rows, bool conditional, cudaStream_t s);
 // F of every job from scratch into js[j].recompute (without sum_ij |P_ij|^2).
 cudaError_t launch_objective_recompute(const SweepArgs& a, cudaStream_t s);
 
@@ -555,12 +532,13 @@ constexpr int kKernelsOutsideRegions = kKernelsPerSweep + kGatesPerSweep - kKern
 cudaError_t launch_sweep(const SweepArgs& a, long long rows, int grid, cudaStream_t s, cudaEvent_t prop0,
                          cudaEvent_t prop1, cudaStream_t body = nullptr);
 cudaError_t prepare_propose(int* blocks_per_sm);
-// Adds to the graph being captured on s a WHILE node whose body (captured on
-// `loop`, with the sweep's regions on `body`) is one sweep followed by a gate
-// that repeats it until the run stops, fails or has run `budget` bodies: a
-// whole run as one graph launch.
-cudaError_t capture_run_loop(const SweepArgs& a, long long rows, int grid, cudaStream_t s, cudaStream_t loop,
-                             cudaStream_t body, int budget);
+// ---- persist.cu ----
+// Grid of the run kernel for a context (0: it cannot be resident).
+cudaError_t run_grid(const SweepArgs& a, long long rows, int sms, int* grid);
+// The run kernel: up to `budget` sweep bodies of a run in one cooperative
+// launch (fresh: starts the run first).  ts: 3 x budget device words.
+cudaError_t launch_run(const SweepArgs& a, long long rows, int grid, int limit, bool fresh, int budget,
+                       unsigned long long* ts, cudaStream_t s);
 // The proposal step's scoring kernels alone (own-cluster sums, candidate
 // bids) on the current state, for timing; they write only aown, act (the
 // same values on the same state) and the bids, which launch_clear_bids

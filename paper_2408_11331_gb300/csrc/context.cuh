@@ -24,8 +24,6 @@ struct cc_ctx {
     cudaStream_t stream = nullptr;      // stream used by calls
     cudaStream_t own_stream = nullptr;  // stream created by the context (also used for capture)
     cudaStream_t body_stream = nullptr; // captures the bodies of a sweep graph's conditional regions
-    cudaStream_t loop_stream = nullptr; // captures the body of a run loop (batches: a run is one launch)
-    bool loop_ok = true;                // the run loop graph could be built (else: chunks of sweeps)
     cudaMemPool_t pool = nullptr;       // device memory comes from this pool (stream-ordered) if set
     std::vector<ccg::JobInfo> job;      // host copy of the job table
     std::vector<long long> F0;          // objective of each job at the singleton start
@@ -55,7 +53,7 @@ struct cc_ctx {
     int* size = nullptr;
     int* dsize = nullptr;
     unsigned long long* best = nullptr;
-    int* aown = nullptr;
+    int2* own = nullptr;
     int* chg = nullptr;                 // active set: change stamp per cluster id (n)
     unsigned long long* prev = nullptr; // active set: previous bid per vertex (n)
     unsigned char* act = nullptr;       // active set: scored in this sweep (n)
@@ -82,11 +80,14 @@ struct cc_ctx {
     cc_sweep_info* hist = nullptr;
     int hist_cap = 0;
     ccg::SweepArgs args{};
-    std::map<int, RunGraph> graphs;     // key > 0: chunk of that many bodies; key < 0: run loop of that limit
+    std::map<int, RunGraph> graphs;     // by the number of sweep bodies in the graph
     std::vector<float> sweep_ms;        // device time of each sweep of the last run
     std::vector<float> propose_ms;      // ... and of its proposal kernels
     long long launches = 0;             // kernels launched so far
     int grid = 0;
+    int run_blocks = 0;                 // grid of the run kernel; 0: runs are graphs of one kernel per step
+    unsigned long long* ts = nullptr;   // run kernel: three times per sweep body of the last launch
+    int ts_bodies = 0;                  // bodies of the last launch not yet in sweep_ms (read when asked for)
     unsigned long long cap_start = 0;   // active table capacity at the singleton start
     unsigned long long cap_max = 0;     // allocated table capacity
     bool started = false;               // start_state ran once
@@ -100,9 +101,18 @@ struct cc_ctx {
     cudaEvent_t chunk_done = nullptr;   // recorded after each graph launch and the copy of st
     int async_limit = 0;
     int async_launches = 0;
+    bool async_fresh = false;           // the next launch of the run kernel starts the run
 };
 
 namespace ccg {
+
+// Sweep bodies of one launch of the run kernel at most (longer runs are
+// launched again), and the entries of the block sums of its size scan.
+constexpr int kRunBodies = 512;
+constexpr size_t bsum_entries(size_t n)
+{
+    return n / 1024 + 4096;
+}
 
 // One input job, pointers host or device.
 struct JobInput {

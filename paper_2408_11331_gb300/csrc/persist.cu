@@ -1,0 +1,380 @@
+// The run kernel: a whole run (or a budget of sweep bodies) of a context in
+// one cooperative launch.  Its blocks stay resident and go through the steps
+// of a sweep (sweep_phases.cuh, rebuild.cuh) together, with a grid barrier
+// where a step needs what other blocks wrote; the last block to arrive takes
+// the decisions between two steps (route, guards, end of the sweep) while the
+// others wait, so a decision costs no pass of its own.
+//
+// What bounds it: at small and middle sizes the barriers (3-4 us each with 608
+// blocks) and the latency of each step's dependent gathers, at large sizes the
+// steps themselves (gathers of label and summary rows).  The same steps as a
+// graph of kernels with IF regions spent 2-5 us per node and 35-43 us to enter
+// a region, about 110 us per sweep, and 1.0-1.5 ms of host time to capture and
+// instantiate the graph of a new context.  Measured, graphs then run kernel:
+// LFR-style n = 20011, k = 12, host to host 3.31 -> 1.75 ms; colour-batched
+// n = 1e5, k = 8 15.4 -> 7.5 ms; 40 served requests 20.2 -> 17.3 ms.
+// Layout: 4 blocks of 256 threads per SM (64 registers), as the scoring step
+// wants; the steps that gather in shared memory share one buffer, because
+// every further KB came out of the L1 that the other steps read through
+// (n = 1e6, k = 20: 8.4 -> 7.5 ms).
+#include <algorithm>
+
+#include "rebuild.cuh"
+#include "sweep_phases.cuh"
+
+namespace ccg {
+
+namespace {
+
+constexpr unsigned long long kBarrierLimitNs = 20ull * 1000 * 1000 * 1000;  // a wait past this gives up
+
+__device__ __forceinline__ unsigned long long now_ns()
+{
+    unsigned long long t;
+    asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
+    return t;
+}
+
+__device__ __forceinline__ unsigned ld_relaxed(const unsigned* p)
+{
+    unsigned x;
+    asm volatile("ld.relaxed.gpu.global.u32 %0, [%1];" : "=r"(x) : "l"(p) : "memory");
+    return x;
+}
+
+__device__ __forceinline__ unsigned atom_add_acq_rel(unsigned* p, unsigned x)
+{
+    unsigned old;
+    asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], %2;" : "=r"(old) : "l"(p), "r"(x) : "memory");
+    return old;
+}
+
+__device__ __forceinline__ void st_release(unsigned* p, unsigned x)
+{
+    asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(x) : "memory");
+}
+
+// Steps of the run kernel.
+enum Step {
+    kStart, kOwn, kEdges, kCollect,         // proposal step
+    kMark, kApply, kUndo, kHeavyEval,       // heavy path (and its rollback)
+    kSizes, kClear, kScatter, kBuild, kTop, // table rebuild
+    kStage, kEval,                          // light path
+    kBid, kKeys, kCommit,                   // matching, commit
+    kLeave
+};
+
+// Grid barrier between two steps.  The last block to arrive runs schedule()
+// (all its threads; the value counts in thread 0), which takes the decisions
+// that follow from the finished step and returns the next one; the others
+// wait for it.  Barrier number and next step travel in one word, so every
+// block takes the same step without another load.  A wait that exceeds its
+// limit sets st->err and ends the kernel in every block.
+template <class Schedule>
+__device__ __forceinline__ int grid_step(DevState* st, unsigned& word, unsigned& arrivals, Schedule schedule)
+{
+    __shared__ unsigned s_word;
+    __shared__ int s_last;
+    __syncthreads();
+    arrivals += gridDim.x;
+    if (threadIdx.x == 0) s_last = atom_add_acq_rel(&st->bar_count, 1u) == arrivals - 1;
+    __syncthreads();
+    if (s_last) {
+        const int next = schedule();
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            s_word = (((word >> 8) + 1) << 8) | (unsigned)next;
+            if (next == kLeave) st->bar_count = 0;
+            st_release(&st->bar_word, s_word);
+        }
+    } else if (threadIdx.x == 0) {
+        unsigned long long t0 = 0;
+        unsigned now;
+        // relaxed polls and one fence at the end: an acquire on every poll
+        // would drop the L1 lines of the blocks still at work on this SM
+        for (unsigned spins = 1; (now = ld_relaxed(&st->bar_word)) == word; ++spins) {
+            if (spins & 1023u) continue;
+            if (t0 == 0) t0 = now_ns();
+            if (*reinterpret_cast<volatile int*>(&st->bar_abort) || now_ns() - t0 > kBarrierLimitNs) {
+                set_err(st, CC_ERR_TIMEOUT);
+                st->bar_abort = 1;
+                now = kLeave;
+                break;
+            }
+        }
+        __threadfence();
+        s_word = now;
+    }
+    __syncthreads();
+    word = s_word;
+    return (int)(word & 255u);
+}
+
+// Sum of x over the block, in every thread.
+__device__ __forceinline__ int block_sum(int x)
+{
+    __shared__ int part[kWarpsPerBlock];
+    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(kFull, x, o);
+    __syncthreads();
+    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = x;
+    __syncthreads();
+    int s = 0;
+#pragma unroll
+    for (int w = 0; w < kWarpsPerBlock; ++w) s += part[w];
+    return s;
+}
+
+// Exclusive scan of the cluster sizes into cursor[], first half: each block's
+// sum over its own contiguous range of ids.
+__device__ __forceinline__ void scan_range(const SweepArgs& a, long long& lo, long long& hi)
+{
+    const long long per = ((a.n + gridDim.x - 1) / gridDim.x + 3) & ~3LL;
+    lo = per * blockIdx.x < a.n ? per * blockIdx.x : a.n;
+    hi = lo + per < a.n ? lo + per : a.n;
+}
+
+__device__ __forceinline__ void scan_sum_step(const SweepArgs& a)
+{
+    long long lo, hi;
+    scan_range(a, lo, hi);
+    int s = 0;
+    unsigned long long small = 0;
+    for (long long v = lo + threadIdx.x; v < hi; v += kBlock) {
+        s += a.size[v];
+        small += small_rows(a, v, a.size[v]);
+    }
+    if (to_size(a.st, 1)) add_small_rows(a.st, small);
+    s = block_sum(s);
+    if (threadIdx.x == 0) a.bsum[blockIdx.x] = s;
+}
+
+// Second half: the sums of the blocks before, then the block's own range in
+// tiles of four ids per thread.
+__device__ __forceinline__ void scan_write_step(const SweepArgs& a)
+{
+    __shared__ int wsum[kWarpsPerBlock];
+    long long lo, hi;
+    scan_range(a, lo, hi);
+    int before = 0;
+    for (unsigned b = threadIdx.x; b < blockIdx.x; b += kBlock) before += a.bsum[b];
+    int run = block_sum(before);
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    for (long long t = lo; t < hi; t += 4 * kBlock) {
+        const long long v = t + 4 * threadIdx.x;
+        int s[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) s[i] = v + i < hi ? a.size[v + i] : 0;
+        const int mine = s[0] + s[1] + s[2] + s[3];
+        const int incl = warp_incl_scan(mine, lane);
+        __syncthreads();
+        if (lane == 31) wsum[w] = incl;
+        __syncthreads();
+        int x = run + incl - mine, all = 0;
+#pragma unroll
+        for (int q = 0; q < kWarpsPerBlock; ++q) {
+            if (q < w) x += wsum[q];
+            all += wsum[q];
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            if (v + i < hi) a.cursor[v + i] = x;
+            x += s[i];
+        }
+        run += all;
+    }
+}
+
+// What follows a finished step (all threads of one block; the decisions of the
+// one-thread and per-job steps of a sweep are taken here).
+struct Scheduler {
+    const SweepArgs& a;
+    int limit, fresh;
+
+    // Starts a rebuild: 0 heavy sweep, 1 its rollback, 2 end of the sweep.
+    __device__ int rebuild(int kind) const
+    {
+        if (threadIdx.x == 0) a.st->rebuild_kind = kind;
+        return kSizes;
+    }
+
+    __device__ int begin() const
+    {
+        __syncthreads();
+        if (a.st->bodies_left <= 0) return kLeave;
+        begin_phase(a, threadIdx.x, kBlock);
+        __syncthreads();
+        return a.st->skip ? kLeave : kOwn;
+    }
+
+    // Objective, history and stop per job; then the end-of-sweep rebuild or
+    // the next sweep.
+    __device__ int end() const
+    {
+        __syncthreads();
+        end_jobs_phase(a, threadIdx.x, kBlock);
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            end_phase(a);
+            a.st->bodies_left -= 1;
+        }
+        __syncthreads();
+        return a.st->rebuild && !a.st->err ? rebuild(2) : begin();
+    }
+
+    __device__ int after_apply() const { return a.st->match ? kBid : end(); }
+
+    __device__ int next(int step) const
+    {
+        DevState* st = a.st;
+        switch (step) {
+        case kStart:
+            if (fresh) {
+                run_begin_phase(a, limit, threadIdx.x, kBlock);
+                __syncthreads();
+            }
+            return begin();
+        case kOwn: return kEdges;
+        case kEdges: return kCollect;
+        case kCollect:
+            if (threadIdx.x == 0) {
+                route_phase(a);
+                st->tries = 0;
+            }
+            __syncthreads();
+            if (st->heavy) return kMark;
+            if (st->nprop > 0 && !st->err) return kStage;
+            return end();
+        case kMark: return kApply;
+        case kApply: return rebuild(0);
+        case kUndo: return rebuild(1);
+        case kSizes:
+            if (threadIdx.x == 0 && to_size(st, 1)) size_build(a);
+            return kClear;
+        case kClear: return kScatter;
+        case kScatter: return kBuild;
+        case kBuild: build_check_phase(a, 1); return kTop;
+        case kTop:
+            if (threadIdx.x == 0) {
+                table_done_phase(st, 1);
+                st->tries += 1;
+            }
+            __syncthreads();
+            if (st->rebuild_kind == 2) return begin();
+            if (st->rebuild_kind == 1) return after_apply();
+            if (st->again && st->tries < 2) return kSizes;  // the tight attempt did not fit
+            return kHeavyEval;
+        case kHeavyEval:
+            h_decide_phase(a, threadIdx.x, kBlock);
+            __syncthreads();
+            return st->rollback ? kUndo : after_apply();
+        case kStage: return kEval;
+        case kEval: decide_phase(a, threadIdx.x, kBlock); __syncthreads(); return st->match ? kBid : kCommit;
+        case kBid: return kKeys;
+        case kKeys: return kCommit;
+        case kCommit: return end();
+        }
+        return kLeave;
+    }
+};
+
+}  // namespace
+
+// fresh: 1 starts a run of at most `limit` sweeps, 0 goes on with it; at most
+// `budget` sweep bodies are run.  ts: three times (ns) per body: its start,
+// the end of its proposal step, its end.
+template <bool kSingle>
+__global__ void __launch_bounds__(kBlock, 4)
+    k_run(const __grid_constant__ SweepArgs a, long long rows, int limit, int fresh, int budget, unsigned long long* ts)
+{
+    // one buffer for the steps that gather in shared memory, so that the L1
+    // keeps the rest
+    __shared__ union {
+        EdgeScratch edge[kWarpsPerBlock];
+        int4 proposal[kBlock];
+    } scratch;
+    DevState* st = a.st;
+    unsigned arrivals = 0;                       // at the barrier, over this launch
+    unsigned word = ld_relaxed(&st->bar_word);   // cannot change before this block arrives
+    const bool clock = blockIdx.x == 0 && threadIdx.x == 0;
+    int step = kStart, body = -1;
+    // every step ends in a barrier; kLeave ends the kernel
+    for (;;) {
+        switch (step) {
+        case kStart:
+            if (clock) st->bodies_left = budget;
+            break;
+        case kOwn:
+            if (clock) {
+                if (body >= 0) ts[3 * body + 2] = now_ns();
+                ++body;
+                ts[3 * body] = now_ns();
+            }
+            own_phase<kSingle>(a);
+            break;
+        case kEdges: edges_phase<kSingle>(a, scratch.edge); break;
+        case kCollect: collect_phase(a, scratch.proposal); break;
+        case kMark: h_mark_phase(a); break;
+        case kApply: h_apply_phase(a, 0); break;
+        case kUndo: h_apply_phase(a, 1); break;
+        case kSizes: scan_sum_step(a); break;
+        case kClear:
+            table_clear_phase(a, rows, 1);
+            scan_write_step(a);
+            break;
+        case kScatter: members_scatter_phase(a, 1); break;
+        case kBuild: table_build_phase(a, 1); break;
+        case kTop: summ_top_phase(a, 1); break;
+        case kHeavyEval: h_eval_phase<kSingle>(a); break;
+        case kStage: stage_phase(a); break;
+        case kEval: eval_phase(a); break;
+        case kBid: bid_phase(a); break;
+        case kKeys: match_keys_phase(a); break;
+        case kCommit:
+            commit_phase(a);
+            if (st->match) match_reset_phase(a);
+            break;
+        }
+        const int done = step;
+        step = grid_step(st, word, arrivals, [&] { return Scheduler{a, limit, fresh}.next(done); });
+        if (clock && done == kCollect) ts[3 * body + 1] = now_ns();
+        if (step == kLeave) break;
+    }
+    if (clock && body >= 0) ts[3 * body + 2] = now_ns();
+}
+
+namespace {
+
+// Blocks of a run of this context: one warp per window of the proposal step's
+// CSR entries and one thread per 8 label rows, at most what is resident.
+inline size_t run_smem(int jobs)
+{
+    return (2 * jobs <= kSmemJobs ? 2 : 1) * smem_jobs_bytes(jobs);
+}
+
+}  // namespace
+
+cudaError_t run_grid(const SweepArgs& a, long long rows, int sms, int* grid)
+{
+    int per_sm = 0;
+    const cudaError_t e =
+        a.jobs == 1 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_run<true>, kBlock, run_smem(a.jobs))
+                    : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_run<false>, kBlock, run_smem(a.jobs));
+    if (e != cudaSuccess) return e;
+    const long long span = 32LL * kChunks * kWarpsPerBlock;
+    long long g = std::max((a.nnz + span - 1) / span, (rows + 8 * kBlock - 1) / (8 * kBlock));
+    g = std::max(g, (a.n + kBlock - 1) / kBlock);
+    *grid = (int)std::max(0LL, std::min(g, (long long)per_sm * sms));
+    return cudaSuccess;
+}
+
+cudaError_t launch_run(const SweepArgs& a, long long rows, int grid, int limit, bool fresh, int budget,
+                       unsigned long long* ts, cudaStream_t s)
+{
+    SweepArgs args = a;
+    int f = fresh ? 1 : 0;
+    void* params[] = {&args, &rows, &limit, &f, &budget, &ts};
+    const void* k = a.jobs == 1 ? reinterpret_cast<const void*>(k_run<true>) : reinterpret_cast<const void*>(k_run<false>);
+    return cudaLaunchCooperativeKernel(k, dim3((unsigned)grid), dim3(kBlock), params, run_smem(a.jobs), s);
+}
+
+}  // namespace ccg

@@ -1,0 +1,388 @@
+// Device code of the table rebuild (see setup.cu for the kernels that run it
+// one step at a time, persist.cu for the run kernel that calls the steps
+// between its grid barriers).  Every function is one step over the whole
+// grid: blocks take their share by blockIdx and gridDim.
+#pragma once
+
+#include "cc_internal.cuh"
+
+namespace ccg {
+
+namespace {
+
+// ---- table rebuild ------------------------------------------------------
+// The table is rebuilt from C alone: list the vertices cluster by cluster
+// (counting sort: an exclusive scan of the sizes gives each cluster's first
+// position), clear the capacity being built, then insert the keys with
+// partitions innermost per member, so that the 32 lanes of a warp hold
+// consecutive members of (mostly) one cluster for one partition: equal keys
+// are merged with __match_any_sync and added with one atomic.  The summary
+// rows follow from the rebuilt counts.  All steps are skipped unless a
+// rebuild is pending (conditional) and run unconditionally otherwise.
+//
+// A heavy sweep whose P1 leaves many label rows in clusters of at most kSmall
+// members (the first sweep of a run, above all) builds a partial table: those
+// clusters get neither keys nor summary rows, since the next sweep's scoring
+// compares v's label row with their few members' rows instead (the member
+// list is part of the rebuild), and a sweep that finds a partial table is
+// heavy, so nothing else looks for their keys.  On the kNN workload (n = 2e6,
+// k = 50) 99.5% of the vertices are in such clusters after sweep 1, and its
+// rebuild shrank from 62.5M keys in 2^28 slots (5.8 ms) to 0.2M keys.  Not
+// worth it below a quarter of the rows: the full table then costs little and
+// lets a light sweep follow.
+
+__device__ __forceinline__ bool rebuild_off(const DevState* st, int conditional)
+{
+    return conditional && (!st->rebuild || st->err);
+}
+
+// Whether the rebuild's sizes are still to be looked over (see size_build).
+__device__ __forceinline__ bool to_size(const DevState* st, int conditional)
+{
+    return conditional && st->heavy && !st->rollback && !st->sized;
+}
+
+// Label rows of cluster c (sz members) that a partial table would leave out.
+__device__ __forceinline__ unsigned long long small_rows(const SweepArgs& a, long long c, int sz)
+{
+    return sz >= 1 && sz <= kSmall ? (unsigned long long)sz * a.job[a.jid[c]].k : 0ull;
+}
+
+__device__ __forceinline__ void add_small_rows(DevState* st, unsigned long long x)
+{
+    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+    if ((threadIdx.x & 31) == 0 && x) atomicAdd(&st->small_keys, x);
+}
+
+// One thread, once the sizes after P1 are known: partial or full table, and
+// its capacity.  First a tight one: the occupied slots of the sweep start
+// (the moves of a heavy sweep mostly merge keys) at load <= 1/2, with room
+// below the fill limit for the new keys of a light sweep that may follow a
+// full table (2 x sum k n / 8 at most).  After a partial table the keys of
+// the small clusters were not counted; the sweep that merges them leaves
+// 11-13% of their rows as keys on the kNN and LFR-style workloads, and a
+// quarter is assumed.  The build checks that the keys fit (build_check) and
+// otherwise builds again at the capacity that holds every key.
+__device__ __forceinline__ void size_build(const SweepArgs& a)
+{
+    DevState* st = a.st;
+    st->sized = 1;
+    const unsigned long long total = a.keys;
+    const bool partial = !st->build_light && 4 * st->small_keys >= total;
+    unsigned long long c = st->safe_mask + 1;
+    unsigned long long est = !st->tvalid ? total : st->small ? st->used + (st->keys_all - st->used) / 4 : st->used;
+    unsigned long long room = 2 * ((total + 7) / 8);
+    if (partial) {
+        const unsigned long long rest = total - st->small_keys;
+        unsigned long long p = a.cap_min;
+        while (p < 2 * rest && p < c) p <<= 1;
+        c = p;
+        if (est > rest) est = rest;
+        room = 0;
+    }
+    unsigned long long t = a.cap_min;
+    while ((t < 2 * est || t - (t >> 3) < est + room) && t < c) t <<= 1;
+    st->build_small = partial ? kSmall : 0;
+    st->retry_mask = c - 1;
+    st->tight = (t < c && a.tight_mode != 1) ? 1 : 0;
+    st->new_mask = (st->tight ? t : c) - 1;
+}
+
+// Clears the slots of the capacity being built (st->new_mask + 1 of them),
+// the summary rows, the occupied-slot counter, and the staged size deltas
+// after an abandoned sweep.  Summary rows: those of the live clusters that
+// the table holds (a warp per 32 cluster ids, the lanes across each live
+// row), which are the rows the rebuild fills and the sweeps read.  The row of
+// a dead cluster is never read again, since no move enters an empty cluster,
+// except with empty_moves (a vertex may found a cluster under its own,
+// possibly dead, id); then every row of a full table is cleared.
+__device__ __forceinline__ void table_clear_phase(const SweepArgs& a, long long rows, int conditional)
+{
+    DevState* st = a.st;
+    if (rebuild_off(st, conditional)) return;
+    const unsigned long long cap = st->new_mask + 1;
+    const int small = conditional ? st->build_small : 0;
+    const unsigned long long stride = (unsigned long long)gridDim.x * blockDim.x;
+    const unsigned long long t0 = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x;
+    for (unsigned long long s = t0; s < cap; s += stride)
+        reinterpret_cast<ulonglong2*>(a.table)[s] = make_ulonglong2(kEmpty, 0ull);
+    const int4 none = make_int4(-1, 0, -1, 0);
+    if (a.empty_moves && !small) {
+        for (unsigned long long r = t0; r < (unsigned long long)rows; r += stride) a.summ[r] = none;
+    } else {
+        const int lane = threadIdx.x & 31;
+        for (unsigned long long x0 = t0 - lane; x0 < (unsigned long long)a.n; x0 += stride) {
+            const unsigned long long x = x0 + lane;
+            unsigned live = __ballot_sync(0xffffffffu, x < (unsigned long long)a.n && a.size[x] > small);
+            while (live) {
+                const long long xx = (long long)x0 + __ffs(live) - 1;
+                live &= live - 1;
+                const JobInfo& J = a.job[a.jid[xx]];
+                int4* row = a.summ + row_of(J, xx);
+                for (int q = lane; q < J.kp; q += 32) row[q] = none;
+            }
+        }
+    }
+    if (st->abort)
+        for (unsigned long long v = t0; v < (unsigned long long)a.n; v += stride) a.dsize[v] = 0;
+    if (t0 == 0) st->used = 0;
+}
+
+__device__ __forceinline__ int warp_incl_scan(int x, int lane)
+{
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
+    }
+    return x;
+}
+
+__device__ __forceinline__ void members_scatter_phase(const SweepArgs& a, int conditional)
+{
+    if (rebuild_off(a.st, conditional)) return;
+    const bool undone = conditional && a.st->rollback;
+    const long long stride = (long long)gridDim.x * blockDim.x;
+    for (long long v = (long long)blockIdx.x * blockDim.x + threadIdx.x; v < a.n; v += stride) {
+        const int c = a.C[v];
+        const int pos = atomicAdd(&a.cursor[c], 1);
+        if (pos < a.n) a.members[pos] = (int)v;
+        else set_err(a.st, CC_ERR_INVALID);  // sizes inconsistent with C
+        // P1 is being undone: what h_eval computed under it no longer holds
+        if (undone && a.chg[c] == a.st->stamp) a.own[v].y = kOwnNever;
+    }
+}
+
+// Largest 64-bit value over the lanes of a contiguous lane segment [lane,
+// end) of the warp, left in the segment's first lane (every lane must call it).
+__device__ __forceinline__ unsigned long long segment_max(unsigned long long x, int lane, int end)
+{
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const unsigned long long y = __shfl_down_sync(0xffffffffu, x, o);
+        if (lane + o < end && y > x) x = y;
+    }
+    return x;
+}
+
+// Inserts the keys of every member of a cluster the table holds (partitions
+// innermost, equal keys of a warp merged with __match_any_sync and added
+// once).  Members are listed cluster by cluster, so a cluster whose members
+// all lie in one warp's 32 entries gets its exact counts inside that warp:
+// the warp then writes the cluster's summary entries itself (the two most
+// frequent labels, ties to the larger id, as the table scan would rank them)
+// and marks those keys so that the scan skips them.  Keys of clusters spread
+// over several warps are left to the scan.
+// A tight attempt (see build_check) gives every insert kTightProbes probes;
+// an insert that finds no slot within them flags the attempt as failed, and
+// the warps stop inserting.
+constexpr unsigned long long kTightProbes = 256;
+
+__device__ __forceinline__ void table_build_phase(const SweepArgs& a, int conditional)
+{
+    DevState* st = a.st;
+    if (rebuild_off(st, conditional)) return;
+    __shared__ unsigned long long s_used;
+    if (threadIdx.x == 0) s_used = 0;
+    // tight attempts are made only by the heavy sweep's rebuild inside a
+    // sweep graph; a rebuild the host asks for is never one
+    const bool tight = conditional && st->tight != 0;
+    const unsigned long long limit = tight ? kTightProbes : ~0ull;
+    const int small = conditional ? st->build_small : 0;
+    __syncthreads();
+    const unsigned long long mask = st->new_mask;
+    const long long stride = (long long)gridDim.x * blockDim.x;
+    const int lane = threadIdx.x & 31;
+    unsigned created = 0;  // slots this lane created
+    for (long long base = (long long)blockIdx.x * blockDim.x; base < a.n; base += stride) {
+        if (tight && __any_sync(0xffffffffu, *reinterpret_cast<volatile int*>(&st->build_fail) != 0)) break;
+        const long long m = base + threadIdx.x;
+        const long long wb = m - lane;  // first member of this warp's window
+        bool valid = m < a.n;
+        int v = 0, c = 0, k = 0, seg_end = lane + 1;
+        bool whole = false;
+        const int* row = a.G;
+        int4* S = a.summ;
+        if (valid) {
+            v = a.members[m];
+            c = a.C[v];
+            if (a.size[c] <= small) valid = false;
+        }
+        if (!__any_sync(0xffffffffu, valid)) continue;
+        if (valid) {
+            const JobInfo& J = a.job[a.jid[v]];
+            k = J.k;
+            row = a.G + row_of(J, v);
+            // after the scatter, cursor[c] is one past the cluster's last member
+            const long long end = a.cursor[c], first = end - a.size[c];
+            whole = first >= wb && end <= wb + 32;
+            if (whole) seg_end = (int)(end - wb);
+            S = a.summ + row_of(J, c);
+        }
+        const int hl = whole ? (int)((long long)a.cursor[c] - a.size[c] - wb) : lane;  // the cluster's first lane
+        const bool head = whole && hl == lane;
+        // the warp's whole clusters need the summary maxima; a warp without
+        // any skips them
+        const bool any_whole = __any_sync(0xffffffffu, whole);
+        const int4* G4 = reinterpret_cast<const int4*>(row);
+        // lanes holding members of this lane's cluster (a contiguous run)
+        const int cl = valid ? c : -1 - lane;
+        const int up = __shfl_up_sync(0xffffffffu, cl, 1);
+        const unsigned heads = __ballot_sync(0xffffffffu, lane == 0 || up != cl);
+        const int run0 = 31 - __clz(heads & (0xffffffffu >> (31 - lane)));
+        const unsigned above = lane == 31 ? 0u : heads & (0xfffffffeu << lane);
+        const unsigned run = (0xffffffffu << run0) & (above ? (1u << (__ffs(above) - 1)) - 1u : 0xffffffffu);
+        // a whole cluster's new slots are marked (their summary entry is final;
+        // the scan clears the mark before any sweep stages deltas); such a
+        // key is added once
+        const unsigned long long mark = whole ? (1ull << 32) : 0ull;
+        // four partitions at a time: one quad of the label row, and the four
+        // keys' first CASes issued before any result is used
+        for (int i0 = 0; i0 < a.kmax; i0 += 4) {
+            int4 g4 = make_int4(0, 0, 0, 0);
+            if (valid && i0 < k) g4 = __ldg(G4 + (i0 >> 2));
+            const int gq[4] = {g4.x, g4.y, g4.z, g4.w};
+            // only the labels, the counts (a byte each) and the leader bits
+            // stay live; keys and slots are computed again for each probe
+            unsigned cnts = 0, pend = 0;
+#pragma unroll
+            for (int b = 0; b < 4; ++b) {
+                const bool on = valid && i0 + b < k;
+                const unsigned same = __match_any_sync(0xffffffffu, on ? gq[b] : -1) & run;
+                cnts |= (unsigned)__popc(same) << (8 * b);
+                pend |= (on && (__ffs(same) - 1) == lane) ? 1u << b : 0u;
+            }
+            // probe round p: the p-th slot of every key not placed yet, all
+            // of them in flight together (a lane's keys collide one by one,
+            // but the warp waits only for its longest chain, not for their sum)
+            for (unsigned long long p = 0; pend; ++p) {
+                if (p > mask || p >= limit) {
+                    if (tight) st->build_fail = 1;
+                    else set_err(st, CC_ERR_TABLE_FULL);
+                    break;
+                }
+                unsigned long long old[4];
+#pragma unroll
+                for (int b = 0; b < 4; ++b)
+                    if (pend >> b & 1u) {
+                        const unsigned long long key = ckey(c, gq[b]);
+                        old[b] = atomicCAS(&a.table[(hash_key(key) + p) & mask].key, kEmpty, key);
+                    }
+#pragma unroll
+                for (int b = 0; b < 4; ++b)
+                    if (pend >> b & 1u) {
+                        const unsigned long long key = ckey(c, gq[b]);
+                        if (old[b] != kEmpty && old[b] != key) continue;
+                        created += old[b] == kEmpty;
+                        // {count, mark}: nothing waits for the sum
+                        atomicAdd(reinterpret_cast<unsigned long long*>(&a.table[(hash_key(key) + p) & mask].cnt),
+                                  mark | (cnts >> (8 * b) & 255u));
+                        pend &= ~(1u << b);
+                    }
+            }
+            if (!any_whole) continue;
+            // summary entries of the whole clusters: the two largest (count, label)
+#pragma unroll
+            for (int b = 0; b < 4; ++b) {
+                const bool on = valid && i0 + b < k;
+                const unsigned long long mine =
+                    (whole && on) ? ((unsigned long long)(cnts >> (8 * b) & 255u) << 32) | (unsigned)gq[b] : 0ull;
+                const unsigned long long top1 = segment_max(mine, lane, seg_end);
+                const unsigned long long t1 = __shfl_sync(0xffffffffu, top1, hl);
+                const unsigned long long other = (mine != 0 && (unsigned)mine != (unsigned)t1) ? mine : 0ull;
+                const unsigned long long top2 = segment_max(other, lane, seg_end);
+                if (head && on) {
+                    const int d2 = top2 ? (int)(unsigned)top2 : -1, m2 = (int)(top2 >> 32);
+                    S[i0 + b] = make_int4((int)(unsigned)top1, (int)(top1 >> 32), d2, m2);
+                }
+            }
+        }
+    }
+    // one add per block: st->used is a single word that every block updates
+    for (int o = 16; o > 0; o >>= 1) created += __shfl_xor_sync(0xffffffffu, created, o);
+    if (lane == 0 && created) atomicAdd(&s_used, (unsigned long long)created);
+    __syncthreads();
+    if (threadIdx.x == 0 && s_used) atomicAdd(&st->used, s_used);
+}
+
+// Summary rows of the rebuilt table for the keys the build left unmarked
+// (clusters spread over several warps).  Each half of a row entry reads as
+// one unsigned 64-bit value (count << 32 | label id); every such slot offers
+// its (count, label) to the entry, which keeps the two largest by a 16-byte
+// compare-and-swap (ties to the larger id; cleared entries hold count 0 and
+// label -1, below any real key).  Content does not depend on the order of
+// the offers.  Marked slots only get their mark cleared.
+__device__ __forceinline__ void summ_top_phase(const SweepArgs& a, int conditional)
+{
+    DevState* st = a.st;
+    if (rebuild_off(st, conditional) || st->again) return;
+    const unsigned long long cap = st->new_mask + 1;
+    const unsigned long long stride = (unsigned long long)gridDim.x * blockDim.x;
+    for (unsigned long long s = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x; s < cap; s += stride) {
+        const ulonglong2 e = reinterpret_cast<const ulonglong2*>(a.table)[s];
+        const int cnt = (int)(unsigned)(e.y & 0xffffffffull);
+        if (e.x == kEmpty || cnt <= 0) continue;
+        if ((e.y >> 32) != 0) {
+            a.table[s].dlt = 0;  // summary done by the build
+            continue;
+        }
+        const int x = (int)(e.x >> 32), g = (int)(unsigned)(e.x & 0xffffffffull);
+        const int job = a.jid[x];
+        const JobInfo& J = a.job[job];
+        int4* E = a.summ + row_of(J, x) + (g >> J.lshift);
+        const unsigned long long kn = ((unsigned long long)(unsigned)cnt << 32) | (unsigned)g;
+        const volatile unsigned long long* Ev = reinterpret_cast<const volatile unsigned long long*>(E);
+        ulonglong2 cur = make_ulonglong2(Ev[0], Ev[1]);
+        // lock-free: every failed swap means another offer went in; bounded
+        // all the same
+        for (int tries = 0; kn > cur.y; ++tries) {
+            if (tries >= (1 << 20)) {
+                set_err(st, CC_ERR_INVALID);
+                break;
+            }
+            const ulonglong2 nv = kn > cur.x ? make_ulonglong2(kn, cur.x) : make_ulonglong2(cur.x, kn);
+            const ulonglong2 old = entry_cas(E, cur, nv);
+            if (old.x == cur.x && old.y == cur.y) break;
+            cur = old;
+        }
+    }
+}
+
+// Check of a tight attempt, after its build: the table must have taken every
+// key within the probe limit, at load <= 1/2, with room left below the fill
+// limit for the new keys of a light sweep (at most 2 x sum_j k_j n_j / 8).
+// (if it is a full one).  Otherwise the attempt is dropped (the summary pass
+// and the done step skip it) and the rebuild runs again at the capacity that
+// holds every key it can meet.  One thread.
+__device__ __forceinline__ void build_check_phase(const SweepArgs& a, int conditional)
+{
+    DevState* st = a.st;
+    if (threadIdx.x != 0 || rebuild_off(st, conditional)) return;
+    int fail = 0;
+    if (conditional && st->tight) {
+        const unsigned long long cap = st->new_mask + 1, fill = cap - (cap >> 3);
+        const unsigned long long room = st->build_small ? 0 : 2 * ((a.keys + 7) / 8);
+        fail = st->build_fail || st->used > cap / 2 || st->used + room > fill || a.tight_mode == 2;
+    }
+    if (fail) st->new_mask = st->retry_mask;
+    st->again = fail;
+    st->tight = 0;
+    st->build_fail = 0;
+}
+
+__device__ __forceinline__ void table_done_phase(DevState* st, int conditional)
+{
+    if (rebuild_off(st, conditional) || st->again) return;
+    st->live = (long long)st->used;
+    st->mask = st->new_mask;
+    st->small = conditional ? st->build_small : 0;
+    st->keys_all = st->used + (st->small ? st->small_keys : 0);
+    st->rebuild = 0;
+    st->abort = 0;
+    st->rebuilds += 1;
+    st->tvalid = 1;
+}
+
+}  // namespace
+
+}  // namespace ccg

@@ -8,7 +8,7 @@
 #include <climits>
 #include <vector>
 
-#include "cc_internal.cuh"
+#include "rebuild.cuh"
 
 namespace ccg {
 
@@ -227,17 +227,9 @@ __global__ void k_init_state(SweepArgs a)
         a.dsize[v] = 0;
         a.best[v] = kEmpty;
         a.chg[v] = -2;  // stamps start at 0: never "the previous sweep"
+        a.own[v] = make_int2(0, kOwnNever);
         a.prev[v] = kEmpty;
         a.act[v] = 1;
-    }
-}
-
-__global__ void k_summ_singletons(SweepArgs a, long long rows)
-{
-    const long long stride = (long long)gridDim.x * blockDim.x;
-    for (long long r = (long long)blockIdx.x * blockDim.x + threadIdx.x; r < rows; r += stride) {
-        const int g = a.G[r];
-        a.summ[r] = make_int4(g, g >= 0 ? 1 : 0, -1, 0);
     }
 }
 
@@ -248,6 +240,7 @@ __global__ void k_sizes_zero(SweepArgs a)
         a.size[v] = 0;
         a.dsize[v] = 0;
         a.best[v] = kEmpty;
+        a.own[v].y = kOwnNever;
     }
 }
 
@@ -263,70 +256,7 @@ __global__ void k_count_sizes(SweepArgs a)
     }
 }
 
-// ---- table rebuild ------------------------------------------------------
-// The table is rebuilt from C alone: clear the capacity being built, list the
-// vertices cluster by cluster (counting sort: an exclusive scan of the sizes
-// gives each cluster's first position), then insert the keys with partitions
-// innermost per member, so that the 32 lanes of a warp hold consecutive
-// members of (mostly) one cluster for one partition: equal keys are merged
-// with __match_any_sync and added with one atomic.  The summary rows follow
-// from the rebuilt counts.  All kernels are skipped unless a rebuild is
-// pending (conditional) and run unconditionally otherwise.
-
-__device__ __forceinline__ bool rebuild_off(const DevState* st, int conditional)
-{
-    return conditional && (!st->rebuild || st->err);
-}
-
-// Clears the slots of the capacity being built (st->new_mask + 1 of them),
-// the summary rows, the occupied-slot counter, and the staged size deltas
-// after an abandoned sweep.  Summary rows: those of the live clusters (a warp
-// per 32 cluster ids, the lanes across each live row), which are the rows the
-// rebuild fills and the sweeps read.  The row of a dead cluster is never read
-// again, since no move enters an empty cluster, except with empty_moves (a
-// vertex may found a cluster under its own, possibly dead, id); then, and
-// when the table did not hold the counts of C before (a new start), every row
-// is cleared.
-__global__ void k_table_clear(SweepArgs a, long long rows, int conditional)
-{
-    DevState* st = a.st;
-    if (rebuild_off(st, conditional)) return;
-    const unsigned long long cap = st->new_mask + 1;
-    const unsigned long long stride = (unsigned long long)gridDim.x * blockDim.x;
-    const unsigned long long t0 = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x;
-    for (unsigned long long s = t0; s < cap; s += stride)
-        reinterpret_cast<ulonglong2*>(a.table)[s] = make_ulonglong2(kEmpty, 0ull);
-    const int4 none = make_int4(-1, 0, -1, 0);
-    if (a.empty_moves || !st->tvalid) {
-        for (unsigned long long r = t0; r < (unsigned long long)rows; r += stride) a.summ[r] = none;
-    } else {
-        const int lane = threadIdx.x & 31;
-        for (unsigned long long x0 = t0 - lane; x0 < (unsigned long long)a.n; x0 += stride) {
-            const unsigned long long x = x0 + lane;
-            unsigned live = __ballot_sync(0xffffffffu, x < (unsigned long long)a.n && a.size[x] > 0);
-            while (live) {
-                const long long xx = (long long)x0 + __ffs(live) - 1;
-                live &= live - 1;
-                const JobInfo& J = a.job[a.jid[xx]];
-                int4* row = a.summ + row_of(J, xx);
-                for (int q = lane; q < J.kp; q += 32) row[q] = none;
-            }
-        }
-    }
-    if (st->abort)
-        for (unsigned long long v = t0; v < (unsigned long long)a.n; v += stride) a.dsize[v] = 0;
-    if (t0 == 0) st->used = 0;
-}
-
-__device__ __forceinline__ int warp_incl_scan(int x, int lane)
-{
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const int y = __shfl_up_sync(0xffffffffu, x, o);
-        if (lane >= o) x += y;
-    }
-    return x;
-}
+// ---- table rebuild: the steps of rebuild.cuh as kernels --------------------
 
 // Block sums of size[] over blocks of 1024 entries.
 __global__ void __launch_bounds__(1024) k_scan_blocks(SweepArgs a, int conditional)
@@ -336,6 +266,7 @@ __global__ void __launch_bounds__(1024) k_scan_blocks(SweepArgs a, int condition
     const long long i = (long long)blockIdx.x * 1024 + threadIdx.x;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     int x = i < a.n ? a.size[i] : 0;
+    if (to_size(a.st, conditional)) add_small_rows(a.st, i < a.n ? small_rows(a, i, x) : 0);
     for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
     if (lane == 0) wsum[w] = x;
     __syncthreads();
@@ -352,6 +283,7 @@ __global__ void __launch_bounds__(1024) k_scan_sums(SweepArgs a, int nb, int con
 {
     if (rebuild_off(a.st, conditional)) return;
     __shared__ int wsum[32];
+    if (threadIdx.x == 0 && to_size(a.st, conditional)) size_build(a);
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const int per = (nb + 1023) / 1024;
     const int lo = threadIdx.x * per, hi = min(nb, lo + per);
@@ -386,240 +318,34 @@ __global__ void __launch_bounds__(1024) k_scan_write(SweepArgs a, int conditiona
     if (i < a.n) a.cursor[i] = a.bsum[blockIdx.x] + x - v + (w > 0 ? wsum[w - 1] : 0);
 }
 
+__global__ void k_table_clear(SweepArgs a, long long rows, int conditional)
+{
+    table_clear_phase(a, rows, conditional);
+}
+
 __global__ void k_members_scatter(SweepArgs a, int conditional)
 {
-    if (rebuild_off(a.st, conditional)) return;
-    const long long stride = (long long)gridDim.x * blockDim.x;
-    for (long long v = (long long)blockIdx.x * blockDim.x + threadIdx.x; v < a.n; v += stride) {
-        const int pos = atomicAdd(&a.cursor[a.C[v]], 1);
-        if (pos < a.n) a.members[pos] = (int)v;
-        else set_err(a.st, CC_ERR_INVALID);  // sizes inconsistent with C
-    }
+    members_scatter_phase(a, conditional);
 }
 
-// Largest 64-bit value over the lanes of a contiguous lane segment [lane,
-// end) of the warp, left in the segment's first lane (every lane must call it).
-__device__ __forceinline__ unsigned long long segment_max(unsigned long long x, int lane, int end)
+__global__ void __launch_bounds__(kSetupBlock, 6) k_table_build(SweepArgs a, int conditional)
 {
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const unsigned long long y = __shfl_down_sync(0xffffffffu, x, o);
-        if (lane + o < end && y > x) x = y;
-    }
-    return x;
+    table_build_phase(a, conditional);
 }
 
-// Inserts every member's keys (partitions innermost, equal keys of a warp
-// merged with __match_any_sync and added once).  Members are listed cluster
-// by cluster, so a cluster whose members all lie in one warp's 32 entries
-// gets its exact counts inside that warp: the warp then writes the cluster's
-// summary entries itself (the two most frequent labels, ties to the larger
-// id, as the table scan would rank them), adds its keys' -2 n^2 to the job's
-// F' in a heavy sweep (eval), and marks those keys so that the scan skips
-// them.  Keys of clusters spread over several warps are left to the scan.
-// A tight attempt (see k_build_check) gives every insert kTightProbes probes;
-// an insert that finds no slot within them flags the attempt as failed, and
-// the warps stop inserting.
-constexpr unsigned long long kTightProbes = 256;
-
-__global__ void __launch_bounds__(kSetupBlock, 4) k_table_build(SweepArgs a, int conditional, int eval)
+__global__ void k_summ_top(SweepArgs a, int conditional)
 {
-    extern __shared__ long long dyn_jobs[];
-    DevState* st = a.st;
-    if (rebuild_off(st, conditional)) return;
-    __shared__ unsigned long long s_used;
-    if (threadIdx.x == 0) s_used = 0;
-    // tight attempts are made only by the heavy sweep's rebuild inside a
-    // sweep graph; a rebuild the host asks for is never one
-    const bool tight = conditional && st->tight != 0;
-    const unsigned long long limit = tight ? kTightProbes : ~0ull;
-    const bool ev = eval && st->heavy;
-    JobAcc acc(ev ? job_smem_init(a.jobs, dyn_jobs) : nullptr, &a.js[0].recompute, kJobStride);
-    __syncthreads();
-    const unsigned long long mask = st->new_mask;
-    const long long stride = (long long)gridDim.x * blockDim.x;
-    const int lane = threadIdx.x & 31;
-    unsigned long long used = 0;  // slots this warp created (lane 0 counts)
-    for (long long base = (long long)blockIdx.x * blockDim.x; base < a.n; base += stride) {
-        if (tight && __any_sync(0xffffffffu, *reinterpret_cast<volatile int*>(&st->build_fail) != 0)) break;
-        const long long m = base + threadIdx.x;
-        const long long wb = m - lane;  // first member of this warp's window
-        const bool valid = m < a.n;
-        int v = 0, c = 0, k = 0, job = 0, seg_end = lane + 1;
-        bool whole = false;
-        const int* row = a.G;
-        int4* S = a.summ;
-        if (valid) {
-            v = a.members[m];
-            c = a.C[v];
-            job = a.jid[v];
-            const JobInfo& J = a.job[job];
-            k = J.k;
-            row = a.G + row_of(J, v);
-            // after the scatter, cursor[c] is one past the cluster's last member
-            const long long end = a.cursor[c], first = end - a.size[c];
-            whole = first >= wb && end <= wb + 32;
-            if (whole) seg_end = (int)(end - wb);
-            S = a.summ + row_of(J, c);
-        }
-        const int hl = whole ? (int)((long long)a.cursor[c] - a.size[c] - wb) : lane;  // the cluster's first lane
-        const bool head = whole && hl == lane;
-        // the warp's whole clusters need the summary maxima; a warp without
-        // any skips them
-        const bool any_whole = __any_sync(0xffffffffu, whole);
-        const int4* G4 = reinterpret_cast<const int4*>(row);
-        const ulonglong2 empty = make_ulonglong2(kEmpty, 0ull);
-        const unsigned long long mark = whole ? (1ull << 32) : 0ull;
-        // four partitions at a time: one quad of the label row, and the four
-        // keys' first CASes issued before any result is used
-        for (int i0 = 0; i0 < a.kmax; i0 += 4) {
-            int4 g4 = make_int4(0, 0, 0, 0);
-            if (valid && i0 < k) g4 = __ldg(G4 + (i0 >> 2));
-            const int gq[4] = {g4.x, g4.y, g4.z, g4.w};
-            unsigned long long key[4], h[4];
-            int cnt[4];
-            bool lead[4];
-            ulonglong2 old[4];
-#pragma unroll
-            for (int b = 0; b < 4; ++b) {
-                const bool on = valid && i0 + b < k;
-                key[b] = on ? ckey(c, gq[b]) : kEmpty;
-                const unsigned same = __match_any_sync(0xffffffffu, key[b]);
-                cnt[b] = __popc(same);
-                lead[b] = on && (__ffs(same) - 1) == lane;
-                h[b] = hash_key(key[b]) & mask;
-            }
-#pragma unroll
-            for (int b = 0; b < 4; ++b)
-                if (lead[b]) old[b] = slot_cas(a.table + h[b], empty, make_ulonglong2(key[b], mark | (unsigned)cnt[b]));
-#pragma unroll
-            for (int b = 0; b < 4; ++b) {
-                bool ins = false;
-                if (lead[b]) {
-                    if (table_build_finish(a.table, mask, key[b], cnt[b], &ins, whole ? 1 : 0, limit, h[b], old[b]) <
-                        0) {
-                        if (tight) st->build_fail = 1;
-                        else set_err(st, CC_ERR_TABLE_FULL);
-                    }
-                    if (ev && whole) acc.add(job, -2LL * cnt[b] * cnt[b]);
-                }
-                used += __popc(__ballot_sync(0xffffffffu, ins));
-            }
-            if (!any_whole) continue;
-            // summary entries of the whole clusters: the two largest (count, label)
-#pragma unroll
-            for (int b = 0; b < 4; ++b) {
-                const bool on = valid && i0 + b < k;
-                const unsigned long long mine =
-                    (whole && on) ? ((unsigned long long)(unsigned)cnt[b] << 32) | (unsigned)gq[b] : 0ull;
-                const unsigned long long top1 = segment_max(mine, lane, seg_end);
-                const unsigned long long t1 = __shfl_sync(0xffffffffu, top1, hl);
-                const unsigned long long other = (mine != 0 && (unsigned)mine != (unsigned)t1) ? mine : 0ull;
-                const unsigned long long top2 = segment_max(other, lane, seg_end);
-                if (head && on) {
-                    const int d2 = top2 ? (int)(unsigned)top2 : -1, m2 = (int)(top2 >> 32);
-                    S[i0 + b] = make_int4((int)(unsigned)top1, (int)(top1 >> 32), d2, m2);
-                }
-            }
-        }
-    }
-    // one add per block: st->used is a single word that every block updates
-    if (lane == 0 && used) atomicAdd(&s_used, used);
-    if (ev) job_acc_finish(acc, a.jobs);
-    __syncthreads();
-    if (threadIdx.x == 0 && s_used) atomicAdd(&st->used, s_used);
+    summ_top_phase(a, conditional);
 }
 
-// Summary rows of the rebuilt table for the keys the build left unmarked
-// (clusters spread over several warps).  Each half of a row entry reads as
-// one unsigned 64-bit value (count << 32 | label id); every such slot offers
-// its (count, label) to the entry, which keeps the two largest by a 16-byte
-// compare-and-swap (ties to the larger id; cleared entries hold count 0 and
-// label -1, below any real key).  Content does not depend on the order of
-// the offers.  Marked slots only get their mark cleared.
-// With eval set (the first rebuild of a heavy sweep) this pass also adds
-// -2 sum n^2 over the unmarked keys to each job's recompute (the table part
-// of F'; the build added the marked ones).
-__global__ void k_summ_top(SweepArgs a, int conditional, int eval)
-{
-    extern __shared__ long long dyn_jobs[];
-    DevState* st = a.st;
-    if (rebuild_off(st, conditional) || st->again) return;
-    const bool ev = eval && st->heavy;
-    JobAcc acc(ev ? job_smem_init(a.jobs, dyn_jobs) : nullptr, &a.js[0].recompute, kJobStride);
-    const unsigned long long cap = st->new_mask + 1;
-    const unsigned long long stride = (unsigned long long)gridDim.x * blockDim.x;
-    for (unsigned long long s = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x; s < cap; s += stride) {
-        const ulonglong2 e = reinterpret_cast<const ulonglong2*>(a.table)[s];
-        const int cnt = (int)(unsigned)(e.y & 0xffffffffull);
-        if (e.x == kEmpty || cnt <= 0) continue;
-        if ((e.y >> 32) != 0) {
-            a.table[s].dlt = 0;  // summary and F' part done by the build
-            continue;
-        }
-        const int x = (int)(e.x >> 32), g = (int)(unsigned)(e.x & 0xffffffffull);
-        const int job = a.jid[x];
-        const JobInfo& J = a.job[job];
-        int4* E = a.summ + row_of(J, x) + (g >> J.lshift);
-        const unsigned long long kn = ((unsigned long long)(unsigned)cnt << 32) | (unsigned)g;
-        const volatile unsigned long long* Ev = reinterpret_cast<const volatile unsigned long long*>(E);
-        ulonglong2 cur = make_ulonglong2(Ev[0], Ev[1]);
-        // lock-free: every failed swap means another offer went in; bounded
-        // all the same
-        for (int tries = 0; kn > cur.y; ++tries) {
-            if (tries >= (1 << 20)) {
-                set_err(st, CC_ERR_INVALID);
-                break;
-            }
-            const ulonglong2 nv = kn > cur.x ? make_ulonglong2(kn, cur.x) : make_ulonglong2(cur.x, kn);
-            const ulonglong2 old = entry_cas(E, cur, nv);
-            if (old.x == cur.x && old.y == cur.y) break;
-            cur = old;
-        }
-        if (ev) acc.add(job, -2LL * cnt * cnt);
-    }
-    if (ev) job_acc_finish(acc, a.jobs);
-}
-
-// Check of a tight attempt, after its build: the table must have taken every
-// key within the probe limit, at load <= 1/2, with room left below the fill
-// limit for the new keys of a light sweep (at most 2 x sum_j k_j n_j / 8).
-// Otherwise the attempt is dropped (its part of F' is cleared; the summary
-// pass and the done step skip it) and the rebuild runs again at the capacity
-// that holds every key the sweep can create.  One block.
 __global__ void k_build_check(SweepArgs a, int conditional)
 {
-    DevState* st = a.st;
-    if (rebuild_off(st, conditional)) return;
-    __shared__ int fail;
-    if (threadIdx.x == 0) {
-        fail = 0;
-        if (conditional && st->tight) {
-            const unsigned long long cap = st->new_mask + 1, fill = cap - (cap >> 3);
-            const unsigned long long room = 2 * ((a.keys + 7) / 8);
-            fail = st->build_fail || st->used > cap / 2 || st->used + room > fill || a.tight_mode == 2;
-        }
-    }
-    __syncthreads();
-    if (fail)
-        for (int j = threadIdx.x; j < a.jobs; j += blockDim.x) a.js[j].recompute = 0;
-    if (threadIdx.x == 0) {
-        if (fail) st->new_mask = st->safe_mask;
-        st->again = fail;
-        st->tight = 0;
-        st->build_fail = 0;
-    }
+    build_check_phase(a, conditional);
 }
 
 __global__ void k_table_done(DevState* st, int conditional)
 {
-    if (rebuild_off(st, conditional) || st->again) return;
-    st->live = (long long)st->used;
-    st->mask = st->new_mask;
-    st->rebuild = 0;
-    st->abort = 0;
-    st->rebuilds += 1;
-    st->tvalid = 1;
+    table_done_phase(st, conditional);
 }
 
 // F of every job without sum_ij |P_ij|^2: k sum_c s_c^2 - 2 sum_keys n^2.
@@ -845,12 +571,6 @@ cudaError_t launch_init_state(const SweepArgs& a, cudaStream_t s)
     return cudaGetLastError();
 }
 
-cudaError_t launch_singleton_summaries(const SweepArgs& a, long long rows, cudaStream_t s)
-{
-    k_summ_singletons<<<grid_for(rows), kSetupBlock, 0, s>>>(a, rows);
-    return cudaGetLastError();
-}
-
 cudaError_t launch_state_from_ids(const SweepArgs& a, cudaStream_t s)
 {
     k_sizes_zero<<<grid_for(a.n), kSetupBlock, 0, s>>>(a);
@@ -858,19 +578,18 @@ cudaError_t launch_state_from_ids(const SweepArgs& a, cudaStream_t s)
     return cudaGetLastError();
 }
 
-cudaError_t launch_table_rebuild(const SweepArgs& a, long long rows, bool conditional, cudaStream_t s, bool eval)
+cudaError_t launch_table_rebuild(const SweepArgs& a, long long rows, bool conditional, cudaStream_t s)
 {
     const int c = conditional ? 1 : 0;
     const int nb = (int)((a.n + 1023) / 1024);
-    k_table_clear<<<grid_for(std::max((long long)a.mask_max + 1, rows)), kSetupBlock, 0, s>>>(a, rows, c);
     k_scan_blocks<<<nb, 1024, 0, s>>>(a, c);
     k_scan_sums<<<1, 1024, 0, s>>>(a, nb, c);
     k_scan_write<<<nb, 1024, 0, s>>>(a, c);
+    k_table_clear<<<grid_for(std::max((long long)a.mask_max + 1, rows)), kSetupBlock, 0, s>>>(a, rows, c);
     k_members_scatter<<<grid_for(a.n), kSetupBlock, 0, s>>>(a, c);
-    k_table_build<<<grid_for(a.n), kSetupBlock, eval ? smem_jobs_bytes(a.jobs) : 0, s>>>(a, c, eval ? 1 : 0);
-    k_build_check<<<1, 256, 0, s>>>(a, c);
-    k_summ_top<<<grid_for((long long)a.mask_max + 1), kSetupBlock, eval ? smem_jobs_bytes(a.jobs) : 0, s>>>(a, c,
-                                                                                                 eval ? 1 : 0);
+    k_table_build<<<grid_for(a.n), kSetupBlock, 0, s>>>(a, c);
+    k_build_check<<<1, 32, 0, s>>>(a, c);
+    k_summ_top<<<grid_for((long long)a.mask_max + 1), kSetupBlock, 0, s>>>(a, c);
     k_table_done<<<1, 1, 0, s>>>(a.st, c);
     return cudaGetLastError();
 }
