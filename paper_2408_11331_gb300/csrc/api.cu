@@ -808,6 +808,7 @@ cc_status create_common(int jobs, const JobInput* in, bool on_device, const cc_o
         la.lmask = lcap - 1;
         la.rows = rows;
         la.st = c->st;
+        la.classes = &c->st->classes;
         la.part_sq = c->part_sq;
         la.part_slog = c->part_slog;
         if (e == cudaSuccess) e = cudaMemsetAsync(c->part_sq, 0, sizeof(long long) * pjob.size(), c->stream);
@@ -818,6 +819,7 @@ cc_status create_common(int jobs, const JobInput* in, bool on_device, const cc_o
         cleanup();
         if (e != cudaSuccess) return bail(cuda_fail(c, e, "label compaction"));
         if (s.err) return bail(fail(c, CC_ERR_INVALID, "malformed CSR: columns must lie in [0, n)"));
+        c->classes = s.classes;
     }
     std::vector<JobState> js;
     if (read_jobs(c, js) != CC_OK) return bail(CC_ERR_CUDA);
@@ -940,7 +942,12 @@ __global__ void k_first(long long n, int* first)
 __global__ void k_first_min(long long n, const int* __restrict__ C, int* first)
 {
     const long long stride = (long long)gridDim.x * blockDim.x;
-    for (long long v = (long long)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += stride) atomicMin(&first[C[v]], (int)v);
+    // vertices come roughly in order, so most find a smaller one there already
+    // and need no atomic (adds and minima of one word take about 10 ns each)
+    for (long long v = (long long)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += stride) {
+        int* f = &first[C[v]];
+        if (__ldcg(f) > (int)v) atomicMin(f, (int)v);
+    }
 }
 
 __global__ void k_flags(long long n, const int* __restrict__ C, const int* __restrict__ first, int* flag, int* blocksum)
@@ -1162,8 +1169,10 @@ __global__ void k_load_state(SweepArgs a, long long vo, long long ncap, long lon
 __global__ void k_first_min_job(long long n, long long vo, const int* __restrict__ C, int* first)
 {
     const long long stride = (long long)gridDim.x * blockDim.x;
-    for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < n; t += stride)
-        atomicMin(&first[C[vo + t]], (int)t);
+    for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < n; t += stride) {
+        int* f = &first[C[vo + t]];
+        if (__ldcg(f) > (int)t) atomicMin(f, (int)t);
+    }
 }
 
 __global__ void k_flags_job(long long n, long long vo, const int* __restrict__ C, const int* __restrict__ first,
@@ -1231,6 +1240,200 @@ cc_status renumber(cc_ctx* c, int** labels)
     c->launches += 6;
     CC_CUDA(c, cudaGetLastError());
     *labels = lab;
+    return CC_OK;
+}
+
+// Capacity - 1 of the rebuild before the distance reductions, which read the
+// whole table: no more than the keys of C need (they are known while the table
+// holds its counts), by the rule of a full rebuild in a sweep (load <= 1/2 and
+// room for a light sweep; size_build in rebuild.cuh).  At the capacity in use
+// the clear and the two scans of 2^27 slots took 1.0 of 2.0 ms (kNN n = 1e6,
+// k = 50).
+unsigned long long metrics_mask(const cc_ctx* c, const DevState& s)
+{
+    if (!s.tvalid || s.small) return full_mask(c, s);
+    const unsigned long long live = s.live > 0 ? (unsigned long long)s.live : 0;
+    const unsigned long long room = 2 * (((unsigned long long)c->keys + 7) / 8);
+    unsigned long long cap = std::min<unsigned long long>(1024, s.mask + 1);
+    while (cap < s.mask + 1 && (cap < 2 * live || cap - (cap >> 3) < live + room)) cap <<= 1;
+    return cap - 1;
+}
+
+// Distances of the consensus to every input partition, from a table rebuilt
+// at the given capacity (which makes the summary rows exact maxima).
+cc_status metrics(cc_ctx* c, unsigned long long mask, cc_partition_metrics* out)
+{
+    CC_CUDA(c, cudaMemcpyAsync(&c->st->new_mask, &mask, sizeof(mask), cudaMemcpyHostToDevice, c->stream));
+    CC_CUDA(c, launch_table_rebuild(c->args, c->rows, false, c->stream, mask + 1));
+    c->launches += kKernelsPerRebuild;
+    const int P = c->parts, J = c->jobs;
+    // class maxima: a hash of the classes, unless that is no smaller than one
+    // int per label id
+    unsigned long long ccap = 64;
+    while (ccap < 2ull * (unsigned long long)c->classes) ccap <<= 1;
+    if (sizeof(Slot) * ccap >= sizeof(int) * (unsigned long long)c->nlabels) ccap = 0;
+    const size_t maxima = ccap ? sizeof(Slot) * (size_t)ccap : sizeof(int) * (size_t)c->nlabels;
+    const size_t sums = (sizeof(long long) * 3 + sizeof(double)) * (size_t)P +
+                        (sizeof(long long) + sizeof(double)) * (size_t)J;
+    const size_t head = (sums + 15) & ~size_t(15);
+    unsigned char* buf = nullptr;
+    CC_CUDA(c, c->pool ? cudaMallocFromPoolAsync((void**)&buf, head + maxima, c->pool, c->stream)
+                       : cudaMalloc((void**)&buf, head + maxima));
+    MetricsArgs m{};
+    long long* sq = reinterpret_cast<long long*>(buf);
+    long long* sjc = sq + P;
+    long long* sjl = sjc + P;
+    long long* csq = sjl + P;
+    double* slog = reinterpret_cast<double*>(csq + J);
+    double* cslog = slog + P;
+    m.pfirst = c->d_pfirst;
+    m.lbase = c->d_lbase;
+    m.nlabels = c->nlabels;
+    if (ccap) m.cmap = reinterpret_cast<Slot*>(buf + head);
+    else m.lmax = reinterpret_cast<int*>(buf + head);
+    m.cmask = ccap ? ccap - 1 : 0;
+    m.sq = sq;
+    m.slog = slog;
+    m.sjc = sjc;
+    m.sjl = sjl;
+    m.csq = csq;
+    m.cslog = cslog;
+    // one copy back for the sums, one for the partitions' own
+    std::vector<unsigned char> h(sums);
+    std::vector<long long> h_psq(P);
+    std::vector<double> h_pslog(P);
+    cudaError_t e = cudaMemsetAsync(buf, 0, head + (ccap ? 0 : maxima), c->stream);
+    if (e == cudaSuccess && ccap) e = launch_empty_slots(m.cmap, ccap, c->stream);
+    if (e == cudaSuccess) e = launch_metrics(c->args, m, P, mask + 1, c->stream);
+    c->launches += ccap ? 4 : 3;
+    auto get = [&](void* dst, const void* src, size_t n) {
+        if (e == cudaSuccess) e = cudaMemcpyAsync(dst, src, n, cudaMemcpyDeviceToHost, c->stream);
+    };
+    DevState s;
+    get(h.data(), buf, sums);
+    get(h_psq.data(), c->part_sq, sizeof(long long) * P);
+    get(h_pslog.data(), c->part_slog, sizeof(double) * P);
+    get(&s, c->st, sizeof(s));
+    if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
+    if (c->pool) cudaFreeAsync(buf, c->stream);
+    else cudaFree(buf);
+    if (e != cudaSuccess) return cuda_fail(c, e, "metrics");
+    const long long* h_sq = reinterpret_cast<const long long*>(h.data());
+    const long long *h_sjc = h_sq + P, *h_sjl = h_sjc + P, *h_csq = h_sjl + P;
+    const double* h_slog = reinterpret_cast<const double*>(h_csq + J);
+    const double* h_cslog = h_slog + P;
+    for (int j = 0; j < J; ++j) {
+        const JobInfo& Jb = c->job[j];
+        const double n = (double)Jb.n;
+        for (int i = 0; i < Jb.k; ++i) {
+            const int p = c->pfirst[j] + i;
+            cc_partition_metrics& o = out[p];
+            o.mirkin = h_csq[j] + h_psq[p] - 2 * h_sq[p];
+            o.split_join = 2 * Jb.n - h_sjc[p] - h_sjl[p];
+            o.rand_distance = Jb.n > 1 ? (double)o.mirkin / (n * (n - 1.0)) : 0.0;
+            o.vi = (h_cslog[j] + h_pslog[p] - 2.0 * h_slog[p]) / n;
+        }
+    }
+    return check_device_error(c, s);
+}
+
+// The distances between all input partitions from dense matrices, one per
+// pair of partitions (see metrics.cu); *done is false, and nothing was done,
+// where a matrix would be large for the vertices it counts (many classes: it
+// is cleared and read twice, so up to 16 cells per vertex, and 2^18 for the
+// smallest jobs) or the memory is not there.
+cc_status pair_distances(cc_ctx* c, cc_partition_metrics* out, bool* done)
+{
+    const int k = c->job[0].k;
+    const long long n = c->job[0].n;
+    constexpr long long kCells = 1LL << 26;   // cells counted at once (256 MB)
+    constexpr size_t kPairs = 32768;
+    const size_t ids_bytes = rounded(sizeof(int) * (size_t)n * k), log_bytes = sizeof(double) * kLogTable;
+    const size_t cls_bytes = rounded(sizeof(int) * (size_t)k);
+    unsigned char* buf = nullptr;
+    auto lacking = [&](cudaError_t e) {
+        cudaGetLastError();
+        return e == cudaErrorMemoryAllocation ? CC_OK : cuda_fail(c, e, "partition distances");
+    };
+    cudaError_t e = cudaMalloc((void**)&buf, ids_bytes + log_bytes + cls_bytes);
+    if (e != cudaSuccess) return lacking(e);
+    int* ids = reinterpret_cast<int*>(buf);
+    double* nlogn = reinterpret_cast<double*>(buf + ids_bytes);
+    int* classes = reinterpret_cast<int*>(buf + ids_bytes + log_bytes);
+    std::vector<int> kc(k);
+    std::vector<long long> psq(k);
+    std::vector<double> pslog(k);
+    e = cudaMemsetAsync(classes, 0, cls_bytes, c->stream);
+    if (e == cudaSuccess) e = launch_pair_ids(c->args, ids, classes, nlogn, c->stream);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(kc.data(), classes, sizeof(int) * k, cudaMemcpyDeviceToHost, c->stream);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(psq.data(), c->part_sq, sizeof(long long) * k, cudaMemcpyDeviceToHost, c->stream);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(pslog.data(), c->part_slog, sizeof(double) * k, cudaMemcpyDeviceToHost, c->stream);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
+    c->launches += 3;
+    const long long kmax = e == cudaSuccess ? *std::max_element(kc.begin(), kc.end()) : 0;
+    if (e == cudaSuccess && kmax * kmax > std::min(16 * n + (1LL << 18), kCells)) {
+        cudaFree(buf);
+        return CC_OK;
+    }
+    long long total = 0;
+    for (int a = 0; a < k; ++a)
+        for (int b = a + 1; b < k; ++b) total += (long long)kc[a] * kc[b];
+    const size_t pairs_all = (size_t)k * (k - 1) / 2, pairs_most = std::max<size_t>(1, std::min(pairs_all, kPairs));
+    const size_t cells_bytes = rounded(sizeof(int) * (size_t)std::max<long long>(1, std::min(total, kCells)));
+    const size_t desc_bytes = rounded(sizeof(PairDesc) * pairs_most), sum_bytes = rounded(sizeof(PairSums) * pairs_most);
+    unsigned char* work = nullptr;
+    if (e == cudaSuccess) {
+        e = cudaMalloc((void**)&work, cells_bytes + desc_bytes + sum_bytes);
+        if (e != cudaSuccess) {
+            cudaFree(buf);
+            return lacking(e);
+        }
+    }
+    int* cells = reinterpret_cast<int*>(work);
+    PairDesc* d_pairs = reinterpret_cast<PairDesc*>(work + cells_bytes);
+    PairSums* d_sums = reinterpret_cast<PairSums*>(work + cells_bytes + desc_bytes);
+    std::vector<PairDesc> pairs;
+    std::vector<PairSums> sums;
+    long long used = 0;
+    auto flush = [&]() {
+        if (pairs.empty() || e != cudaSuccess) return;
+        sums.resize(pairs.size());
+        e = cudaMemcpyAsync(d_pairs, pairs.data(), sizeof(PairDesc) * pairs.size(), cudaMemcpyHostToDevice, c->stream);
+        if (e == cudaSuccess) e = cudaMemsetAsync(cells, 0, sizeof(int) * (size_t)used, c->stream);
+        if (e == cudaSuccess) e = cudaMemsetAsync(d_sums, 0, sizeof(PairSums) * pairs.size(), c->stream);
+        if (e == cudaSuccess)
+            e = launch_pairs(n, ids, d_pairs, (int)pairs.size(), (int)kmax, cells, nlogn, d_sums, c->stream);
+        if (e == cudaSuccess)
+            e = cudaMemcpyAsync(sums.data(), d_sums, sizeof(PairSums) * pairs.size(), cudaMemcpyDeviceToHost, c->stream);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
+        c->launches += 3;
+        for (size_t p = 0; p < pairs.size() && e == cudaSuccess; ++p) {
+            const int a = pairs[p].a, b = pairs[p].b;
+            const PairSums& q = sums[p];
+            cc_partition_metrics o;
+            o.mirkin = psq[a] + psq[b] - 2 * q.sq;
+            o.split_join = 2 * n - q.rows - q.cols;
+            o.rand_distance = n > 1 ? (double)o.mirkin / ((double)n * ((double)n - 1.0)) : 0.0;
+            o.vi = (pslog[a] + pslog[b] - 2.0 * q.slog) / (double)n;
+            out[(size_t)a * k + b] = out[(size_t)b * k + a] = o;
+        }
+        pairs.clear();
+        used = 0;
+    };
+    for (int a = 0; a < k && e == cudaSuccess; ++a) {
+        out[(size_t)a * k + a] = cc_partition_metrics{0, 0, 0.0, 0.0};
+        for (int b = a + 1; b < k; ++b) {
+            const long long cells_ab = (long long)kc[a] * kc[b];
+            if (used + cells_ab > kCells || pairs.size() == kPairs) flush();
+            pairs.push_back(PairDesc{a, b, kc[a], kc[b], used});
+            used += cells_ab;
+        }
+    }
+    flush();
+    cudaFree(work);
+    cudaFree(buf);
+    if (e != cudaSuccess) return cuda_fail(c, e, "partition distances");
+    *done = true;
     return CC_OK;
 }
 
@@ -1463,6 +1666,7 @@ cc_status ctx_load_job(cc_ctx* c, int j, const JobInput& in)
     la.lmask = lcap - 1;
     la.rows = n * J.kp;
     la.st = tst;
+    la.classes = &tst->classes;
     la.part_sq = c->part_sq + c->pfirst[j];
     la.part_slog = c->part_slog + c->pfirst[j];
     if (e == cudaSuccess) e = launch_label_kernels(la, c->stream);
@@ -1498,6 +1702,7 @@ cc_status ctx_load_job(cc_ctx* c, int j, const JobInput& in)
     c->job[j] = J;
     c->psq[j] = psq;
     c->F0[j] = psq - k * n;
+    c->classes += chk.classes;  // (an upper bound: the finished job's still count)
     c->async_launches = 0;  // the run's launch budget starts again
     return CC_OK;
 }
@@ -1844,74 +2049,11 @@ cc_status cc_batch_result(cc_ctx* c, int32_t job, int32_t* labels_out, int64_t* 
 cc_status cc_metrics(cc_ctx* c, cc_partition_metrics* out)
 {
     if (!c || !out) return fail(c, CC_ERR_INVALID, "null argument");
-    // a rebuild at the current capacity makes the summary rows exact maxima
     DevState pre;
     cc_status r = read_state(c, &pre);
     if (r != CC_OK) return r;
     if (pre.err) return check_device_error(c, pre);
-    const unsigned long long nm = full_mask(c, pre);
-    CC_CUDA(c, cudaMemcpyAsync(&c->st->new_mask, &nm, sizeof(nm), cudaMemcpyHostToDevice, c->stream));
-    CC_CUDA(c, launch_table_rebuild(c->args, c->rows, false, c->stream));
-    c->launches += kKernelsPerRebuild;
-    const int P = c->parts, J = c->jobs;
-    const size_t bytes = sizeof(int) * (size_t)c->nlabels + (sizeof(long long) * 3 + sizeof(double)) * (size_t)P +
-                         (sizeof(long long) + sizeof(double)) * (size_t)J + 64;
-    unsigned char* buf = nullptr;
-    CC_CUDA(c, c->pool ? cudaMallocFromPoolAsync((void**)&buf, bytes, c->pool, c->stream) : cudaMalloc((void**)&buf, bytes));
-    MetricsArgs m{};
-    long long* sq = reinterpret_cast<long long*>(buf);
-    long long* sjc = sq + P;
-    long long* sjl = sjc + P;
-    long long* csq = sjl + P;
-    double* slog = reinterpret_cast<double*>(csq + J);
-    double* cslog = slog + P;
-    int* lmax = reinterpret_cast<int*>(cslog + J);
-    m.pfirst = c->d_pfirst;
-    m.lbase = c->d_lbase;
-    m.nlabels = c->nlabels;
-    m.lmax = lmax;
-    m.sq = sq;
-    m.slog = slog;
-    m.sjc = sjc;
-    m.sjl = sjl;
-    m.csq = csq;
-    m.cslog = cslog;
-    std::vector<long long> h_sq(P), h_sjc(P), h_sjl(P), h_csq(J), h_psq(P);
-    std::vector<double> h_slog(P), h_cslog(J), h_pslog(P);
-    cudaError_t e = cudaMemsetAsync(buf, 0, bytes, c->stream);
-    if (e == cudaSuccess) e = launch_metrics(c->args, m, P, c->stream);
-    c->launches += 3;
-    auto get = [&](void* dst, const void* src, size_t n) {
-        if (e == cudaSuccess) e = cudaMemcpyAsync(dst, src, n, cudaMemcpyDeviceToHost, c->stream);
-    };
-    get(h_sq.data(), sq, sizeof(long long) * P);
-    get(h_sjc.data(), sjc, sizeof(long long) * P);
-    get(h_sjl.data(), sjl, sizeof(long long) * P);
-    get(h_csq.data(), csq, sizeof(long long) * J);
-    get(h_slog.data(), slog, sizeof(double) * P);
-    get(h_cslog.data(), cslog, sizeof(double) * J);
-    get(h_psq.data(), c->part_sq, sizeof(long long) * P);
-    get(h_pslog.data(), c->part_slog, sizeof(double) * P);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
-    if (c->pool) cudaFreeAsync(buf, c->stream);
-    else cudaFree(buf);
-    if (e != cudaSuccess) return cuda_fail(c, e, "metrics");
-    for (int j = 0; j < J; ++j) {
-        const JobInfo& Jb = c->job[j];
-        const double n = (double)Jb.n;
-        for (int i = 0; i < Jb.k; ++i) {
-            const int p = c->pfirst[j] + i;
-            cc_partition_metrics& o = out[p];
-            o.mirkin = h_csq[j] + h_psq[p] - 2 * h_sq[p];
-            o.split_join = 2 * Jb.n - h_sjc[p] - h_sjl[p];
-            o.rand_distance = Jb.n > 1 ? (double)o.mirkin / (n * (n - 1.0)) : 0.0;
-            o.vi = (h_cslog[j] + h_pslog[p] - 2.0 * h_slog[p]) / n;
-        }
-    }
-    DevState s;
-    r = read_state(c, &s);
-    if (r != CC_OK) return r;
-    return check_device_error(c, s);
+    return metrics(c, metrics_mask(c, pre), out);
 }
 
 cc_status cc_partition_distances(cc_ctx* c, cc_partition_metrics* out)
@@ -1919,12 +2061,15 @@ cc_status cc_partition_distances(cc_ctx* c, cc_partition_metrics* out)
     if (!c || !out) return fail(c, CC_ERR_INVALID, "null argument");
     cc_status r = need_single(c);
     if (r != CC_OK) return r;
-    const int k = c->job[0].k;
-    const long long n = c->n;
     DevState pre;
     r = read_state(c, &pre);
     if (r != CC_OK) return r;
     if (pre.err) return check_device_error(c, pre);
+    bool done = false;
+    r = pair_distances(c, out, &done);
+    if (r != CC_OK || done) return r;
+    const int k = c->job[0].k;
+    const long long n = c->n;
     // the consensus is kept aside and restored; each input partition in turn
     // becomes the consensus, and the distance reductions give its row
     int* saved = c->scratch;
@@ -1934,9 +2079,8 @@ cc_status cc_partition_distances(cc_ctx* c, cc_partition_metrics* out)
     for (int a = 0; a < k && r == CC_OK; ++a) {
         CC_CUDA(c, launch_ids_from_partition(c->args, n, 0, a, c->stream));
         CC_CUDA(c, launch_state_from_ids(c->args, c->stream));
-        CC_CUDA(c, cudaMemcpyAsync(&c->st->mask, &full, sizeof(full), cudaMemcpyHostToDevice, c->stream));
         c->launches += 3;
-        r = cc_metrics(c, row.data());
+        r = metrics(c, full, row.data());
         for (int i = 0; r == CC_OK && i < k; ++i) out[(size_t)a * k + i] = row[i];
     }
     // restore C, its sizes and its table at the capacity it had

@@ -131,6 +131,7 @@ struct DevState {
     unsigned long long retry_mask;  // heavy sweep: capacity - 1 of the second attempt of its rebuild
     int many;                    // 1: many vertices may move (the sweep before moved more than 1/8 of the label rows)
     int match;                   // 1: some job of this sweep falls back to the matching
+    long long classes;           // label classes of all partitions (set at creation)
     // run kernel (persist.cu); written between two steps only
     int rebuild_kind;            // the running rebuild: 0 heavy sweep, 1 its rollback, 2 end of the sweep
     int tries;                   // rebuild attempts of this heavy sweep
@@ -444,6 +445,7 @@ struct LabelArgs {
     unsigned long long lmask;
     long long rows;             // entries of G
     DevState* st;
+    long long* classes;         // label classes of all partitions together
     long long* part_sq;         // per global partition: sum_l |P_il|^2
     double* part_slog;          // per global partition: sum_l |P_il| log |P_il|
 };
@@ -457,7 +459,12 @@ cudaError_t launch_init_state(const SweepArgs& a, cudaStream_t s);
 cudaError_t launch_state_from_ids(const SweepArgs& a, cudaStream_t s);
 // Rebuild of the table and summary rows from C into st->new_mask + 1 slots,
 // then st->mask = st->new_mask.  conditional: only if st->rebuild is set.
-cudaError_t launch_table_rebuild(const SweepArgs& a, long long rows, bool conditional, cudaStream_t s);
+// cap: capacity being built, where the host knows it (0: any up to the
+// allocated one), for the size of the grids.
+cudaError_t launch_table_rebuild(const SweepArgs& a, long long rows, bool conditional, cudaStream_t s,
+                                 unsigned long long cap = 0);
+// Slots of an empty table.
+cudaError_t launch_empty_slots(Slot* t, unsigned long long cap, cudaStream_t s);
 // F of every job from scratch into js[j].recompute (without sum_ij |P_ij|^2).
 cudaError_t launch_objective_recompute(const SweepArgs& a, cudaStream_t s);
 
@@ -468,13 +475,18 @@ cudaError_t launch_objective_recompute(const SweepArgs& a, cudaStream_t s);
 // j's partition i is P = pfirst[j] + i): sq[P] = sum n(c,i,l)^2, slog[P] =
 // sum n log n, sjc[P] = sum over clusters c of max_l n(c,i,l), sjl[P] = sum
 // over classes l of max_c n(c,i,l); per job: csq[j] = sum |c|^2, cslog[j] =
-// sum |c| log |c|.  lmax: one int per label id of every job (job j's ids start
-// at lbase[j]); all outputs zeroed by the caller.
+// sum |c| log |c|.  The class maxima are kept in cmap, a hash of the class ids
+// with cmask + 1 entries (keys kEmpty, counts 0 at the start), or, where the
+// jobs have so many classes that it would be no smaller (cmask 0), in lmax, one
+// int per label id of every job (job j's ids start at lbase[j]); all outputs
+// zeroed by the caller.
 struct MetricsArgs {
     const int* pfirst;
     const long long* lbase;
     long long nlabels;      // entries of lmax
     int* lmax;
+    Slot* cmap;
+    unsigned long long cmask;
     long long* sq;
     double* slog;
     long long* sjc;
@@ -482,7 +494,30 @@ struct MetricsArgs {
     long long* csq;
     double* cslog;
 };
-cudaError_t launch_metrics(const SweepArgs& a, const MetricsArgs& m, int parts, cudaStream_t s);
+// cap: slots of the table in use.
+cudaError_t launch_metrics(const SweepArgs& a, const MetricsArgs& m, int parts, unsigned long long cap, cudaStream_t s);
+
+// Pair (a, b) of input partitions with ka and kb classes: its ka x kb matrix
+// starts at cells[off]; its sums.
+struct PairDesc {
+    int a, b, ka, kb;
+    long long off;
+};
+struct PairSums {
+    long long sq;    // sum of n^2 over the cells
+    long long rows;  // sum of the row maxima
+    long long cols;  // sum of the column maxima
+    double slog;     // sum of n log n
+};
+constexpr int kLogTable = 4096;  // entries of the table of n log n
+// ids (k n ints): rank of each vertex's class per partition of job 0,
+// partition-major; classes (k ints, zeroed by the caller): classes per
+// partition; nlogn: kLogTable doubles.
+cudaError_t launch_pair_ids(const SweepArgs& a, int* ids, int* classes, double* nlogn, cudaStream_t s);
+// Sums of `count` pairs (at most 65535; cells and out zeroed by the caller;
+// kmax: the most classes of a partition).
+cudaError_t launch_pairs(long long n, const int* ids, const PairDesc* pairs, int count, int kmax, int* cells,
+                         const double* nlogn, PairSums* out, cudaStream_t s);
 // C of job j's n vertices := its input partition i (cluster id = least vertex of the class).
 cudaError_t launch_ids_from_partition(const SweepArgs& a, long long n, int j, int i, cudaStream_t s);
 

@@ -37,6 +37,7 @@ struct cc_ctx {
     std::vector<long long> lbase;       // first label id of each job in a job-concatenated id space
     long long nlabels = 0;              // sum_j k_j 2^s_j
     int parts = 0;                      // sum_j k_j
+    long long classes = 0;              // label classes of all partitions (at most)
     int* d_pfirst = nullptr;
     long long* d_lbase = nullptr;
     long long* part_sq = nullptr;       // per global partition: sum_l |P_il|^2

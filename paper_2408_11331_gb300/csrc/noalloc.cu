@@ -61,7 +61,7 @@ __global__ void k_na_first(int n, const int* __restrict__ ids, int* first, int* 
     for (long long v = (long long)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += stride) {
         const int c = ids[v];
         if (c < 0 || c >= n) *flag = 1;
-        else atomicMin(&first[c], (int)v);
+        else if (__ldcg(&first[c]) > (int)v) atomicMin(&first[c], (int)v);
     }
 }
 

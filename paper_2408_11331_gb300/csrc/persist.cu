@@ -291,6 +291,7 @@ __global__ void __launch_bounds__(kBlock, 4)
     __shared__ union {
         EdgeScratch edge[kWarpsPerBlock];
         int4 proposal[kBlock];
+        TileCount tile;
     } scratch;
     DevState* st = a.st;
     unsigned arrivals = 0;                       // at the barrier, over this launch
@@ -321,7 +322,7 @@ __global__ void __launch_bounds__(kBlock, 4)
             table_clear_phase(a, rows, 1);
             scan_write_step(a);
             break;
-        case kScatter: members_scatter_phase(a, 1); break;
+        case kScatter: members_scatter_phase(a, 1, &scratch.tile); break;
         case kBuild: table_build_phase(a, 1); break;
         case kTop: summ_top_phase(a, 1); break;
         case kHeavyEval: h_eval_phase<kSingle>(a); break;

@@ -138,18 +138,67 @@ __device__ __forceinline__ int warp_incl_scan(int x, int lane)
     return x;
 }
 
-__device__ __forceinline__ void members_scatter_phase(const SweepArgs& a, int conditional)
+// Cluster ids of a tile of vertices counted in shared memory, so that a block
+// adds to a cluster's word in global memory once per tile instead of once per
+// vertex: adds to one word take about 10 ns each, and the largest clusters
+// hold several percent of the vertices (n = 1e6, 200 clusters: 233 -> 45 us).
+constexpr int kTile = 4 * kBlock;
+struct TileCount {
+    int key[2 * kTile], cnt[2 * kTile];
+};
+
+// All threads of the block; ids: this thread's four (-1: none).  Leaves the
+// entry of each in slot and its number among the tile's equal ones in rank.
+__device__ __forceinline__ void tile_count(TileCount* tc, const int (&id)[4], int (&slot)[4], int (&rank)[4])
+{
+    for (int s = threadIdx.x; s < 2 * kTile; s += kBlock) {
+        tc->key[s] = -1;
+        tc->cnt[s] = 0;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+        slot[q] = rank[q] = 0;
+        if (id[q] < 0) continue;
+        int h = (int)(((unsigned)id[q] * 0x9E3779B1u) >> 16) & (2 * kTile - 1);
+        // at most kTile ids in twice as many entries: an empty one is found
+        for (int p = 0; p < 2 * kTile; ++p) {
+            const int old = atomicCAS(&tc->key[h], -1, id[q]);
+            if (old == -1 || old == id[q]) break;
+            h = (h + 1) & (2 * kTile - 1);
+        }
+        slot[q] = h;
+        rank[q] = atomicAdd(&tc->cnt[h], 1);
+    }
+    __syncthreads();
+}
+
+__device__ __forceinline__ void members_scatter_phase(const SweepArgs& a, int conditional, TileCount* tc)
 {
     if (rebuild_off(a.st, conditional)) return;
     const bool undone = conditional && a.st->rollback;
-    const long long stride = (long long)gridDim.x * blockDim.x;
-    for (long long v = (long long)blockIdx.x * blockDim.x + threadIdx.x; v < a.n; v += stride) {
-        const int c = a.C[v];
-        const int pos = atomicAdd(&a.cursor[c], 1);
-        if (pos < a.n) a.members[pos] = (int)v;
-        else set_err(a.st, CC_ERR_INVALID);  // sizes inconsistent with C
-        // P1 is being undone: what h_eval computed under it no longer holds
-        if (undone && a.chg[c] == a.st->stamp) a.own[v].y = kOwnNever;
+    for (long long t0 = (long long)blockIdx.x * kTile; t0 < a.n; t0 += (long long)gridDim.x * kTile) {
+        int id[4], slot[4], rank[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const long long v = t0 + q * kBlock + threadIdx.x;
+            id[q] = v < a.n ? a.C[v] : -1;
+        }
+        tile_count(tc, id, slot, rank);
+        for (int s = threadIdx.x; s < 2 * kTile; s += kBlock)
+            if (tc->cnt[s]) tc->cnt[s] = atomicAdd(&a.cursor[tc->key[s]], tc->cnt[s]);
+        __syncthreads();
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const long long v = t0 + q * kBlock + threadIdx.x;
+            if (id[q] < 0) continue;
+            const int pos = tc->cnt[slot[q]] + rank[q];
+            if (pos < a.n) a.members[pos] = (int)v;
+            else set_err(a.st, CC_ERR_INVALID);  // sizes inconsistent with C
+            // P1 is being undone: what h_eval computed under it no longer holds
+            if (undone && a.chg[id[q]] == a.st->stamp) a.own[v].y = kOwnNever;
+        }
+        __syncthreads();
     }
 }
 

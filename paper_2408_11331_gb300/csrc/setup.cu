@@ -205,8 +205,10 @@ __global__ void k_label_sumsq(LabelArgs a, unsigned long long cap)
     const LSlot* m = static_cast<const LSlot*>(a.lmap);
     JobAcc acc(job_smem_init(a.jobs, dyn_jobs), &a.js[0].partition_sq, kJobStride);
     const unsigned long long stride = (unsigned long long)gridDim.x * blockDim.x;
+    int classes = 0;
     for (unsigned long long s = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x; s < cap; s += stride) {
         if (m[s].key == kEmpty) continue;
+        ++classes;
         const long long c = m[s].cnt;
         const int P = (int)(m[s].key >> 32);
         acc.add(a.pjob[P], c * c);
@@ -214,6 +216,9 @@ __global__ void k_label_sumsq(LabelArgs a, unsigned long long cap)
         atomicAdd(a.part_slog + P, (double)c * log((double)c));
     }
     job_acc_finish(acc, a.jobs);
+    for (int o = 16; o > 0; o >>= 1) classes += __shfl_xor_sync(0xffffffffu, classes, o);
+    if ((threadIdx.x & 31) == 0 && classes)
+        atomicAdd(reinterpret_cast<unsigned long long*>(a.classes), (unsigned long long)classes);
 }
 
 // ---- state ----------------------------------------------------------------
@@ -245,14 +250,25 @@ __global__ void k_sizes_zero(SweepArgs a)
 }
 
 // Sizes from a given consensus; an id outside its vertex's job sets an error.
-__global__ void k_count_sizes(SweepArgs a)
+__global__ void __launch_bounds__(kBlock) k_count_sizes(SweepArgs a)
 {
-    const long long stride = (long long)gridDim.x * blockDim.x;
-    for (long long v = (long long)blockIdx.x * blockDim.x + threadIdx.x; v < a.n; v += stride) {
-        const JobInfo& J = a.job[a.jid[v]];
-        const long long c = a.C[v];
-        if (c < J.vo || c >= J.vo + J.n) set_err(a.st, CC_ERR_INVALID);
-        else atomicAdd(&a.size[c], 1);
+    __shared__ TileCount tc;
+    for (long long t0 = (long long)blockIdx.x * kTile; t0 < a.n; t0 += (long long)gridDim.x * kTile) {
+        int id[4], slot[4], rank[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const long long v = t0 + q * kBlock + threadIdx.x;
+            id[q] = -1;
+            if (v >= a.n) continue;
+            const JobInfo& J = a.job[a.jid[v]];
+            const long long c = a.C[v];
+            if (c < J.vo || c >= J.vo + J.n) set_err(a.st, CC_ERR_INVALID);
+            else id[q] = (int)c;
+        }
+        tile_count(&tc, id, slot, rank);
+        for (int s = threadIdx.x; s < 2 * kTile; s += kBlock)
+            if (tc.cnt[s]) atomicAdd(&a.size[tc.key[s]], tc.cnt[s]);
+        __syncthreads();
     }
 }
 
@@ -325,7 +341,8 @@ __global__ void k_table_clear(SweepArgs a, long long rows, int conditional)
 
 __global__ void k_members_scatter(SweepArgs a, int conditional)
 {
-    members_scatter_phase(a, conditional);
+    __shared__ TileCount tc;
+    members_scatter_phase(a, conditional, &tc);
 }
 
 __global__ void __launch_bounds__(kSetupBlock, 6) k_table_build(SweepArgs a, int conditional)
@@ -574,22 +591,37 @@ cudaError_t launch_init_state(const SweepArgs& a, cudaStream_t s)
 cudaError_t launch_state_from_ids(const SweepArgs& a, cudaStream_t s)
 {
     k_sizes_zero<<<grid_for(a.n), kSetupBlock, 0, s>>>(a);
-    k_count_sizes<<<grid_for(a.n), kSetupBlock, 0, s>>>(a);
+    k_count_sizes<<<grid_for(a.n, kTile), kBlock, 0, s>>>(a);
     return cudaGetLastError();
 }
 
-cudaError_t launch_table_rebuild(const SweepArgs& a, long long rows, bool conditional, cudaStream_t s)
+__global__ void k_empty_slots(Slot* t, unsigned long long cap)
 {
+    const unsigned long long stride = (unsigned long long)gridDim.x * blockDim.x;
+    for (unsigned long long s = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x; s < cap; s += stride)
+        reinterpret_cast<ulonglong2*>(t)[s] = make_ulonglong2(kEmpty, 0ull);
+}
+
+cudaError_t launch_empty_slots(Slot* t, unsigned long long cap, cudaStream_t s)
+{
+    k_empty_slots<<<grid_for((long long)cap), kSetupBlock, 0, s>>>(t, cap);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_table_rebuild(const SweepArgs& a, long long rows, bool conditional, cudaStream_t s,
+                                 unsigned long long cap)
+{
+    const long long slots = cap ? (long long)cap : (long long)a.mask_max + 1;
     const int c = conditional ? 1 : 0;
     const int nb = (int)((a.n + 1023) / 1024);
     k_scan_blocks<<<nb, 1024, 0, s>>>(a, c);
     k_scan_sums<<<1, 1024, 0, s>>>(a, nb, c);
     k_scan_write<<<nb, 1024, 0, s>>>(a, c);
-    k_table_clear<<<grid_for(std::max((long long)a.mask_max + 1, rows)), kSetupBlock, 0, s>>>(a, rows, c);
-    k_members_scatter<<<grid_for(a.n), kSetupBlock, 0, s>>>(a, c);
+    k_table_clear<<<grid_for(std::max(slots, rows)), kSetupBlock, 0, s>>>(a, rows, c);
+    k_members_scatter<<<grid_for(a.n, kTile), kBlock, 0, s>>>(a, c);
     k_table_build<<<grid_for(a.n), kSetupBlock, 0, s>>>(a, c);
     k_build_check<<<1, 32, 0, s>>>(a, c);
-    k_summ_top<<<grid_for((long long)a.mask_max + 1), kSetupBlock, 0, s>>>(a, c);
+    k_summ_top<<<grid_for(slots), kSetupBlock, 0, s>>>(a, c);
     k_table_done<<<1, 1, 0, s>>>(a.st, c);
     return cudaGetLastError();
 }
