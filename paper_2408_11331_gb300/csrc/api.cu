@@ -722,18 +722,17 @@ cc_status create_common(int jobs, const JobInput* in, bool on_device, const cc_o
     js0[jobs].stop = 1;
     CC_TRY(cudaMemcpyAsync(c->js, js0.data(), sizeof(JobState) * ((size_t)jobs + 1), cudaMemcpyHostToDevice,
                            c->stream));
-    js0.clear();
 
     const cudaMemcpyKind kind = on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
     // staging: offsets of every job whole (n + 1 each), labels partition-major per job
     {
         long long* offstage = nullptr;
-        long long* d_eo = nullptr;
         int* labels = nullptr;
-        long long* d_lo = nullptr;
-        int* d_pjob = nullptr;
+        unsigned char* d_meta = nullptr;
+        DevState* tst = nullptr;
         void* lmap = nullptr;
-        const unsigned long long lcap = plan.lcap;
+        const unsigned long long most = std::min(plan.lcap, 1ull << 32);
+        unsigned long long lcap = label_map_slots(keys, most);
         std::vector<void*> temp;
         auto tmalloc = [&](void** p, size_t bytes) {
             bytes = bytes > 0 ? bytes : 16;
@@ -748,13 +747,27 @@ cc_status create_common(int jobs, const JobInput* in, bool on_device, const cc_o
                 cudaStreamSynchronize(c->stream);
                 for (void* p : temp) cudaFree(p);
             }
+            temp.clear();
         };
+        // the tables of the assembly and the labels, one copy to the device
+        LabelTiles tl;
+        for (int j = 0; j < jobs; ++j) label_tiles(tl, in[j].n, in[j].k);
+        std::vector<unsigned char> meta;
+        auto put = [&](const void* p, size_t bytes) {
+            const size_t at = (meta.size() + 15) & ~size_t(15);
+            meta.resize(at + bytes);
+            std::memcpy(meta.data() + at, p, bytes);
+            return at;
+        };
+        const size_t at_eo = put(eo.data(), sizeof(long long) * (jobs + 1));
+        const size_t at_lo = put(lo.data(), sizeof(long long) * (jobs + 1));
+        const size_t at_pjob = put(pjob.data(), sizeof(int) * pjob.size());
+        const size_t at_tile = put(tl.tile0.data(), sizeof(int) * (size_t)jobs);
+        const size_t at_turn = put(tl.turn0.data(), sizeof(int) * (size_t)jobs);
         cudaError_t e = tmalloc((void**)&offstage, sizeof(long long) * ((size_t)N + jobs));
-        if (e == cudaSuccess) e = tmalloc((void**)&d_eo, sizeof(long long) * (jobs + 1));
         if (e == cudaSuccess) e = tmalloc((void**)&labels, sizeof(int) * (size_t)keys);
-        if (e == cudaSuccess) e = tmalloc((void**)&d_lo, sizeof(long long) * (jobs + 1));
-        if (e == cudaSuccess) e = tmalloc((void**)&d_pjob, sizeof(int) * pjob.size());
-        int* d_pfirst = c->d_pfirst;
+        if (e == cudaSuccess) e = tmalloc((void**)&d_meta, meta.size());
+        if (e == cudaSuccess) e = tmalloc((void**)&tst, sizeof(DevState));
         if (e == cudaSuccess) e = tmalloc(&lmap, 16 * lcap);
         for (int j = 0; j < jobs && e == cudaSuccess; ++j) {
             const JobInfo& J = c->job[j];
@@ -764,16 +777,14 @@ cc_status create_common(int jobs, const JobInput* in, bool on_device, const cc_o
             if (e == cudaSuccess)
                 e = cudaMemcpyAsync(labels + lo[j], in[j].labels, sizeof(int) * (size_t)(lo[j + 1] - lo[j]), kind, c->stream);
         }
-        if (e == cudaSuccess) e = cudaMemcpyAsync(d_eo, eo.data(), sizeof(long long) * (jobs + 1), cudaMemcpyHostToDevice, c->stream);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(d_lo, lo.data(), sizeof(long long) * (jobs + 1), cudaMemcpyHostToDevice, c->stream);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(d_pjob, pjob.data(), sizeof(int) * pjob.size(), cudaMemcpyHostToDevice, c->stream);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(d_pfirst, pfirst.data(), sizeof(int) * jobs, cudaMemcpyHostToDevice, c->stream);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(d_meta, meta.data(), meta.size(), cudaMemcpyHostToDevice, c->stream);
+        if (e == cudaSuccess) e = cudaMemcpyAsync(c->d_pfirst, pfirst.data(), sizeof(int) * jobs, cudaMemcpyHostToDevice, c->stream);
         AssemblyArgs as{};
         as.jobs = jobs;
         as.n = N;
         as.nnz = NNZ;
         as.offstage = offstage;
-        as.eo = d_eo;
+        as.eo = reinterpret_cast<long long*>(d_meta + at_eo);
         as.job = c->d_job;
         as.off = c->off;
         as.col = c->col;
@@ -781,45 +792,56 @@ cc_status create_common(int jobs, const JobInput* in, bool on_device, const cc_o
         as.jid = c->jid;
         as.st = c->st;
         if (e == cudaSuccess) e = launch_assemble(as, c->stream);
-        DevState s;
-        if (e == cudaSuccess) e = cudaMemcpyAsync(&s, c->st, sizeof(s), cudaMemcpyDeviceToHost, c->stream);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
-        if (e != cudaSuccess) {
-            cleanup();
-            return bail(cuda_fail(c, e, "input assembly"));
-        }
-        if (s.err) {
-            cleanup();
-            return bail(fail(c, CC_ERR_INVALID, "malformed CSR: offsets must start at 0, end at nnz and not decrease; "
-                                                "columns must lie in [0, n)"));
-        }
-        e = launch_assemble_edges(as, c->stream);
         LabelArgs la{};
         la.jobs = jobs;
-        la.total = keys;
-        la.labels = labels;
-        la.lo = d_lo;
-        la.pjob = d_pjob;
-        la.pfirst = d_pfirst;
+            la.labels = labels;
+        la.lo = reinterpret_cast<long long*>(d_meta + at_lo);
+        la.pjob = reinterpret_cast<int*>(d_meta + at_pjob);
+        la.pfirst = c->d_pfirst;
         la.job = c->d_job;
         la.js = c->js;
         la.G = c->G;
-        la.lmap = lmap;
-        la.lmask = lcap - 1;
-        la.rows = rows;
-        la.st = c->st;
-        la.classes = &c->st->classes;
+        la.slots = reinterpret_cast<unsigned*>(c->summ);  // the summary rows are written by the first rebuild
+        la.tiles = tl.tiles;
+        la.turns = tl.turns;
+        la.tile0 = reinterpret_cast<int*>(d_meta + at_tile);
+        la.turn0 = reinterpret_cast<int*>(d_meta + at_turn);
+        la.st = tst;
+        la.classes = &tst->classes;
         la.part_sq = c->part_sq;
         la.part_slog = c->part_slog;
-        if (e == cudaSuccess) e = cudaMemsetAsync(c->part_sq, 0, sizeof(long long) * pjob.size(), c->stream);
-        if (e == cudaSuccess) e = cudaMemsetAsync(c->part_slog, 0, sizeof(double) * pjob.size(), c->stream);
-        if (e == cudaSuccess) e = launch_compact_labels(la, c->stream);
-        if (e == cudaSuccess) e = cudaMemcpyAsync(&s, c->st, sizeof(s), cudaMemcpyDeviceToHost, c->stream);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
+        DevState s, t;
+        for (bool again = true; again && e == cudaSuccess;) {
+            la.lmap = lmap;
+            la.lmask = lcap - 1;
+            la.limit = lcap < most ? kLabelProbes : ~0ull;
+            e = cudaMemsetAsync(tst, 0, sizeof(DevState), c->stream);
+            if (e == cudaSuccess) e = cudaMemsetAsync(c->part_sq, 0, sizeof(long long) * pjob.size(), c->stream);
+            if (e == cudaSuccess) e = cudaMemsetAsync(c->part_slog, 0, sizeof(double) * pjob.size(), c->stream);
+            if (e == cudaSuccess) e = launch_label_kernels(la, c->stream);
+            if (e == cudaSuccess) e = cudaMemcpyAsync(&s, c->st, sizeof(s), cudaMemcpyDeviceToHost, c->stream);
+            if (e == cudaSuccess) e = cudaMemcpyAsync(&t, tst, sizeof(t), cudaMemcpyDeviceToHost, c->stream);
+            if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
+            again = e == cudaSuccess && !s.err && t.err == CC_ERR_TABLE_FULL && lcap < most;
+            if (again) {
+                // many classes: the map that holds any number of them
+                temp.pop_back();
+                if (c->pool) cudaFreeAsync(lmap, c->own_stream);
+                else cudaFree(lmap);
+                lcap = most;
+                e = tmalloc(&lmap, 16 * lcap);
+                if (e == cudaSuccess)
+                    e = cudaMemcpyAsync(c->js, js0.data(), sizeof(JobState) * ((size_t)jobs + 1), cudaMemcpyHostToDevice,
+                                        c->stream);
+            }
+        }
         cleanup();
-        if (e != cudaSuccess) return bail(cuda_fail(c, e, "label compaction"));
-        if (s.err) return bail(fail(c, CC_ERR_INVALID, "malformed CSR: columns must lie in [0, n)"));
-        c->classes = s.classes;
+        if (e != cudaSuccess) return bail(cuda_fail(c, e, "input assembly"));
+        if (s.err)
+            return bail(fail(c, CC_ERR_INVALID, "malformed CSR: offsets must start at 0, end at nnz and not decrease; "
+                                                "columns must lie in [0, n)"));
+        if (t.err) return bail(fail(c, (cc_status)t.err, "label compaction failed"));
+        c->classes = t.classes;
     }
     std::vector<JobState> js;
     if (read_jobs(c, js) != CC_OK) return bail(CC_ERR_CUDA);
@@ -1578,8 +1600,12 @@ cc_status ctx_load_job(cc_ctx* c, int j, const JobInput& in)
     J.lshift = 0;
     while ((1LL << J.lshift) < n) ++J.lshift;
     const long long eo = c->eo[j], keys = n * k;
+    // (the map that holds any number of classes: a second attempt would need
+    // a wait before the keys go in)
     unsigned long long lcap = 64;
     while (lcap < 2ull * (unsigned long long)keys + 64) lcap <<= 1;
+    LabelTiles tl;
+    label_tiles(tl, n, (int)k);
     // staging, from the context's pool when it has one (stream-ordered)
     std::vector<void*> temp;
     auto tmalloc = [&](void** p, size_t bytes) {
@@ -1648,13 +1674,11 @@ cc_status ctx_load_job(cc_ctx* c, int j, const JobInput& in)
     k_load_src<<<g, 256, 0, c->stream>>>(J.vo, n, eo, nnz, nnzcap, ro, c->src);
     // labels: compacted as at creation, into the place's rows
     e = cudaGetLastError();
-    if (e == cudaSuccess) e = cudaMemsetAsync(c->G + J.go, 0xff, sizeof(int) * (size_t)(n * J.kp), c->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(c->part_sq + c->pfirst[j], 0, sizeof(long long) * (size_t)k, c->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(c->part_slog + c->pfirst[j], 0, sizeof(double) * (size_t)k, c->stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(&c->js[j], 0, sizeof(JobState), c->stream);
     LabelArgs la{};
     la.jobs = 1;
-    la.total = keys;
     la.labels = lab;
     la.lo = lo;
     la.pjob = pjob;
@@ -1664,7 +1688,12 @@ cc_status ctx_load_job(cc_ctx* c, int j, const JobInput& in)
     la.G = c->G;
     la.lmap = lmap;
     la.lmask = lcap - 1;
-    la.rows = n * J.kp;
+    la.limit = ~0ull;
+    la.slots = reinterpret_cast<unsigned*>(c->summ + J.go);  // the place's summary rows, written afterwards
+    la.tiles = tl.tiles;
+    la.turns = tl.turns;
+    la.tile0 = pjob;  // (zeros: the one job's first tiles)
+    la.turn0 = pjob;
     la.st = tst;
     la.classes = &tst->classes;
     la.part_sq = c->part_sq + c->pfirst[j];

@@ -35,6 +35,7 @@
 
 #include <cstdint>
 #include <string>
+#include <vector>
 #include <cuda_runtime.h>
 
 #include "cc.h"
@@ -424,16 +425,14 @@ struct AssemblyArgs {
     int* jid;
     DevState* st;
 };
+// (the second does nothing once the first has found the offsets malformed).
 cudaError_t launch_assemble(const AssemblyArgs& a, cudaStream_t s);
-// Second half of the assembly (source array, union columns), once the offsets are valid.
-cudaError_t launch_assemble_edges(const AssemblyArgs& a, cudaStream_t s);
 
 // Label compaction of all jobs: labels staged partition-major per job (job j's
 // k_j x n_j block at lo_j); pjob maps a global partition index (sum of the
 // earlier k plus i) to its job, pfirst the job to its first global partition.
 struct LabelArgs {
     int jobs;
-    long long total;            // sum_j k_j n_j
     const int* labels;          // staged labels
     const long long* lo;        // J + 1: first staged label of each job
     const int* pjob;            // global partition -> job
@@ -443,15 +442,30 @@ struct LabelArgs {
     int* G;
     void* lmap;                 // 16-byte slots, lmask + 1 of them
     unsigned long long lmask;
-    long long rows;             // entries of G
+    unsigned long long limit;   // probes of an insert before st->err is set to CC_ERR_TABLE_FULL
+    unsigned* slots;            // scratch: the map entry of every staged label (total)
+    int tiles, turns;           // tiles of the two passes over the labels, and the first of each job
+    const int* tile0;
+    const int* turn0;
     DevState* st;
     long long* classes;         // label classes of all partitions together
     long long* part_sq;         // per global partition: sum_l |P_il|^2
     double* part_slog;          // per global partition: sum_l |P_il| log |P_il|
 };
-cudaError_t launch_compact_labels(const LabelArgs& a, cudaStream_t s);
-// The same without filling G with -1 first (the caller has set the rows the
-// jobs of `a` write, and only those, to -1).
+// Slots of the label map to try first: a quarter of the labels (or 2^16), as
+// partitions mostly have few classes for their vertices; `most` holds any.
+// An insert that needs more than kLabelProbes probes there gives up
+// (st->err = CC_ERR_TABLE_FULL) and the compaction is run again with `most`.
+constexpr unsigned long long kLabelProbes = 64;
+unsigned long long label_map_slots(long long keys, unsigned long long most);
+// Tiles of the passes over the labels, job by job.
+struct LabelTiles {
+    std::vector<int> tile0, turn0;
+    int tiles = 0, turns = 0;
+};
+void label_tiles(LabelTiles& t, long long n, int k);
+// Fills G (padding included), part_sq, part_slog, classes (added to) and the
+// jobs' partition_sq (added to).  At most 2^32 map slots.
 cudaError_t launch_label_kernels(const LabelArgs& a, cudaStream_t s);
 
 cudaError_t launch_init_state(const SweepArgs& a, cudaStream_t s);

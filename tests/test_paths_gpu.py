@@ -84,3 +84,21 @@ def test_sweeps_around_the_run_kernel(cc, n, k, opts):
             assert job.objective_recompute() == ref.stats[min(s, ref.sweeps - 1)]["F"]
         job.run_until_converged(20)
         np.testing.assert_array_equal(job.cluster_ids(), ref.C)
+
+
+# many classes (more than the first label map takes: 2^16 entries, or a quarter
+# of the labels), one class, and a mix, against the oracle's run
+@pytest.mark.parametrize("n,k,kinds", [(30011, 6, "sssooo"), (70003, 2, "ss"), (1023, 3, "oso"), (1025, 5, "soooo")])
+def test_label_maps(cc, n, k, kinds):
+    rng = np.random.default_rng(n)
+    lab = np.stack([rng.permutation(n).astype(np.int32) - n // 2 if q == "s" else (np.arange(n) // 37).astype(np.int32)
+                    for q in kinds])
+    ro, col = _graph(rng, n)
+    ref = oracle.sync_run(ro, col, lab, 4)
+    with cc.Consensus(ro, col, lab) as job, cc.ConsensusBatch([(ro, col, lab), (ro, col, lab[:1])]) as batch:
+        job.run_until_converged(4)
+        assert job.history() == ref.stats
+        np.testing.assert_array_equal(job.cluster_ids(), ref.C)
+        batch.run_until_converged(4)
+        assert batch.history(0) == ref.stats
+        np.testing.assert_array_equal(batch.cluster_ids()[:n], ref.C)
