@@ -37,11 +37,25 @@ cc_status cuda_fail(cc_ctx* c, cudaError_t e, const char* what)
         if (e_ != cudaSuccess) return cuda_fail(c, e_, #expr); \
     } while (0)
 
+// Device bytes of one allocation of `bytes` (each starts on a multiple of
+// 512 bytes).
+inline size_t rounded(size_t bytes)
+{
+    return (std::max<size_t>(bytes, 16) + 511) & ~size_t(511);
+}
+
 template <typename T>
 cudaError_t dalloc(cc_ctx* c, T** p, size_t count)
 {
+    // from the context's block, which was allocated for everything the plan
+    // counts
+    const size_t bytes = rounded(count * sizeof(T));
+    if (c->block_used + bytes <= c->block_bytes) {
+        *p = reinterpret_cast<T*>(c->block + c->block_used);
+        c->block_used += bytes;
+        return cudaSuccess;
+    }
     void* q = nullptr;
-    const size_t bytes = count * sizeof(T) > 0 ? count * sizeof(T) : 16;
     cudaError_t e = c->pool ? cudaMallocFromPoolAsync(&q, bytes, c->pool, c->own_stream) : cudaMalloc(&q, bytes);
     if (e != cudaSuccess) return e;
     c->allocs.push_back(q);
@@ -465,13 +479,6 @@ cc_status run(cc_ctx* c, int limit, int* done)
     return CC_OK;
 }
 
-// Device bytes of one allocation of `bytes` (allocations are rounded up to
-// 512 bytes or more).
-inline size_t rounded(size_t bytes)
-{
-    return (std::max<size_t>(bytes, 16) + 511) & ~size_t(511);
-}
-
 }  // namespace
 
 namespace ccg {
@@ -573,8 +580,10 @@ void finish_plan(Plan& p, const cc_options& opt)
         const size_t cls[] = {4 * N, 4 * N, 4 * (size_t)p.nnz, 4 * (N + 2), 8 * (N + 2), 16 * (N + 2) + 8};
         for (size_t b : cls) p.persistent += rounded(b);
     }
-    const size_t tmp[] = {8 * (N + J), 8 * (J + 1), 4 * (size_t)p.keys, 8 * (J + 1), 4 * (size_t)p.parts, 4 * J,
-                          16 * (size_t)p.lcap};
+    // (both label maps: the first one tried stays until the second is done)
+    const size_t tmp[] = {8 * (N + J), 8 * (J + 1), 4 * (size_t)p.keys, 8 * (J + 1), 4 * (size_t)p.parts, 8 * J + 64,
+                          sizeof(DevState), 16 * (size_t)p.lcap,
+                          16 * (size_t)label_map_slots((long long)p.keys, p.lcap)};
     for (size_t b : tmp) p.temporary += rounded(b);
 }
 
@@ -670,6 +679,16 @@ cc_status create_common(int jobs, const JobInput* in, bool on_device, const cc_o
     const unsigned long long cap = plan.cap_max;
     c->cap_max = cap;
 
+    // one allocation for the whole context: 36 of them, and their release, took
+    // 3.5 ms for a context of 1.7 GB
+    {
+        void* q = nullptr;
+        CC_TRY(pool ? cudaMallocFromPoolAsync(&q, plan.persistent, pool, c->own_stream) : cudaMalloc(&q, plan.persistent));
+        c->allocs.push_back(q);
+        c->bytes += plan.persistent;
+        c->block = static_cast<unsigned char*>(q);
+        c->block_bytes = plan.persistent;
+    }
     CC_TRY(dalloc(c, &c->d_job, (size_t)jobs + 1));
     CC_TRY(dalloc(c, &c->d_pfirst, (size_t)jobs));
     CC_TRY(dalloc(c, &c->d_lbase, (size_t)jobs + 1));
@@ -764,11 +783,15 @@ cc_status create_common(int jobs, const JobInput* in, bool on_device, const cc_o
         const size_t at_pjob = put(pjob.data(), sizeof(int) * pjob.size());
         const size_t at_tile = put(tl.tile0.data(), sizeof(int) * (size_t)jobs);
         const size_t at_turn = put(tl.turn0.data(), sizeof(int) * (size_t)jobs);
-        cudaError_t e = tmalloc((void**)&offstage, sizeof(long long) * ((size_t)N + jobs));
-        if (e == cudaSuccess) e = tmalloc((void**)&labels, sizeof(int) * (size_t)keys);
-        if (e == cudaSuccess) e = tmalloc((void**)&d_meta, meta.size());
-        if (e == cudaSuccess) e = tmalloc((void**)&tst, sizeof(DevState));
-        if (e == cudaSuccess) e = tmalloc(&lmap, 16 * lcap);
+        const size_t off_b = rounded(sizeof(long long) * ((size_t)N + jobs)), lab_b = rounded(sizeof(int) * (size_t)keys);
+        const size_t meta_b = rounded(meta.size()), st_b = rounded(sizeof(DevState));
+        unsigned char* stage = nullptr;
+        cudaError_t e = tmalloc((void**)&stage, off_b + lab_b + meta_b + st_b + 16 * lcap);
+        offstage = reinterpret_cast<long long*>(stage);
+        labels = reinterpret_cast<int*>(stage + off_b);
+        d_meta = stage + off_b + lab_b;
+        tst = reinterpret_cast<DevState*>(stage + off_b + lab_b + meta_b);
+        lmap = stage + off_b + lab_b + meta_b + st_b;
         for (int j = 0; j < jobs && e == cudaSuccess; ++j) {
             const JobInfo& J = c->job[j];
             e = cudaMemcpyAsync(offstage + J.vo + j, in[j].row_off, sizeof(long long) * ((size_t)J.n + 1), kind, c->stream);
@@ -825,9 +848,6 @@ cc_status create_common(int jobs, const JobInput* in, bool on_device, const cc_o
             again = e == cudaSuccess && !s.err && t.err == CC_ERR_TABLE_FULL && lcap < most;
             if (again) {
                 // many classes: the map that holds any number of them
-                temp.pop_back();
-                if (c->pool) cudaFreeAsync(lmap, c->own_stream);
-                else cudaFree(lmap);
                 lcap = most;
                 e = tmalloc(&lmap, 16 * lcap);
                 if (e == cudaSuccess)
@@ -1627,15 +1647,26 @@ cc_status ctx_load_job(cc_ctx* c, int j, const JobInput& in)
     void* lmap = nullptr;
     JobInfo* dj = nullptr;
     DevState* tst = nullptr;
-    cudaError_t e = tmalloc((void**)&ro, sizeof(long long) * ((size_t)n + 1));
-    if (e == cudaSuccess) e = tmalloc((void**)&col, sizeof(int) * (size_t)nnz);
-    if (e == cudaSuccess) e = tmalloc((void**)&lab, sizeof(int) * (size_t)keys);
-    if (e == cudaSuccess) e = tmalloc((void**)&lo, sizeof(long long) * 2);
-    if (e == cudaSuccess) e = tmalloc((void**)&pjob, sizeof(int) * (size_t)k);
-    if (e == cudaSuccess) e = tmalloc((void**)&pfirst, sizeof(int));
-    if (e == cudaSuccess) e = tmalloc(&lmap, 16 * (size_t)lcap);
-    if (e == cudaSuccess) e = tmalloc((void**)&dj, sizeof(JobInfo));
-    if (e == cudaSuccess) e = tmalloc((void**)&tst, sizeof(DevState));
+    const size_t ro_b = rounded(sizeof(long long) * ((size_t)n + 1)), col_b = rounded(sizeof(int) * (size_t)nnz);
+    const size_t lab_b = rounded(sizeof(int) * (size_t)keys), small_b = 512, pjob_b = rounded(sizeof(int) * (size_t)k);
+    const size_t map_b = 16 * (size_t)lcap, st_b = rounded(sizeof(DevState));
+    unsigned char* stage = nullptr;
+    cudaError_t e = tmalloc((void**)&stage, ro_b + col_b + lab_b + pjob_b + map_b + st_b + 3 * small_b);
+    unsigned char* at = stage;
+    auto part = [&](size_t bytes) {
+        unsigned char* p = at;
+        at += bytes;
+        return p;
+    };
+    ro = reinterpret_cast<long long*>(part(ro_b));
+    col = reinterpret_cast<int*>(part(col_b));
+    lab = reinterpret_cast<int*>(part(lab_b));
+    pjob = reinterpret_cast<int*>(part(pjob_b));
+    lmap = part(map_b);
+    tst = reinterpret_cast<DevState*>(part(st_b));
+    lo = reinterpret_cast<long long*>(part(small_b));
+    pfirst = reinterpret_cast<int*>(part(small_b));
+    dj = reinterpret_cast<JobInfo*>(part(small_b));
     const long long lo_h[2] = {0, keys};
     const int zero = 0;
     DevState s0;

@@ -94,6 +94,8 @@ struct cc_ctx {
     bool started = false;               // start_state ran once
     cc_options opt{};
     std::vector<void*> allocs;
+    unsigned char* block = nullptr;     // the allocation that holds the context's arrays
+    size_t block_bytes = 0, block_used = 0;
     size_t bytes = 0;                   // device bytes held
     std::string err;
     // a run driven without blocking (ctx_async_*)
