@@ -116,6 +116,20 @@ cc_status read_state(cc_ctx* c, DevState* out)
     return CC_OK;
 }
 
+// The control block and the job records in one copy (they lie next to each
+// other, see create_common).
+cc_status read_state_jobs(cc_ctx* c, DevState* out, std::vector<JobState>& js)
+{
+    const size_t at = (size_t)(reinterpret_cast<unsigned char*>(c->js) - reinterpret_cast<unsigned char*>(c->st));
+    std::vector<unsigned char> h(at + sizeof(JobState) * (size_t)c->jobs);
+    CC_CUDA(c, cudaMemcpyAsync(h.data(), c->st, h.size(), cudaMemcpyDeviceToHost, c->stream));
+    CC_CUDA(c, cudaStreamSynchronize(c->stream));
+    js.resize(c->jobs);
+    std::memcpy(out, h.data(), sizeof(DevState));
+    std::memcpy(js.data(), h.data() + at, sizeof(JobState) * (size_t)c->jobs);
+    return CC_OK;
+}
+
 cc_status read_jobs(cc_ctx* c, std::vector<JobState>& out)
 {
     out.resize(c->jobs);
@@ -174,44 +188,18 @@ cc_status objective_recompute(cc_ctx* c, std::vector<long long>& F)
     return check_device_error(c, s);
 }
 
-// Singleton start of every job: C[v] = v, sizes 1, F = F0, history cleared.
+// Singleton start of every job: C[v] = v, sizes 1, F = F0, history cleared
+// (one kernel; a device-side failure of an earlier run is cleared).
 cc_status start_state(cc_ctx* c)
 {
-    DevState s;
-    std::memset(&s, 0, sizeof(s));
-    if (c->started) {
-        DevState prev;
-        cc_status rp = read_state(c, &prev);
-        if (rp != CC_OK) return rp;
-        s.rebuilds = prev.rebuilds;
-        s.retries = prev.retries;
-        s.region_launches = prev.region_launches;
-    }
-    c->started = true;
-    s.stop = 1;
-    s.cls = 0;
-    s.ncls = c->ncls;
-    s.new_mask = c->cap_start - 1;
-    s.mask = c->cap_start - 1;
-    std::vector<JobState> js(c->jobs);
-    for (int j = 0; j < c->jobs; ++j) {
-        std::memset(&js[j], 0, sizeof(JobState));
-        js[j].F = c->F0[j];
-        js[j].partition_sq = c->psq[j];
-        js[j].stop = 1;
-    }
-    CC_CUDA(c, cudaMemcpyAsync(c->st, &s, sizeof(s), cudaMemcpyHostToDevice, c->stream));
-    CC_CUDA(c, cudaMemcpyAsync(c->js, js.data(), sizeof(JobState) * c->jobs, cudaMemcpyHostToDevice, c->stream));
-    CC_CUDA(c, launch_init_state(c->args, c->stream));
-    if (c->opt.sweep_mode == 1) {
-        // staged deltas need the singleton counts in the table from the start
-        CC_CUDA(c, launch_table_rebuild(c->args, c->rows, false, c->stream));
-        c->launches += 1 + kKernelsPerRebuild;
-    } else {
-        // the first sweep rebuilds the table and the summary rows itself (it
-        // is always heavy); singletons are scored from the label rows
-        c->launches += 1;
-    }
+    CC_CUDA(c, launch_init_state(c->args, c->ncls, c->cap_start - 1, c->stream));
+    c->launches += 1;
+    // the first sweep rebuilds the table and the summary rows itself (it is
+    // always heavy), and singletons are scored from the label rows; staged
+    // deltas need the singleton counts in the table from the start
+    if (c->opt.sweep_mode != 1) return CC_OK;
+    CC_CUDA(c, launch_table_rebuild(c->args, c->rows, false, c->stream));
+    c->launches += kKernelsPerRebuild;
     DevState r;
     cc_status rc = read_state(c, &r);
     if (rc != CC_OK) return rc;
@@ -362,7 +350,7 @@ cc_status tune_lanes(cc_ctx* c)
 
 // A run as launches of the run kernel: one unless the run is very long, or
 // the context's lanes are to be timed after its first sweep.
-cc_status run_kernel(cc_ctx* c, int limit, DevState* out)
+cc_status run_kernel(cc_ctx* c, int limit, DevState* out, std::vector<JobState>& js)
 {
     DevState& st = *out;
     long long left = (long long)limit * c->ncls + 64;  // 64: sweeps abandoned for lack of table space and retried
@@ -373,7 +361,7 @@ cc_status run_kernel(cc_ctx* c, int limit, DevState* out)
         if (r != CC_OK) return r;
         CC_CUDA(c, launch_run(c->args, c->rows, c->run_blocks, limit, fresh, budget, c->ts, c->stream));
         c->launches += 1;
-        r = read_state(c, &st);
+        r = read_state_jobs(c, &st, js);
         if (r != CC_OK) return r;
         c->ts_bodies = st.run_bodies - before;
         before = st.run_bodies;
@@ -391,7 +379,7 @@ cc_status run_kernel(cc_ctx* c, int limit, DevState* out)
 
 // A run as graphs of one kernel per step: up to kChunk sweeps unrolled per
 // graph, launched until the device says the run has stopped.
-cc_status run_graphs(cc_ctx* c, int limit, DevState* out)
+cc_status run_graphs(cc_ctx* c, int limit, DevState* out, std::vector<JobState>& js)
 {
     DevState& st = *out;
     CC_CUDA(c, launch_run_begin(c->args, limit, c->stream));
@@ -406,7 +394,7 @@ cc_status run_graphs(cc_ctx* c, int limit, DevState* out)
         if (r != CC_OK) return r;
         CC_CUDA(c, cudaGraphLaunch(g1->exec, c->stream));
         c->launches += c->opt.no_regions ? kKernelsPerSweep : kKernelsOutsideRegions;
-        r = read_state(c, &st);
+        r = read_state_jobs(c, &st, js);
         if (r != CC_OK) return r;
         if (st.run_bodies > 0) {
             float x = 0.f, y = 0.f;
@@ -435,7 +423,7 @@ cc_status run_graphs(cc_ctx* c, int limit, DevState* out)
     for (long long launch = 0; launch < budget && !(before > 0 && (st.stop || st.err)); ++launch) {
         CC_CUDA(c, cudaGraphLaunch(g->exec, c->stream));
         c->launches += (long long)chunk * (c->opt.no_regions ? kKernelsPerSweep : kKernelsOutsideRegions);
-        r = read_state(c, &st);
+        r = read_state_jobs(c, &st, js);
         if (r != CC_OK) return r;
         const int ran = st.run_bodies - before;
         for (int b = 0; b < ran && b < chunk; ++b) {
@@ -458,14 +446,12 @@ cc_status run(cc_ctx* c, int limit, int* done)
     c->propose_ms.clear();
     c->ts_bodies = 0;
     DevState st;
-    cc_status r = c->run_blocks > 0 ? run_kernel(c, limit, &st) : run_graphs(c, limit, &st);
+    std::vector<JobState> js;
+    cc_status r = c->run_blocks > 0 ? run_kernel(c, limit, &st, js) : run_graphs(c, limit, &st, js);
     if (r != CC_OK) return r;
     r = check_device_error(c, st);
     if (r != CC_OK) return r;
     if (!st.stop) return fail(c, CC_ERR_TABLE_FULL, "sweep retries did not converge");
-    std::vector<JobState> js;
-    r = read_jobs(c, js);
-    if (r != CC_OK) return r;
     int most = 0;
     for (const JobState& s : js) most = std::max(most, s.run_sweeps);
     if (done) *done = most;
@@ -694,7 +680,8 @@ cc_status create_common(int jobs, const JobInput* in, bool on_device, const cc_o
     CC_TRY(dalloc(c, &c->d_lbase, (size_t)jobs + 1));
     CC_TRY(dalloc(c, &c->part_sq, (size_t)plan.parts));
     CC_TRY(dalloc(c, &c->part_slog, (size_t)plan.parts));
-    CC_TRY(dalloc(c, &c->js, (size_t)jobs + 1));
+    CC_TRY(dalloc(c, &c->st, 1));
+    CC_TRY(dalloc(c, &c->js, (size_t)jobs + 1));  // next to st: both are read in one copy
     CC_TRY(dalloc(c, &c->off, (size_t)N + 1));
     CC_TRY(dalloc(c, &c->col, (size_t)NNZ));
     CC_TRY(dalloc(c, &c->src, (size_t)NNZ));
@@ -720,7 +707,6 @@ cc_status create_common(int jobs, const JobInput* in, bool on_device, const cc_o
     CC_TRY(dalloc(c, &c->bsum, bsum_entries((size_t)N)));
     CC_TRY(dalloc(c, &c->scratch, 3 * (size_t)N + (size_t)N / 1024 + 64));
     CC_TRY(dalloc(c, &c->ts, 3 * (size_t)kRunBodies));
-    CC_TRY(dalloc(c, &c->st, 1));
     CC_TRY(dalloc(c, &c->hist, (size_t)jobs * c->hist_cap));
     {
         // entry `jobs` is an idle job (no vertices, k = 0, always stopped) for
@@ -865,12 +851,8 @@ cc_status create_common(int jobs, const JobInput* in, bool on_device, const cc_o
     }
     std::vector<JobState> js;
     if (read_jobs(c, js) != CC_OK) return bail(CC_ERR_CUDA);
-    c->F0.resize(jobs);
     c->psq.resize(jobs);
-    for (int j = 0; j < jobs; ++j) {
-        c->psq[j] = js[j].partition_sq;
-        c->F0[j] = c->psq[j] - (long long)c->job[j].k * c->job[j].n;
-    }
+    for (int j = 0; j < jobs; ++j) c->psq[j] = js[j].partition_sq;
     c->cap_start = plan.cap_start;
 
     SweepArgs& a = c->args;
@@ -960,7 +942,10 @@ cc_status create_common(int jobs, const JobInput* in, bool on_device, const cc_o
     int per_sm = 0;
     CC_TRY(prepare_propose(&per_sm));
     if (per_sm < 1) return bail(fail(c, CC_ERR_INVALID, "proposal kernel cannot be resident"));
-    c->grid = c->sms * per_sm;
+    // grids of the sweep graphs: what is resident, or less for a small job (a
+    // launch of 608 blocks for 1000 vertices costs 1 us more than one of 14)
+    const long long fit = std::max({(NNZ + 1023) / 1024, (rows + 2047) / 2048, (N + kBlock - 1) / kBlock});
+    c->grid = (int)std::min<long long>(fit, (long long)c->sms * per_sm);
     if (!c->opt.no_regions && (jobs > 1 || c->opt.colour_batched || rows >= kRunKernelRows))
         CC_TRY(run_grid(a, rows, c->sms, &c->run_blocks));
 
@@ -1761,7 +1746,6 @@ cc_status ctx_load_job(cc_ctx* c, int j, const JobInput& in)
     if (e != cudaSuccess) return cuda_fail(c, e, "load job: records");
     c->job[j] = J;
     c->psq[j] = psq;
-    c->F0[j] = psq - k * n;
     c->classes += chk.classes;  // (an upper bound: the finished job's still count)
     c->async_launches = 0;  // the run's launch budget starts again
     return CC_OK;

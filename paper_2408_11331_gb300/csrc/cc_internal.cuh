@@ -468,7 +468,7 @@ void label_tiles(LabelTiles& t, long long n, int k);
 // jobs' partition_sq (added to).  At most 2^32 map slots.
 cudaError_t launch_label_kernels(const LabelArgs& a, cudaStream_t s);
 
-cudaError_t launch_init_state(const SweepArgs& a, cudaStream_t s);
+cudaError_t launch_init_state(const SweepArgs& a, int ncls, unsigned long long mask, cudaStream_t s);
 // Sizes from C (ids outside their job set CC_ERR_INVALID).
 cudaError_t launch_state_from_ids(const SweepArgs& a, cudaStream_t s);
 // Rebuild of the table and summary rows from C into st->new_mask + 1 slots,

@@ -26,7 +26,6 @@ struct cc_ctx {
     cudaStream_t body_stream = nullptr; // captures the bodies of a sweep graph's conditional regions
     cudaMemPool_t pool = nullptr;       // device memory comes from this pool (stream-ordered) if set
     std::vector<ccg::JobInfo> job;      // host copy of the job table
-    std::vector<long long> F0;          // objective of each job at the singleton start
     std::vector<long long> psq;         // sum_ij |P_ij|^2 of each job
     std::vector<int> pfirst;            // first global partition of each job
     std::vector<long long> eo;          // first CSR entry of each job (jobs + 1)
@@ -91,7 +90,6 @@ struct cc_ctx {
     int ts_bodies = 0;                  // bodies of the last launch not yet in sweep_ms (read when asked for)
     unsigned long long cap_start = 0;   // active table capacity at the singleton start
     unsigned long long cap_max = 0;     // allocated table capacity
-    bool started = false;               // start_state ran once
     cc_options opt{};
     std::vector<void*> allocs;
     unsigned char* block = nullptr;     // the allocation that holds the context's arrays

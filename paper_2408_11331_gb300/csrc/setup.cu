@@ -281,9 +281,28 @@ __global__ void k_label_sumsq(LabelArgs a, unsigned long long cap)
 
 // ---- state ----------------------------------------------------------------
 
-__global__ void k_init_state(SweepArgs a)
+// The control block, the job records and the vertices at the singleton start.
+// The counters since creation stay (rebuilds, retries, kernels in regions).
+__global__ void k_init_state(SweepArgs a, int ncls, unsigned long long mask)
 {
     const long long stride = (long long)gridDim.x * blockDim.x;
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        DevState s{};
+        s.rebuilds = a.st->rebuilds;
+        s.retries = a.st->retries;
+        s.region_launches = a.st->region_launches;
+        s.stop = 1;
+        s.ncls = ncls;
+        s.mask = s.new_mask = mask;
+        *a.st = s;
+    }
+    for (long long j = (long long)blockIdx.x * blockDim.x + threadIdx.x; j < a.jobs; j += stride) {
+        JobState s{};
+        s.partition_sq = a.js[j].partition_sq;
+        s.F = s.partition_sq - (long long)a.job[j].k * a.job[j].n;
+        s.stop = 1;
+        a.js[j] = s;
+    }
     for (long long v = (long long)blockIdx.x * blockDim.x + threadIdx.x; v < a.n; v += stride) {
         a.C[v] = (int)v;
         a.size[v] = 1;
@@ -640,9 +659,9 @@ cudaError_t launch_label_kernels(const LabelArgs& a, cudaStream_t s)
     return cudaGetLastError();
 }
 
-cudaError_t launch_init_state(const SweepArgs& a, cudaStream_t s)
+cudaError_t launch_init_state(const SweepArgs& a, int ncls, unsigned long long mask, cudaStream_t s)
 {
-    k_init_state<<<grid_for(a.n), kSetupBlock, 0, s>>>(a);
+    k_init_state<<<grid_for(a.n), kSetupBlock, 0, s>>>(a, ncls, mask);
     return cudaGetLastError();
 }
 
