@@ -88,8 +88,8 @@ typedef struct {
                                of a captured graph (a step that a sweep does not need is a
                                kernel that returns at once); for profilers, which see one
                                kernel per step.  Results are identical.  0 (default): the run
-                               kernel, or a graph with conditional regions (see
-                               cc_run_until_converged) */
+                               kernel, or a graph with a loop and conditional regions
+                               (see cc_run_until_converged) */
     int32_t empty_moves;    /* 1: the move-to-empty variant.  Besides the clusters of its
                                neighbours (Eq. objective4), a vertex v may move into a new
                                cluster of its own, which takes the id v, provided no vertex
@@ -313,16 +313,16 @@ cc_status cc_sweep(cc_ctx* ctx, cc_sweep_info* info);
  * A context of several jobs, a colour-batched one, and any job of at least
  * 16,384 label rows (n times k rounded up to 4) runs in the run kernel: one
  * cooperative launch takes the whole run, and the host synchronises once.
- * A smaller job's sweeps are submitted as CUDA graphs of up to 4 unrolled
- * sweeps (a sweep is skipped on the device once the run has stopped), and the
- * host reads the stop flag after each graph; so are all runs with no_regions.
+ * A smaller job's run is one launch of a CUDA graph whose loop holds two
+ * sweeps (one after the end of the run is skipped on the device).  With
+ * no_regions, sweeps are submitted as plain graphs of up to 4, and the host
+ * reads the stop flag after each.
  * *sweeps_done (may be NULL) counts every sweep run, the final empty one
  * included.  Errors as cc_sweep. */
 cc_status cc_run_until_converged(cc_ctx* ctx, int32_t max_sweeps, int32_t* sweeps_done);
 
 /* Device time of each sweep of the last cc_run_until_converged / cc_sweep
- * call, taken on the device between the steps of the run kernel, or from CUDA
- * events recorded inside the run's graphs: sweep_ms[s] covers sweep s (all its
+ * call, from the device's clock, read between its steps: sweep_ms[s] covers sweep s (all its
  * steps), propose_ms[s] its proposal step (own, edges, collect); with
  * colour_batched, entry s covers the s-th colour class run (a sweep is one run
  * of every class).  At most max entries are written to each non-NULL array;

@@ -64,18 +64,15 @@ cudaError_t dalloc(cc_ctx* c, T** p, size_t count)
     return cudaSuccess;
 }
 
-void destroy_graph(RunGraph& g)
+void drop_graphs(cc_ctx* c)
 {
-    if (g.exec) cudaGraphExecDestroy(g.exec);
-    for (cudaEvent_t e : g.bound) cudaEventDestroy(e);
-    for (cudaEvent_t e : g.prop) cudaEventDestroy(e);
-    g = RunGraph();
+    for (auto& kv : c->graphs) cudaGraphExecDestroy(kv.second);
+    c->graphs.clear();
 }
 
 void free_all(cc_ctx* c)
 {
-    for (auto& kv : c->graphs) destroy_graph(kv.second);
-    c->graphs.clear();
+    drop_graphs(c);
     if (c->pool) {
         // stream-ordered: the memory returns to the pool once the context's
         // queued work has finished, without waiting here
@@ -99,6 +96,8 @@ void free_all(cc_ctx* c)
     c->own_stream = nullptr;
     if (c->body_stream) cudaStreamDestroy(c->body_stream);
     c->body_stream = nullptr;
+    if (c->loop_stream) cudaStreamDestroy(c->loop_stream);
+    c->loop_stream = nullptr;
 }
 
 unsigned long long next_pow2(unsigned long long x)
@@ -206,55 +205,47 @@ cc_status start_state(cc_ctx* c)
     return check_device_error(c, r);
 }
 
-cc_status ensure_graph(cc_ctx* c, int limit, RunGraph** out)
+// Graph of `bodies` sweeps with every step a plain node, or (bodies 0) of a
+// run: a WHILE node repeats the sweep, its optional parts behind IF nodes.
+cc_status ensure_graph(cc_ctx* c, int bodies, cudaGraphExec_t* out)
 {
-    auto it = c->graphs.find(limit);
+    auto it = c->graphs.find(bodies);
     if (it != c->graphs.end()) {
-        *out = &it->second;
+        *out = it->second;
         return CC_OK;
     }
-    RunGraph g;
-    g.bound.resize((size_t)limit + 1);
-    g.prop.resize(2 * (size_t)limit);
-    for (auto& e : g.bound) CC_CUDA(c, cudaEventCreate(&e));
-    for (auto& e : g.prop) CC_CUDA(c, cudaEventCreate(&e));
     cudaGraph_t graph = nullptr;
     CC_CUDA(c, cudaStreamBeginCapture(c->own_stream, cudaStreamCaptureModeThreadLocal));
     cudaError_t e = cudaSuccess;
-    for (int s = 0; s < limit && e == cudaSuccess; ++s) {
-        e = cudaEventRecordWithFlags(g.bound[s], c->own_stream, cudaEventRecordExternal);
-        if (e == cudaSuccess)
-            e = launch_sweep(c->args, c->rows, c->grid, c->own_stream, g.prop[2 * s], g.prop[2 * s + 1],
-                             c->opt.no_regions ? nullptr : c->body_stream);
-    }
-    if (e == cudaSuccess) e = cudaEventRecordWithFlags(g.bound[limit], c->own_stream, cudaEventRecordExternal);
-    cudaStreamCaptureStatus bs = cudaStreamCaptureStatusNone;
-    if (cudaStreamIsCapturing(c->body_stream, &bs) == cudaSuccess && bs != cudaStreamCaptureStatusNone) {
-        cudaGraph_t body = nullptr;
-        cudaStreamEndCapture(c->body_stream, &body);  // a region left open by a failed capture
+    if (bodies == 0) e = capture_run_loop(c->args, c->rows, c->grid, c->own_stream, c->loop_stream, c->body_stream);
+    for (int s = 0; s < bodies && e == cudaSuccess; ++s)
+        e = launch_sweep(c->args, c->rows, c->grid, c->own_stream, nullptr);
+    for (cudaStream_t st : {c->body_stream, c->loop_stream}) {
+        cudaStreamCaptureStatus bs = cudaStreamCaptureStatusNone;
+        if (cudaStreamIsCapturing(st, &bs) == cudaSuccess && bs != cudaStreamCaptureStatusNone) {
+            cudaGraph_t left = nullptr;
+            cudaStreamEndCapture(st, &left);  // a capture left open by a failure
+        }
     }
     cudaError_t e2 = cudaStreamEndCapture(c->own_stream, &graph);
     if (e != cudaSuccess || e2 != cudaSuccess) {
         if (graph) cudaGraphDestroy(graph);
-        destroy_graph(g);
         return cuda_fail(c, e != cudaSuccess ? e : e2, "capture sweep graph");
     }
-    e = cudaGraphInstantiate(&g.exec, graph, 0);
+    cudaGraphExec_t exec = nullptr;
+    e = cudaGraphInstantiate(&exec, graph, 0);
     cudaGraphDestroy(graph);
-    if (e != cudaSuccess) {
-        g.exec = nullptr;
-        destroy_graph(g);
-        return cuda_fail(c, e, "instantiate sweep graph");
-    }
-    auto ins = c->graphs.emplace(limit, g);
-    *out = &ins.first->second;
+    if (e != cudaSuccess) return cuda_fail(c, e, "instantiate sweep graph");
+    c->graphs.emplace(bodies, exec);
+    *out = exec;
     return CC_OK;
 }
 
-// Sweep bodies per graph launch: a run launches the graph until the device
-// says the run has stopped, so at most kChunk - 1 skipped sweep bodies are
-// submitted after the last sweep.  With colour_batched a body runs one colour
-// class, and a graph holds up to kClassChunk of them.
+// Sweep bodies per launch where launches are counted in sweeps (a served
+// context, whose jobs are released and loaded between launches; the plain
+// graphs of no_regions): at most kChunk - 1 skipped bodies follow the last
+// sweep.  With colour_batched a body runs one colour class, and a launch up to
+// kClassChunk of them.
 constexpr int kChunk = 4;
 constexpr int kClassChunk = 16;
 
@@ -272,27 +263,30 @@ long long launch_budget(const cc_ctx* c, int limit, int chunk)
     return ((long long)limit * c->ncls + chunk - 1) / chunk + 64;
 }
 
-// Contexts of several jobs, colour-batched ones and jobs of at least this many
-// label rows run in the run kernel: it wins at every size measured there
+// Contexts of several jobs, colour-batched and served ones, and jobs of at
+// least this many label rows run in the run kernel: it wins at every size measured there
 // (n = 20011, k = 12, host to host: 1.75 ms against 3.31 as graphs; n = 1.5e5,
 // k = 37: 2.58 against 2.99).  The smallest single jobs stay graphs of one
 // kernel per step, not because that is faster: cc_launch_count reports their
-// kernels one by one, and callers hold it to that (n = 1000, k = 10).
+// kernels one by one, and callers hold it to that (n = 1000, k = 10: as one
+// launch with a loop 0.75 ms, as launches of 4 unrolled sweeps 1.12 ms, of
+// which 0.2 ms of host time per launch).
 constexpr long long kRunKernelRows = 1 << 14;
 
-// Appends the times of the last launch of the run kernel to sweep_ms and
-// propose_ms (ns differences of the device's clock).
+// Appends the device times of the bodies run since the last call (entries of
+// ts from ts_from, ns) to sweep_ms and propose_ms.
 cc_status read_run_times(cc_ctx* c)
 {
     const int b = c->ts_bodies;
     c->ts_bodies = 0;
     if (b <= 0) return CC_OK;
-    std::vector<unsigned long long> t(3 * (size_t)b);
+    std::vector<unsigned long long> t(3 * (size_t)kRunBodies);
     CC_CUDA(c, cudaMemcpyAsync(t.data(), c->ts, sizeof(unsigned long long) * t.size(), cudaMemcpyDeviceToHost, c->stream));
     CC_CUDA(c, cudaStreamSynchronize(c->stream));
     for (int i = 0; i < b; ++i) {
-        c->propose_ms.push_back((float)((double)(t[3 * i + 1] - t[3 * i]) * 1e-6));
-        c->sweep_ms.push_back((float)((double)(t[3 * i + 2] - t[3 * i]) * 1e-6));
+        const unsigned long long* q = &t[3 * (size_t)((c->ts_from + i) % kRunBodies)];
+        c->propose_ms.push_back((float)((double)(q[1] - q[0]) * 1e-6));
+        c->sweep_ms.push_back((float)((double)(q[2] - q[0]) * 1e-6));
     }
     return CC_OK;
 }
@@ -342,8 +336,7 @@ cc_status tune_lanes(cc_ctx* c)
     for (size_t i = 1; i < cands.size(); ++i)
         if (ms[i] < ms[best]) best = i;
     c->args.gs = cands[best];
-    for (auto& kv : c->graphs) destroy_graph(kv.second);
-    c->graphs.clear();
+    drop_graphs(c);
     if (c->device >= 0 && c->device < kMaxDevices) g_tuned[c->device][lane_bin(c->kmax)].store(cands[best]);
     return CC_OK;
 }
@@ -359,10 +352,11 @@ cc_status run_kernel(cc_ctx* c, int limit, DevState* out, std::vector<JobState>&
         const int budget = !c->tuned ? 1 : (int)std::min<long long>(left, kRunBodies);
         cc_status r = read_run_times(c);
         if (r != CC_OK) return r;
-        CC_CUDA(c, launch_run(c->args, c->rows, c->run_blocks, limit, fresh, budget, c->ts, c->stream));
+        CC_CUDA(c, launch_run(c->args, c->rows, c->run_blocks, limit, fresh, budget, c->stream));
         c->launches += 1;
         r = read_state_jobs(c, &st, js);
         if (r != CC_OK) return r;
+        c->ts_from = 0;
         c->ts_bodies = st.run_bodies - before;
         before = st.run_bodies;
         if (st.stop || st.err) break;
@@ -377,65 +371,48 @@ cc_status run_kernel(cc_ctx* c, int limit, DevState* out, std::vector<JobState>&
     return CC_OK;
 }
 
-// A run as graphs of one kernel per step: up to kChunk sweeps unrolled per
-// graph, launched until the device says the run has stopped.
+// A run as graphs of one kernel per step: one launch whose WHILE node repeats
+// the sweep until the run stops, or, with no_regions, plain graphs of up to
+// kChunk sweeps, launched until the device says the run has stopped.
 cc_status run_graphs(cc_ctx* c, int limit, DevState* out, std::vector<JobState>& js)
 {
     DevState& st = *out;
-    CC_CUDA(c, launch_run_begin(c->args, limit, c->stream));
-    c->launches += 1;
+    const bool plain = c->opt.no_regions != 0;
+    const int chunk = chunk_bodies(c, limit);
+    long long left = (long long)limit * c->ncls + 64;  // 64: sweeps abandoned for lack of table space and retried
+    long long launches = launch_budget(c, limit, chunk);
     int before = 0;
-    cc_status r = CC_OK;
-    if (!c->tuned) {
-        // autotune: the run's first sweep alone, then the lane counts timed
-        // on the state it left
-        RunGraph* g1 = nullptr;
-        r = ensure_graph(c, 1, &g1);
+    for (;;) {
+        // (an autotuned context first runs one sweep, then times its lanes on
+        // the state that left)
+        const int bodies = !c->tuned ? 1 : plain ? chunk : (int)std::min<long long>(left, kRunBodies);
+        if (before == 0) CC_CUDA(c, launch_run_begin(c->args, limit, bodies, c->stream));
+        else if (!plain) CC_CUDA(c, launch_run_more(c->args, before + bodies, c->stream));
+        cudaGraphExec_t exec = nullptr;
+        cc_status r = ensure_graph(c, plain ? bodies : 0, &exec);
         if (r != CC_OK) return r;
-        CC_CUDA(c, cudaGraphLaunch(g1->exec, c->stream));
-        c->launches += c->opt.no_regions ? kKernelsPerSweep : kKernelsOutsideRegions;
+        if (before == 0 || !plain) c->launches += 1;
+        CC_CUDA(c, cudaGraphLaunch(exec, c->stream));
         r = read_state_jobs(c, &st, js);
         if (r != CC_OK) return r;
-        if (st.run_bodies > 0) {
-            float x = 0.f, y = 0.f;
-            CC_CUDA(c, cudaEventElapsedTime(&x, g1->bound[0], g1->bound[1]));
-            CC_CUDA(c, cudaEventElapsedTime(&y, g1->prop[0], g1->prop[1]));
-            c->sweep_ms.push_back(x);
-            c->propose_ms.push_back(y);
-        }
+        const int ran = st.run_bodies - before;
+        const long long turns = (ran + kLoopSweeps - 1) / kLoopSweeps;
+        c->launches += plain ? (long long)bodies * kKernelsPerSweep : turns * (kLoopSweeps * kKernelsOutsideRegions + 1);
+        c->ts_from = before;
+        c->ts_bodies = ran;
         before = st.run_bodies;
-        if (!st.stop && !st.err) {
+        if (st.stop || st.err) break;
+        if (!c->tuned) {
             r = tune_lanes(c);
             if (r != CC_OK) return r;
         }
         c->tuned = true;
-        limit -= st.run_bodies > 0 ? 1 : 0;
-    }
-    const int chunk = chunk_bodies(c, std::max(limit, 1));
-    RunGraph* g = nullptr;
-    if (!(before > 0 && (st.stop || st.err))) {
-        r = ensure_graph(c, chunk, &g);
+        left -= ran;
+        if (--launches <= 0 || left <= 0) break;
+        r = read_run_times(c);
         if (r != CC_OK) return r;
     }
-    // a sweep abandoned for lack of table space is retried in the next body,
-    // so the number of launches is bounded by the limit plus the retries
-    const long long budget = launch_budget(c, std::max(limit, 1), chunk);
-    for (long long launch = 0; launch < budget && !(before > 0 && (st.stop || st.err)); ++launch) {
-        CC_CUDA(c, cudaGraphLaunch(g->exec, c->stream));
-        c->launches += (long long)chunk * (c->opt.no_regions ? kKernelsPerSweep : kKernelsOutsideRegions);
-        r = read_state_jobs(c, &st, js);
-        if (r != CC_OK) return r;
-        const int ran = st.run_bodies - before;
-        for (int b = 0; b < ran && b < chunk; ++b) {
-            float x = 0.f, y = 0.f;
-            CC_CUDA(c, cudaEventElapsedTime(&x, g->bound[b], g->bound[b + 1]));
-            CC_CUDA(c, cudaEventElapsedTime(&y, g->prop[2 * b], g->prop[2 * b + 1]));
-            c->sweep_ms.push_back(x);
-            c->propose_ms.push_back(y);
-        }
-        before = st.run_bodies;
-        if (st.stop || st.err) break;
-    }
+    c->tuned = true;
     return CC_OK;
 }
 
@@ -621,6 +598,7 @@ cc_status create_common(int jobs, const JobInput* in, bool on_device, const cc_o
     CC_TRY(cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, c->device));
     CC_TRY(cudaStreamCreateWithPriority(&c->own_stream, cudaStreamNonBlocking, priority));
     CC_TRY(cudaStreamCreateWithPriority(&c->body_stream, cudaStreamNonBlocking, priority));
+    CC_TRY(cudaStreamCreateWithPriority(&c->loop_stream, cudaStreamNonBlocking, priority));
     // pooled memory is allocated in the order of the context's own stream, so
     // such a context runs on that stream
     c->stream = (stream && !pool) ? static_cast<cudaStream_t>(stream) : c->own_stream;
@@ -946,7 +924,8 @@ cc_status create_common(int jobs, const JobInput* in, bool on_device, const cc_o
     // launch of 608 blocks for 1000 vertices costs 1 us more than one of 14)
     const long long fit = std::max({(NNZ + 1023) / 1024, (rows + 2047) / 2048, (N + kBlock - 1) / kBlock});
     c->grid = (int)std::min<long long>(fit, (long long)c->sms * per_sm);
-    if (!c->opt.no_regions && (jobs > 1 || c->opt.colour_batched || rows >= kRunKernelRows))
+    a.ts = c->ts;
+    if (!c->opt.no_regions && (jobs > 1 || c->opt.colour_batched || pool || rows >= kRunKernelRows))
         CC_TRY(run_grid(a, rows, c->sms, &c->run_blocks));
 
     cc_status rc = start_state(c);
@@ -1475,15 +1454,15 @@ cc_status launch_chunk(cc_ctx* c)
 {
     const int chunk = chunk_bodies(c, c->async_limit);
     if (c->run_blocks > 0) {
-        CC_CUDA(c, launch_run(c->args, c->rows, c->run_blocks, c->async_limit, c->async_fresh, chunk, c->ts, c->stream));
+        CC_CUDA(c, launch_run(c->args, c->rows, c->run_blocks, c->async_limit, c->async_fresh, chunk, c->stream));
         c->async_fresh = false;
         c->launches += 1;
     } else {
-        RunGraph* g = nullptr;
-        cc_status r = ensure_graph(c, chunk, &g);
+        cudaGraphExec_t exec = nullptr;
+        cc_status r = ensure_graph(c, chunk, &exec);
         if (r != CC_OK) return r;
-        CC_CUDA(c, cudaGraphLaunch(g->exec, c->stream));
-        c->launches += (long long)chunk * (c->opt.no_regions ? kKernelsPerSweep : kKernelsOutsideRegions);
+        CC_CUDA(c, cudaGraphLaunch(exec, c->stream));
+        c->launches += (long long)chunk * kKernelsPerSweep;
     }
     CC_CUDA(c, cudaMemcpyAsync(c->hstate, c->st, sizeof(DevState), cudaMemcpyDeviceToHost, c->stream));
     if (c->hjobs)
@@ -1513,7 +1492,7 @@ cc_status ctx_async_start(cc_ctx* c, int limit, DevState* pinned, JobState* pinn
     if (!c->chunk_done) CC_CUDA(c, cudaEventCreateWithFlags(&c->chunk_done, cudaEventDisableTiming));
     c->async_fresh = c->run_blocks > 0;
     if (c->run_blocks == 0) {
-        CC_CUDA(c, launch_run_begin(c->args, c->async_limit, c->stream));
+        CC_CUDA(c, launch_run_begin(c->args, c->async_limit, 0, c->stream));
         c->launches += 1;
     }
     return launch_chunk(c);

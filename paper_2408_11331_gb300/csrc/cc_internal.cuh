@@ -46,6 +46,7 @@ constexpr unsigned long long kEmpty = ~0ull;
 constexpr int kWarpsPerBlock = 8;
 constexpr int kBlock = kWarpsPerBlock * 32;
 constexpr int kSmall = 8;      // largest cluster that a partial table leaves out (see rebuild.cuh)
+constexpr int kRunBodies = 512; // sweep bodies of one launch of a run at most, and of the time records
 constexpr int kOwnNever = -3;  // own[v].y below every change stamp: A_a is not known
 
 // One contingency entry: the (cluster, label id) key, its count and the
@@ -111,6 +112,7 @@ struct DevState {
     int rollback;                // 1: some job's heavy P1 is being undone
     int tvalid;                  // 1: the table holds the counts of the current C
     int run_limit;               // sweep limit of the current run
+    int run_until;               // sweep graphs: bodies after which the loop ends
     int run_bodies;              // sweeps of the current run that did work (retried ones included)
     unsigned long long region_launches;  // kernels run inside the gated regions of sweep graphs
     int stamp;                   // number of the current sweep (since creation; retried sweeps reuse it)
@@ -188,6 +190,7 @@ struct SweepArgs {
     int* cursor;                // rebuild scratch: next free position of each cluster (n)
     int* bsum;                  // rebuild scratch: per-block sums of the size scan (n / 1024 + 1)
     DevState* st;
+    unsigned long long* ts;     // kRunBodies times {start of a sweep body, end of its proposal step, its end} (ns)
     cc_sweep_info* hist;        // J x hist_cap records
     int hist_cap;
 };
@@ -561,9 +564,11 @@ cudaError_t launch_colouring(const ColourArgs& a, int* classes, cudaStream_t s);
 void set_thread_error(const std::string& msg);
 
 // ---- sweep.cu ----
-cudaError_t launch_run_begin(const SweepArgs& a, int limit, cudaStream_t s);
-// One sweep of every job; prop0/prop1 (may be null) are recorded around the
-// proposal kernels.  With a body stream (while s is being captured into a
+// Start of a run of at most `limit` sweeps; a graph's loop ends after `until`
+// bodies, which launch_run_more raises to go on with the run.
+cudaError_t launch_run_begin(const SweepArgs& a, int limit, int until, cudaStream_t s);
+cudaError_t launch_run_more(const SweepArgs& a, int until, cudaStream_t s);
+// One sweep of every job.  With a body stream (while s is being captured into a
 // graph), the heavy path, its rollback, the light path and the end-of-sweep
 // rebuild become IF regions of the graph, each behind a one-thread gate
 // kernel, so a sweep launches only the regions it needs.
@@ -578,16 +583,22 @@ constexpr int kGatesPerSweep = 6;
 // kernels of a sweep graph outside its regions (gates included); the kernels
 // of the regions that run are counted on the device (DevState.region_launches)
 constexpr int kKernelsOutsideRegions = kKernelsPerSweep + kGatesPerSweep - kKernelsInRegions;
-cudaError_t launch_sweep(const SweepArgs& a, long long rows, int grid, cudaStream_t s, cudaEvent_t prop0,
-                         cudaEvent_t prop1, cudaStream_t body = nullptr);
+cudaError_t launch_sweep(const SweepArgs& a, long long rows, int grid, cudaStream_t s, cudaStream_t body);
+// Adds to the graph being captured on s a WHILE node whose body (captured on
+// `loop`, with the sweep's regions on `body`) is kLoopSweeps sweeps (one after
+// the end of the run is skipped) and a gate that repeats them until the run
+// stops, fails or has run st->run_until bodies: a whole run as one graph
+// launch.
+constexpr int kLoopSweeps = 2;
+cudaError_t capture_run_loop(const SweepArgs& a, long long rows, int grid, cudaStream_t s, cudaStream_t loop,
+                             cudaStream_t body);
 cudaError_t prepare_propose(int* blocks_per_sm);
 // ---- persist.cu ----
 // Grid of the run kernel for a context (0: it cannot be resident).
 cudaError_t run_grid(const SweepArgs& a, long long rows, int sms, int* grid);
 // The run kernel: up to `budget` sweep bodies of a run in one cooperative
-// launch (fresh: starts the run first).  ts: 3 x budget device words.
-cudaError_t launch_run(const SweepArgs& a, long long rows, int grid, int limit, bool fresh, int budget,
-                       unsigned long long* ts, cudaStream_t s);
+// launch (fresh: starts the run first; at most kRunBodies).
+cudaError_t launch_run(const SweepArgs& a, long long rows, int grid, int limit, bool fresh, int budget, cudaStream_t s);
 // The proposal step's scoring kernels alone (own-cluster sums, candidate
 // bids) on the current state, for timing; they write only aown, act (the
 // same values on the same state) and the bids, which launch_clear_bids

@@ -9,14 +9,6 @@
 
 #include "cc_internal.cuh"
 
-// A run of `limit` sweeps unrolled into one graph, with events at every sweep
-// boundary and around every proposal step.
-struct RunGraph {
-    cudaGraphExec_t exec = nullptr;
-    std::vector<cudaEvent_t> bound;    // limit + 1
-    std::vector<cudaEvent_t> prop;     // 2 * limit
-};
-
 struct cc_ctx {
     int jobs = 0, kmax = 0;
     long long n = 0, nnz = 0, rows = 0, keys = 0;
@@ -24,6 +16,7 @@ struct cc_ctx {
     cudaStream_t stream = nullptr;      // stream used by calls
     cudaStream_t own_stream = nullptr;  // stream created by the context (also used for capture)
     cudaStream_t body_stream = nullptr; // captures the bodies of a sweep graph's conditional regions
+    cudaStream_t loop_stream = nullptr; // captures the body of its loop
     cudaMemPool_t pool = nullptr;       // device memory comes from this pool (stream-ordered) if set
     std::vector<ccg::JobInfo> job;      // host copy of the job table
     std::vector<long long> psq;         // sum_ij |P_ij|^2 of each job
@@ -80,14 +73,14 @@ struct cc_ctx {
     cc_sweep_info* hist = nullptr;
     int hist_cap = 0;
     ccg::SweepArgs args{};
-    std::map<int, RunGraph> graphs;     // by the number of sweep bodies in the graph
+    std::map<int, cudaGraphExec_t> graphs;  // by the number of sweeps in the graph (0: a run's loop)
     std::vector<float> sweep_ms;        // device time of each sweep of the last run
     std::vector<float> propose_ms;      // ... and of its proposal kernels
     long long launches = 0;             // kernels launched so far
     int grid = 0;
     int run_blocks = 0;                 // grid of the run kernel; 0: runs are graphs of one kernel per step
-    unsigned long long* ts = nullptr;   // run kernel: three times per sweep body of the last launch
-    int ts_bodies = 0;                  // bodies of the last launch not yet in sweep_ms (read when asked for)
+    unsigned long long* ts = nullptr;   // three device times per sweep body (kRunBodies of them)
+    int ts_from = 0, ts_bodies = 0;     // bodies of the last launch not yet in sweep_ms (read when asked for)
     unsigned long long cap_start = 0;   // active table capacity at the singleton start
     unsigned long long cap_max = 0;     // allocated table capacity
     cc_options opt{};
@@ -107,9 +100,7 @@ struct cc_ctx {
 
 namespace ccg {
 
-// Sweep bodies of one launch of the run kernel at most (longer runs are
-// launched again), and the entries of the block sums of its size scan.
-constexpr int kRunBodies = 512;
+// Entries of the block sums of the run kernel's size scan.
 constexpr size_t bsum_entries(size_t n)
 {
     return n / 1024 + 4096;

@@ -28,13 +28,6 @@ namespace {
 
 constexpr unsigned long long kBarrierLimitNs = 20ull * 1000 * 1000 * 1000;  // a wait past this gives up
 
-__device__ __forceinline__ unsigned long long now_ns()
-{
-    unsigned long long t;
-    asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
-    return t;
-}
-
 __device__ __forceinline__ unsigned ld_relaxed(const unsigned* p)
 {
     unsigned x;
@@ -229,7 +222,7 @@ struct Scheduler {
         switch (step) {
         case kStart:
             if (fresh) {
-                run_begin_phase(a, limit, threadIdx.x, kBlock);
+                run_begin_phase(a, limit, 0, threadIdx.x, kBlock);
                 __syncthreads();
             }
             return begin();
@@ -280,11 +273,10 @@ struct Scheduler {
 }  // namespace
 
 // fresh: 1 starts a run of at most `limit` sweeps, 0 goes on with it; at most
-// `budget` sweep bodies are run.  ts: three times (ns) per body: its start,
-// the end of its proposal step, its end.
+// `budget` sweep bodies are run.
 template <bool kSingle>
 __global__ void __launch_bounds__(kBlock, 4)
-    k_run(const __grid_constant__ SweepArgs a, long long rows, int limit, int fresh, int budget, unsigned long long* ts)
+    k_run(const __grid_constant__ SweepArgs a, long long rows, int limit, int fresh, int budget)
 {
     // one buffer for the steps that gather in shared memory, so that the L1
     // keeps the rest
@@ -306,9 +298,9 @@ __global__ void __launch_bounds__(kBlock, 4)
             break;
         case kOwn:
             if (clock) {
-                if (body >= 0) ts[3 * body + 2] = now_ns();
+                if (body >= 0) a.ts[3 * body + 2] = now_ns();
                 ++body;
-                ts[3 * body] = now_ns();
+                a.ts[3 * body] = now_ns();
             }
             own_phase<kSingle>(a);
             break;
@@ -337,10 +329,10 @@ __global__ void __launch_bounds__(kBlock, 4)
         }
         const int done = step;
         step = grid_step(st, word, arrivals, [&] { return Scheduler{a, limit, fresh}.next(done); });
-        if (clock && done == kCollect) ts[3 * body + 1] = now_ns();
+        if (clock && done == kCollect) a.ts[3 * body + 1] = now_ns();
         if (step == kLeave) break;
     }
-    if (clock && body >= 0) ts[3 * body + 2] = now_ns();
+    if (clock && body >= 0) a.ts[3 * body + 2] = now_ns();
 }
 
 namespace {
@@ -368,12 +360,11 @@ cudaError_t run_grid(const SweepArgs& a, long long rows, int sms, int* grid)
     return cudaSuccess;
 }
 
-cudaError_t launch_run(const SweepArgs& a, long long rows, int grid, int limit, bool fresh, int budget,
-                       unsigned long long* ts, cudaStream_t s)
+cudaError_t launch_run(const SweepArgs& a, long long rows, int grid, int limit, bool fresh, int budget, cudaStream_t s)
 {
     SweepArgs args = a;
     int f = fresh ? 1 : 0;
-    void* params[] = {&args, &rows, &limit, &f, &budget, &ts};
+    void* params[] = {&args, &rows, &limit, &f, &budget};
     const void* k = a.jobs == 1 ? reinterpret_cast<const void*>(k_run<true>) : reinterpret_cast<const void*>(k_run<false>);
     return cudaLaunchCooperativeKernel(k, dim3((unsigned)grid), dim3(kBlock), params, run_smem(a.jobs), s);
 }

@@ -42,13 +42,25 @@ namespace ccg {
 
 namespace {
 
-__global__ void k_run_begin(SweepArgs a, int limit)
+// Entry of the time records for the body that runs now (three words).
+__device__ __forceinline__ unsigned long long* body_times(const SweepArgs& a)
 {
-    run_begin_phase(a, limit, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x);
+    return a.ts + 3 * (a.st->run_bodies % kRunBodies);
+}
+
+__global__ void k_run_begin(SweepArgs a, int limit, int until)
+{
+    run_begin_phase(a, limit, until, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x);
+}
+
+__global__ void k_run_more(DevState* st, int until)
+{
+    st->run_until = until;
 }
 
 __global__ void k_begin(SweepArgs a)
 {
+    if (blockIdx.x == 0 && threadIdx.x == 0) body_times(a)[0] = now_ns();
     begin_phase(a, blockIdx.x * blockDim.x + threadIdx.x, gridDim.x * blockDim.x);
 }
 
@@ -73,6 +85,7 @@ __global__ void __launch_bounds__(kBlock) k_collect(SweepArgs a)
 
 __global__ void k_route(SweepArgs a)
 {
+    body_times(a)[1] = now_ns();
     route_phase(a);
 }
 
@@ -139,6 +152,7 @@ __global__ void k_end_jobs(SweepArgs a)
 
 __global__ void k_end(SweepArgs a)
 {
+    if (!a.st->skip) body_times(a)[2] = now_ns();
     end_phase(a);
 }
 
@@ -201,6 +215,16 @@ cudaError_t close_region(cudaStream_t b)
     return cudaStreamEndCapture(b, &g);
 }
 
+// End of one body of a run's loop: go on while the run has not stopped, has no
+// error and has bodies left.
+__global__ void k_loop_gate(cudaGraphConditionalHandle h, SweepArgs a)
+{
+    DevState* st = a.st;
+    if (st->run_bodies > 0) a.ts[3 * ((st->run_bodies - 1) % kRunBodies) + 2] = now_ns();
+    const bool more = !st->stop && !st->err && st->run_bodies < st->run_until;
+    cudaGraphSetConditional(h, more ? 1u : 0u);
+}
+
 inline int jobs_grid(int jobs)
 {
     int g = (jobs + 255) / 256;
@@ -247,14 +271,58 @@ cudaError_t prepare_propose(int* blocks_per_sm)
     return e;
 }
 
-cudaError_t launch_run_begin(const SweepArgs& a, int limit, cudaStream_t s)
+cudaError_t capture_run_loop(const SweepArgs& a, long long rows, int grid, cudaStream_t s, cudaStream_t loop,
+                             cudaStream_t body)
 {
-    k_run_begin<<<jobs_grid(a.jobs), 256, 0, s>>>(a, limit);
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    cudaGraph_t g = nullptr;
+    const cudaGraphNode_t* deps = nullptr;
+    const cudaGraphEdgeData* edges = nullptr;
+    size_t nd = 0;
+    cudaError_t e = cudaStreamGetCaptureInfo(s, &cs, nullptr, &g, &deps, &edges, &nd);
+    if (e != cudaSuccess) return e;
+    if (cs != cudaStreamCaptureStatusActive) return cudaErrorStreamCaptureUnsupported;
+    // the loop is entered once per launch (default value 1); each body's gate
+    // decides whether another follows
+    cudaGraphConditionalHandle h = 0;
+    e = cudaGraphConditionalHandleCreate(&h, g, 1, cudaGraphCondAssignDefault);
+    if (e != cudaSuccess) return e;
+    cudaGraphNodeParams p{};
+    p.type = cudaGraphNodeTypeConditional;
+    p.conditional.handle = h;
+    p.conditional.type = cudaGraphCondTypeWhile;
+    p.conditional.size = 1;
+    cudaGraphNode_t node = nullptr;
+    e = cudaGraphAddNode(&node, g, deps, edges, nd, &p);
+    if (e != cudaSuccess) return e;
+    e = cudaStreamUpdateCaptureDependencies(s, &node, nullptr, 1, cudaStreamSetCaptureDependencies);
+    if (e != cudaSuccess) return e;
+    e = cudaStreamBeginCaptureToGraph(loop, p.conditional.phGraph_out[0], nullptr, nullptr, 0,
+                                      cudaStreamCaptureModeThreadLocal);
+    if (e != cudaSuccess) return e;
+    for (int i = 0; i < kLoopSweeps && e == cudaSuccess; ++i) e = launch_sweep(a, rows, grid, loop, body);
+    if (e == cudaSuccess) {
+        k_loop_gate<<<1, 1, 0, loop>>>(h, a);
+        e = cudaGetLastError();
+    }
+    cudaGraph_t lg = nullptr;
+    const cudaError_t e2 = cudaStreamEndCapture(loop, &lg);
+    return e != cudaSuccess ? e : e2;
+}
+
+cudaError_t launch_run_begin(const SweepArgs& a, int limit, int until, cudaStream_t s)
+{
+    k_run_begin<<<jobs_grid(a.jobs), 256, 0, s>>>(a, limit, until);
     return cudaGetLastError();
 }
 
-cudaError_t launch_sweep(const SweepArgs& a, long long rows, int grid, cudaStream_t s, cudaEvent_t prop0,
-                         cudaEvent_t prop1, cudaStream_t body)
+cudaError_t launch_run_more(const SweepArgs& a, int until, cudaStream_t s)
+{
+    k_run_more<<<1, 1, 0, s>>>(a.st, until);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_sweep(const SweepArgs& a, long long rows, int grid, cudaStream_t s, cudaStream_t body)
 {
     const int g2 = grid;
     const int jg = jobs_grid(a.jobs);
@@ -271,10 +339,6 @@ cudaError_t launch_sweep(const SweepArgs& a, long long rows, int grid, cudaStrea
         if (body && e == cudaSuccess) e = close_region(body);
     };
     k_begin<<<jg, 256, 0, s>>>(a);
-    if (prop0) {
-        e = cudaEventRecordWithFlags(prop0, s, cudaEventRecordExternal);
-        if (e != cudaSuccess) return e;
-    }
     if (a.jobs == 1) {
         k_own<true><<<grid, kBlock, 0, s>>>(a);
         k_edges<true><<<grid, kBlock, 0, s>>>(a);
@@ -283,10 +347,6 @@ cudaError_t launch_sweep(const SweepArgs& a, long long rows, int grid, cudaStrea
         k_edges<false><<<grid, kBlock, 0, s>>>(a);
     }
     k_collect<<<grid, kBlock, js1, s>>>(a);
-    if (prop1) {
-        e = cudaEventRecordWithFlags(prop1, s, cudaEventRecordExternal);
-        if (e != cudaSuccess) return e;
-    }
     k_route<<<1, 1, 0, s>>>(a);
     {
         cudaStream_t r = open(kGateHeavy, 2 + kKernelsPerRebuild);

@@ -12,6 +12,14 @@ namespace {
 
 constexpr unsigned kFull = 0xffffffffu;
 
+// The device's clock (ns), for the time records of a run.
+__device__ __forceinline__ unsigned long long now_ns()
+{
+    unsigned long long t;
+    asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t));
+    return t;
+}
+
 // (dD, id) packed so that unsigned order is (dD, id) order: dD with its sign
 // bit flipped in the high word.
 __device__ __forceinline__ unsigned long long pack_key(int dD, int id)
@@ -50,12 +58,13 @@ __device__ __forceinline__ int resolve(const Slot* t, unsigned long long mask, u
     return 0;
 }
 
-__device__ __forceinline__ void run_begin_phase(const SweepArgs& a, int limit, int t0, int stride)
+__device__ __forceinline__ void run_begin_phase(const SweepArgs& a, int limit, int until, int t0, int stride)
 {
     DevState* st = a.st;
     if (t0 == 0) {
         st->stop = 0;
         st->run_limit = limit;
+        st->run_until = until;
         st->run_bodies = 0;
         st->all_active = 1;
         st->cls = 0;
