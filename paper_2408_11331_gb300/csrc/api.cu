@@ -857,6 +857,7 @@ cc_status create_common(int jobs, const JobInput* in, bool on_device, const cc_o
     a.keys = (unsigned long long)keys;
     a.sweep_mode = c->opt.sweep_mode;
     a.gs = c->opt.lanes > 0 ? c->opt.lanes : lanes_for_k(kmax);
+    a.gs_set = c->opt.lanes > 0 ? 1 : 0;
     // autotune: a choice made earlier on this device for the same lane bin is
     // used as it is; otherwise the first run times the candidates
     c->tuned = true;
@@ -922,7 +923,7 @@ cc_status create_common(int jobs, const JobInput* in, bool on_device, const cc_o
     if (per_sm < 1) return bail(fail(c, CC_ERR_INVALID, "proposal kernel cannot be resident"));
     // grids of the sweep graphs: what is resident, or less for a small job (a
     // launch of 608 blocks for 1000 vertices costs 1 us more than one of 14)
-    const long long fit = std::max({(NNZ + 1023) / 1024, (rows + 2047) / 2048, (N + kBlock - 1) / kBlock});
+    const long long fit = std::max({(NNZ + kBlock - 1) / kBlock, (rows + 2047) / 2048, (N + kBlock - 1) / kBlock});
     c->grid = (int)std::min<long long>(fit, (long long)c->sms * per_sm);
     a.ts = c->ts;
     if (!c->opt.no_regions && (jobs > 1 || c->opt.colour_batched || pool || rows >= kRunKernelRows))

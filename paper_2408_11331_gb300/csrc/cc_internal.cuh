@@ -169,6 +169,7 @@ struct SweepArgs {
     unsigned long long keys;     // sum_j k_j n_j: no C has more live keys
     int sweep_mode;              // 0 automatic, 1 always staged deltas, 2 always rebuild
     int gs;                      // lanes that score one item (a power of two, 1..32)
+    int gs_set;                  // 1: set by the caller (cc_options.lanes)
     int active_set;              // 1: score only the active vertices (cc_options.active_set)
     int empty_moves;             // 1: a vertex may also move into a new cluster with its own id (cc_options.empty_moves)
     int tight_mode;              // cc_options.tight_rebuild: 0 tight attempt first, 1 never, 2 always dropped
@@ -193,6 +194,30 @@ struct SweepArgs {
     unsigned long long* ts;     // kRunBodies times {start of a sweep body, end of its proposal step, its end} (ns)
     cc_sweep_info* hist;        // J x hist_cap records
     int hist_cap;
+};
+
+// The block's share of a step's items (each one warp's work, of uneven cost):
+// kWarpsPerBlock consecutive ones of every gridDim.x times that many, which
+// its warps take one after another from a counter in shared memory, so that
+// they end together.  start() is called by the whole block, next() by a whole
+// warp; the items are used up when next() passes their number.
+struct WarpQueue {
+    int* taken;  // shared
+
+    __device__ __forceinline__ void start() const
+    {
+        __syncthreads();
+        if (threadIdx.x == 0) *taken = 0;
+        __syncthreads();
+    }
+
+    __device__ __forceinline__ long long next() const
+    {
+        int i = 0;
+        if ((threadIdx.x & 31) == 0) i = atomicAdd(taken, 1);
+        i = __shfl_sync(0xffffffffu, i, 0);
+        return ((long long)(i / kWarpsPerBlock) * gridDim.x + blockIdx.x) * kWarpsPerBlock + i % kWarpsPerBlock;
+    }
 };
 
 // Row of vertex / cluster x (a union vertex id) of job J in G or summ.
@@ -232,15 +257,15 @@ __device__ __forceinline__ unsigned long long ckey(int c, int g)
     return ((unsigned long long)(unsigned)c << 32) | (unsigned)g;
 }
 
-// Keeps the summary row of the slot's (cluster, partition) exact after its
-// count changed by d: only the counts of the row's two labels are stored.
-__device__ __forceinline__ void summ_update(const SweepArgs& a, unsigned long long key, int d)
+// Keeps the summary entry of (cluster x, partition p) of job J exact after the
+// count of label g there changed by d: only the counts of the entry's two
+// labels are stored.
+__device__ __forceinline__ void summ_update(const SweepArgs& a, const JobInfo& J, int x, int p, int g, int d)
 {
-    const int x = (int)(key >> 32), g = (int)(unsigned)(key & 0xffffffffull);
-    const JobInfo& J = a.job[a.jid[x]];
-    int4* S = a.summ + row_of(J, x) + (g >> J.lshift);
-    if (S->x == g) atomicAdd(&S->y, d);
-    else if (S->z == g) atomicAdd(&S->w, d);
+    int4* S = a.summ + row_of(J, x) + p;
+    const int d1 = S->x, d2 = S->z;
+    if (d1 == g) atomicAdd(&S->y, d);
+    else if (d2 == g) atomicAdd(&S->w, d);
 }
 
 __device__ __forceinline__ void set_err(DevState* st, int code)

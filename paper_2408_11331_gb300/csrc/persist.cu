@@ -86,6 +86,7 @@ __device__ __forceinline__ int grid_step(DevState* st, unsigned& word, unsigned&
         // relaxed polls and one fence at the end: an acquire on every poll
         // would drop the L1 lines of the blocks still at work on this SM
         for (unsigned spins = 1; (now = ld_relaxed(&st->bar_word)) == word; ++spins) {
+            __nanosleep(100);
             if (spins & 1023u) continue;
             if (t0 == 0) t0 = now_ns();
             if (*reinterpret_cast<volatile int*>(&st->bar_abort) || now_ns() - t0 > kBarrierLimitNs) {
@@ -196,7 +197,8 @@ struct Scheduler {
         if (a.st->bodies_left <= 0) return kLeave;
         begin_phase(a, threadIdx.x, kBlock);
         __syncthreads();
-        return a.st->skip ? kLeave : kOwn;
+        // the own step only serves these options
+        return a.st->skip ? kLeave : a.active_set || a.empty_moves ? kOwn : kEdges;
     }
 
     // Objective, history and stop per job; then the end-of-sweep rebuild or
@@ -289,21 +291,20 @@ __global__ void __launch_bounds__(kBlock, 4)
     unsigned arrivals = 0;                       // at the barrier, over this launch
     unsigned word = ld_relaxed(&st->bar_word);   // cannot change before this block arrives
     const bool clock = blockIdx.x == 0 && threadIdx.x == 0;
-    int step = kStart, body = -1;
+    int step = kStart, last = kStart, body = -1;
     // every step ends in a barrier; kLeave ends the kernel
     for (;;) {
+        if (clock && (step == kOwn || (step == kEdges && last != kOwn))) {
+            // a sweep begins
+            if (body >= 0) a.ts[3 * body + 2] = now_ns();
+            ++body;
+            a.ts[3 * body] = now_ns();
+        }
         switch (step) {
         case kStart:
             if (clock) st->bodies_left = budget;
             break;
-        case kOwn:
-            if (clock) {
-                if (body >= 0) a.ts[3 * body + 2] = now_ns();
-                ++body;
-                a.ts[3 * body] = now_ns();
-            }
-            own_phase<kSingle>(a);
-            break;
+        case kOwn: own_phase<kSingle>(a); break;
         case kEdges: edges_phase<kSingle>(a, scratch.edge); break;
         case kCollect: collect_phase(a, scratch.proposal); break;
         case kMark: h_mark_phase(a); break;
@@ -331,14 +332,15 @@ __global__ void __launch_bounds__(kBlock, 4)
         step = grid_step(st, word, arrivals, [&] { return Scheduler{a, limit, fresh}.next(done); });
         if (clock && done == kCollect) a.ts[3 * body + 1] = now_ns();
         if (step == kLeave) break;
+        last = done;
     }
     if (clock && body >= 0) a.ts[3 * body + 2] = now_ns();
 }
 
 namespace {
 
-// Blocks of a run of this context: one warp per window of the proposal step's
-// CSR entries and one thread per 8 label rows, at most what is resident.
+// Blocks of a run of this context: one thread per CSR entry or vertex and per
+// 8 label rows, at most what is resident.
 inline size_t run_smem(int jobs)
 {
     return (2 * jobs <= kSmemJobs ? 2 : 1) * smem_jobs_bytes(jobs);
@@ -353,8 +355,7 @@ cudaError_t run_grid(const SweepArgs& a, long long rows, int sms, int* grid)
         a.jobs == 1 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_run<true>, kBlock, run_smem(a.jobs))
                     : cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_run<false>, kBlock, run_smem(a.jobs));
     if (e != cudaSuccess) return e;
-    const long long span = 32LL * kChunks * kWarpsPerBlock;
-    long long g = std::max((a.nnz + span - 1) / span, (rows + 8 * kBlock - 1) / (8 * kBlock));
+    long long g = std::max((a.nnz + kBlock - 1) / kBlock, (rows + 8 * kBlock - 1) / (8 * kBlock));
     g = std::max(g, (a.n + kBlock - 1) / kBlock);
     *grid = (int)std::max(0LL, std::min(g, (long long)per_sm * sms));
     return cudaSuccess;

@@ -227,6 +227,24 @@ __device__ __forceinline__ unsigned long long segment_max(unsigned long long x, 
 // the warps stop inserting.
 constexpr unsigned long long kTightProbes = 256;
 
+// Claims an empty slot for key if on; returns the key found there (key itself
+// where off).  One predicated instruction, so that several follow each other
+// without waiting for a result.
+__device__ __forceinline__ unsigned long long key_cas_if(unsigned on, unsigned long long* slot, unsigned long long key)
+{
+    unsigned long long old = key;
+    asm volatile(
+        "{\n\t"
+        ".reg .pred p;\n\t"
+        "setp.ne.u32 p, %3, 0;\n\t"
+        "@p atom.relaxed.gpu.global.cas.b64 %0, [%1], %4, %2;\n\t"
+        "}"
+        : "+l"(old)
+        : "l"(slot), "l"(key), "r"(on), "l"(kEmpty)
+        : "memory");
+    return old;
+}
+
 __device__ __forceinline__ void table_build_phase(const SweepArgs& a, int conditional)
 {
     DevState* st = a.st;
@@ -238,15 +256,24 @@ __device__ __forceinline__ void table_build_phase(const SweepArgs& a, int condit
     const bool tight = conditional && st->tight != 0;
     const unsigned long long limit = tight ? kTightProbes : ~0ull;
     const int small = conditional ? st->build_small : 0;
-    __syncthreads();
     const unsigned long long mask = st->new_mask;
-    const long long stride = (long long)gridDim.x * blockDim.x;
     const int lane = threadIdx.x & 31;
     unsigned created = 0;  // slots this lane created
-    for (long long base = (long long)blockIdx.x * blockDim.x; base < a.n; base += stride) {
+    // an item is a window of 32 members and a run of quads of partitions: a
+    // window alone is too long a chain (one round of inserts per quad) for
+    // the warps to end together when they get only a few each
+    const long long nwarps = (long long)gridDim.x * kWarpsPerBlock, windows = (a.n + 31) >> 5;
+    const int kq = (a.kmax + 3) >> 2;
+    const int parts = (int)max(1LL, min((long long)kq, (8 * nwarps + windows - 1) / windows));
+    const int run_q = (kq + parts - 1) / parts;
+    __shared__ int s_taken;
+    const WarpQueue queue{&s_taken};
+    queue.start();
+    for (long long item = queue.next(); item < windows * parts; item = queue.next()) {
         if (tight && __any_sync(0xffffffffu, *reinterpret_cast<volatile int*>(&st->build_fail) != 0)) break;
-        const long long m = base + threadIdx.x;
-        const long long wb = m - lane;  // first member of this warp's window
+        const long long window = item / parts;
+        const int first_i = 4 * run_q * (int)(item - window * parts), last_i = min(a.kmax, first_i + 4 * run_q);
+        const long long wb = window * 32, m = wb + lane;  // the warp's members
         bool valid = m < a.n;
         int v = 0, c = 0, k = 0, seg_end = lane + 1;
         bool whole = false;
@@ -261,6 +288,11 @@ __device__ __forceinline__ void table_build_phase(const SweepArgs& a, int condit
         if (valid) {
             const JobInfo& J = a.job[a.jid[v]];
             k = J.k;
+            if (k <= first_i) valid = false;
+        }
+        if (!__any_sync(0xffffffffu, valid)) continue;
+        if (valid) {
+            const JobInfo& J = a.job[a.jid[v]];
             row = a.G + row_of(J, v);
             // after the scatter, cursor[c] is one past the cluster's last member
             const long long end = a.cursor[c], first = end - a.size[c];
@@ -287,7 +319,7 @@ __device__ __forceinline__ void table_build_phase(const SweepArgs& a, int condit
         const unsigned long long mark = whole ? (1ull << 32) : 0ull;
         // four partitions at a time: one quad of the label row, and the four
         // keys' first CASes issued before any result is used
-        for (int i0 = 0; i0 < a.kmax; i0 += 4) {
+        for (int i0 = first_i; i0 < last_i; i0 += 4) {
             int4 g4 = make_int4(0, 0, 0, 0);
             if (valid && i0 < k) g4 = __ldg(G4 + (i0 >> 2));
             const int gq[4] = {g4.x, g4.y, g4.z, g4.w};
@@ -312,11 +344,10 @@ __device__ __forceinline__ void table_build_phase(const SweepArgs& a, int condit
                 }
                 unsigned long long old[4];
 #pragma unroll
-                for (int b = 0; b < 4; ++b)
-                    if (pend >> b & 1u) {
-                        const unsigned long long key = ckey(c, gq[b]);
-                        old[b] = atomicCAS(&a.table[(hash_key(key) + p) & mask].key, kEmpty, key);
-                    }
+                for (int b = 0; b < 4; ++b) {
+                    const unsigned long long key = ckey(c, gq[b]);
+                    old[b] = key_cas_if(pend >> b & 1u, &a.table[(hash_key(key) + p) & mask].key, key);
+                }
 #pragma unroll
                 for (int b = 0; b < 4; ++b)
                     if (pend >> b & 1u) {

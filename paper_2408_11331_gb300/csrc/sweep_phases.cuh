@@ -380,20 +380,26 @@ __device__ __forceinline__ void own_phase(const SweepArgs& a)
 // One window of CSR entries of one warp in shared memory: kChunks chunks of
 // 32 entries are gathered before scoring, so that the scoring rounds (32 / gs
 // candidates each) run nearly full.  Candidates: singletons from the front,
-// other clusters from the back.  Slots: the distinct vertices of the window.
+// other clusters from the back.  Slots: the distinct vertices of the window,
+// kSlots of them scored at a time (more in one window are rare).  The size
+// matters: four blocks' scratch (29 KB each) leave 96 KB of the SM's memory to
+// the L1 that the gathers of rows go through; at 40 KB (64 KB of L1) the step
+// took 7% longer, with no L1 to speak of 54%.
 constexpr int kChunks = 4;
 constexpr int kSpan = 32 * kChunks;
+constexpr int kSlots = 64;
 static_assert(16 * kSmall <= kSpan, "the pairs of 16 small candidates must fit the scratch");
 struct EdgeScratch {
-    unsigned long long ubest[kSpan];  // slot: upper bound on the vertex's final bid
-    int x[kSpan];                     // candidate: cluster,
-    int w[kSpan];                     //   its size (singleton: its vertex),
-    int lo[kSpan];                    //   least dD (small clusters: the members of the pairs),
-    int part[kSpan];                  //   exact part of A_x
-    int v[kSpan];                     // slot: vertex,
-    int base[kSpan];                  //   2 (A_a - k) - k (|a| - 1), so dD = base + k |x| - 2 A_x,
-    unsigned top[kSpan];              //   its largest candidate: |x| << 7 | index (0: none)
-    unsigned char slot[kSpan], list[kSpan], pair[kSpan];
+    unsigned long long ubest[kSlots];  // slot: upper bound on the vertex's final bid
+    int base[kSlots];                  //   2 (A_a - k) - k (|a| - 1), so dD = base + k |x| - 2 A_x
+    int v[kSpan];                      // vertex of each slot of the window
+    int x[kSpan];                      // candidate: cluster,
+    int w[kSpan];                      //   its size (singleton: its vertex),
+    int lo[kSpan];                     //   least dD.  Before that: the clusters of the slots, then each slot's
+                                       //   largest candidate (|x| << 7 | index); small clusters: members of the pairs
+    int part[kSpan];                   //   exact part of A_x
+    unsigned char slot[kSpan];         //   its slot, | 128 if it is its vertex's largest
+    unsigned char list[kSpan], pair[kSpan];
 };
 
 // The proposal step's scoring.  CSR entries 32 at a time per warp: each lane
@@ -443,8 +449,17 @@ __device__ __forceinline__ void edges_phase(const SweepArgs& a, EdgeScratch* sh)
         eidx = a.eidx + e0;
         count = a.eoff[st->cls + 1] - e0;
     }
-    const unsigned windows = (unsigned)((count + kSpan - 1) / kSpan);
-    for (unsigned win = blockIdx.x * kWarpsPerBlock + w; win < windows; win += gridDim.x * kWarpsPerBlock) {
+    // entries of a window: fewer than kSpan where that leaves warps idle (a
+    // small job, a colour class), for the window's latency is then the step's
+    const unsigned nwarps = gridDim.x * kWarpsPerBlock;
+    const int span = count >= (long long)kSpan * nwarps
+                         ? kSpan
+                         : 32 * (int)max(1LL, min((long long)kChunks, (count + 32 * nwarps - 1) / (32 * nwarps)));
+    const long long windows = (count + span - 1) / span;
+    __shared__ int s_taken;
+    const WarpQueue queue{&s_taken};
+    queue.start();
+    for (long long win = queue.next(); win < windows; win = queue.next()) {
         int ns = 0, nt = 0, slots = 0;
         // the loads of all kChunks chunks first (entries, then clusters, then
         // sizes), so that their latencies overlap; then each chunk's votes
@@ -452,10 +467,10 @@ __device__ __forceinline__ void edges_phase(const SweepArgs& a, EdgeScratch* sh)
         int vc[kChunks], uc[kChunks], xc[kChunks], sc[kChunks];
 #pragma unroll
         for (int c = 0; c < kChunks; ++c) {
-            const long long ep = (long long)win * kSpan + c * 32 + lane;
+            const long long ep = win * span + c * 32 + lane;
             vc[c] = -1;
             uc[c] = -1;
-            if (ep < count) {
+            if (ep < count && c * 32 < span) {
                 const long long e = eidx ? (long long)__ldg(eidx + ep) : ep;
                 vc[c] = __ldg(a.src + e);
                 uc[c] = __ldg(a.col + e);
@@ -498,7 +513,7 @@ __device__ __forceinline__ void edges_phase(const SweepArgs& a, EdgeScratch* sh)
             const int slot = slots + __popc(heads & (lt | (1u << lane))) - 1;
             if (head) {
                 es.v[slot] = v;
-                es.top[slot] = (unsigned)es.part[c * 32 + lane];
+                es.lo[slot] = es.part[c * 32 + lane];
             }
             slots += __popc(heads);
             before = __shfl_sync(kFull, v, 31 - __clz(kept));
@@ -515,225 +530,239 @@ __device__ __forceinline__ void edges_phase(const SweepArgs& a, EdgeScratch* sh)
         }
         __syncwarp();
         if (slots == 0) continue;
-        // A_a per slot: a lane per slot reads what is known; the rest is
-        // computed by groups of lanes
-        for (int s0 = 0; s0 < slots; s0 += 32) {
-            const int s = s0 + lane;
-            bool stale = false;
-            if (s < slots) {
-                const int v = es.v[s], cv = (int)es.top[s];
-                const int2 o = a.own[v];
-                const int chg = a.chg[cv], sa = a.size[cv];
-                const unsigned long long b0 = __ldcg(a.best + v);
-                const int k = kSingle ? J0.k : a.job[__ldg(a.jid + v)].k;
-                stale = !own_valid(o, chg);
-                es.base[s] = 2 * (o.x - k) - k * (sa - 1);
-                es.ubest[s] = b0;
-                if (!stale) es.top[s] = 0;
-            }
-            unsigned todo = __ballot_sync(kFull, stale);
-            __syncwarp();
-            while (todo) {
-                // the group's slot: the grp-th stale one
-                unsigned t = todo;
-                for (int i = 0; i < grp; ++i) t &= t - 1;
-                const bool on = t != 0;
-                const int q = on ? s0 + __ffs(t) - 1 : 0;
-                const int v = es.v[q];
-                const JobInfo J = kSingle ? J0 : a.job[__ldg(a.jid + v)];
-                const int cv = on ? (int)es.top[q] : 0, sa = on ? a.size[cv] : 1;
-                int part = 0;
-                if (on) part = own_part(a, J, mask, small, v, cv, sa, l, gs);
-                part = group_sum(part, gs);
-                if (on && l == 0) {
-                    a.own[v] = make_int2(part, a.chg[cv]);
-                    es.base[q] = 2 * (part - J.k) - J.k * (sa - 1);
-                    es.top[q] = 0;
+        for (int sb = 0; sb < slots; sb += kSlots) {
+            const int count_s = min(slots - sb, kSlots);
+            auto in_batch = [&](int f) { return ((f & 127) & ~(kSlots - 1)) == sb; };
+            // A_a per slot: a lane per slot reads what is known; the rest is
+            // computed by groups of lanes
+            for (int s0 = 0; s0 < count_s; s0 += 32) {
+                const int s = s0 + lane;
+                bool stale = false;
+                int v = 0, cv = 0, chg = 0, sa = 1;
+                if (s < count_s) {
+                    v = es.v[sb + s];
+                    cv = sb == 0 ? es.lo[s] : a.C[v];  // (the later slots' clusters have been overwritten)
+                    const int2 o = a.own[v];
+                    chg = a.chg[cv];
+                    sa = a.size[cv];
+                    const unsigned long long b0 = __ldcg(a.best + v);
+                    const int k = kSingle ? J0.k : a.job[__ldg(a.jid + v)].k;
+                    stale = !own_valid(o, chg);
+                    es.base[s] = 2 * (o.x - k) - k * (sa - 1);
+                    es.ubest[s] = b0;
                 }
-                for (int i = 0; i < per && todo; ++i) todo &= todo - 1;
-            }
-        }
-        __syncwarp();
-        // the largest candidate of each slot
-        if (many) {
-            for (int c0 = 0; c0 < nt; c0 += 32) {
-                const int q = kSpan - 1 - (c0 + lane);
-                if (c0 + lane < nt) atomicMax(&es.top[es.slot[q]], ((unsigned)es.w[q] << 7) | (unsigned)q);
+                unsigned todo = __ballot_sync(kFull, stale);
+                __syncwarp();
+                if (s < count_s) es.lo[s] = 0;
+                while (todo) {
+                    // the group's slot: the grp-th stale one
+                    unsigned t = todo;
+                    for (int i = 0; i < grp; ++i) t &= t - 1;
+                    const bool on = t != 0;
+                    const int q = on ? __ffs(t) - 1 : lane;
+                    const int vq = __shfl_sync(kFull, v, q), cq = __shfl_sync(kFull, cv, q);
+                    const int sq = __shfl_sync(kFull, sa, q), hq = __shfl_sync(kFull, chg, q);
+                    const JobInfo J = kSingle ? J0 : a.job[__ldg(a.jid + vq)];
+                    int part = 0;
+                    if (on) part = own_part(a, J, mask, small, vq, cq, sq, l, gs);
+                    part = group_sum(part, gs);
+                    if (on && l == 0) {
+                        a.own[vq] = make_int2(part, hq);
+                        es.base[s0 + q] = 2 * (part - J.k) - J.k * (sq - 1);
+                    }
+                    for (int i = 0; i < per && todo; ++i) todo &= todo - 1;
+                }
             }
             __syncwarp();
-        }
-        // the clusters: the largest ones first, then the others (all at once
-        // when few vertices moved in the sweep before: the bounds then rule
-        // out little)
-        for (int pass = many ? 0 : 1; pass < 2; ++pass) {
-            // list: candidates above `small` from the front, others from the back
-            int nl = 0, nm = 0;
-            for (int c0 = 0; c0 < nt; c0 += 32) {
-                const int q = kSpan - 1 - (c0 + lane);
-                bool on = c0 + lane < nt, big = true;
-                if (on) {
-                    const int s = es.slot[q], sx = es.w[q];
-                    const int k = kSingle ? J0.k : a.job[__ldg(a.jid + es.v[s])].k;
-                    // A_x <= k |x|
-                    const int lo = es.base[s] - k * sx;
-                    on = (!many || ((es.top[s] & 127u) == (unsigned)q) == (pass == 0)) && lo < 0 &&
-                         pack_key(lo, es.x[q]) < es.ubest[s];
-                    big = sx > small;
+            // the largest candidate of each slot
+            if (many) {
+                for (int c0 = 0; c0 < nt; c0 += 32) {
+                    const int q = kSpan - 1 - (c0 + lane);
+                    if (c0 + lane < nt && in_batch(es.slot[q]))
+                        atomicMax(reinterpret_cast<unsigned*>(&es.lo[es.slot[q] & (kSlots - 1)]),
+                                  ((unsigned)es.w[q] << 7) | (unsigned)q);
                 }
-                const unsigned bb = __ballot_sync(kFull, on && big), bm = __ballot_sync(kFull, on && !big);
-                if (on) {
-                    const int p = big ? nl + __popc(bb & lt) : kSpan - 1 - (nm + __popc(bm & lt));
-                    es.list[p] = (unsigned char)q;
+                __syncwarp();
+                for (int c0 = 0; c0 < nt; c0 += 32) {
+                    const int q = kSpan - 1 - (c0 + lane);
+                    if (c0 + lane < nt && in_batch(es.slot[q]) && (es.lo[es.slot[q] & (kSlots - 1)] & 127) == q)
+                        es.slot[q] |= 128;
                 }
-                nl += __popc(bb);
-                nm += __popc(bm);
+                __syncwarp();
             }
-            __syncwarp();
-            // small clusters: every (candidate, member) pair is one row
-            // compare, 16 candidates at a time (at most 16 kSmall pairs), so
-            // that the rounds run full and no load waits for another
-            for (int c0 = 0; c0 < nm; c0 += 16) {
-                const bool mine = lane < 16 && c0 + lane < nm;
-                const int q = mine ? (int)es.list[kSpan - 1 - (c0 + lane)] : 0;
-                const int sx = mine ? es.w[q] : 0;
-                int end = sx;  // pairs up to and including this lane's
-                for (int o = 1; o < 16; o <<= 1) {
-                    const int y = __shfl_up_sync(kFull, end, o);
-                    if (lane >= o) end += y;
+            // the clusters: the largest ones first, then the others (all at once
+            // when few vertices moved in the sweep before: the bounds then rule
+            // out little)
+            for (int pass = many ? 0 : 1; pass < 2; ++pass) {
+                // list: candidates above `small` from the front, others from the back
+                int nl = 0, nm = 0;
+                for (int c0 = 0; c0 < nt; c0 += 32) {
+                    const int q = kSpan - 1 - (c0 + lane);
+                    bool on = c0 + lane < nt, big = true;
+                    if (on) {
+                        const int f = es.slot[q], s = f & (kSlots - 1), sx = es.w[q];
+                        const int k = kSingle ? J0.k : a.job[__ldg(a.jid + es.v[f & 127])].k;
+                        // A_x <= k |x|
+                        const int lo = es.base[s] - k * sx;
+                        on = in_batch(f) && (!many || (f >= 128) == (pass == 0)) && lo < 0 &&
+                             pack_key(lo, es.x[q]) < es.ubest[s];
+                        big = sx > small;
+                    }
+                    const unsigned bb = __ballot_sync(kFull, on && big), bm = __ballot_sync(kFull, on && !big);
+                    if (on) {
+                        const int p = big ? nl + __popc(bb & lt) : kSpan - 1 - (nm + __popc(bm & lt));
+                        es.list[p] = (unsigned char)q;
+                    }
+                    nl += __popc(bb);
+                    nm += __popc(bm);
                 }
-                const int pairs = __shfl_sync(kFull, end, 15);
-                if (mine) {
-                    const int* mem = a.members + (a.cursor[es.x[q]] - sx);
-                    es.part[q] = 0;
-                    for (int m = 0; m < sx; ++m) {
-                        es.lo[end - sx + m] = mem[m];
-                        es.pair[end - sx + m] = (unsigned char)q;
+                __syncwarp();
+                // small clusters: every (candidate, member) pair is one row
+                // compare, 16 candidates at a time (at most 16 kSmall pairs), so
+                // that the rounds run full and no load waits for another
+                for (int c0 = 0; c0 < nm; c0 += 16) {
+                    const bool mine = lane < 16 && c0 + lane < nm;
+                    const int q = mine ? (int)es.list[kSpan - 1 - (c0 + lane)] : 0;
+                    const int sx = mine ? es.w[q] : 0;
+                    int end = sx;  // pairs up to and including this lane's
+                    for (int o = 1; o < 16; o <<= 1) {
+                        const int y = __shfl_up_sync(kFull, end, o);
+                        if (lane >= o) end += y;
+                    }
+                    const int pairs = __shfl_sync(kFull, end, 15);
+                    if (mine) {
+                        const int* mem = a.members + (a.cursor[es.x[q]] - sx);
+                        es.part[q] = 0;
+                        for (int m = 0; m < sx; ++m) {
+                            es.lo[end - sx + m] = mem[m];
+                            es.pair[end - sx + m] = (unsigned char)q;
+                        }
+                    }
+                    __syncwarp();
+                    for (int r0 = 0; r0 < pairs; r0 += pr) {
+                        const bool valid = r0 + lane / gr < pairs;
+                        const int p = valid ? r0 + lane / gr : 0;
+                        const int pq = es.pair[p], v = es.v[es.slot[pq] & 127];
+                        const JobInfo J = kSingle ? J0 : a.job[__ldg(a.jid + v)];
+                        int part = 0;
+                        if (valid) part = row_part(a.G + row_of(J, es.lo[p]), a.G + row_of(J, v), J.kp >> 2, lr, gr);
+                        part = group_sum(part, gr);
+                        if (valid && lr == 0) atomicAdd(&es.part[pq], part - (J.kp - J.k));
+                    }
+                    __syncwarp();
+                    if (mine) {
+                        const int v = es.v[es.slot[q] & 127], s = es.slot[q] & (kSlots - 1), x = es.x[q];
+                        const int k = kSingle ? J0.k : a.job[__ldg(a.jid + v)].k;
+                        const int dD = es.base[s] + k * sx - 2 * es.part[q];
+                        const unsigned long long key = pack_key(dD, x);
+                        if (dD < 0 && key < es.ubest[s]) {
+                            atomicMin(&es.ubest[s], key);
+                            atomicMin(&a.best[v], key);
+                        }
+                    }
+                    __syncwarp();
+                }
+                // larger clusters: their summary rows
+                int no = 0;  // left open by the summary
+                for (int r0 = 0; r0 < nl; r0 += per) {
+                    const bool valid = r0 + grp < nl;
+                    const int q = valid ? (int)es.list[r0 + grp] : 0;
+                    const int f = valid ? (int)es.slot[q] : 0, s = f & (kSlots - 1);
+                    const int v = valid ? es.v[f & 127] : 0, x = valid ? es.x[q] : 0, sx = valid ? es.w[q] : 0;
+                    const JobInfo J = kSingle ? J0 : a.job[valid ? __ldg(a.jid + v) : 0];
+                    int part = 0, ub = 0;
+                    if (valid) summary_part(a, J, a.G + row_of(J, v), x, sx, l, gs, part, ub);
+                    part = group_sum(part, gs);
+                    ub = group_sum(ub, gs);
+                    bool open = false;
+                    if (valid && l == 0) {
+                        const int top = es.base[s] + J.k * sx;  // dD = top - 2 A
+                        const int lo = top - 2 * ub, hi = top - 2 * part;
+                        const unsigned long long key = pack_key(hi, x);
+                        if (hi < 0 && key < es.ubest[s]) atomicMin(&es.ubest[s], key);
+                        if (ub == part) {
+                            if (hi < 0 && key <= es.ubest[s]) atomicMin(&a.best[v], key);
+                        } else if (lo < 0) {
+                            es.lo[q] = lo;
+                            es.part[q] = part;
+                            open = true;
+                        }
+                    }
+                    // the list entries of this round are read already: the open
+                    // ones go back to the front
+                    const unsigned bal = __ballot_sync(kFull, open);
+                    __syncwarp();
+                    if (open) es.list[no + __popc(bal & lt)] = (unsigned char)q;
+                    no += __popc(bal);
+                }
+                __syncwarp();
+                // probes of the open ones still below the bound, in full rounds
+                int np = 0;
+                for (int c0 = 0; c0 < no; c0 += 32) {
+                    const int q = c0 + lane < no ? (int)es.list[c0 + lane] : 0;
+                    const bool on = c0 + lane < no && pack_key(es.lo[q], es.x[q]) < es.ubest[es.slot[q] & (kSlots - 1)];
+                    const unsigned bal = __ballot_sync(kFull, on);
+                    __syncwarp();
+                    if (on) es.list[np + __popc(bal & lt)] = (unsigned char)q;
+                    np += __popc(bal);
+                }
+                __syncwarp();
+                for (int r0 = 0; r0 < np; r0 += per) {
+                    const bool valid = r0 + grp < np;
+                    const int q = valid ? (int)es.list[r0 + grp] : 0;
+                    const int f = valid ? (int)es.slot[q] : 0, s = f & (kSlots - 1);
+                    const int v = valid ? es.v[f & 127] : 0, x = valid ? es.x[q] : 0, sx = valid ? es.w[q] : 0;
+                    const JobInfo J = kSingle ? J0 : a.job[valid ? __ldg(a.jid + v) : 0];
+                    int pb = 0;
+                    if (valid) pb = probe_part(a, J, a.table, mask, a.G + row_of(J, v), x, sx, l, gs);
+                    pb = group_sum(pb, gs);
+                    if (valid && l == 0) {
+                        const int dD = es.base[s] + J.k * sx - 2 * (es.part[q] + pb);
+                        const unsigned long long key = pack_key(dD, x);
+                        if (dD < 0 && key <= es.ubest[s]) {
+                            atomicMin(&es.ubest[s], key);
+                            atomicMin(&a.best[v], key);
+                        }
                     }
                 }
                 __syncwarp();
-                for (int r0 = 0; r0 < pairs; r0 += pr) {
-                    const bool valid = r0 + lane / gr < pairs;
-                    const int p = valid ? r0 + lane / gr : 0;
-                    const int pq = es.pair[p], v = es.v[es.slot[pq]];
-                    const JobInfo J = kSingle ? J0 : a.job[__ldg(a.jid + v)];
-                    int part = 0;
-                    if (valid) part = row_part(a.G + row_of(J, es.lo[p]), a.G + row_of(J, v), J.kp >> 2, lr, gr);
-                    part = group_sum(part, gr);
-                    if (valid && lr == 0) atomicAdd(&es.part[pq], part - (J.kp - J.k));
+            }
+            // singletons
+            int nl = 0;
+            for (int c0 = 0; c0 < ns; c0 += 32) {
+                const int q = c0 + lane;
+                bool on = q < ns;
+                if (on) {
+                    const int f = es.slot[q], s = f & (kSlots - 1);
+                    const int k = kSingle ? J0.k : a.job[__ldg(a.jid + es.v[f])].k;
+                    const int lo = es.base[s] - k;
+                    on = in_batch(f) && lo < 0 && pack_key(lo, es.x[q]) < es.ubest[s];
                 }
-                __syncwarp();
-                if (mine) {
-                    const int s = es.slot[q], v = es.v[s], x = es.x[q];
-                    const int k = kSingle ? J0.k : a.job[__ldg(a.jid + v)].k;
-                    const int dD = es.base[s] + k * sx - 2 * es.part[q];
-                    const unsigned long long key = pack_key(dD, x);
+                const unsigned bal = __ballot_sync(kFull, on);
+                if (on) es.list[nl + __popc(bal & lt)] = (unsigned char)q;
+                nl += __popc(bal);
+            }
+            __syncwarp();
+            for (int r0 = 0; r0 < nl; r0 += pr) {
+                const bool valid = r0 + lane / gr < nl;
+                const int q = valid ? (int)es.list[r0 + lane / gr] : 0;
+                const int f = valid ? (int)es.slot[q] : 0, s = f & (kSlots - 1);
+                const int v = valid ? es.v[f] : 0;
+                const JobInfo J = kSingle ? J0 : a.job[valid ? __ldg(a.jid + v) : 0];
+                int part = 0;
+                if (valid) part = row_part(a.G + row_of(J, es.w[q]), a.G + row_of(J, v), J.kp >> 2, lr, gr);
+                part = group_sum(part, gr);
+                if (valid && lr == 0) {
+                    const int dD = es.base[s] + J.k - 2 * (part - (J.kp - J.k));
+                    const unsigned long long key = pack_key(dD, es.x[q]);
                     if (dD < 0 && key < es.ubest[s]) {
                         atomicMin(&es.ubest[s], key);
                         atomicMin(&a.best[v], key);
                     }
                 }
-                __syncwarp();
-            }
-            // larger clusters: their summary rows
-            int no = 0;  // left open by the summary
-            for (int r0 = 0; r0 < nl; r0 += per) {
-                const bool valid = r0 + grp < nl;
-                const int q = valid ? (int)es.list[r0 + grp] : 0;
-                const int s = valid ? (int)es.slot[q] : 0;
-                const int v = valid ? es.v[s] : 0, x = valid ? es.x[q] : 0, sx = valid ? es.w[q] : 0;
-                const JobInfo J = kSingle ? J0 : a.job[valid ? __ldg(a.jid + v) : 0];
-                int part = 0, ub = 0;
-                if (valid) summary_part(a, J, a.G + row_of(J, v), x, sx, l, gs, part, ub);
-                part = group_sum(part, gs);
-                ub = group_sum(ub, gs);
-                bool open = false;
-                if (valid && l == 0) {
-                    const int top = es.base[s] + J.k * sx;  // dD = top - 2 A
-                    const int lo = top - 2 * ub, hi = top - 2 * part;
-                    const unsigned long long key = pack_key(hi, x);
-                    if (hi < 0 && key < es.ubest[s]) atomicMin(&es.ubest[s], key);
-                    if (ub == part) {
-                        if (hi < 0 && key <= es.ubest[s]) atomicMin(&a.best[v], key);
-                    } else if (lo < 0) {
-                        es.lo[q] = lo;
-                        es.part[q] = part;
-                        open = true;
-                    }
-                }
-                // the list entries of this round are read already: the open
-                // ones go back to the front
-                const unsigned bal = __ballot_sync(kFull, open);
-                __syncwarp();
-                if (open) es.list[no + __popc(bal & lt)] = (unsigned char)q;
-                no += __popc(bal);
-            }
-            __syncwarp();
-            // probes of the open ones still below the bound, in full rounds
-            int np = 0;
-            for (int c0 = 0; c0 < no; c0 += 32) {
-                const int q = c0 + lane < no ? (int)es.list[c0 + lane] : 0;
-                const bool on = c0 + lane < no && pack_key(es.lo[q], es.x[q]) < es.ubest[es.slot[q]];
-                const unsigned bal = __ballot_sync(kFull, on);
-                __syncwarp();
-                if (on) es.list[np + __popc(bal & lt)] = (unsigned char)q;
-                np += __popc(bal);
-            }
-            __syncwarp();
-            for (int r0 = 0; r0 < np; r0 += per) {
-                const bool valid = r0 + grp < np;
-                const int q = valid ? (int)es.list[r0 + grp] : 0;
-                const int s = valid ? (int)es.slot[q] : 0;
-                const int v = valid ? es.v[s] : 0, x = valid ? es.x[q] : 0, sx = valid ? es.w[q] : 0;
-                const JobInfo J = kSingle ? J0 : a.job[valid ? __ldg(a.jid + v) : 0];
-                int pb = 0;
-                if (valid) pb = probe_part(a, J, a.table, mask, a.G + row_of(J, v), x, sx, l, gs);
-                pb = group_sum(pb, gs);
-                if (valid && l == 0) {
-                    const int dD = es.base[s] + J.k * sx - 2 * (es.part[q] + pb);
-                    const unsigned long long key = pack_key(dD, x);
-                    if (dD < 0 && key <= es.ubest[s]) {
-                        atomicMin(&es.ubest[s], key);
-                        atomicMin(&a.best[v], key);
-                    }
-                }
             }
             __syncwarp();
         }
-        // singletons
-        int nl = 0;
-        for (int c0 = 0; c0 < ns; c0 += 32) {
-            const int q = c0 + lane;
-            bool on = q < ns;
-            if (on) {
-                const int s = es.slot[q];
-                const int k = kSingle ? J0.k : a.job[__ldg(a.jid + es.v[s])].k;
-                const int lo = es.base[s] - k;
-                on = lo < 0 && pack_key(lo, es.x[q]) < es.ubest[s];
-            }
-            const unsigned bal = __ballot_sync(kFull, on);
-            if (on) es.list[nl + __popc(bal & lt)] = (unsigned char)q;
-            nl += __popc(bal);
-        }
-        __syncwarp();
-        for (int r0 = 0; r0 < nl; r0 += pr) {
-            const bool valid = r0 + lane / gr < nl;
-            const int q = valid ? (int)es.list[r0 + lane / gr] : 0;
-            const int s = valid ? (int)es.slot[q] : 0;
-            const int v = valid ? es.v[s] : 0;
-            const JobInfo J = kSingle ? J0 : a.job[valid ? __ldg(a.jid + v) : 0];
-            int part = 0;
-            if (valid) part = row_part(a.G + row_of(J, es.w[q]), a.G + row_of(J, v), J.kp >> 2, lr, gr);
-            part = group_sum(part, gr);
-            if (valid && lr == 0) {
-                const int dD = es.base[s] + J.k - 2 * (part - (J.kp - J.k));
-                const unsigned long long key = pack_key(dD, es.x[q]);
-                if (dD < 0 && key < es.ubest[s]) {
-                    atomicMin(&es.ubest[s], key);
-                    atomicMin(&a.best[v], key);
-                }
-            }
-        }
-        __syncwarp();
     }
 }
 
@@ -898,9 +927,10 @@ __device__ __forceinline__ void h_eval_phase(const SweepArgs& a)
     const int lane = threadIdx.x & 31, l = lane & (gs - 1), grp = lane / gs;
     const int step = 32 - small;
     const JobInfo J0 = first_job(a);
-    const long long nwarps = (long long)gridDim.x * kWarpsPerBlock;
-    for (long long wb = ((long long)blockIdx.x * kWarpsPerBlock + (threadIdx.x >> 5)) * step; wb < a.n;
-         wb += nwarps * step) {
+    __shared__ int s_taken;
+    const WarpQueue queue{&s_taken};
+    queue.start();
+    for (long long wb = queue.next() * step; wb < a.n; wb = queue.next() * step) {
         const long long idx = wb + lane;
         const int v = idx < a.n ? a.members[idx] : 0;
         // (a place holding a smaller job leaves vertices to the idle job)
@@ -1022,15 +1052,39 @@ __device__ __forceinline__ void count_inserts(DevState* st, int mine, unsigned l
     }
 }
 
-// The light-path kernels give each proposal a group of gs lanes: the lanes
-// split the job's partitions, and the group's first lane does the per-proposal
-// work (flags, sizes, bids, sums).  Items of one warp: 32 / gs proposals.
+// The light-path steps give each proposal a group of lanes: the lanes split
+// the job's partitions, and the group's first lane does the per-proposal work
+// (flags, sizes, bids, sums).  A partition is a chain of dependent loads and
+// atomics (find the slot, exchange, add, look at the summary: about 2.5 us), so
+// when the proposals leave threads idle a group gets more lanes than the
+// scoring's gs, up to one per partition (colour classes of n = 1e5, k = 8:
+// stage + evaluate + commit 85 -> 35 us); a lane count set by the caller stays.
+__device__ __forceinline__ int proposal_lanes(const SweepArgs& a, long long np)
+{
+    int gs = a.gs;
+    if (a.gs_set) return gs;
+    const long long threads = (long long)gridDim.x * blockDim.x;
+    while (gs < 32 && gs < a.kmax && 2 * gs * np <= threads) gs <<= 1;
+    return gs;
+}
+
 #define PROPOSAL_LOOP(np)                                                                                  \
-    const int gs = a.gs, per = 32 / gs;                                                                   \
+    const int gs = proposal_lanes(a, np), per = 32 / gs;                                                  \
     const int lane = threadIdx.x & 31, l = lane & (gs - 1);                                               \
     const long long warp0 = ((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5;                      \
     const long long nwarp = ((long long)gridDim.x * blockDim.x) >> 5;                                     \
     for (long long b0 = warp0 * per; b0 < (np); b0 += nwarp * per)
+
+// Slots of two keys (-1: absent), their first probes in flight together.
+__device__ __forceinline__ void table_find_pair(const Slot* t, unsigned long long mask, unsigned long long ka,
+                                                unsigned long long kb, long long& sa, long long& sb)
+{
+    const unsigned long long ha = hash_key(ka) & mask, hb = hash_key(kb) & mask;
+    const unsigned long long a = *reinterpret_cast<const volatile unsigned long long*>(&t[ha].key);
+    const unsigned long long b = *reinterpret_cast<const volatile unsigned long long*>(&t[hb].key);
+    sa = a == ka ? (long long)ha : a == kEmpty ? -1 : table_find(t, mask, ka);
+    sb = b == kb ? (long long)hb : b == kEmpty ? -1 : table_find(t, mask, kb);
+}
 
 __device__ __forceinline__ long long group_sum64(long long x, int gs)
 {
@@ -1070,8 +1124,9 @@ __device__ __forceinline__ void stage_phase(const SweepArgs& a)
                 for (int i = l; i < J.k; i += gs) {
                     const int g = gv[i];
                     bool ins = false;
-                    const long long sa = table_find(a.table, mask, ckey(ca, g));
-                    const long long sb = table_find_or_insert(a.table, mask, ckey(cb, g), &ins);
+                    long long sa, sb;
+                    table_find_pair(a.table, mask, ckey(ca, g), ckey(cb, g), sa, sb);
+                    if (sb < 0) sb = table_find_or_insert(a.table, mask, ckey(cb, g), &ins);
                     ins_count += ins;
                     if (sa < 0) {
                         set_err(st, CC_ERR_INVALID);  // the vertex's own key must exist
@@ -1113,15 +1168,16 @@ __device__ __forceinline__ void eval_phase(const SweepArgs& a)
             const int* gv = a.G + row_of(J, v);
             for (int i = l; i < J.k; i += gs) {
                 const int g = gv[i];
-                const long long sa = table_find(a.table, mask, ckey(ca, g));
-                const long long sb = table_find(a.table, mask, ckey(cb, g));
+                long long sa, sb;
+                table_find_pair(a.table, mask, ckey(ca, g), ckey(cb, g), sa, sb);
                 if (sa < 0 || sb < 0) {
                     set_err(st, CC_ERR_INVALID);  // staged keys must exist
                     continue;
                 }
                 const Slot* A = a.table + sa;
                 const Slot* B = a.table + sb;
-                keys += -(2LL * A->cnt + A->dlt) + (2LL * B->cnt + B->dlt);
+                const int na = A->cnt, da = A->dlt, nb = B->cnt, db = B->dlt;
+                keys += -(2LL * na + da) + (2LL * nb + db);
             }
             if (l == 0) {
                 job = j;
@@ -1275,21 +1331,20 @@ __device__ __forceinline__ void commit_phase(const SweepArgs& a)
                 }
                 for (int i = l; i < J.k; i += gs) {
                     const int g = gv[i];
-#pragma unroll
-                    for (int side = 0; side < 2; ++side) {
-                        const long long si = table_find(a.table, mask, ckey(side ? cb : ca, g));
-                        if (si < 0) {
-                            set_err(st, CC_ERR_INVALID);
-                            continue;
-                        }
-                        Slot* s = a.table + si;
-                        const int dd = atomicExch(&s->dlt, 0);
-                        if (dd) {
-                            const int old = atomicAdd(&s->cnt, dd);
-                            live += (old == 0) - (old + dd == 0);
-                            summ_update(a, s->key, dd);
-                        }
+                    long long sa, sb;
+                    table_find_pair(a.table, mask, ckey(ca, g), ckey(cb, g), sa, sb);
+                    if (sa < 0 || sb < 0) {
+                        set_err(st, CC_ERR_INVALID);
+                        continue;
                     }
+                    // both sides' atomics in flight together
+                    const int da = atomicExch(&a.table[sa].dlt, 0), db = atomicExch(&a.table[sb].dlt, 0);
+                    const int oa = da ? atomicAdd(&a.table[sa].cnt, da) : 1;
+                    const int ob = db ? atomicAdd(&a.table[sb].cnt, db) : 1;
+                    if (da) live += (oa == 0) - (oa + da == 0);
+                    if (db) live += (ob == 0) - (ob + db == 0);
+                    if (da) summ_update(a, J, ca, i, g, da);
+                    if (db) summ_update(a, J, cb, i, g, db);
                 }
             } else if (mode == 2 && a.pflag[p] == 2) {
                 if (l == 0) {
@@ -1304,8 +1359,8 @@ __device__ __forceinline__ void commit_phase(const SweepArgs& a)
                 }
                 for (int i = l; i < J.k; i += gs) {
                     const int g = gv[i];
-                    const long long sa = table_find(a.table, mask, ckey(ca, g));
-                    const long long sb = table_find(a.table, mask, ckey(cb, g));
+                    long long sa, sb;
+                    table_find_pair(a.table, mask, ckey(ca, g), ckey(cb, g), sa, sb);
                     if (sa < 0 || sb < 0) {
                         set_err(st, CC_ERR_INVALID);
                         continue;
@@ -1313,8 +1368,8 @@ __device__ __forceinline__ void commit_phase(const SweepArgs& a)
                     const int oa = atomicAdd(&a.table[sa].cnt, -1);
                     const int ob = atomicAdd(&a.table[sb].cnt, 1);
                     live += (ob == 0) - (oa == 1);
-                    summ_update(a, ckey(ca, g), -1);
-                    summ_update(a, ckey(cb, g), 1);
+                    summ_update(a, J, ca, i, g, -1);
+                    summ_update(a, J, cb, i, g, 1);
                 }
             }
         }

@@ -102,3 +102,28 @@ def test_label_maps(cc, n, k, kinds):
         batch.run_until_converged(4)
         assert batch.history(0) == ref.stats
         np.testing.assert_array_equal(batch.cluster_ids()[:n], ref.C)
+
+
+# one, two and all vertices per neighbour list: windows of the scoring with 128
+# distinct vertices, with 64, and with one
+@pytest.mark.parametrize("shape", ["matching", "ring", "star"])
+@pytest.mark.parametrize("n,k", [(1000, 3), (5000, 9)])
+def test_sparse_graphs(cc, shape, n, k):
+    rng = np.random.default_rng(n + k)
+    v = np.arange(n)
+    if shape == "matching":
+        ro, col = csr_from_edges(n, v[::2], v[1::2])
+    elif shape == "ring":
+        ro, col = csr_from_edges(n, v, (v + 1) % n)
+    else:
+        ro, col = csr_from_edges(n, np.zeros(n - 1, np.int64), v[1:])
+    lab = np.stack([(v // rng.integers(2, 40) + (rng.random(n) < 0.1) * 7).astype(np.int32) for _ in range(k)])
+    ref = oracle.sync_run(ro, col, lab, 20)
+    for opts in ({}, {"active_set": 1}, {"no_regions": 1}):
+        o = cc.cc_default_options()
+        for f, x in opts.items():
+            setattr(o, f, x)
+        with cc.Consensus(ro, col, lab, o) as job:
+            job.run_until_converged(20)
+            assert job.history() == ref.stats
+            np.testing.assert_array_equal(job.cluster_ids(), ref.C)
