@@ -476,6 +476,7 @@ cc_status plan_jobs(int jobs, const JobInput* in, const cc_options& opt, Plan* o
         p.n += q.n;
         p.nnz += q.nnz;
         p.rows += (long long)q.n * ((q.k + 3) & ~3);
+        p.words16 += (long long)q.n * quads16(q.k);
         p.keys += (long long)q.n * q.k;
         p.parts += q.k;
         p.kmax = std::max(p.kmax, (int)q.k);
@@ -533,7 +534,7 @@ void finish_plan(Plan& p, const cc_options& opt)
         sizeof(JobInfo) * (J + 1), sizeof(JobState) * (J + 1), 8 * (N + 1), 4 * (size_t)p.nnz, 4 * (size_t)p.nnz,
         4 * N, 4 * (size_t)p.rows, 16 * (size_t)p.rows, 4 * N, 4 * N, 4 * N, 8 * N, 8 * N,
         sizeof(Slot) * (size_t)p.cap_max, 4 * N, 4 * N, 4 * N, 4 * N, N, 4 * N, 4 * N, 4 * bsum_entries(N),
-        24 * (size_t)kRunBodies,
+        24 * (size_t)kRunBodies, 16 * (size_t)p.words16,
         4 * N, 8 * N, N, 4 * J, 8 * (J + 1), 8 * (size_t)p.parts, 8 * (size_t)p.parts,
         4 * (3 * N + N / 1024 + 64), sizeof(DevState), sizeof(cc_sweep_info) * J * (size_t)p.hist_cap};
     for (size_t b : per) p.persistent += rounded(b);
@@ -544,7 +545,7 @@ void finish_plan(Plan& p, const cc_options& opt)
         for (size_t b : cls) p.persistent += rounded(b);
     }
     // (both label maps: the first one tried stays until the second is done)
-    const size_t tmp[] = {8 * (N + J), 8 * (J + 1), 4 * (size_t)p.keys, 8 * (J + 1), 4 * (size_t)p.parts, 8 * J + 64,
+    const size_t tmp[] = {8 * (N + J), 8 * (J + 1), 4 * (size_t)p.keys, 8 * (J + 1), 4 * (size_t)p.parts, 8 * J + 64, 4 * (size_t)p.parts,
                           sizeof(DevState), 16 * (size_t)p.lcap,
                           16 * (size_t)label_map_slots((long long)p.keys, p.lcap)};
     for (size_t b : tmp) p.temporary += rounded(b);
@@ -607,7 +608,7 @@ cc_status create_common(int jobs, const JobInput* in, bool on_device, const cc_o
     c->job.resize(jobs);
     std::vector<long long> eo(jobs + 1, 0), lo(jobs + 1, 0);
     std::vector<int> pjob, pfirst(jobs);
-    long long vo = 0, go = 0;
+    long long vo = 0, go = 0, g16 = 0;
     for (int j = 0; j < jobs; ++j) {
         JobInfo& J = c->job[j];
         J.vo = vo;
@@ -617,9 +618,11 @@ cc_status create_common(int jobs, const JobInput* in, bool on_device, const cc_o
         J.kp = (in[j].k + 3) & ~3;
         J.lshift = 0;
         while ((1LL << J.lshift) < J.n) ++J.lshift;
-        J.pad = 0;
+        J.narrow = 1;
+        J.g16 = g16;
         vo += J.n;
         go += J.n * J.kp;
+        g16 += J.n * quads16(J.k);
         eo[j + 1] = eo[j] + in[j].nnz;
         lo[j + 1] = lo[j] + (long long)in[j].k * in[j].n;
         pfirst[j] = (int)pjob.size();
@@ -665,6 +668,7 @@ cc_status create_common(int jobs, const JobInput* in, bool on_device, const cc_o
     CC_TRY(dalloc(c, &c->src, (size_t)NNZ));
     CC_TRY(dalloc(c, &c->jid, (size_t)N));
     CC_TRY(dalloc(c, &c->G, (size_t)rows));
+    CC_TRY(dalloc(c, &c->G16, (size_t)g16));
     CC_TRY(dalloc(c, &c->summ, (size_t)rows));
     CC_TRY(dalloc(c, &c->C, (size_t)N));
     CC_TRY(dalloc(c, &c->size, (size_t)N));
@@ -690,7 +694,7 @@ cc_status create_common(int jobs, const JobInput* in, bool on_device, const cc_o
         // entry `jobs` is an idle job (no vertices, k = 0, always stopped) for
         // the vertices that a slot reloaded with a smaller job leaves unused
         std::vector<JobInfo> jt(c->job);
-        jt.push_back(JobInfo{0, 0, 0, 0, 0, 0, 0});
+        jt.push_back(JobInfo{});
         CC_TRY(cudaMemcpyAsync(c->d_job, jt.data(), sizeof(JobInfo) * ((size_t)jobs + 1), cudaMemcpyHostToDevice,
                                c->stream));
     }
@@ -749,13 +753,14 @@ cc_status create_common(int jobs, const JobInput* in, bool on_device, const cc_o
         const size_t at_turn = put(tl.turn0.data(), sizeof(int) * (size_t)jobs);
         const size_t off_b = rounded(sizeof(long long) * ((size_t)N + jobs)), lab_b = rounded(sizeof(int) * (size_t)keys);
         const size_t meta_b = rounded(meta.size()), st_b = rounded(sizeof(DevState));
+        const size_t parts_b = rounded(sizeof(int) * pjob.size());
         unsigned char* stage = nullptr;
-        cudaError_t e = tmalloc((void**)&stage, off_b + lab_b + meta_b + st_b + 16 * lcap);
+        cudaError_t e = tmalloc((void**)&stage, off_b + lab_b + meta_b + st_b + parts_b + 16 * lcap);
         offstage = reinterpret_cast<long long*>(stage);
         labels = reinterpret_cast<int*>(stage + off_b);
         d_meta = stage + off_b + lab_b;
         tst = reinterpret_cast<DevState*>(stage + off_b + lab_b + meta_b);
-        lmap = stage + off_b + lab_b + meta_b + st_b;
+        lmap = stage + off_b + lab_b + meta_b + st_b + parts_b;
         for (int j = 0; j < jobs && e == cudaSuccess; ++j) {
             const JobInfo& J = c->job[j];
             e = cudaMemcpyAsync(offstage + J.vo + j, in[j].row_off, sizeof(long long) * ((size_t)J.n + 1), kind, c->stream);
@@ -788,6 +793,9 @@ cc_status create_common(int jobs, const JobInput* in, bool on_device, const cc_o
         la.job = c->d_job;
         la.js = c->js;
         la.G = c->G;
+        la.G16 = c->G16;
+        la.parts = (int)pjob.size();
+        la.part_n = reinterpret_cast<int*>(reinterpret_cast<unsigned char*>(tst) + st_b);
         la.slots = reinterpret_cast<unsigned*>(c->summ);  // the summary rows are written by the first rebuild
         la.tiles = tl.tiles;
         la.turns = tl.turns;
@@ -802,7 +810,7 @@ cc_status create_common(int jobs, const JobInput* in, bool on_device, const cc_o
             la.lmap = lmap;
             la.lmask = lcap - 1;
             la.limit = lcap < most ? kLabelProbes : ~0ull;
-            e = cudaMemsetAsync(tst, 0, sizeof(DevState), c->stream);
+            e = cudaMemsetAsync(tst, 0, st_b + parts_b, c->stream);
             if (e == cudaSuccess) e = cudaMemsetAsync(c->part_sq, 0, sizeof(long long) * pjob.size(), c->stream);
             if (e == cudaSuccess) e = cudaMemsetAsync(c->part_slog, 0, sizeof(double) * pjob.size(), c->stream);
             if (e == cudaSuccess) e = launch_label_kernels(la, c->stream);
@@ -845,6 +853,7 @@ cc_status create_common(int jobs, const JobInput* in, bool on_device, const cc_o
     a.job = c->d_job;
     a.js = c->js;
     a.G = c->G;
+    a.G16 = c->G16;
     a.summ = c->summ;
     a.C = c->C;
     a.size = c->size;
@@ -1616,7 +1625,7 @@ cc_status ctx_load_job(cc_ctx* c, int j, const JobInput& in)
     const size_t lab_b = rounded(sizeof(int) * (size_t)keys), small_b = 512, pjob_b = rounded(sizeof(int) * (size_t)k);
     const size_t map_b = 16 * (size_t)lcap, st_b = rounded(sizeof(DevState));
     unsigned char* stage = nullptr;
-    cudaError_t e = tmalloc((void**)&stage, ro_b + col_b + lab_b + pjob_b + map_b + st_b + 3 * small_b);
+    cudaError_t e = tmalloc((void**)&stage, ro_b + col_b + lab_b + 2 * pjob_b + map_b + st_b + 3 * small_b);
     unsigned char* at = stage;
     auto part = [&](size_t bytes) {
         unsigned char* p = at;
@@ -1627,6 +1636,7 @@ cc_status ctx_load_job(cc_ctx* c, int j, const JobInput& in)
     col = reinterpret_cast<int*>(part(col_b));
     lab = reinterpret_cast<int*>(part(lab_b));
     pjob = reinterpret_cast<int*>(part(pjob_b));
+    int* part_n = reinterpret_cast<int*>(part(pjob_b));
     lmap = part(map_b);
     tst = reinterpret_cast<DevState*>(part(st_b));
     lo = reinterpret_cast<long long*>(part(small_b));
@@ -1640,7 +1650,7 @@ cc_status ctx_load_job(cc_ctx* c, int j, const JobInput& in)
     if (e == cudaSuccess && nnz > 0) e = cudaMemcpyAsync(col, in.col, sizeof(int) * (size_t)nnz, cudaMemcpyHostToDevice, c->stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(lab, in.labels, sizeof(int) * (size_t)keys, cudaMemcpyHostToDevice, c->stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(lo, lo_h, sizeof(lo_h), cudaMemcpyHostToDevice, c->stream);
-    if (e == cudaSuccess) e = cudaMemsetAsync(pjob, 0, sizeof(int) * (size_t)k, c->stream);
+    if (e == cudaSuccess) e = cudaMemsetAsync(pjob, 0, 2 * pjob_b, c->stream);  // (part_n follows it)
     if (e == cudaSuccess) e = cudaMemcpyAsync(pfirst, &zero, sizeof(int), cudaMemcpyHostToDevice, c->stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(dj, &J, sizeof(JobInfo), cudaMemcpyHostToDevice, c->stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(tst, &s0, sizeof(DevState), cudaMemcpyHostToDevice, c->stream);
@@ -1682,6 +1692,9 @@ cc_status ctx_load_job(cc_ctx* c, int j, const JobInput& in)
     la.job = dj;
     la.js = c->js + j;
     la.G = c->G;
+    la.G16 = c->G16;
+    la.parts = (int)k;
+    la.part_n = part_n;
     la.lmap = lmap;
     la.lmask = lcap - 1;
     la.limit = ~0ull;
@@ -1720,7 +1733,7 @@ cc_status ctx_load_job(cc_ctx* c, int j, const JobInput& in)
     jsr.partition_sq = psq;
     jsr.F = psq - k * n;
     e = cudaMemcpyAsync(&c->js[j], &jsr, sizeof(JobState), cudaMemcpyHostToDevice, c->stream);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(c->d_job + j, &J, sizeof(JobInfo), cudaMemcpyHostToDevice, c->stream);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(c->d_job + j, dj, sizeof(JobInfo), cudaMemcpyDeviceToDevice, c->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);  // jsr and J are host locals
     cleanup();
     if (e != cudaSuccess) return cuda_fail(c, e, "load job: records");

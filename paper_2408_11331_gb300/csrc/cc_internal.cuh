@@ -14,6 +14,8 @@
 //   jid   int32[N]     job of each vertex (and of each cluster id)
 //   G     int32[...]   compacted label ids, vertex-major: job j's rows start at go_j,
 //                      kp_j = k_j rounded up to 4 ints each (16-byte rows, padding -1);
+//   G16   16-bit numbers of the same classes, counted from 0 within each partition, in
+//                      rows of quads16(k_j) 16-byte words (valid where JobInfo::narrow);
 //                      g = (i << s_j) | rep, rep the job-local index of the least vertex
 //                      carrying that label in partition i and 2^s_j >= n_j, so g names
 //                      (partition, label) within the job and g < 2 k_j n_j.
@@ -65,7 +67,8 @@ struct JobInfo {
     int k;          // input partitions
     int kp;         // k rounded up to 4
     int lshift;     // s_j
-    int pad;
+    int narrow;     // 1: every partition has fewer than 2^16 - 1 classes, so G16 holds the labels too
+    long long g16;  // first 16-byte word of the job's rows in G16
 };
 
 // Per-job state of the current run.
@@ -157,6 +160,7 @@ struct SweepArgs {
     const JobInfo* job;         // J
     JobState* js;               // J
     const int* G;
+    const int4* G16;            // label rows again, as 16-bit class numbers (JobInfo::narrow)
     int4* summ;
     int* C;
     int* size;
@@ -219,6 +223,15 @@ struct WarpQueue {
         return ((long long)(i / kWarpsPerBlock) * gridDim.x + blockIdx.x) * kWarpsPerBlock + i % kWarpsPerBlock;
     }
 };
+
+// 16-bit label rows: a job's rows are quads16(k) 16-byte words each, eight
+// class numbers to a word.
+constexpr int kNoClass16 = 0xffff;  // the padding, and the first number that does not fit
+
+__host__ __device__ __forceinline__ int quads16(int k)
+{
+    return (k + 7) >> 3;
+}
 
 // Row of vertex / cluster x (a union vertex id) of job J in G or summ.
 __device__ __forceinline__ long long row_of(const JobInfo& J, long long x)
@@ -465,9 +478,12 @@ struct LabelArgs {
     const long long* lo;        // J + 1: first staged label of each job
     const int* pjob;            // global partition -> job
     const int* pfirst;          // J: first global partition of each job
-    const JobInfo* job;
+    JobInfo* job;               // (narrow is cleared where a partition has too many classes)
     JobState* js;
     int* G;
+    int4* G16;
+    int parts;                  // partitions of all jobs
+    int* part_n;                // per global partition: its classes (zeroed)
     void* lmap;                 // 16-byte slots, lmask + 1 of them
     unsigned long long lmask;
     unsigned long long limit;   // probes of an insert before st->err is set to CC_ERR_TABLE_FULL

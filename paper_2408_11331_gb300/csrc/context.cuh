@@ -46,6 +46,7 @@ struct cc_ctx {
     int* size = nullptr;
     int* dsize = nullptr;
     unsigned long long* best = nullptr;
+    int4* G16 = nullptr;
     int2* own = nullptr;
     int* chg = nullptr;                 // active set: change stamp per cluster id (n)
     unsigned long long* prev = nullptr; // active set: previous bid per vertex (n)
@@ -119,7 +120,7 @@ struct JobInput {
 // Sizes of a context for a set of jobs, and the device bytes it holds.
 struct Plan {
     int jobs = 0, kmax = 0, hist_cap = 0;
-    long long n = 0, nnz = 0, rows = 0, keys = 0, parts = 0;
+    long long n = 0, nnz = 0, rows = 0, keys = 0, parts = 0, words16 = 0;
     unsigned long long cap_max = 0, cap_start = 0, lcap = 0;
     size_t persistent = 0;  // held until cc_destroy
     size_t temporary = 0;   // held during creation only
@@ -130,7 +131,7 @@ struct Plan {
 cc_status plan_jobs(int jobs, const JobInput* in, const cc_options& opt, Plan* out, std::string* msg);
 cc_status check_options(const cc_options& opt, std::string* msg);
 // Fills the capacities and byte counts of a plan from its totals (jobs, n,
-// nnz, rows, keys, parts, kmax).
+// nnz, rows, words16, keys, parts, kmax).
 void finish_plan(Plan& p, const cc_options& opt);
 // Lanes that score one (vertex, candidate) pair for partitions of count k.
 int lanes_for_k(int k);

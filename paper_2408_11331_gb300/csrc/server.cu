@@ -106,6 +106,7 @@ Plan job_totals(const JobInput& q)
     p.n = q.n;
     p.nnz = q.nnz;
     p.rows = (long long)q.n * ((q.k + 3) & ~3);
+    p.words16 = (long long)q.n * quads16(q.k);
     p.keys = (long long)q.n * q.k;
     p.parts = q.k;
     p.kmax = q.k;
@@ -118,6 +119,7 @@ void add_totals(Plan& a, const Plan& b)
     a.n += b.n;
     a.nnz += b.nnz;
     a.rows += b.rows;
+    a.words16 += b.words16;
     a.keys += b.keys;
     a.parts += b.parts;
     a.kmax = std::max(a.kmax, b.kmax);

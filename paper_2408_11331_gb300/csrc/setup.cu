@@ -220,21 +220,102 @@ __global__ void __launch_bounds__(kBlock) k_label_insert(LabelArgs a)
     }
 }
 
-// G[row(v) + i] = (i << s_j) | rep(i, label), padding entries -1: tiles of 64
+// The classes numbered within their partition (the number replaces the raw
+// label in the class's key), sum_i sum_j |P_ij|^2 of every job and the sums per
+// partition.  With at most kSmemParts partitions a block counts its tile's
+// classes and adds up its sums in shared memory, so that a partition's words
+// take an add per tile instead of one per class (n = 1e6, k = 20: 96 us; the
+// sums alone, with an add per class, took 85).
+constexpr int kSmemParts = 512;
+__global__ void __launch_bounds__(kBlock) k_label_classes(LabelArgs a, unsigned long long cap)
+{
+    extern __shared__ long long dyn_jobs[];
+    __shared__ int s_n[kSmemParts], s_base[kSmemParts];
+    __shared__ unsigned long long s_sq[kSmemParts];
+    __shared__ double s_slog[kSmemParts];
+    LSlot* m = static_cast<LSlot*>(a.lmap);
+    JobAcc acc(job_smem_init(a.jobs, dyn_jobs), &a.js[0].partition_sq, kJobStride);
+    const bool shared = a.parts <= kSmemParts;
+    if (shared)
+        for (int P = threadIdx.x; P < a.parts; P += kBlock) {
+            s_sq[P] = 0;
+            s_slog[P] = 0;
+        }
+    int classes = 0;
+    for (unsigned long long b0 = (unsigned long long)blockIdx.x * kTile; b0 < cap; b0 += (unsigned long long)gridDim.x * kTile) {
+        if (shared)
+            for (int P = threadIdx.x; P < a.parts; P += kBlock) s_n[P] = 0;
+        __syncthreads();
+        int part[4], rank[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const unsigned long long s = b0 + q * kBlock + threadIdx.x;
+            part[q] = -1;
+            if (s >= cap) continue;
+            const ulonglong2 e = reinterpret_cast<const ulonglong2*>(m)[s];
+            if (e.x == kEmpty) continue;
+            ++classes;
+            const int P = part[q] = (int)(e.x >> 32);
+            const long long c = (long long)(e.y >> 32);
+            acc.add(a.pjob[P], c * c);
+            const double cl = (double)c * log((double)c);
+            if (shared) {
+                rank[q] = atomicAdd(&s_n[P], 1);
+                atomicAdd(&s_sq[P], (unsigned long long)(c * c));
+                atomicAdd(&s_slog[P], cl);
+            } else {
+                rank[q] = atomicAdd(&a.part_n[P], 1);
+                atomicAdd(reinterpret_cast<unsigned long long*>(a.part_sq + P), (unsigned long long)(c * c));
+                atomicAdd(a.part_slog + P, cl);
+            }
+        }
+        if (shared) {
+            __syncthreads();
+            for (int P = threadIdx.x; P < a.parts; P += kBlock)
+                if (s_n[P]) s_base[P] = atomicAdd(&a.part_n[P], s_n[P]);
+            __syncthreads();
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int P = part[q];
+            if (P < 0) continue;
+            const int id = shared ? s_base[P] + rank[q] : rank[q];
+            m[b0 + q * kBlock + threadIdx.x].key = ((unsigned long long)(unsigned)P << 32) | (unsigned)id;
+            if (id >= kNoClass16) a.job[a.pjob[P]].narrow = 0;
+        }
+    }
+    __syncthreads();
+    if (shared)
+        for (int P = threadIdx.x; P < a.parts; P += kBlock)
+            if (s_sq[P]) {
+                atomicAdd(reinterpret_cast<unsigned long long*>(a.part_sq + P), s_sq[P]);
+                atomicAdd(a.part_slog + P, s_slog[P]);
+            }
+    job_acc_finish(acc, a.jobs);
+    for (int o = 16; o > 0; o >>= 1) classes += __shfl_xor_sync(0xffffffffu, classes, o);
+    if ((threadIdx.x & 31) == 0 && classes)
+        atomicAdd(reinterpret_cast<unsigned long long*>(a.classes), (unsigned long long)classes);
+}
+
+// G[row(v) + i] = (i << s_j) | rep(i, label), padding entries -1, and the same
+// rows as 16-bit class numbers, padding kNoClass16: tiles of 64
 // vertices and 32 partitions, turned in shared memory from the partitions'
 // order to the vertices' (written straight, each label was a 4-byte store to
-// a sector of its own: n = 1e6, k = 20: 719 us, now 91).
+// a sector of its own: n = 1e6, k = 20: 719 us, 91 turned, 107 with the
+// 16-bit rows).
 constexpr int kTurn = 64;
 __global__ void __launch_bounds__(kBlock) k_label_assign(LabelArgs a)
 {
     if (a.st->err) return;
     __shared__ int turn[kTurn][33];
-    const LSlot* m = static_cast<const LSlot*>(a.lmap);
+    __shared__ __align__(4) unsigned short turn16[kTurn][34];
+    const ulonglong2* m = static_cast<const ulonglong2*>(a.lmap);
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     for (int tile = blockIdx.x; tile < a.turns; tile += gridDim.x) {
         const int j = upper_index32(a.turn0, a.jobs, tile);
         const JobInfo J = a.job[j];
-        const int v0 = (tile - a.turn0[j]) * kTurn;
+        const int v0 = (tile - a.turn0[j]) * kTurn, words = quads16(J.k) * 4;
+        unsigned* const rows16 = reinterpret_cast<unsigned*>(a.G16 + J.g16);
         for (int i0 = 0; i0 < J.kp; i0 += 32) {
 #pragma unroll
             for (int r = 0; r < 4; ++r) {
@@ -243,40 +324,28 @@ __global__ void __launch_bounds__(kBlock) k_label_assign(LabelArgs a)
 #pragma unroll
                 for (int h = 0; h < kTurn; h += 32) {
                     const int vl = h + lane;
-                    int g = -1;
-                    if (i < J.k && v0 + vl < J.n) g = (i << J.lshift) | m[a.slots[t0 + vl]].rep;
+                    int g = -1, id = kNoClass16;
+                    if (i < J.k && v0 + vl < J.n) {
+                        const ulonglong2 e = m[a.slots[t0 + vl]];
+                        g = (i << J.lshift) | (int)(unsigned)(e.y & 0xffffffffull);
+                        id = (int)(unsigned)(e.x & 0xffffffffull);
+                    }
                     turn[vl][w * 4 + r] = g;
+                    turn16[vl][w * 4 + r] = (unsigned short)id;
                 }
             }
             __syncthreads();
-            for (int vl = w; vl < kTurn; vl += kWarpsPerBlock)
-                if (v0 + vl < J.n && i0 + lane < J.kp) a.G[J.go + (long long)(v0 + vl) * J.kp + i0 + lane] = turn[vl][lane];
+            for (int vl = w; vl < kTurn; vl += kWarpsPerBlock) {
+                if (v0 + vl >= J.n) break;
+                if (i0 + lane < J.kp) a.G[J.go + (long long)(v0 + vl) * J.kp + i0 + lane] = turn[vl][lane];
+                // two 16-bit entries per lane
+                if (lane < 16 && i0 / 2 + lane < words)
+                    rows16[(long long)(v0 + vl) * words + i0 / 2 + lane] =
+                        *reinterpret_cast<const unsigned*>(&turn16[vl][2 * lane]);
+            }
             __syncthreads();
         }
     }
-}
-
-// sum_i sum_j |P_ij|^2 of every job.
-__global__ void k_label_sumsq(LabelArgs a, unsigned long long cap)
-{
-    extern __shared__ long long dyn_jobs[];
-    const LSlot* m = static_cast<const LSlot*>(a.lmap);
-    JobAcc acc(job_smem_init(a.jobs, dyn_jobs), &a.js[0].partition_sq, kJobStride);
-    const unsigned long long stride = (unsigned long long)gridDim.x * blockDim.x;
-    int classes = 0;
-    for (unsigned long long s = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x; s < cap; s += stride) {
-        if (m[s].key == kEmpty) continue;
-        ++classes;
-        const long long c = m[s].cnt;
-        const int P = (int)(m[s].key >> 32);
-        acc.add(a.pjob[P], c * c);
-        atomicAdd(reinterpret_cast<unsigned long long*>(a.part_sq + P), (unsigned long long)(c * c));
-        atomicAdd(a.part_slog + P, (double)c * log((double)c));
-    }
-    job_acc_finish(acc, a.jobs);
-    for (int o = 16; o > 0; o >>= 1) classes += __shfl_xor_sync(0xffffffffu, classes, o);
-    if ((threadIdx.x & 31) == 0 && classes)
-        atomicAdd(reinterpret_cast<unsigned long long*>(a.classes), (unsigned long long)classes);
 }
 
 // ---- state ----------------------------------------------------------------
@@ -654,8 +723,8 @@ cudaError_t launch_label_kernels(const LabelArgs& a, cudaStream_t s)
     const unsigned long long cap = a.lmask + 1;
     k_lmap_clear<<<grid_for((long long)cap), kSetupBlock, 0, s>>>(m, cap);
     k_label_insert<<<grid_for(a.tiles, 1), kBlock, 0, s>>>(a);
+    k_label_classes<<<grid_for((long long)cap, kTile), kBlock, smem_jobs_bytes(a.jobs), s>>>(a, cap);
     k_label_assign<<<grid_for(a.turns, 1), kBlock, 0, s>>>(a);
-    k_label_sumsq<<<grid_for((long long)cap), kSetupBlock, smem_jobs_bytes(a.jobs), s>>>(a, cap);
     return cudaGetLastError();
 }
 

@@ -127,3 +127,29 @@ def test_sparse_graphs(cc, shape, n, k):
             job.run_until_converged(20)
             assert job.history() == ref.stats
             np.testing.assert_array_equal(job.cluster_ids(), ref.C)
+
+
+# 16-bit label rows hold partitions of up to 65535 classes, and up to 512
+# partitions are counted in shared memory: both sides of both lines, alone and
+# next to a job of the other kind
+@pytest.mark.parametrize("n,classes", [(66001, [65535, 900, 65534]), (66001, [900, 65536, 900]), (301, [40] * 512),
+                                       (301, [40] * 513)])
+def test_label_rows(cc, n, classes):
+    rng = np.random.default_rng(len(classes) + classes[0])
+    base = np.arange(n) // 33
+    lab = np.stack([np.where(np.arange(n) < K, np.arange(n), rng.integers(0, K, n)) if K > 1000 else
+                    np.where(rng.random(n) < 0.2, rng.integers(0, K, n), base % K) for K in classes]).astype(np.int32)
+    ro, col = _graph(rng, n)
+    small = make_config("lfr", n=2000, k=9, cmin=10, cmax=300, max_deg=100, seed=n)
+    jobs = [(ro, col, lab), (small["row_off"], small["col"], small["labels"])]
+    refs = [oracle.sync_run(*j, 6) for j in jobs]
+    with cc.Consensus(*jobs[0]) as job, cc.ConsensusBatch(jobs) as batch:
+        job.run_until_converged(6)
+        assert job.history() == refs[0].stats
+        np.testing.assert_array_equal(job.cluster_ids(), refs[0].C)
+        want, got = oracle.metrics(lab, refs[0].C), job.metrics()
+        for f in ("mirkin", "split_join"):
+            np.testing.assert_array_equal(got[f], want[f])
+        batch.run_until_converged(6)
+        assert [batch.history(j) for j in range(2)] == [r.stats for r in refs]
+        np.testing.assert_array_equal(batch.cluster_ids(), np.concatenate([r.C for r in refs]))
