@@ -14,11 +14,11 @@
 //   jid   int32[N]     job of each vertex (and of each cluster id)
 //   G     int32[...]   compacted label ids, vertex-major: job j's rows start at go_j,
 //                      kp_j = k_j rounded up to 4 ints each (16-byte rows, padding -1);
-//   G16   16-bit numbers of the same classes, counted from 0 within each partition, in
-//                      rows of quads16(k_j) 16-byte words (valid where JobInfo::narrow);
 //                      g = (i << s_j) | rep, rep the job-local index of the least vertex
 //                      carrying that label in partition i and 2^s_j >= n_j, so g names
 //                      (partition, label) within the job and g < 2 k_j n_j.
+//   G16   int4[...]    the same labels as 16-bit class numbers, counted from 0 within each
+//                      partition: rows of quads16(k_j) words (valid where JobInfo::narrow)
 //   summ  int4[...]    same layout as G, one row per cluster id: per partition i
 //                      {d1, m1, d2, m2}: the two label ids that were most frequent in the
 //                      cluster at the last table rebuild (d1 first; -1 where the cluster

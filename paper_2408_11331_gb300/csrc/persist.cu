@@ -358,7 +358,6 @@ __global__ void __launch_bounds__(kBlock, 4)
     // keeps the rest
     __shared__ union {
         EdgeScratch edge[kWarpsPerBlock];
-        int4 proposal[kBlock];
         TileCount tile;
     } scratch;
     DevState* st = a.st;
@@ -380,7 +379,7 @@ __global__ void __launch_bounds__(kBlock, 4)
             break;
         case kOwn: own_step<kSingle>(a); break;
         case kEdges: edges_phase<kSingle>(a, scratch.edge); break;
-        case kCollect: collect_phase(a, scratch.proposal); break;
+        case kCollect: collect_phase(a); break;
         case kMark: mark_step(a); break;
         case kApply: apply_step(a, 0); break;
         case kUndo: apply_step(a, 1); break;

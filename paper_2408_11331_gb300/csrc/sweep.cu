@@ -79,8 +79,7 @@ __global__ void __launch_bounds__(kBlock, 4) k_edges(SweepArgs a)
 
 __global__ void __launch_bounds__(kBlock) k_collect(SweepArgs a)
 {
-    __shared__ int4 sbuf[kBlock];
-    collect_phase(a, sbuf);
+    collect_phase(a);
 }
 
 __global__ void k_route(SweepArgs a)

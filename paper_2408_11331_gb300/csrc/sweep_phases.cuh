@@ -815,60 +815,88 @@ __device__ __forceinline__ void edges_phase(const SweepArgs& a, EdgeScratch* sh)
 }
 
 // Turns the bids into the proposal list (v, a, b, dD), counts them per job and
-// clears best[].  Each block gathers its proposals in shared memory (sbuf, one
-// entry per thread) and appends them with one global atomic.
-__device__ __forceinline__ void collect_phase(const SweepArgs& a, int4* sbuf)
+// clears best[].  A block takes tiles of one vertex per thread, or of four
+// where that still gives every block one, and one range of the list per tile:
+// adds to the list's length go through one after another, about 6 ns each, and
+// were most of the step with small tiles and a sum per warp for the job's
+// count (n = 1e6: 22 us; with fewer tiles than blocks, n = 1.5e5, large ones
+// took 13 us instead of 11).  With one job the length is the job's count, and
+// route_phase copies it.
+__device__ __forceinline__ void collect_phase(const SweepArgs& a)
 {
+    constexpr int kPer = 4;
     extern __shared__ long long dyn_jobs[];
     DevState* st = a.st;
     if (st->skip) return;
     __shared__ int s_cnt, s_keys;
     __shared__ unsigned long long s_base;
+    const bool many_jobs = a.jobs > 1;
     JobAcc acc(job_smem_init(a.jobs, dyn_jobs), reinterpret_cast<long long*>(&a.js[0].nprop), kJobStride);
-    const long long stride = (long long)gridDim.x * blockDim.x;
-    for (long long b0 = (long long)blockIdx.x * blockDim.x; b0 < a.n; b0 += stride) {
+    const int lane = threadIdx.x & 31;
+    const unsigned lt = (1u << lane) - 1u;
+    const int per = a.n >= (long long)gridDim.x * (kPer * kBlock) ? kPer : 1;
+    const long long stride = (long long)gridDim.x * (per * kBlock);
+    for (long long b0 = (long long)blockIdx.x * (per * kBlock) + threadIdx.x; b0 - threadIdx.x < a.n; b0 += stride) {
         if (threadIdx.x == 0) {
             s_cnt = 0;
             s_keys = 0;
         }
         __syncthreads();
-        const long long v = b0 + threadIdx.x;
-        if (v < a.n) {
-            unsigned long long key = a.best[v];
-            if (key != kEmpty) a.best[v] = kEmpty;
-            if (a.active_set) {
+        unsigned long long key[kPer];
+        int rank[kPer], total = 0, keys = 0;
+#pragma unroll
+        for (int q = 0; q < kPer; ++q) {
+            const long long v = b0 + q * kBlock;
+            key[q] = q < per && v < a.n ? a.best[v] : kEmpty;
+        }
+#pragma unroll
+        for (int q = 0; q < kPer; ++q) {
+            const long long v = b0 + q * kBlock;
+            if (q > 0 && q >= per) break;
+            if (key[q] != kEmpty) a.best[v] = kEmpty;
+            if (a.active_set && v < a.n) {
                 // a vertex scored only on its changed candidates keeps its
                 // previous bid if that is still the least; a vertex of a
                 // stopped job bids nothing
-                if (a.js[a.jid[v]].stop) key = kEmpty;
-                else if (!st->all_active && !a.act[v] && a.prev[v] < key) key = a.prev[v];
-                a.prev[v] = key;
+                if (a.js[a.jid[v]].stop) key[q] = kEmpty;
+                else if (!st->all_active && !a.act[v] && a.prev[v] < key[q]) key[q] = a.prev[v];
+                a.prev[v] = key[q];
             }
-            if (key != kEmpty) {
+            const unsigned on = __ballot_sync(kFull, key[q] != kEmpty);
+            rank[q] = total + __popc(on & lt);
+            total += __popc(on);
+            if (many_jobs && key[q] != kEmpty) {
                 const int job = a.jid[v];
                 acc.add(job, 1);
-                const int p = atomicAdd(&s_cnt, 1);
-                atomicAdd(&s_keys, a.job[job].k);
-                sbuf[p] = make_int4((int)v, a.C[v], (int)(unsigned)(key & 0xffffffffull), key_gain(key));
+                keys += a.job[job].k;
             }
         }
+        if (many_jobs)
+            for (int o = 16; o > 0; o >>= 1) keys += __shfl_xor_sync(kFull, keys, o);
+        int base = 0;
+        if (lane == 0 && total) {
+            base = atomicAdd(&s_cnt, total);
+            if (many_jobs) atomicAdd(&s_keys, keys);
+        }
+        base = __shfl_sync(kFull, base, 0);
         __syncthreads();
         if (threadIdx.x == 0 && s_cnt > 0) {
             s_base = atomicAdd(&st->nprop, (unsigned long long)s_cnt);
-            atomicAdd(&st->pkeys, (unsigned long long)s_keys);
+            if (many_jobs) atomicAdd(&st->pkeys, (unsigned long long)s_keys);
         }
         __syncthreads();
-        for (int p = threadIdx.x; p < s_cnt; p += blockDim.x) {
-            const int4 q = sbuf[p];
-            const unsigned long long jj = s_base + p;
-            a.pv[jj] = q.x;
-            a.pa[jj] = q.y;
-            a.pb[jj] = q.z;
-            a.pg[jj] = q.w;
-        }
-        __syncthreads();
+#pragma unroll
+        for (int q = 0; q < kPer; ++q)
+            if (key[q] != kEmpty) {
+                const long long v = b0 + q * kBlock;
+                const unsigned long long p = s_base + (unsigned)(base + rank[q]);
+                a.pv[p] = (int)v;
+                a.pa[p] = a.C[v];
+                a.pb[p] = (int)(unsigned)(key[q] & 0xffffffffull);
+                a.pg[p] = key_gain(key[q]);
+            }
     }
-    job_acc_finish(acc, a.jobs);
+    if (many_jobs) job_acc_finish(acc, a.jobs);
 }
 
 // ---- heavy sweeps --------------------------------------------------------
@@ -888,7 +916,12 @@ __device__ __forceinline__ void route_phase(const SweepArgs& a)
     const unsigned long long total_keys = a.keys;
     DevState* st = a.st;
     st->heavy = 0;
-    if (st->skip || st->err || st->nprop == 0) return;
+    if (st->skip) return;
+    if (a.jobs == 1) {
+        a.js[0].nprop = st->nprop;
+        st->pkeys = st->nprop * (unsigned long long)a.job[0].k;
+    }
+    if (st->err || st->nprop == 0) return;
     // light when the proposals move at most 1/8 of all label rows (for one
     // job: |P| <= n / 8)
     const bool light = a.sweep_mode == 1 || (a.sweep_mode == 0 && st->pkeys * 8 <= total_keys);
