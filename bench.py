@@ -64,12 +64,12 @@ UNIT = "edge-partitions/s"
 # changed since).
 NOMINAL_HBM_GBS = 7900.0  # GB300 HBM3e, nominal (the roofline's peak is the measured copy rate)
 
-PROPOSAL_TRAFFIC = {"knn_n2000000_k50": 47.90e9, "lfr_n1000000_k20": 3.648e9}
+PROPOSAL_TRAFFIC = {"knn_n2000000_k50": 12.06e9, "lfr_n1000000_k20": 2.802e9}
 PROPOSAL_TRAFFIC_SOURCE = {
     "knn_n2000000_k50": "ncu dram__bytes_read.sum + dram__bytes_write.sum of k_own, k_edges, k_collect over one "
-                        "run at n=500000 (11.706 GB), scaled by nnz (x4.0921)",
+                        "run at n=500000 (2.946 GB), scaled by nnz (x4.0921)",
     "lfr_n1000000_k20": "ncu dram__bytes_read.sum + dram__bytes_write.sum of k_own, k_edges, k_collect over one "
-                        "run at n=500000 (1.824 GB), scaled by nnz (x2.0002)"}
+                        "run at n=500000 (1.401 GB), scaled by nnz (x2.0002)"}
 
 
 def parse():
@@ -443,7 +443,7 @@ def single_job(args, c, local, dist, rank, world, extras=True):
     achieved = float(np.sum(balg[:n_sw])) / (prop_total_ms / 1e3) / 1e9
     traffic = PROPOSAL_TRAFFIC.get(c["name"])
     out["roofline"] = {
-        "kernel": "proposal step (k_own + k_edges + k_collect, one launch each per sweep)",
+        "kernel": "proposal step (own, edges and collect of every sweep, inside the run kernel)",
         "bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s", "frac": achieved / peak,
         "traffic": traffic,
         "achieved_kind": "algorithmic: unit-cost bytes of the method per step / proposal-kernel time",

@@ -279,7 +279,7 @@ cc_status cc_job_labels(cc_ctx* ctx, int32_t job, int32_t* out);
 /* The batch calls under the names of the interface's first description
  * (a batch context is a cc_ctx from cc_batch_create):
  * cc_batch_run  = cc_run_until_converged without the sweep count: the whole
- *                 run of every job (one graph launch for a batch context).
+ *                 run of every job (one launch for a batch context).
  * cc_batch_result = job `job`'s consensus labels (int32[n_j] host, as
  *                 cc_job_labels) and objective (as cc_job_objective); either
  *                 output may be NULL, not both.  Errors as those calls. */
@@ -454,7 +454,7 @@ cc_status cc_server_create(const cc_server_options* sopt, const cc_options* opt,
 cc_status cc_server_submit(cc_server* s, const cc_job_desc* job, int32_t* labels_out, int64_t* ticket);
 
 /* Advances the server: harvests the contexts whose jobs have all stopped,
- * queues the next graph launch of those still running and admits waiting
+ * queues the next launch of those still running and admits waiting
  * jobs.  wait != 0: if nothing finished and nothing was admitted, keeps
  * polling (at most about a second) until something does.  Up to max_done
  * tickets of jobs done since the last report are written to done (*n_done
