@@ -1157,13 +1157,13 @@ __global__ void k_load_check_fill(DevState* st, unsigned long long new_keys)
 // Singleton state of the place's vertices (stamped as changed in the sweep
 // just run, so that the next sweep computes their own-cluster sums) and the
 // summary rows of the new job's label rows; the run goes on.
-__global__ void k_load_state(SweepArgs a, long long vo, long long ncap, long long go, long long rows)
+__global__ void k_load_state(SweepArgs a, JobInfo J, long long ncap)
 {
     const long long stride = (long long)gridDim.x * blockDim.x;
     const long long t0 = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     const int stamp = a.st->stamp;
     for (long long t = t0; t < ncap; t += stride) {
-        const long long v = vo + t;
+        const long long v = J.vo + t;
         a.C[v] = (int)v;
         a.size[v] = 1;
         a.dsize[v] = 0;
@@ -1173,9 +1173,9 @@ __global__ void k_load_state(SweepArgs a, long long vo, long long ncap, long lon
         a.prev[v] = kEmpty;
         a.act[v] = 1;
     }
-    for (long long r = t0; r < rows; r += stride) {
-        const int g = a.G[go + r];
-        a.summ[go + r] = make_int4(g, g >= 0 ? 1 : 0, -1, 0);
+    for (long long r = t0; r < J.n * J.kp; r += stride) {
+        const int g = a.G[J.go + r], i = (int)(r % J.kp);
+        a.summ[J.go + r - i + summ_at(J, i)] = make_int4(g, g >= 0 ? 1 : 0, -1, 0);
     }
     if (t0 == 0) a.st->stop = 0;
 }
@@ -1711,7 +1711,7 @@ cc_status ctx_load_job(cc_ctx* c, int j, const JobInput& in)
     // singleton state of the place's vertices, their summary rows, and a
     // table rebuild in the next sweep
     if (e == cudaSuccess) {
-        k_load_state<<<g, 256, 0, c->stream>>>(c->args, J.vo, ncap, J.go, n * J.kp);
+        k_load_state<<<g, 256, 0, c->stream>>>(c->args, J, ncap);
         k_load_check_fill<<<1, 1, 0, c->stream>>>(c->st, (unsigned long long)keys);
         k_load_keys<<<g, 256, 0, c->stream>>>(c->args, J, J.vo);
         e = cudaGetLastError();

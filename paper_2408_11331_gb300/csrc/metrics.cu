@@ -154,7 +154,7 @@ __global__ void k_met_clusters(SweepArgs a, MetricsArgs m, int parts)
         const int4* S = a.summ + row_of(J, x);
         const int P0 = m.pfirst[j];
         for (int i = 0; i < J.k; ++i)
-            atomicAdd(reinterpret_cast<unsigned long long*>(sjc + P0 + i), (unsigned long long)S[i].y);
+            atomicAdd(reinterpret_cast<unsigned long long*>(sjc + P0 + i), (unsigned long long)S[summ_at(J, i)].y);
     }
     if (shared) {
         __syncthreads();

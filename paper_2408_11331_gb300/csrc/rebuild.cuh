@@ -373,7 +373,7 @@ __device__ __forceinline__ void table_build_phase(const SweepArgs& a, int condit
                 const unsigned long long top2 = segment_max(other, lane, seg_end);
                 if (head && on) {
                     const int d2 = top2 ? (int)(unsigned)top2 : -1, m2 = (int)(top2 >> 32);
-                    S[i0 + b] = make_int4((int)(unsigned)top1, (int)(top1 >> 32), d2, m2);
+                    S[b * ((k + 3) >> 2) + (i0 >> 2)] = make_int4((int)(unsigned)top1, (int)(top1 >> 32), d2, m2);
                 }
             }
         }
@@ -409,7 +409,7 @@ __device__ __forceinline__ void summ_top_phase(const SweepArgs& a, int condition
         const int x = (int)(e.x >> 32), g = (int)(unsigned)(e.x & 0xffffffffull);
         const int job = a.jid[x];
         const JobInfo& J = a.job[job];
-        int4* E = a.summ + row_of(J, x) + (g >> J.lshift);
+        int4* E = a.summ + row_of(J, x) + summ_at(J, g >> J.lshift);
         const unsigned long long kn = ((unsigned long long)(unsigned)cnt << 32) | (unsigned)g;
         const volatile unsigned long long* Ev = reinterpret_cast<const volatile unsigned long long*>(E);
         ulonglong2 cur = make_ulonglong2(Ev[0], Ev[1]);

@@ -132,7 +132,7 @@ __device__ __forceinline__ int group_sum(int x, int gs)
 
 // The partitions of a job are scored four at a time ("quads"): partition
 // 4q + t is component t of quad q of v's label row (one int4 load) and entry
-// 4q + t of x's summary row (one int4 {d1, m1, d2, m2} per partition).  Rows
+// q + t kp / 4 of x's summary row (one int4 {d1, m1, d2, m2} per partition).  Rows
 // are kp = k rounded up to 4 entries; the padding (label -1, summary {-1, 0,
 // -1, 0}) adds nothing to the sums below and is never probed.  Lane l of a
 // group takes quads l, l + gs, ...  (One partition per lane, with contiguous
@@ -163,7 +163,7 @@ __device__ __forceinline__ void summary_part(const SweepArgs& a, const JobInfo& 
     const int kq = J.kp >> 2;
     for (int q = l; q < kq; q += gs) {
         const int4 g = __ldg(G4 + q);
-        const int4 e0 = S4[4 * q], e1 = S4[4 * q + 1], e2 = S4[4 * q + 2], e3 = S4[4 * q + 3];
+        const int4 e0 = S4[q], e1 = S4[q + kq], e2 = S4[q + 2 * kq], e3 = S4[q + 3 * kq];
         summary_one(g.x, e0, sx, ex, open);
         summary_one(g.y, e1, sx, ex, open);
         summary_one(g.z, e2, sx, ex, open);
@@ -198,10 +198,10 @@ __device__ __forceinline__ int probe_part(const SweepArgs& a, const JobInfo& J, 
         const int4 g = __ldg(G4 + q);
         ulonglong2 ev[4];
         bool on[4];
-        on[0] = probe_start(table, mask, x, g.x, S4[4 * q], sx, ev[0]);
-        on[1] = probe_start(table, mask, x, g.y, S4[4 * q + 1], sx, ev[1]);
-        on[2] = probe_start(table, mask, x, g.z, S4[4 * q + 2], sx, ev[2]);
-        on[3] = probe_start(table, mask, x, g.w, S4[4 * q + 3], sx, ev[3]);
+        on[0] = probe_start(table, mask, x, g.x, S4[q], sx, ev[0]);
+        on[1] = probe_start(table, mask, x, g.y, S4[q + kq], sx, ev[1]);
+        on[2] = probe_start(table, mask, x, g.z, S4[q + 2 * kq], sx, ev[2]);
+        on[3] = probe_start(table, mask, x, g.w, S4[q + 3 * kq], sx, ev[3]);
         const int gq[4] = {g.x, g.y, g.z, g.w};
 #pragma unroll
         for (int b = 0; b < 4; ++b)
