@@ -49,18 +49,6 @@ struct __align__(16) LSlot {
     int cnt;
 };
 
-// Largest index i with key[i] <= x among key[0..count) (key[0] <= x assumed).
-__device__ __forceinline__ int upper_index(const long long* key, int count, long long x)
-{
-    int lo = 0, hi = count - 1;
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if (key[mid] <= x) lo = mid;
-        else hi = mid - 1;
-    }
-    return lo;
-}
-
 __device__ __forceinline__ int job_of_vertex(const JobInfo* job, int jobs, long long v)
 {
     int lo = 0, hi = jobs - 1;
