@@ -50,7 +50,8 @@ typedef enum {
     CC_ERR_CUDA = 3,       /* a CUDA runtime call or kernel failed */
     CC_ERR_OVERFLOW = 4,   /* 3 k n + k >= 2^31: an int32 gain could overflow */
     CC_ERR_TABLE_FULL = 5, /* the contingency hash ran out of slots (bounded probing gave up) */
-    CC_ERR_TIMEOUT = 6     /* a block of the run kernel waited more than 20 s for the others */
+    CC_ERR_TIMEOUT = 6     /* a block of the run kernel waited too long for the others (see
+                              cc_set_wait_limit) */
 } cc_status;
 
 typedef struct {
@@ -288,6 +289,14 @@ cc_status cc_batch_result(cc_ctx* ctx, int32_t job, int32_t* labels_out, int64_t
 
 /* Uses the given cudaStream_t (NULL: the context's own) for later calls. */
 cc_status cc_set_stream(cc_ctx* ctx, void* stream);
+
+/* Longest time (ns, >= 0) that a block of the run kernel waits for the others
+ * before the run ends with CC_ERR_TIMEOUT; 20 s in a new context.  0: no
+ * wait at all, so that a run of more than one block ends so (to try a caller's
+ * handling of the error).  After CC_ERR_TIMEOUT the consensus is that of some
+ * moment inside a sweep; cc_reset and cc_set_cluster_ids make the context
+ * usable again.  Errors: CC_ERR_INVALID (ns < 0). */
+cc_status cc_set_wait_limit(cc_ctx* ctx, int64_t ns);
 
 /* Returns the context to the singleton start (C[v] = v, F = F0) with the
  * inputs kept resident; the sweep history is cleared. */

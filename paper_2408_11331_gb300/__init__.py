@@ -88,6 +88,9 @@ class Consensus:
     def set_stream(self, stream: int = 0):
         _native.cc_set_stream(self._ctx, stream)
 
+    def set_wait_limit(self, ns: int):
+        _native.cc_set_wait_limit(self._ctx, ns)
+
     def reset(self):
         _native.cc_reset(self._ctx)
 
@@ -180,6 +183,9 @@ class ConsensusBatch:
 
     def set_stream(self, stream: int = 0):
         _native.cc_set_stream(self._ctx, stream)
+
+    def set_wait_limit(self, ns: int):
+        _native.cc_set_wait_limit(self._ctx, ns)
 
     def reset(self):
         _native.cc_reset(self._ctx)

@@ -20,7 +20,7 @@ STATUS_NAMES = {0: "CC_OK", 1: "CC_ERR_INVALID", 2: "CC_ERR_OOM", 3: "CC_ERR_CUD
                 5: "CC_ERR_TABLE_FULL", 6: "CC_ERR_TIMEOUT"}
 
 # Every symbol include/cc.h declares; the CPU test suite checks the library exports them.
-EXPORTS = ("cc_default_options", "cc_create", "cc_create_dev", "cc_set_stream", "cc_reset", "cc_set_cluster_ids", "cc_sweep",
+EXPORTS = ("cc_default_options", "cc_create", "cc_create_dev", "cc_set_stream", "cc_set_wait_limit", "cc_reset", "cc_set_cluster_ids", "cc_sweep",
            "cc_run_until_converged", "cc_last_run_timing", "cc_table_stats", "cc_launch_count", "cc_history", "cc_objective", "cc_objective_recompute",
            "cc_consensus_labels", "cc_cluster_ids", "cc_cluster_ids_dev", "cc_last_error", "cc_destroy",
            "cc_batch_create", "cc_job_count", "cc_job_objective", "cc_job_history", "cc_job_labels",
@@ -101,6 +101,8 @@ def load_library(path: str = LIB_PATH) -> ctypes.CDLL:
                                   c.POINTER(P)]
     lib.cc_set_stream.restype = c.c_int
     lib.cc_set_stream.argtypes = [P, P]
+    lib.cc_set_wait_limit.restype = c.c_int
+    lib.cc_set_wait_limit.argtypes = [P, c.c_int64]
     lib.cc_reset.restype = c.c_int
     lib.cc_reset.argtypes = [P]
     lib.cc_set_cluster_ids.restype = c.c_int
@@ -298,6 +300,10 @@ def cc_batch_result(ctx, job: int, n: int) -> tuple[np.ndarray, int]:
 
 def cc_set_stream(ctx, stream: int = 0):
     _check(lib.cc_set_stream(ctx, ctypes.c_void_p(stream or None)), ctx)
+
+
+def cc_set_wait_limit(ctx, ns: int):
+    _check(lib.cc_set_wait_limit(ctx, ns), ctx)
 
 
 def cc_reset(ctx):

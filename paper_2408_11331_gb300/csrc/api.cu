@@ -3,6 +3,7 @@
 // and the output calls.
 #include <algorithm>
 #include <atomic>
+#include <cstddef>
 #include <cstdio>
 #include <cstring>
 #include <map>
@@ -129,6 +130,16 @@ cc_status read_state_jobs(cc_ctx* c, DevState* out, std::vector<JobState>& js)
     return CC_OK;
 }
 
+// After a run kernel that gave up a wait (s: its control block): its blocks
+// left the barrier's count in the middle of a step, and a launch that started
+// from it would release barriers before all of its blocks have arrived.
+cc_status clear_barrier(cc_ctx* c, const DevState& s)
+{
+    static_assert(offsetof(DevState, bar_abort) == offsetof(DevState, bar_count) + 4, "cleared together");
+    if (s.bar_abort) CC_CUDA(c, cudaMemsetAsync(&c->st->bar_count, 0, 8, c->stream));
+    return CC_OK;
+}
+
 cc_status read_jobs(cc_ctx* c, std::vector<JobState>& out)
 {
     out.resize(c->jobs);
@@ -141,6 +152,7 @@ cc_status check_device_error(cc_ctx* c, const DevState& s)
 {
     if (s.err == CC_ERR_TABLE_FULL) return fail(c, CC_ERR_TABLE_FULL, "contingency hash is full");
     if (s.err == CC_ERR_INVALID) return fail(c, CC_ERR_INVALID, "inconsistent contingency state");
+    if (s.err == CC_ERR_TIMEOUT) return fail(c, CC_ERR_TIMEOUT, "a block of the run kernel waited too long for the others");
     if (s.err != 0) return fail(c, (cc_status)s.err, "device-side failure");
     return CC_OK;
 }
@@ -273,6 +285,8 @@ long long launch_budget(const cc_ctx* c, int limit, int chunk)
 // which 0.2 ms of host time per launch).
 constexpr long long kRunKernelRows = 1 << 14;
 
+constexpr unsigned long long kWaitLimitNs = 20ull * 1000 * 1000 * 1000;  // see cc_set_wait_limit
+
 // Appends the device times of the bodies run since the last call (entries of
 // ts from ts_from, ns) to sweep_ms and propose_ms.
 cc_status read_run_times(cc_ctx* c)
@@ -355,6 +369,7 @@ cc_status run_kernel(cc_ctx* c, int limit, DevState* out, std::vector<JobState>&
         CC_CUDA(c, launch_run(c->args, c->rows, c->run_blocks, limit, fresh, budget, c->stream));
         c->launches += 1;
         r = read_state_jobs(c, &st, js);
+        if (r == CC_OK) r = clear_barrier(c, st);
         if (r != CC_OK) return r;
         c->ts_from = 0;
         c->ts_bodies = st.run_bodies - before;
@@ -895,6 +910,7 @@ cc_status create_common(int jobs, const JobInput* in, bool on_device, const cc_o
     a.st = c->st;
     a.hist = c->hist;
     a.hist_cap = c->hist_cap;
+    a.wait_ns = kWaitLimitNs;
 
     if (c->opt.colour_batched) {
         CC_TRY(dalloc(c, &c->colour, (size_t)N));
@@ -1833,6 +1849,13 @@ cc_status cc_set_stream(cc_ctx* c, void* stream)
     return CC_OK;
 }
 
+cc_status cc_set_wait_limit(cc_ctx* c, int64_t ns)
+{
+    if (!c || ns < 0) return fail(c, CC_ERR_INVALID, c ? "the wait limit must not be negative" : "ctx is NULL");
+    c->args.wait_ns = (unsigned long long)ns;
+    return CC_OK;
+}
+
 cc_status cc_reset(cc_ctx* c)
 {
     if (!c) return fail(nullptr, CC_ERR_INVALID, "ctx is NULL");
@@ -1880,6 +1903,8 @@ cc_status cc_set_cluster_ids(cc_ctx* c, const int32_t* C)
     for (int j = 0; j < c->jobs; ++j) {
         js[j].F = F[j];
         js[j].stop = 1;
+        // (a colour-batched sweep that ended on an error left its totals)
+        js[j].t_prop = js[j].t_p1 = js[j].t_dFp1 = js[j].t_fb = js[j].t_moves = 0;
     }
     CC_CUDA(c, cudaMemcpyAsync(c->js, js.data(), sizeof(JobState) * c->jobs, cudaMemcpyHostToDevice, c->stream));
     int one = 1;

@@ -142,9 +142,9 @@ struct DevState {
     int rebuild_kind;            // the running rebuild: 0 heavy sweep, 1 its rollback, 2 end of the sweep
     int tries;                   // rebuild attempts of this heavy sweep
     int bodies_left;             // sweep bodies the launch may still run
-    unsigned bar_count;          // blocks that have arrived at the barrier
     unsigned bar_word;           // barriers passed << 8 | step that follows
-    int bar_abort;               // 1: a block gave up waiting; every block leaves
+    unsigned bar_count;          // blocks that have arrived at the barrier; 0 between launches (left over where
+    int bar_abort;               //    a block gave up waiting (1: every block leaves): the host clears both)
 };
 
 // Arguments of the kernels (passed by value).
@@ -198,6 +198,7 @@ struct SweepArgs {
     unsigned long long* ts;     // kRunBodies times {start of a sweep body, end of its proposal step, its end} (ns)
     cc_sweep_info* hist;        // J x hist_cap records
     int hist_cap;
+    unsigned long long wait_ns; // run kernel: longest wait of a block at a barrier (cc_set_wait_limit)
 };
 
 // The block's share of a step's items (each one warp's work, of uneven cost):

@@ -26,8 +26,6 @@ namespace ccg {
 
 namespace {
 
-constexpr unsigned long long kBarrierLimitNs = 20ull * 1000 * 1000 * 1000;  // a wait past this gives up
-
 __device__ __forceinline__ unsigned ld_relaxed(const unsigned* p)
 {
     unsigned x;
@@ -61,10 +59,13 @@ enum Step {
 // (all its threads; the value counts in thread 0), which takes the decisions
 // that follow from the finished step and returns the next one; the others
 // wait for it.  Barrier number and next step travel in one word, so every
-// block takes the same step without another load.  A wait that exceeds its
-// limit sets st->err and ends the kernel in every block.
+// block takes the same step without another load.  A wait that exceeds
+// wait_ns sets st->err and ends the kernel in every block: the blocks still at
+// work finish their step and at most one more, for no later barrier sees all
+// of them.
 template <class Schedule>
-__device__ __forceinline__ int grid_step(DevState* st, unsigned& word, unsigned& arrivals, Schedule schedule)
+__device__ __forceinline__ int grid_step(DevState* st, unsigned long long wait_ns, unsigned& word, unsigned& arrivals,
+                                         Schedule schedule)
 {
     __shared__ unsigned s_word;
     __shared__ int s_last;
@@ -87,9 +88,9 @@ __device__ __forceinline__ int grid_step(DevState* st, unsigned& word, unsigned&
         // would drop the L1 lines of the blocks still at work on this SM
         for (unsigned spins = 1; (now = ld_relaxed(&st->bar_word)) == word; ++spins) {
             __nanosleep(100);
-            if (spins & 1023u) continue;
+            if ((spins & 1023u) && wait_ns) continue;
             if (t0 == 0) t0 = now_ns();
-            if (*reinterpret_cast<volatile int*>(&st->bar_abort) || now_ns() - t0 > kBarrierLimitNs) {
+            if (*reinterpret_cast<volatile int*>(&st->bar_abort) || !wait_ns || now_ns() - t0 > wait_ns) {
                 set_err(st, CC_ERR_TIMEOUT);
                 st->bar_abort = 1;
                 now = kLeave;
@@ -399,7 +400,7 @@ __global__ void __launch_bounds__(kBlock, 4)
             break;
         }
         const int done = step;
-        step = grid_step(st, word, arrivals, [&] { return Scheduler{a, limit, fresh}.next(done); });
+        step = grid_step(st, a.wait_ns, word, arrivals, [&] { return Scheduler{a, limit, fresh}.next(done); });
         if (clock && done == kCollect) a.ts[3 * body + 1] = now_ns();
         if (step == kLeave) break;
         last = done;
