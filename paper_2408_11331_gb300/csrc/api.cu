@@ -388,31 +388,31 @@ cc_status run_kernel(cc_ctx* c, int limit, DevState* out, std::vector<JobState>&
 
 // A run as graphs of one kernel per step: one launch whose WHILE node repeats
 // the sweep until the run stops, or, with no_regions, plain graphs of up to
-// kChunk sweeps, launched until the device says the run has stopped.
+// kChunk sweeps, launched until the device says the run has stopped.  An
+// autotuned context runs its first sweep alone (a plain graph of one body: the
+// loop holds kLoopSweeps) and times its lanes on the state that left.
 cc_status run_graphs(cc_ctx* c, int limit, DevState* out, std::vector<JobState>& js)
 {
     DevState& st = *out;
-    const bool plain = c->opt.no_regions != 0;
     const int chunk = chunk_bodies(c, limit);
     long long left = (long long)limit * c->ncls + 64;  // 64: sweeps abandoned for lack of table space and retried
     long long launches = launch_budget(c, limit, chunk);
     int before = 0;
     for (;;) {
-        // (an autotuned context first runs one sweep, then times its lanes on
-        // the state that left)
-        const int bodies = !c->tuned ? 1 : plain ? chunk : (int)std::min<long long>(left, kRunBodies);
+        const bool loop = c->tuned && !c->opt.no_regions;
+        const int bodies = !c->tuned ? 1 : loop ? (int)std::min<long long>(left, kRunBodies) : chunk;
         if (before == 0) CC_CUDA(c, launch_run_begin(c->args, limit, bodies, c->stream));
-        else if (!plain) CC_CUDA(c, launch_run_more(c->args, before + bodies, c->stream));
+        else if (loop) CC_CUDA(c, launch_run_more(c->args, before + bodies, c->stream));
         cudaGraphExec_t exec = nullptr;
-        cc_status r = ensure_graph(c, plain ? bodies : 0, &exec);
+        cc_status r = ensure_graph(c, loop ? 0 : bodies, &exec);
         if (r != CC_OK) return r;
-        if (before == 0 || !plain) c->launches += 1;
+        if (before == 0 || loop) c->launches += 1;
         CC_CUDA(c, cudaGraphLaunch(exec, c->stream));
         r = read_state_jobs(c, &st, js);
         if (r != CC_OK) return r;
         const int ran = st.run_bodies - before;
         const long long turns = (ran + kLoopSweeps - 1) / kLoopSweeps;
-        c->launches += plain ? (long long)bodies * kKernelsPerSweep : turns * (kLoopSweeps * kKernelsOutsideRegions + 1);
+        c->launches += loop ? turns * (kLoopSweeps * kKernelsOutsideRegions + 1) : (long long)bodies * kKernelsPerSweep;
         c->ts_from = before;
         c->ts_bodies = ran;
         before = st.run_bodies;

@@ -1,5 +1,10 @@
-"""The run kernel beside the ordinary run: waits that run out, against the
-oracle (whole numbers, exact)."""
+"""The run kernel and the graphs of a run beside the ordinary run: waits that
+run out, the autotuned first sweep (against the oracle where there are results;
+whole numbers, exact)."""
+import os
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 
@@ -8,6 +13,7 @@ from workloads import make_config
 
 pytestmark = pytest.mark.gpu
 
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 SECOND = 10**9
 
 
@@ -86,3 +92,32 @@ def test_batch_after_a_timeout(cc):
 def test_wait_limit_must_not_be_negative(cc):
     with cc.Consensus(*_job(40, 3)) as job, pytest.raises(cc.CCError):
         job.set_wait_limit(-1)
+
+
+# The lanes are timed after the first sweep of the first run.  Pairs of vertices
+# with the same labels merge in that sweep and the second finds nothing to do,
+# so a run that does two sweeps before it times them never times them.  (A
+# process of its own: the choices are remembered per process.)
+@pytest.mark.parametrize("n", [1000, 40000])
+@pytest.mark.parametrize("no_regions", [0, 1])
+def test_autotune_after_the_first_sweep(cc, n, no_regions):
+    code = f"""
+import ctypes, numpy as np, paper_2408_11331_gb300 as cc
+def record():
+    r = (ctypes.c_int32 * 6)()
+    cc._native._check(cc._native.lib.cc_autotune_record(6, r))
+    return list(r)
+n = {n}
+v = np.arange(n)
+col = (v ^ 1).astype(np.int32)
+lab = np.tile((v // 2).astype(np.int32), (10, 1))
+o = cc.cc_default_options()
+o.autotune, o.no_regions = 1, {no_regions}
+assert not any(record())
+with cc.Consensus(np.arange(n + 1, dtype=np.int64), col, lab, o) as job:
+    assert job.run_until_converged(20) == 2
+    assert np.array_equal(job.cluster_ids(), v // 2 * 2)
+    assert len(job.last_run_timing()[0]) == 2
+assert record()[0] > 0, record()
+"""
+    subprocess.run([sys.executable, "-c", code], check=True, cwd=ROOT, timeout=120)
