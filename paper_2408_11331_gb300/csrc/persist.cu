@@ -410,15 +410,25 @@ __global__ void __launch_bounds__(kBlock, 4)
 
 namespace {
 
-// Blocks of a run of this context: one thread per CSR entry or vertex and per
-// 8 label rows, at most what is resident.
 inline size_t run_smem(int jobs)
 {
     return (2 * jobs <= kSmemJobs ? 2 : 1) * smem_jobs_bytes(jobs);
 }
 
+// Places for blocks that a run leaves free, so that the caller's kernels on
+// other streams find one: four blocks of a run take all registers of an SM, and
+// with every place taken a small kernel waited for the end of the run (n =
+// 300,007, k = 24: 1224 us, now 47).  Two of 608 cost the run nothing (n = 1e6,
+// k = 20: 6.96 ms both), eight cost it 1%.
+inline int spare_blocks(int resident)
+{
+    return std::min(2, resident / 64);
+}
+
 }  // namespace
 
+// Blocks of a run of this context: one thread per CSR entry or vertex and per
+// 8 label rows, at most what is resident beside the spare ones.
 cudaError_t run_grid(const SweepArgs& a, long long rows, int sms, int* grid)
 {
     int per_sm = 0;
@@ -428,7 +438,8 @@ cudaError_t run_grid(const SweepArgs& a, long long rows, int sms, int* grid)
     if (e != cudaSuccess) return e;
     long long g = std::max((a.nnz + kBlock - 1) / kBlock, (rows + 8 * kBlock - 1) / (8 * kBlock));
     g = std::max(g, (a.n + kBlock - 1) / kBlock);
-    *grid = (int)std::max(0LL, std::min(g, (long long)per_sm * sms));
+    const int resident = per_sm * sms;
+    *grid = (int)std::max(0LL, std::min(g, (long long)resident - spare_blocks(resident)));
     return cudaSuccess;
 }
 

@@ -4,6 +4,8 @@ whole numbers, exact)."""
 import os
 import subprocess
 import sys
+import threading
+import time
 
 import numpy as np
 import pytest
@@ -121,3 +123,42 @@ with cc.Consensus(np.arange(n + 1, dtype=np.int64), col, lab, o) as job:
 assert record()[0] > 0, record()
 """
     subprocess.run([sys.executable, "-c", code], check=True, cwd=ROOT, timeout=120)
+
+
+# The caller's own kernels on another stream run beside a run, not after it.
+def test_other_streams_run_beside_a_run(cc):
+    torch = pytest.importorskip("torch")
+    job = cc.Consensus(*_job(200003, 24))
+    job.run_until_converged(20)
+    started = time.perf_counter()
+    job.reset()
+    job.run_until_converged(20)
+    run_s = time.perf_counter() - started
+    stop = threading.Event()
+
+    def runs():
+        while not stop.is_set():
+            job.reset()
+            job.run_until_converged(20)
+
+    other, x = torch.cuda.Stream(), torch.zeros(64, device="cuda")
+    with torch.cuda.stream(other):
+        x.add_(1)
+    torch.cuda.synchronize()
+    thread = threading.Thread(target=runs)
+    thread.start()
+    waits = []
+    try:
+        for _ in range(100):
+            t0 = time.perf_counter()
+            with torch.cuda.stream(other):
+                x.add_(1)
+            other.synchronize()
+            waits.append(time.perf_counter() - t0)
+            time.sleep(run_s / 3)
+    finally:
+        stop.set()
+        thread.join()
+        job.close()
+    # half a run on average where it waits for the end of the run
+    assert np.median(waits) < run_s / 6, (np.median(waits), run_s)
