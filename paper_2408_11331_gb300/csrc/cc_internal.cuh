@@ -648,8 +648,10 @@ cudaError_t capture_run_loop(const SweepArgs& a, long long rows, int grid, cudaS
                              cudaStream_t body);
 cudaError_t prepare_propose(int* blocks_per_sm);
 // ---- persist.cu ----
-// Grid of the run kernel for a context (0: it cannot be resident).
-cudaError_t run_grid(const SweepArgs& a, long long rows, int sms, int* grid);
+// Blocks of the run kernel: *most are resident at a time on `sms` SMs beside the
+// spare places (0: it cannot run), *want is what this context's work fills (one
+// thread per CSR entry or vertex and per 8 label rows).
+cudaError_t run_grid(const SweepArgs& a, long long rows, int sms, int* most, int* want);
 // The run kernel: up to `budget` sweep bodies of a run in one cooperative
 // launch (fresh: starts the run first; at most kRunBodies).
 cudaError_t launch_run(const SweepArgs& a, long long rows, int grid, int limit, bool fresh, int budget, cudaStream_t s);

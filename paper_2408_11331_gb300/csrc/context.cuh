@@ -79,7 +79,9 @@ struct cc_ctx {
     std::vector<float> propose_ms;      // ... and of its proposal kernels
     long long launches = 0;             // kernels launched so far
     int grid = 0;
-    int run_blocks = 0;                 // grid of the run kernel; 0: runs are graphs of one kernel per step
+    int run_blocks = 0;                 // most blocks of the run kernel; 0: runs are graphs of one kernel per step
+    int run_want = 0;                   // blocks that the context's work fills
+    int in_flight = 0;                  // blocks of its launch of the run kernel that may still run
     unsigned long long* ts = nullptr;   // three device times per sweep body (kRunBodies of them)
     int ts_from = 0, ts_bodies = 0;     // bodies of the last launch not yet in sweep_ms (read when asked for)
     unsigned long long cap_start = 0;   // active table capacity at the singleton start

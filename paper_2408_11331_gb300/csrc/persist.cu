@@ -427,9 +427,7 @@ inline int spare_blocks(int resident)
 
 }  // namespace
 
-// Blocks of a run of this context: one thread per CSR entry or vertex and per
-// 8 label rows, at most what is resident beside the spare ones.
-cudaError_t run_grid(const SweepArgs& a, long long rows, int sms, int* grid)
+cudaError_t run_grid(const SweepArgs& a, long long rows, int sms, int* most, int* want)
 {
     int per_sm = 0;
     const cudaError_t e =
@@ -439,7 +437,8 @@ cudaError_t run_grid(const SweepArgs& a, long long rows, int sms, int* grid)
     long long g = std::max((a.nnz + kBlock - 1) / kBlock, (rows + 8 * kBlock - 1) / (8 * kBlock));
     g = std::max(g, (a.n + kBlock - 1) / kBlock);
     const int resident = per_sm * sms;
-    *grid = (int)std::max(0LL, std::min(g, (long long)resident - spare_blocks(resident)));
+    *most = resident - spare_blocks(resident);
+    *want = (int)std::min(g, 1LL << 20);
     return cudaSuccess;
 }
 

@@ -162,3 +162,54 @@ def test_other_streams_run_beside_a_run(cc):
         job.close()
     # half a run on average where it waits for the end of the run
     assert np.median(waits) < run_s / 6, (np.median(waits), run_s)
+
+
+# Contexts that run at the same time share the GPU, so the number of blocks of a
+# launch depends on the others in flight; the results do not.
+def test_runs_in_threads(cc):
+    sizes = [(1500, 12), (6007, 9), (20011, 12), (3001, 33), (60001, 8), (6007, 20), (900, 40), (20011, 4), (40, 3)]
+    jobs = [_job(n, k) for n, k in sizes]
+    refs = [oracle.sync_run(*j, 20) for j in jobs]
+    wrong = []
+
+    def work(i):
+        with cc.Consensus(*jobs[i]) as job:
+            for _ in range(12):
+                job.reset()
+                sweeps = job.run_until_converged(20)
+                if (sweeps, job.history()) != (refs[i].sweeps, refs[i].stats) or not np.array_equal(job.cluster_ids(), refs[i].C):
+                    wrong.append(i)
+
+    threads = [threading.Thread(target=work, args=(i,)) for i in range(len(jobs))]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not wrong
+
+
+# Two contexts that each fill the GPU alone: run together they take less than
+# one after the other.
+def test_two_runs_overlap(cc):
+    jobs = [cc.Consensus(*_job(20011, 12, seed)) for seed in (1, 2, 3, 4)]
+
+    def work(job):
+        for _ in range(30):
+            job.reset()
+            job.run_until_converged(20)
+
+    def wall(groups):
+        threads = [threading.Thread(target=lambda g=g: [work(j) for j in g]) for g in groups]
+        t0 = time.perf_counter()
+        for t in threads:
+            t.start()
+        for t in threads:
+            t.join()
+        return time.perf_counter() - t0
+
+    wall([jobs])
+    alone = min(wall([jobs]) for _ in range(3))
+    together = min(wall([[j] for j in jobs]) for _ in range(3))
+    for j in jobs:
+        j.close()
+    assert together < 0.75 * alone, (together, alone)  # one after the other: 0.9
