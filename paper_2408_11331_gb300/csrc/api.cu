@@ -10,6 +10,8 @@
 #include <string>
 #include <vector>
 
+#include <cudaTypedefs.h>
+
 #include "context.cuh"
 
 using namespace ccg;
@@ -391,9 +393,45 @@ cudaError_t launch_share(cc_ctx* c, int limit, bool fresh, int budget)
         f.blocks.fetch_add(grid);
         c->in_flight = grid;
     }
-    const cudaError_t e = launch_run(c->args, c->rows, grid, limit, fresh, budget, c->stream);
+    cudaError_t e = launch_run(c->args, c->rows, grid, limit, fresh, budget, c->stream);
+    // (fewer places than size_run counted: any grid gives the same results)
+    while (e == cudaErrorCooperativeLaunchTooLarge && grid > 1) {
+        cudaGetLastError();
+        c->run_blocks = grid /= 2;
+        e = launch_run(c->args, c->rows, grid, limit, fresh, budget, c->stream);
+    }
     if (e != cudaSuccess) end_flight(c);
     return e;
+}
+
+// SMs that kernels on stream s may use: the device's, or those of its green
+// context (a part of the GPU that the caller has set aside).
+int stream_sms(cudaStream_t s, int device_sms)
+{
+    static const auto entry = [](const char* name) -> void* {
+        void* f = nullptr;
+        cudaDriverEntryPointQueryResult found = cudaDriverEntryPointSymbolNotFound;
+        const cudaError_t e = cudaGetDriverEntryPointByVersion(name, &f, 12040, cudaEnableDefault, &found);
+        if (e != cudaSuccess) cudaGetLastError();
+        return e == cudaSuccess && found == cudaDriverEntryPointSuccess ? f : nullptr;
+    };
+    static const auto of_stream = reinterpret_cast<PFN_cuStreamGetGreenCtx_v12040>(entry("cuStreamGetGreenCtx"));
+    static const auto resource = reinterpret_cast<PFN_cuGreenCtxGetDevResource_v12040>(entry("cuGreenCtxGetDevResource"));
+    CUgreenCtx g = nullptr;
+    CUdevResource r{};
+    if (!of_stream || !resource || of_stream(s, &g) != CUDA_SUCCESS || !g ||
+        resource(g, &r, CU_DEV_RESOURCE_TYPE_SM) != CUDA_SUCCESS || r.sm.smCount < 1)
+        return device_sms;
+    return std::min(device_sms, (int)r.sm.smCount);
+}
+
+// Most blocks of the run kernel on the context's stream.  Its blocks wait for one
+// another, so the launch must not count SMs that the stream cannot use.
+cudaError_t size_run(cc_ctx* c)
+{
+    c->run_blocks = 0;
+    if (!c->run_kernel) return cudaSuccess;
+    return run_grid(c->args, c->rows, stream_sms(c->stream, c->sms), &c->run_blocks, &c->run_want);
 }
 
 // A run as launches of the run kernel: one unless the run is very long, or
@@ -993,8 +1031,8 @@ cc_status create_common(int jobs, const JobInput* in, bool on_device, const cc_o
     const long long fit = std::max({(NNZ + kBlock - 1) / kBlock, (rows + 2047) / 2048, (N + kBlock - 1) / kBlock});
     c->grid = (int)std::min<long long>(fit, (long long)c->sms * per_sm);
     a.ts = c->ts;
-    if (!c->opt.no_regions && (jobs > 1 || c->opt.colour_batched || pool || rows >= kRunKernelRows))
-        CC_TRY(run_grid(a, rows, c->sms, &c->run_blocks, &c->run_want));
+    c->run_kernel = !c->opt.no_regions && (jobs > 1 || c->opt.colour_batched || pool || rows >= kRunKernelRows);
+    CC_TRY(size_run(c));
 
     cc_status rc = start_state(c);
     if (rc != CC_OK) return bail(rc);
@@ -1890,6 +1928,7 @@ cc_status cc_set_stream(cc_ctx* c, void* stream)
     if (!c) return fail(nullptr, CC_ERR_INVALID, "ctx is NULL");
     CC_CUDA(c, cudaStreamSynchronize(c->stream));
     c->stream = stream ? static_cast<cudaStream_t>(stream) : c->own_stream;
+    CC_CUDA(c, size_run(c));
     return CC_OK;
 }
 

@@ -79,6 +79,7 @@ struct cc_ctx {
     std::vector<float> propose_ms;      // ... and of its proposal kernels
     long long launches = 0;             // kernels launched so far
     int grid = 0;
+    bool run_kernel = false;            // runs go through the run kernel where it can be resident
     int run_blocks = 0;                 // most blocks of the run kernel; 0: runs are graphs of one kernel per step
     int run_want = 0;                   // blocks that the context's work fills
     int in_flight = 0;                  // blocks of its launch of the run kernel that may still run

@@ -1,6 +1,7 @@
 """The run kernel and the graphs of a run beside the ordinary run: waits that
 run out, the autotuned first sweep (against the oracle where there are results;
 whole numbers, exact)."""
+import ctypes
 import os
 import subprocess
 import sys
@@ -213,3 +214,53 @@ def test_two_runs_overlap(cc):
     for j in jobs:
         j.close()
     assert together < 0.75 * alone, (together, alone)  # one after the other: 0.9
+
+
+class _Part:
+    """A stream on some of the device's SMs (a green context)."""
+
+    def __init__(self, sms):
+        self.lib = ctypes.CDLL("libcuda.so.1")
+        self.stream, self.green = ctypes.c_void_p(), ctypes.c_void_p()
+        dev, count, desc = ctypes.c_int(), ctypes.c_uint(1), ctypes.c_void_p()
+        whole, part, rest = (ctypes.create_string_buffer(144) for _ in range(3))  # CUdevResource
+        # (dev, desc and green are read when their call is made: ctypes passes the objects' values then)
+        for call, args in (("cuDeviceGet", (ctypes.byref(dev), 0)),
+                           ("cuDeviceGetDevResource", (dev, whole, 1)),
+                           ("cuDevSmResourceSplitByCount", (part, ctypes.byref(count), whole, rest, 0, sms)),
+                           ("cuDevResourceGenerateDesc", (ctypes.byref(desc), part, 1)),
+                           ("cuGreenCtxCreate", (ctypes.byref(self.green), desc, dev, 1)),
+                           ("cuGreenCtxStreamCreate", (ctypes.byref(self.stream), self.green, 1, 0))):
+            if not hasattr(self.lib, call) or getattr(self.lib, call)(*args) != 0:
+                pytest.skip(f"{call}: no green contexts here")
+
+    def close(self):
+        self.lib.cuStreamDestroy_v2(self.stream)
+        self.lib.cuGreenCtxDestroy(self.green)
+
+
+# On a stream that may use a few of the SMs only, the run kernel's blocks have to
+# fit those: they wait for one another.
+def test_stream_on_part_of_the_gpu(cc):
+    torch = pytest.importorskip("torch")
+    ro, col, lab = _job(20011, 12)
+    ref = oracle.sync_run(ro, col, lab, 20)
+    torch.cuda.init()
+    with cc.Consensus(ro, col, lab) as job:
+        part = _Part(16)
+        job.set_wait_limit(2 * SECOND)
+        for stream in (part.stream.value, 0, part.stream.value):
+            job.set_stream(stream)
+            job.reset()
+            assert job.run_until_converged(20) == ref.sweeps
+            assert job.history() == ref.stats
+            np.testing.assert_array_equal(job.cluster_ids(), ref.C)
+        job.set_stream(0)
+        dev = [torch.from_numpy(np.ascontiguousarray(x)).cuda() for x in (ro, col, lab)]
+        torch.cuda.synchronize()
+        with cc.Consensus.from_device(len(ro) - 1, len(col), dev[0].data_ptr(), dev[1].data_ptr(), len(lab),
+                                      dev[2].data_ptr(), stream=part.stream.value) as other:
+            other.set_wait_limit(2 * SECOND)
+            assert other.run_until_converged(20) == ref.sweeps
+            assert other.history() == ref.stats
+        part.close()
