@@ -240,8 +240,9 @@ typedef struct {
 /* The distances of every job's current consensus to each of its input
  * partitions: out (caller-allocated, sum_j k_j entries) receives job 0's k_0
  * partitions in order, then job 1's, and so on.  Rebuilds the contingency
- * table at its current capacity first (the results of later sweeps do not
- * change).  Errors: CC_ERR_OOM (scratch), CC_ERR_CUDA. */
+ * table first, at the capacity its keys need (the results of later sweeps do
+ * not change).  Scratch of up to 1 MB stays with the context, more is released.
+ * Errors: CC_ERR_OOM (scratch), CC_ERR_CUDA. */
 cc_status cc_metrics(cc_ctx* ctx, cc_partition_metrics* out);
 
 /* Grouping homogeneous partitions (Methods, "Grouping homogeneous

@@ -91,6 +91,8 @@ struct cc_ctx {
     std::vector<void*> allocs;
     unsigned char* block = nullptr;     // the allocation that holds the context's arrays
     size_t block_bytes = 0, block_used = 0;
+    unsigned char* work = nullptr;      // scratch of the distances to the inputs, kept where it is small (in allocs)
+    size_t work_bytes = 0;
     size_t bytes = 0;                   // device bytes held
     std::string err;
     // a run driven without blocking (ctx_async_*)

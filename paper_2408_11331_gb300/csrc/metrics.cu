@@ -44,12 +44,15 @@ __device__ __forceinline__ int job_by_start(const long long* key, int count, lon
 constexpr int kSmemParts = 1024;
 
 // Counts below this many are first counted per partition and value in shared
-// memory (most counts are tiny); 0 bins where the partitions leave no room.
+// memory (most counts are tiny); 0 bins where the partitions leave no room, and
+// in tables of up to kPlainSlots slots, where a block has a few hundred slots and
+// the bins cost more than their adds (n = 1000, k = 10: 11.8 us, 9.7 without).
 constexpr int kCountBins = 64;
+constexpr unsigned long long kPlainSlots = 1ull << 16;
 
-inline int count_bins(int parts)
+inline int count_bins(int parts, unsigned long long cap)
 {
-    const int bins = parts <= kSmemParts ? 8192 / parts : 0;
+    const int bins = parts <= kSmemParts && cap > kPlainSlots ? 8192 / parts : 0;
     return bins > kCountBins ? kCountBins : bins;
 }
 
@@ -346,7 +349,7 @@ cudaError_t launch_ids_from_partition(const SweepArgs& a, long long n, int j, in
 
 cudaError_t launch_metrics(const SweepArgs& a, const MetricsArgs& m, int parts, unsigned long long cap, cudaStream_t s)
 {
-    const int bins = count_bins(parts);
+    const int bins = count_bins(parts, cap);
     const size_t sm = parts <= kSmemParts ? (size_t)parts * (16 + 4 * (size_t)bins) : 0;
     const size_t sm1 = parts <= kSmemParts ? (size_t)parts * 8 : 0;
     k_met_table<<<met_grid((long long)cap), kMetBlock, sm, s>>>(a, m, parts, bins);

@@ -1,0 +1,53 @@
+"""Calls whose way depends on how small the job is, on both sides of each line,
+against the oracle (whole numbers exact; variation of information within the
+rounding of its fp64 sums of at most n log n)."""
+import numpy as np
+import pytest
+
+import oracle
+from workloads.graphs import csr_from_edges
+
+pytestmark = pytest.mark.gpu
+
+VI_TOL = 1e-9  # nats; see test_metrics_gpu.py
+
+
+@pytest.fixture(scope="module")
+def cc():
+    import __graft_entry__
+
+    __graft_entry__.build()
+    import paper_2408_11331_gb300 as m
+
+    return m
+
+
+def _graph(rng, n):
+    u = rng.integers(0, n, 4 * n)
+    return csr_from_edges(n, u, (u + rng.integers(1, max(2, n // 8), 4 * n)) % n)
+
+
+def _same(got, want):
+    for f in ("mirkin", "split_join"):
+        np.testing.assert_array_equal(got[f], want[f])
+    np.testing.assert_allclose(got["rand_distance"], want["rand_distance"], rtol=1e-14, atol=0)
+    np.testing.assert_allclose(got["vi"], want["vi"], rtol=0, atol=VI_TOL)
+
+
+# Tables of 2^16 slots and of 2^17 (counts tallied first), and scratch below and
+# above the megabyte that a context keeps; every call twice, the second on what
+# the first left.
+@pytest.mark.parametrize("n,k,distinct", [(10, 3, False), (2000, 10, False), (4000, 10, False), (4000, 10, True),
+                                          (30011, 9, True)])
+def test_metrics_small_and_large(cc, n, k, distinct):
+    rng = np.random.default_rng(n + k)
+    base = np.arange(n) // 90
+    lab = np.stack([rng.permutation(n) if distinct else np.where(rng.random(n) < 0.2, rng.integers(0, 9, n), base)
+                    for _ in range(k)]).astype(np.int32)
+    with cc.Consensus(*_graph(rng, n), lab) as job:
+        for C in (None, base * 90, rng.integers(0, n, n)):
+            if C is not None:
+                job.set_cluster_ids(C.astype(np.int32))
+            want = oracle.metrics(lab, oracle.singletons(n) if C is None else C.astype(np.int32))
+            for _ in range(2):
+                _same(job.metrics(), want)
