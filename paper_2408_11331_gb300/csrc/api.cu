@@ -118,10 +118,18 @@ cc_status read_state(cc_ctx* c, DevState* out)
     return CC_OK;
 }
 
-// The control block and the job records in one copy (they lie next to each
-// other, see create_common).
+// The control block and the job records: of few jobs in one copy (they lie next
+// to each other, see create_common), which is then taken apart.
 cc_status read_state_jobs(cc_ctx* c, DevState* out, std::vector<JobState>& js)
 {
+    constexpr int kOneCopyJobs = 64;
+    if (c->jobs > kOneCopyJobs) {
+        CC_CUDA(c, cudaMemcpyAsync(out, c->st, sizeof(DevState), cudaMemcpyDeviceToHost, c->stream));
+        js.resize(c->jobs);
+        CC_CUDA(c, cudaMemcpyAsync(js.data(), c->js, sizeof(JobState) * (size_t)c->jobs, cudaMemcpyDeviceToHost, c->stream));
+        CC_CUDA(c, cudaStreamSynchronize(c->stream));
+        return CC_OK;
+    }
     const size_t at = (size_t)(reinterpret_cast<unsigned char*>(c->js) - reinterpret_cast<unsigned char*>(c->st));
     std::vector<unsigned char> h(at + sizeof(JobState) * (size_t)c->jobs);
     CC_CUDA(c, cudaMemcpyAsync(h.data(), c->st, h.size(), cudaMemcpyDeviceToHost, c->stream));

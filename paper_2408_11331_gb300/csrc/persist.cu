@@ -52,8 +52,16 @@ enum Step {
     kSizes, kClear, kScatter, kBuild, kTop, // table rebuild
     kStage, kEval,                          // light path
     kBid, kKeys, kCommit,                   // matching, commit
+    kBegin, kDecide, kHeavyDecide, kEndJobs, // per-job decisions of many jobs
     kLeave
 };
+
+// Up to this many jobs the block that takes the decisions goes through them
+// alone, 256 at a time; more are a step of all blocks.  A step costs a barrier
+// (three of them per sweep), the rounds of one block 1-2 us each.  Runs, alone
+// and as steps: 512 jobs of n = 300 1463 and 1502 us, 1000 of 120 1161 and 1130,
+// 8000 of 60 3086 and 2448, 120,000 of 8 9.45 and 3.12 ms.
+constexpr int kSchedulerJobs = 768;
 
 // Grid barrier between two steps.  The last block to arrive runs schedule()
 // (all its threads; the value counts in thread 0), which takes the decisions
@@ -181,9 +189,11 @@ __device__ __forceinline__ void scan_write_step(const SweepArgs& a)
 
 // What follows a finished step (all threads of one block; the decisions of the
 // one-thread and per-job steps of a sweep are taken here).
+template <bool kSingle>
 struct Scheduler {
     const SweepArgs& a;
-    int limit, fresh;
+
+    __device__ bool many_jobs() const { return !kSingle && a.jobs > kSchedulerJobs; }
 
     // Starts a rebuild: 0 heavy sweep, 1 its rollback, 2 end of the sweep.
     __device__ int rebuild(int kind) const
@@ -196,7 +206,13 @@ struct Scheduler {
     {
         __syncthreads();
         if (a.st->bodies_left <= 0) return kLeave;
+        if (many_jobs()) return kBegin;
         begin_phase(a, threadIdx.x, kBlock);
+        return begun();
+    }
+
+    __device__ int begun() const
+    {
         __syncthreads();
         // the own step only serves these options
         return a.st->skip ? kLeave : a.active_set || a.empty_moves ? kOwn : kEdges;
@@ -207,7 +223,13 @@ struct Scheduler {
     __device__ int end() const
     {
         __syncthreads();
+        if (many_jobs()) return kEndJobs;
         end_jobs_phase(a, threadIdx.x, kBlock);
+        return ended();
+    }
+
+    __device__ int ended() const
+    {
         __syncthreads();
         if (threadIdx.x == 0) {
             end_phase(a);
@@ -223,12 +245,8 @@ struct Scheduler {
     {
         DevState* st = a.st;
         switch (step) {
-        case kStart:
-            if (fresh) {
-                run_begin_phase(a, limit, 0, threadIdx.x, kBlock);
-                __syncthreads();
-            }
-            return begin();
+        case kStart: return begin();
+        case kBegin: return begun();
         case kOwn: return kEdges;
         case kEdges: return kCollect;
         case kCollect:
@@ -260,14 +278,22 @@ struct Scheduler {
             if (st->again && st->tries < 2) return kSizes;  // the tight attempt did not fit
             return kHeavyEval;
         case kHeavyEval:
+            if (many_jobs()) return kHeavyDecide;
             h_decide_phase(a, threadIdx.x, kBlock);
             __syncthreads();
             return st->rollback ? kUndo : after_apply();
+        case kHeavyDecide: return st->rollback ? kUndo : after_apply();
         case kStage: return kEval;
-        case kEval: decide_phase(a, threadIdx.x, kBlock); __syncthreads(); return st->match ? kBid : kCommit;
+        case kEval:
+            if (many_jobs()) return kDecide;
+            decide_phase(a, threadIdx.x, kBlock);
+            __syncthreads();
+            return st->match ? kBid : kCommit;
+        case kDecide: return st->match ? kBid : kCommit;
         case kBid: return kKeys;
         case kKeys: return kCommit;
         case kCommit: return end();
+        case kEndJobs: return ended();
         }
         return kLeave;
     }
@@ -347,6 +373,18 @@ __device__ __noinline__ void match_reset_step(const SweepArgs& a)
     match_reset_phase(a);
 }
 
+// The per-job decisions `step` of many jobs, by all blocks.
+__device__ __noinline__ void jobs_step(const SweepArgs& a, int step)
+{
+    const int t0 = blockIdx.x * kBlock + threadIdx.x, stride = gridDim.x * kBlock;
+    switch (step) {
+    case kBegin: begin_phase(a, t0, stride); break;
+    case kDecide: decide_phase(a, t0, stride); break;
+    case kHeavyDecide: h_decide_phase(a, t0, stride); break;
+    case kEndJobs: end_jobs_phase(a, t0, stride); break;
+    }
+}
+
 }  // namespace
 
 // fresh: 1 starts a run of at most `limit` sweeps, 0 goes on with it; at most
@@ -377,6 +415,7 @@ __global__ void __launch_bounds__(kBlock, 4)
         switch (step) {
         case kStart:
             if (clock) st->bodies_left = budget;
+            if (fresh) run_begin_phase(a, limit, 0, blockIdx.x * kBlock + threadIdx.x, gridDim.x * kBlock);
             break;
         case kOwn: own_step<kSingle>(a); break;
         case kEdges: edges_phase<kSingle>(a, scratch.edge); break;
@@ -398,9 +437,15 @@ __global__ void __launch_bounds__(kBlock, 4)
             commit_phase(a);
             if (st->match) match_reset_step(a);
             break;
+        case kBegin:
+        case kDecide:
+        case kHeavyDecide:
+        case kEndJobs:
+            if (!kSingle) jobs_step(a, step);
+            break;
         }
         const int done = step;
-        step = grid_step(st, a.wait_ns, word, arrivals, [&] { return Scheduler{a, limit, fresh}.next(done); });
+        step = grid_step(st, a.wait_ns, word, arrivals, [&] { return Scheduler<kSingle>{a}.next(done); });
         if (clock && done == kCollect) a.ts[3 * body + 1] = now_ns();
         if (step == kLeave) break;
         last = done;

@@ -13,6 +13,7 @@ import pytest
 
 import oracle
 from workloads import make_config
+from workloads.graphs import csr_from_edges
 
 pytestmark = pytest.mark.gpu
 
@@ -264,3 +265,31 @@ def test_stream_on_part_of_the_gpu(cc):
             assert other.run_until_converged(20) == ref.sweeps
             assert other.history() == ref.stats
         part.close()
+
+
+# Up to 768 jobs one block takes the jobs' decisions, more are a step of all
+# blocks; from random warm starts some jobs fall back to the matching.
+@pytest.mark.parametrize("opts", [{}, {"active_set": 1}, {"colour_batched": 1}, {"sweep_mode": 1}, {"sweep_mode": 2}])
+@pytest.mark.parametrize("count", [768, 769, 1100])
+def test_many_jobs(cc, count, opts):
+    rng = np.random.default_rng(count)
+    kinds, starts = [], []
+    for n, k in [(1, 1), (2, 3), (5, 2), (9, 5), (17, 4), (33, 7), (40, 3), (64, 6), (21, 9), (12, 12), (50, 5), (30, 2)] * 2:
+        u = rng.integers(0, n, 3 * n)
+        ro, col = csr_from_edges(n, u, (u + rng.integers(0, n, 3 * n)) % n)
+        kinds.append((ro, col, rng.integers(0, 1 + n // 4, (k, n)).astype(np.int32)))
+        starts.append(rng.integers(0, n, n).astype(np.int32) // 3 * 3)
+    run = oracle.colour_run if opts.get("colour_batched") else oracle.sync_run
+    warm = [run(*j, 20, C0=c) for j, c in zip(kinds, starts)]
+    assert any(s["fallback"] for r in warm for s in r.stats)
+    fresh = [run(*j, 20) for j in kinds]
+    pick = rng.integers(0, len(kinds), count)
+    with cc.ConsensusBatch([kinds[i] for i in pick], _options(cc, **opts)) as batch:
+        for refs in (fresh, warm, fresh):
+            batch.reset()
+            if refs is warm:
+                batch.set_cluster_ids(np.concatenate([starts[i] for i in pick]))
+            batch.run_until_converged(20)
+            np.testing.assert_array_equal(batch.cluster_ids(), np.concatenate([refs[i].C for i in pick]))
+            for j, i in enumerate(pick):
+                assert batch.history(j) == refs[i].stats
