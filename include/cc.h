@@ -125,7 +125,7 @@ typedef struct {
                                for every value).  0 (default): first a tight capacity, from
                                the occupied slots at the sweep start at load <= 1/2 with room
                                for a following light sweep; a build that does not fit it (an
-                               insert past 256 probes, load above 1/2, or too little room) is
+                               insert past 128 probes, load above 1/2, or too little room) is
                                dropped and redone at the capacity that holds every key the
                                sweep can create.  1: always that safe capacity.  2: the tight
                                attempt is always dropped (for tests of the second attempt) */

@@ -61,7 +61,9 @@ __device__ __forceinline__ void add_small_rows(DevState* st, unsigned long long 
 // full table (2 x sum k n / 8 at most).  After a partial table the keys of
 // the small clusters were not counted; the sweep that merges them leaves
 // 11-13% of their rows as keys on the kNN and LFR-style workloads, and a
-// quarter is assumed.  The build checks that the keys fit (build_check) and
+// quarter is assumed; but three quarters of the rows that are still in small
+// clusters, whose members need not agree on much (jobs with noisy labels that
+// end with such clusters: a light sweep follows, so the table is full).  The build checks that the keys fit (build_check) and
 // otherwise builds again at the capacity that holds every key.
 __device__ __forceinline__ void size_build(const SweepArgs& a)
 {
@@ -79,6 +81,8 @@ __device__ __forceinline__ void size_build(const SweepArgs& a)
         c = p;
         if (est > rest) est = rest;
         room = 0;
+    } else if (st->small && est < st->small_keys / 4 * 3) {
+        est = st->small_keys / 4 * 3;
     }
     unsigned long long t = a.cap_min;
     while ((t < 2 * est || t - (t >> 3) < est + room) && t < c) t <<= 1;
@@ -224,8 +228,13 @@ __device__ __forceinline__ unsigned long long segment_max(unsigned long long x, 
 // over several warps are left to the scan.
 // A tight attempt (see build_check) gives every insert kTightProbes probes;
 // an insert that finds no slot within them flags the attempt as failed, and
-// the warps stop inserting.
-constexpr unsigned long long kTightProbes = 256;
+// the warps stop inserting.  At load 1/2 the longest chain of n keys is about
+// ln n / 0.19 slots (79 for 2^22, 97 for 2^27), so 128 do not fail an attempt
+// that fits; and a warp looks at the flag every 16 probes, for in a table that
+// overflows every chain is long (2500 jobs of n = 100 with random labels, whose
+// clusters merge fewer keys than size_build assumes: the failed attempt took 484
+// of 875 us of its sweep with 256 probes and no look, 128 so).
+constexpr unsigned long long kTightProbes = 128;
 
 // Claims an empty slot for key if on; returns the key found there (key itself
 // where off).  One predicated instruction, so that several follow each other
@@ -342,6 +351,7 @@ __device__ __forceinline__ void table_build_phase(const SweepArgs& a, int condit
                     else set_err(st, CC_ERR_TABLE_FULL);
                     break;
                 }
+                if (tight && (p & 15u) == 15u && *reinterpret_cast<volatile int*>(&st->build_fail)) break;
                 unsigned long long old[4];
 #pragma unroll
                 for (int b = 0; b < 4; ++b) {

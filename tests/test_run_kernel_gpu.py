@@ -293,3 +293,21 @@ def test_many_jobs(cc, count, opts):
             np.testing.assert_array_equal(batch.cluster_ids(), np.concatenate([refs[i].C for i in pick]))
             for j, i in enumerate(pick):
                 assert batch.history(j) == refs[i].stats
+
+
+# Noisy labels: the first sweeps leave clusters of a few members that agree on
+# little, so the table that follows a partial one holds most of their label rows.
+@pytest.mark.parametrize("tight", [0, 1, 2])
+@pytest.mark.parametrize("n,k,classes", [(100, 6, 4), (61, 9, 60), (300, 5, 2)])
+def test_noisy_labels(cc, n, k, classes, tight):
+    rng = np.random.default_rng(n)
+    jobs = []
+    for _ in range(40):
+        u = rng.integers(0, n, 4 * n)
+        ro, col = csr_from_edges(n, u, (u + rng.integers(1, max(2, n // 8), 4 * n)) % n)
+        jobs.append((ro, col, rng.integers(0, classes, (k, n)).astype(np.int32)))
+    refs = [oracle.sync_run(*j, 20) for j in jobs]
+    with cc.ConsensusBatch(jobs, _options(cc, tight_rebuild=tight)) as batch:
+        batch.run_until_converged(20)
+        assert [batch.history(j) for j in range(len(jobs))] == [r.stats for r in refs]
+        np.testing.assert_array_equal(batch.cluster_ids(), np.concatenate([r.C for r in refs]))
