@@ -522,6 +522,44 @@ __global__ void k_objective_recompute(SweepArgs a)
     job_acc_finish(acc, a.jobs);
 }
 
+// The same sum's part of the clusters that a partial table leaves out: their
+// sum_keys n^2 is the sum of A_c over their members, counted inside a warp as in
+// h_eval_phase (windows overlap, so that each small cluster lies whole in the
+// window of its first member).  A full rebuild for the sake of the sum took 165
+// of 235 us (n = 1e5, k = 20, after one sweep; 68 so).
+__global__ void __launch_bounds__(kBlock) k_objective_small(SweepArgs a)
+{
+    extern __shared__ long long dyn_jobs[];
+    JobAcc acc(job_smem_init(a.jobs, dyn_jobs), &a.js[0].recompute, kJobStride);
+    const int small = a.st->small, step = 32 - small, lane = threadIdx.x & 31;
+    const long long stride = (((long long)gridDim.x * blockDim.x) >> 5) * step;
+    long long wb = (((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * step;
+    for (; small > 0 && wb < a.n; wb += stride) {
+        const bool valid = wb + lane < a.n;
+        const int v = valid ? a.members[wb + lane] : 0;
+        const int c = valid ? a.C[v] : 0, sc = valid ? a.size[c] : 0;
+        const long long at = valid ? (long long)a.cursor[c] - sc : 0;  // the cluster's first place in the list
+        const bool on = valid && sc <= small && at >= wb && at < wb + step;
+        if (!__any_sync(0xffffffffu, on)) continue;
+        const unsigned lanes = on ? (~0u >> (32 - sc)) << (int)(at - wb) : 0u;
+        const int job = a.jid[v];
+        const JobInfo J = a.job[job];
+        const int4* row = reinterpret_cast<const int4*>(a.G + row_of(J, v));
+        const int k = on ? J.k : 0;
+        int sum = 0;
+        for (int i = 0; i < a.kmax; i += 4) {
+            // (the padding of a row, -1, counts for nothing: i + b < k)
+            const int4 g4 = i < k ? __ldg(row + (i >> 2)) : make_int4(-1, -1, -1, -1);
+            const int g[4] = {g4.x, g4.y, g4.z, g4.w};
+#pragma unroll
+            for (int b = 0; b < 4; ++b)
+                sum += __popc(__match_any_sync(0xffffffffu, g[b]) & (i + b < k ? lanes : 0u));
+        }
+        if (on) acc.add(job, -2LL * sum);
+    }
+    job_acc_finish(acc, a.jobs);
+}
+
 __global__ void k_zero_recompute(SweepArgs a)
 {
     for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < a.jobs; j += gridDim.x * blockDim.x)
@@ -760,11 +798,12 @@ cudaError_t launch_table_rebuild(const SweepArgs& a, long long rows, bool condit
     return cudaGetLastError();
 }
 
-cudaError_t launch_objective_recompute(const SweepArgs& a, cudaStream_t s)
+cudaError_t launch_objective_recompute(const SweepArgs& a, bool partial, cudaStream_t s)
 {
     k_zero_recompute<<<grid_for(a.jobs), kSetupBlock, 0, s>>>(a);
     const long long work = (long long)a.mask_max + 1 > a.n ? (long long)a.mask_max + 1 : a.n;
     k_objective_recompute<<<grid_for(work), kSetupBlock, smem_jobs_bytes(a.jobs), s>>>(a);
+    if (partial) k_objective_small<<<grid_for(a.n), kBlock, smem_jobs_bytes(a.jobs), s>>>(a);
     return cudaGetLastError();
 }
 

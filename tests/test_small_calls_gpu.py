@@ -5,6 +5,7 @@ import numpy as np
 import pytest
 
 import oracle
+from workloads import make_config
 from workloads.graphs import csr_from_edges
 
 pytestmark = pytest.mark.gpu
@@ -51,3 +52,24 @@ def test_metrics_small_and_large(cc, n, k, distinct):
             want = oracle.metrics(lab, oracle.singletons(n) if C is None else C.astype(np.int32))
             for _ in range(2):
                 _same(job.metrics(), want)
+
+
+# The objective between sweeps, where the table holds the clusters of more than 8
+# members only, without rebuilding it; ragged k, several lanes and one.
+@pytest.mark.parametrize("n,k", [(20011, 12), (6007, 9), (1000, 10), (3001, 33), (40, 3)])
+def test_objective_after_a_partial_table(cc, n, k):
+    c = make_config("lfr", n=n, k=k, cmin=10, cmax=300, max_deg=100, seed=n + k)
+    ro, col, lab = c["row_off"], c["col"], c["labels"]
+    ref = oracle.sync_run(ro, col, lab, 20)
+    with cc.Consensus(ro, col, lab) as job:
+        for s in range(ref.sweeps):
+            job.sweep()
+            before = job.table_stats()
+            assert job.objective_recompute() == ref.stats[s]["F"]
+            assert job.table_stats() == before
+        np.testing.assert_array_equal(job.cluster_ids(), ref.C)
+    o = cc.cc_default_options()
+    o.debug_checks = 1  # the same sums, job by job
+    with cc.ConsensusBatch([(ro, col, lab), (ro, col, lab[:1]), (ro, col, lab[::2])], o) as batch:
+        for s in range(3):
+            batch.sweep()
