@@ -146,30 +146,36 @@ __device__ __forceinline__ int warp_incl_scan(int x, int lane)
 // adds to a cluster's word in global memory once per tile instead of once per
 // vertex: adds to one word take about 10 ns each, and the largest clusters
 // hold several percent of the vertices (n = 1e6, 200 clusters: 233 -> 45 us).
+// A tile is four vertices per thread, or one up to kSmallTiles vertices, where
+// the time is a block's chain of steps (n = 3000: scatter 4.6 -> 2.6 us; n =
+// 100,003 6.4 -> 3.6).
 constexpr int kTile = 4 * kBlock;
+constexpr long long kSmallTiles = 1 << 17;
 struct TileCount {
     int key[2 * kTile], cnt[2 * kTile];
 };
 
-// All threads of the block; ids: this thread's four (-1: none).  Leaves the
+// All threads of the block; ids: this thread's kPer (-1: none).  Leaves the
 // entry of each in slot and its number among the tile's equal ones in rank.
-__device__ __forceinline__ void tile_count(TileCount* tc, const int (&id)[4], int (&slot)[4], int (&rank)[4])
+template <int kPer>
+__device__ __forceinline__ void tile_count(TileCount* tc, const int (&id)[kPer], int (&slot)[kPer], int (&rank)[kPer])
 {
-    for (int s = threadIdx.x; s < 2 * kTile; s += kBlock) {
+    constexpr int kEntries = 2 * kPer * kBlock;
+    for (int s = threadIdx.x; s < kEntries; s += kBlock) {
         tc->key[s] = -1;
         tc->cnt[s] = 0;
     }
     __syncthreads();
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
+    for (int q = 0; q < kPer; ++q) {
         slot[q] = rank[q] = 0;
         if (id[q] < 0) continue;
-        int h = (int)(((unsigned)id[q] * 0x9E3779B1u) >> 16) & (2 * kTile - 1);
-        // at most kTile ids in twice as many entries: an empty one is found
-        for (int p = 0; p < 2 * kTile; ++p) {
+        int h = (int)(((unsigned)id[q] * 0x9E3779B1u) >> 16) & (kEntries - 1);
+        // half as many ids as entries at most: an empty one is found
+        for (int p = 0; p < kEntries; ++p) {
             const int old = atomicCAS(&tc->key[h], -1, id[q]);
             if (old == -1 || old == id[q]) break;
-            h = (h + 1) & (2 * kTile - 1);
+            h = (h + 1) & (kEntries - 1);
         }
         slot[q] = h;
         rank[q] = atomicAdd(&tc->cnt[h], 1);
@@ -177,23 +183,23 @@ __device__ __forceinline__ void tile_count(TileCount* tc, const int (&id)[4], in
     __syncthreads();
 }
 
-__device__ __forceinline__ void members_scatter_phase(const SweepArgs& a, int conditional, TileCount* tc)
+template <int kPer>
+__device__ __forceinline__ void scatter_tiles(const SweepArgs& a, bool undone, TileCount* tc)
 {
-    if (rebuild_off(a.st, conditional)) return;
-    const bool undone = conditional && a.st->rollback;
-    for (long long t0 = (long long)blockIdx.x * kTile; t0 < a.n; t0 += (long long)gridDim.x * kTile) {
-        int id[4], slot[4], rank[4];
+    constexpr int kThis = kPer * kBlock;
+    for (long long t0 = (long long)blockIdx.x * kThis; t0 < a.n; t0 += (long long)gridDim.x * kThis) {
+        int id[kPer], slot[kPer], rank[kPer];
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
+        for (int q = 0; q < kPer; ++q) {
             const long long v = t0 + q * kBlock + threadIdx.x;
             id[q] = v < a.n ? a.C[v] : -1;
         }
         tile_count(tc, id, slot, rank);
-        for (int s = threadIdx.x; s < 2 * kTile; s += kBlock)
+        for (int s = threadIdx.x; s < 2 * kThis; s += kBlock)
             if (tc->cnt[s]) tc->cnt[s] = atomicAdd(&a.cursor[tc->key[s]], tc->cnt[s]);
         __syncthreads();
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
+        for (int q = 0; q < kPer; ++q) {
             const long long v = t0 + q * kBlock + threadIdx.x;
             if (id[q] < 0) continue;
             const int pos = tc->cnt[slot[q]] + rank[q];
@@ -204,6 +210,14 @@ __device__ __forceinline__ void members_scatter_phase(const SweepArgs& a, int co
         }
         __syncthreads();
     }
+}
+
+__device__ __forceinline__ void members_scatter_phase(const SweepArgs& a, int conditional, TileCount* tc)
+{
+    if (rebuild_off(a.st, conditional)) return;
+    const bool undone = conditional && a.st->rollback;
+    if (a.n <= kSmallTiles) scatter_tiles<1>(a, undone, tc);
+    else scatter_tiles<4>(a, undone, tc);
 }
 
 // Largest 64-bit value over the lanes of a contiguous lane segment [lane,

@@ -384,13 +384,15 @@ __global__ void k_sizes_zero(SweepArgs a)
 }
 
 // Sizes from a given consensus; an id outside its vertex's job sets an error.
+template <int kPer>
 __global__ void __launch_bounds__(kBlock) k_count_sizes(SweepArgs a)
 {
+    constexpr int kThis = kPer * kBlock;
     __shared__ TileCount tc;
-    for (long long t0 = (long long)blockIdx.x * kTile; t0 < a.n; t0 += (long long)gridDim.x * kTile) {
-        int id[4], slot[4], rank[4];
+    for (long long t0 = (long long)blockIdx.x * kThis; t0 < a.n; t0 += (long long)gridDim.x * kThis) {
+        int id[kPer], slot[kPer], rank[kPer];
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
+        for (int q = 0; q < kPer; ++q) {
             const long long v = t0 + q * kBlock + threadIdx.x;
             id[q] = -1;
             if (v >= a.n) continue;
@@ -400,7 +402,7 @@ __global__ void __launch_bounds__(kBlock) k_count_sizes(SweepArgs a)
             else id[q] = (int)c;
         }
         tile_count(&tc, id, slot, rank);
-        for (int s = threadIdx.x; s < 2 * kTile; s += kBlock)
+        for (int s = threadIdx.x; s < 2 * kThis; s += kBlock)
             if (tc.cnt[s]) atomicAdd(&a.size[tc.key[s]], tc.cnt[s]);
         __syncthreads();
     }
@@ -763,7 +765,8 @@ cudaError_t launch_init_state(const SweepArgs& a, int ncls, unsigned long long m
 cudaError_t launch_state_from_ids(const SweepArgs& a, cudaStream_t s)
 {
     k_sizes_zero<<<grid_for(a.n), kSetupBlock, 0, s>>>(a);
-    k_count_sizes<<<grid_for(a.n, kTile), kBlock, 0, s>>>(a);
+    if (a.n <= kSmallTiles) k_count_sizes<1><<<grid_for(a.n, kBlock), kBlock, 0, s>>>(a);
+    else k_count_sizes<4><<<grid_for(a.n, kTile), kBlock, 0, s>>>(a);
     return cudaGetLastError();
 }
 
@@ -790,8 +793,9 @@ cudaError_t launch_table_rebuild(const SweepArgs& a, long long rows, bool condit
     k_scan_sums<<<1, 1024, 0, s>>>(a, nb, c);
     k_scan_write<<<nb, 1024, 0, s>>>(a, c);
     k_table_clear<<<grid_for(std::max(slots, rows)), kSetupBlock, 0, s>>>(a, rows, c);
-    k_members_scatter<<<grid_for(a.n, kTile), kBlock, 0, s>>>(a, c);
-    k_table_build<<<grid_for(a.n), kSetupBlock, 0, s>>>(a, c);
+    k_members_scatter<<<grid_for(a.n, a.n <= kSmallTiles ? kBlock : kTile), kBlock, 0, s>>>(a, c);
+    // (a warp per window of 32 members and quad of partitions where the grid has room)
+    k_table_build<<<grid_for((a.n + 31) / 32 * ((a.kmax + 3) / 4), kWarpsPerBlock), kSetupBlock, 0, s>>>(a, c);
     k_build_check<<<1, 32, 0, s>>>(a, c);
     k_summ_top<<<grid_for(slots), kSetupBlock, 0, s>>>(a, c);
     k_table_done<<<1, 1, 0, s>>>(a.st, c);

@@ -73,3 +73,22 @@ def test_objective_after_a_partial_table(cc, n, k):
     with cc.ConsensusBatch([(ro, col, lab), (ro, col, lab[:1]), (ro, col, lab[::2])], o) as batch:
         for s in range(3):
             batch.sweep()
+
+
+# Sizes and member lists of a warm start are counted in tiles of 256 vertices, of
+# 1024 above 2^17 vertices: tile edges, one cluster, many, and two large ones.
+@pytest.mark.parametrize("n", [1, 255, 256, 257, 1025, (1 << 17) - 1, 1 << 17, (1 << 17) + 1])
+def test_warm_start_tiles(cc, n):
+    rng = np.random.default_rng(n)
+    lab = np.stack([np.arange(n) // 50, rng.integers(0, 40, n), np.arange(n) % 7]).astype(np.int32)
+    ro, col = _graph(rng, n) if n > 1 else (np.zeros(2, np.int64), np.empty(0, np.int32))
+    with cc.Consensus(ro, col, lab) as job:
+        for C in (np.zeros(n), np.arange(n)[::-1], rng.integers(0, n, n), np.where(rng.random(n) < 0.9, n - 1, 0)):
+            C = C.astype(np.int32)
+            job.set_cluster_ids(C)
+            assert job.objective() == oracle.objective(lab, C) == job.objective_recompute()
+            np.testing.assert_array_equal(job.cluster_ids(), C)
+            assert job.run_until_converged(1) == 1
+            step = oracle.sync_step(ro, col, lab, C)
+            np.testing.assert_array_equal(job.cluster_ids(), step.C)
+            assert job.history()[-1] == step.stats
