@@ -99,7 +99,9 @@ __global__ void k_assemble_off(AssemblyArgs a)
 // lanes across their entries, each finding its entry's vertex among the 32
 // offsets.  Bound by the writes of src (and the reads of col); a thread per
 // vertex wrote 32 rows at once, 80 bytes apart (n = 1e6, nnz = 2e7: 192 us for
-// sources and columns, now 114).  Skipped when the offsets are malformed.
+// sources and columns, now 114).  In dense graphs of few vertices the entries of
+// 32 vertices are cut into slices, one warp each (gridDim.y; a clique of 3000:
+// creation 2.21 ms with one warp, 0.66 so).  Skipped when the offsets are malformed.
 __global__ void k_assemble_edges(AssemblyArgs a)
 {
     if (a.st->err) return;
@@ -113,7 +115,7 @@ __global__ void k_assemble_edges(AssemblyArgs a)
         const int at = (int)(mine - e0 < e1 - e0 ? mine - e0 : e1 - e0);  // a row holds fewer than 2^31 entries here
         const bool wide = e1 - e0 >= (1LL << 31);
         const JobInfo J = a.job[a.jid[v < a.n ? v : a.n - 1]];
-        for (long long b = e0; b < e1; b += 32) {
+        for (long long b = e0 + 32 * blockIdx.y; b < e1; b += 32 * gridDim.y) {
             const long long e = b + lane;
             // last of the 32 offsets that is not past e
             int l = 0;
@@ -726,7 +728,10 @@ cudaError_t launch_colouring(const ColourArgs& a, int* classes, cudaStream_t s)
 cudaError_t launch_assemble(const AssemblyArgs& a, cudaStream_t s)
 {
     k_assemble_off<<<grid_for(a.n), kSetupBlock, 0, s>>>(a);
-    k_assemble_edges<<<grid_for(a.n), kSetupBlock, 0, s>>>(a);
+    // slices of about 1024 entries where the vertices leave warps idle
+    const long long groups = (a.n + 31) / 32, warps = 16LL * device_sm_count() * kWarpsPerBlock;
+    const long long slices = std::max(1LL, std::min(a.nnz / groups / 1024, warps / groups));
+    k_assemble_edges<<<dim3((unsigned)grid_for(a.n), (unsigned)slices), kSetupBlock, 0, s>>>(a);
     return cudaGetLastError();
 }
 

@@ -92,3 +92,27 @@ def test_warm_start_tiles(cc, n):
             step = oracle.sync_step(ro, col, lab, C)
             np.testing.assert_array_equal(job.cluster_ids(), step.C)
             assert job.history()[-1] == step.stats
+
+
+# Dense graphs are assembled in slices of their vertices' entries: cliques and a
+# graph whose rows are partly empty, alone and behind another job.
+@pytest.mark.parametrize("n,full", [(33, 33), (65, 64), (700, 700), (1500, 1500), (2100, 900)])
+def test_dense_graphs(cc, n, full):
+    rng = np.random.default_rng(n)
+    u, v = np.triu_indices(full, 1)
+    ro, col = csr_from_edges(n, u, v)
+    lab = (np.arange(n)[None, :] // np.array([[7], [9], [40]]) + (rng.random((3, n)) < 0.2)).astype(np.int32)
+    ref = oracle.sync_run(ro, col, lab, 6)
+    other = (*_graph(rng, 50), rng.integers(0, 9, (2, 50)).astype(np.int32))
+    with cc.Consensus(ro, col, lab) as job, cc.ConsensusBatch([other, (ro, col, lab)]) as batch:
+        job.run_until_converged(6)
+        assert job.history() == ref.stats
+        np.testing.assert_array_equal(job.cluster_ids(), ref.C)
+        batch.run_until_converged(6)
+        assert batch.history(1) == ref.stats
+        np.testing.assert_array_equal(batch.cluster_ids()[50:], ref.C)
+    bad = col.copy()
+    bad[len(bad) // 2] = n
+    with pytest.raises(cc.CCError) as e:
+        cc.Consensus(ro, bad, lab)
+    assert e.value.status == 1
