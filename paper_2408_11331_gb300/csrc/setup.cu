@@ -183,6 +183,8 @@ __global__ void __launch_bounds__(kBlock) k_label_insert(LabelArgs a)
     __shared__ TileCount tc;
     LSlot* m = static_cast<LSlot*>(a.lmap);
     for (int tile = blockIdx.x; tile < a.tiles; tile += gridDim.x) {
+        // the map has proved too small: the compaction is run again
+        if (a.limit != ~0ull && __syncthreads_or(*reinterpret_cast<volatile int*>(&a.st->err))) break;
         const int j = upper_index32(a.tile0, a.jobs, tile);
         const int n = (int)a.job[j].n, per = (n + kTile - 1) / kTile, rel = tile - a.tile0[j];
         const int i = rel / per, v0 = (rel - i * per) * kTile;
@@ -223,6 +225,7 @@ __global__ void __launch_bounds__(kBlock) k_label_classes(LabelArgs a, unsigned 
     __shared__ int s_n[kSmemParts], s_base[kSmemParts];
     __shared__ unsigned long long s_sq[kSmemParts];
     __shared__ double s_slog[kSmemParts];
+    if (a.st->err) return;
     LSlot* m = static_cast<LSlot*>(a.lmap);
     JobAcc acc(job_smem_init(a.jobs, dyn_jobs), &a.js[0].partition_sq, kJobStride);
     const bool shared = a.parts <= kSmemParts;

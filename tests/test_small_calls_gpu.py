@@ -116,3 +116,24 @@ def test_dense_graphs(cc, n, full):
     with pytest.raises(cc.CCError) as e:
         cc.Consensus(ro, bad, lab)
     assert e.value.status == 1
+
+
+# More classes than the first label map holds (2^16 entries, or a quarter of the
+# labels): the compaction stops and runs again, and the sums over the classes are
+# those of the second run.
+@pytest.mark.parametrize("n,k,distinct", [(70001, 3, 3), (70001, 3, 1), (30011, 9, 9), (30011, 9, 2)])
+def test_label_map_runs_again(cc, n, k, distinct):
+    rng = np.random.default_rng(n + distinct)
+    lab = np.stack([rng.permutation(n) if i < distinct else np.arange(n) // 41 for i in range(k)]).astype(np.int32)
+    other = (*_graph(rng, 500), rng.integers(0, 30, (4, 500)).astype(np.int32))
+    mine = (*_graph(rng, n), lab)
+    C = (np.arange(n) // 60 * 60).astype(np.int32)
+    with cc.Consensus(*mine) as job, cc.ConsensusBatch([other, mine]) as batch:
+        job.set_cluster_ids(C)
+        _same(job.metrics(), oracle.metrics(lab, C))
+        assert job.objective() == oracle.objective(lab, C)
+        batch.set_cluster_ids(np.concatenate([np.zeros(500, np.int32), C]))
+        got = batch.metrics()
+        _same(got[0], oracle.metrics(other[2], np.zeros(500, np.int32)))
+        _same(got[1], oracle.metrics(lab, C))
+        assert batch.objective(1) == oracle.objective(lab, C)
