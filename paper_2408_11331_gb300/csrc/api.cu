@@ -190,15 +190,14 @@ cc_status objective_recompute(cc_ctx* c, std::vector<long long>& F)
     DevState pre;
     cc_status rp = read_state(c, &pre);
     if (rp != CC_OK) return rp;
-    const bool rebuild = !pre.tvalid, partial = !rebuild && pre.small > 0;
-    if (rebuild) {
+    if (!pre.tvalid) {
         const unsigned long long nm = full_mask(c, pre);
         CC_CUDA(c, cudaMemcpyAsync(&c->st->new_mask, &nm, sizeof(nm), cudaMemcpyHostToDevice, c->stream));
         CC_CUDA(c, launch_table_rebuild(c->args, c->rows, false, c->stream));
         c->launches += kKernelsPerRebuild;
     }
-    CC_CUDA(c, launch_objective_recompute(c->args, partial, c->stream));
-    c->launches += partial ? 3 : 2;
+    CC_CUDA(c, launch_objective_recompute(c->args, c->stream));
+    c->launches += 2;
     std::vector<JobState> js;
     cc_status r = read_jobs(c, js);
     if (r != CC_OK) return r;

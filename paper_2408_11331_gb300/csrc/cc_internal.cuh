@@ -536,9 +536,8 @@ cudaError_t launch_table_rebuild(const SweepArgs& a, long long rows, bool condit
                                  unsigned long long cap = 0);
 // Slots of an empty table.
 cudaError_t launch_empty_slots(Slot* t, unsigned long long cap, cudaStream_t s);
-// F of every job from scratch into js[j].recompute (without sum_ij |P_ij|^2);
-// partial: the table is a partial one (st->small).
-cudaError_t launch_objective_recompute(const SweepArgs& a, bool partial, cudaStream_t s);
+// F of every job from scratch into js[j].recompute (without sum_ij |P_ij|^2).
+cudaError_t launch_objective_recompute(const SweepArgs& a, cudaStream_t s);
 
 // ---- metrics.cu ----
 // Sums for the partition distances of every job's consensus against each of

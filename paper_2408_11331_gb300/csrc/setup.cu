@@ -506,42 +506,17 @@ __global__ void k_table_done(DevState* st, int conditional)
     table_done_phase(st, conditional);
 }
 
-// F of every job without sum_ij |P_ij|^2: k sum_c s_c^2 - 2 sum_keys n^2.
-__global__ void k_objective_recompute(SweepArgs a)
-{
-    extern __shared__ long long dyn_jobs[];
-    JobAcc acc(job_smem_init(a.jobs, dyn_jobs), &a.js[0].recompute, kJobStride);
-    const unsigned long long mask = a.st->mask;
-    const unsigned long long stride = (unsigned long long)gridDim.x * blockDim.x;
-    const unsigned long long t0 = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x;
-    for (unsigned long long t = t0; t < (unsigned long long)a.n; t += stride) {
-        const long long s = a.size[t];
-        if (s > 0) {
-            const int j = a.jid[t];
-            acc.add(j, (long long)a.job[j].k * s * s);
-        }
-    }
-    for (unsigned long long t = t0; t <= mask; t += stride) {
-        const ulonglong2 e = reinterpret_cast<const ulonglong2*>(a.table)[t];
-        const long long c = (int)(unsigned)(e.y & 0xffffffffull);
-        if (e.x != kEmpty && c != 0) acc.add(a.jid[(int)(e.x >> 32)], -2 * c * c);
-    }
-    job_acc_finish(acc, a.jobs);
-}
-
-// The same sum's part of the clusters that a partial table leaves out: their
+// Part of the objective of the clusters that a partial table leaves out: their
 // sum_keys n^2 is the sum of A_c over their members, counted inside a warp as in
 // h_eval_phase (windows overlap, so that each small cluster lies whole in the
 // window of its first member).  A full rebuild for the sake of the sum took 165
 // of 235 us (n = 1e5, k = 20, after one sweep; 68 so).
-__global__ void __launch_bounds__(kBlock) k_objective_small(SweepArgs a)
+__device__ __forceinline__ void objective_small(const SweepArgs& a, int small, JobAcc& acc)
 {
-    extern __shared__ long long dyn_jobs[];
-    JobAcc acc(job_smem_init(a.jobs, dyn_jobs), &a.js[0].recompute, kJobStride);
-    const int small = a.st->small, step = 32 - small, lane = threadIdx.x & 31;
+    const int step = 32 - small, lane = threadIdx.x & 31;
     const long long stride = (((long long)gridDim.x * blockDim.x) >> 5) * step;
     long long wb = (((long long)blockIdx.x * blockDim.x + threadIdx.x) >> 5) * step;
-    for (; small > 0 && wb < a.n; wb += stride) {
+    for (; wb < a.n; wb += stride) {
         const bool valid = wb + lane < a.n;
         const int v = valid ? a.members[wb + lane] : 0;
         const int c = valid ? a.C[v] : 0, sc = valid ? a.size[c] : 0;
@@ -564,6 +539,29 @@ __global__ void __launch_bounds__(kBlock) k_objective_small(SweepArgs a)
         }
         if (on) acc.add(job, -2LL * sum);
     }
+}
+
+// F of every job without sum_ij |P_ij|^2: k sum_c s_c^2 - 2 sum_keys n^2.
+__global__ void k_objective_recompute(SweepArgs a)
+{
+    extern __shared__ long long dyn_jobs[];
+    JobAcc acc(job_smem_init(a.jobs, dyn_jobs), &a.js[0].recompute, kJobStride);
+    const unsigned long long mask = a.st->mask;
+    const unsigned long long stride = (unsigned long long)gridDim.x * blockDim.x;
+    const unsigned long long t0 = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x;
+    for (unsigned long long t = t0; t < (unsigned long long)a.n; t += stride) {
+        const long long s = a.size[t];
+        if (s > 0) {
+            const int j = a.jid[t];
+            acc.add(j, (long long)a.job[j].k * s * s);
+        }
+    }
+    for (unsigned long long t = t0; t <= mask; t += stride) {
+        const ulonglong2 e = reinterpret_cast<const ulonglong2*>(a.table)[t];
+        const long long c = (int)(unsigned)(e.y & 0xffffffffull);
+        if (e.x != kEmpty && c != 0) acc.add(a.jid[(int)(e.x >> 32)], -2 * c * c);
+    }
+    if (a.st->small > 0) objective_small(a, a.st->small, acc);
     job_acc_finish(acc, a.jobs);
 }
 
@@ -810,12 +808,11 @@ cudaError_t launch_table_rebuild(const SweepArgs& a, long long rows, bool condit
     return cudaGetLastError();
 }
 
-cudaError_t launch_objective_recompute(const SweepArgs& a, bool partial, cudaStream_t s)
+cudaError_t launch_objective_recompute(const SweepArgs& a, cudaStream_t s)
 {
     k_zero_recompute<<<grid_for(a.jobs), kSetupBlock, 0, s>>>(a);
     const long long work = (long long)a.mask_max + 1 > a.n ? (long long)a.mask_max + 1 : a.n;
     k_objective_recompute<<<grid_for(work), kSetupBlock, smem_jobs_bytes(a.jobs), s>>>(a);
-    if (partial) k_objective_small<<<grid_for(a.n), kBlock, smem_jobs_bytes(a.jobs), s>>>(a);
     return cudaGetLastError();
 }
 
