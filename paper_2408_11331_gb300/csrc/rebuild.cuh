@@ -248,7 +248,7 @@ __device__ __forceinline__ unsigned long long segment_max(unsigned long long x, 
 // overflows every chain is long (2500 jobs of n = 100 with random labels, whose
 // clusters merge fewer keys than size_build assumes: the failed attempt took 484
 // of 875 us of its sweep with 256 probes and no look, 128 so).
-constexpr unsigned long long kTightProbes = 128;
+constexpr unsigned kTightProbes = 128, kLookProbes = 16;
 
 // Claims an empty slot for key if on; returns the key found there (key itself
 // where off).  One predicated instruction, so that several follow each other
@@ -277,9 +277,9 @@ __device__ __forceinline__ void table_build_phase(const SweepArgs& a, int condit
     // tight attempts are made only by the heavy sweep's rebuild inside a
     // sweep graph; a rebuild the host asks for is never one
     const bool tight = conditional && st->tight != 0;
-    const unsigned long long limit = tight ? kTightProbes : ~0ull;
     const int small = conditional ? st->build_small : 0;
     const unsigned long long mask = st->new_mask;
+    const unsigned first_stop = tight ? kLookProbes : ~0u;  // probes of a key before the first look at the limits
     const int lane = threadIdx.x & 31;
     unsigned created = 0;  // slots this lane created
     // an item is a window of 32 members and a run of quads of partitions: a
@@ -359,13 +359,17 @@ __device__ __forceinline__ void table_build_phase(const SweepArgs& a, int condit
             // probe round p: the p-th slot of every key not placed yet, all
             // of them in flight together (a lane's keys collide one by one,
             // but the warp waits only for its longest chain, not for their sum)
-            for (unsigned long long p = 0; pend; ++p) {
-                if (p > mask || p >= limit) {
-                    if (tight) st->build_fail = 1;
-                    else set_err(st, CC_ERR_TABLE_FULL);
-                    break;
+            unsigned stop = first_stop > mask ? (unsigned)mask + 1u : first_stop;
+            for (unsigned p = 0; pend; ++p) {
+                if (p == stop) {
+                    if (!tight) {
+                        set_err(st, CC_ERR_TABLE_FULL);
+                        break;
+                    }
+                    if (p >= kTightProbes || p > mask) st->build_fail = 1;
+                    if (*reinterpret_cast<volatile int*>(&st->build_fail)) break;
+                    stop = p + kLookProbes > mask ? (unsigned)mask + 1u : p + kLookProbes;
                 }
-                if (tight && (p & 15u) == 15u && *reinterpret_cast<volatile int*>(&st->build_fail)) break;
                 unsigned long long old[4];
 #pragma unroll
                 for (int b = 0; b < 4; ++b) {
