@@ -323,6 +323,8 @@ cc_status cc_sweep(cc_ctx* ctx, cc_sweep_info* info);
  * A context of several jobs, a colour-batched one, and any job of at least
  * 16,384 label rows (n times k rounded up to 4) runs in the run kernel: one
  * cooperative launch takes the whole run, and the host synchronises once.
+ * While other contexts run on the device it takes a share of it, or, for a job
+ * that fills it many times over, runs as the graph below.
  * A smaller job's run is one launch of a CUDA graph whose loop holds two
  * sweeps (one after the end of the run is skipped on the device).  With
  * no_regions, sweeps are submitted as plain graphs of up to 4, and the host

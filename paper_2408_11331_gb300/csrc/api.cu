@@ -365,19 +365,27 @@ cc_status tune_lanes(cc_ctx* c)
     return CC_OK;
 }
 
-// Launches of the run kernel that may still run, and their blocks, per device:
-// a cooperative launch starts once all of its blocks find places, so contexts
-// that run at the same time (threads, the served form) take shares that fit
-// beside each other.  With the whole GPU each they ran one after another, and 8
-// threads got less done than with a kernel per step (per run, kernels per step /
-// whole GPU / shares: n = 5000, k = 20 258 / 382 / 88 us; n = 20,011, k = 12
-// 314 / 559 / 169; n = 100,003, k = 20 803 / 1088 / 727).  The counts only size
-// grids; no result depends on them.
+// Runs in flight and the blocks they hold, per device: a cooperative launch
+// starts once all of its blocks find places, so contexts that run at the same
+// time (threads, the served form) take shares that fit beside each other.  With
+// the whole GPU each they ran one after another, and 8 threads got less done than
+// with a kernel per step (us per run, kernels per step / whole GPU / now: n = 5000,
+// k = 20 258 / 382 / 99; n = 20,011, k = 12 314 / 559 / 177; n = 100,003, k = 20
+// 803 / 1088 / 757).  A share is an equal part, or what is free, but not less
+// than a block for kWorkPerBlock blocks of work: large jobs in small shares end
+// long after the others (the served mix of n up to 2e6: 317 jobs/s with the
+// whole GPU each, 207 with equal parts, 334 so; 322 with 40 in place of 100).
+// Jobs whose work is kManyTimes the GPU run as graphs while others are in flight:
+// their kernels interleave (n = 300,007, k = 20 1957 / 2338 / 1610; n = 1,000,003,
+// k = 12 5586 / 6776 / 5260).  The counts only choose among ways and sizes; no
+// result depends on them.
 struct RunsInFlight {
     std::atomic<int> launches{0}, blocks{0};
 };
 RunsInFlight g_in_flight[kMaxDevices];
 constexpr int kMostShares = 8;
+constexpr int kWorkPerBlock = 100;
+constexpr int kManyTimes = 26;
 
 void end_flight(cc_ctx* c)
 {
@@ -388,8 +396,20 @@ void end_flight(cc_ctx* c)
     c->in_flight = 0;
 }
 
-// Launches the run kernel with this context's share of the GPU: what the others
-// leave free, at least an equal part.  end_flight once the launch has ended.
+// A run as graphs beside other runs (see above): counted with all places.
+bool graphs_beside_others(cc_ctx* c)
+{
+    if (c->device < 0 || c->device >= kMaxDevices || c->run_want / kManyTimes < c->run_blocks) return false;
+    RunsInFlight& f = g_in_flight[c->device];
+    if (f.launches.load() == 0) return false;
+    f.launches.fetch_add(1);
+    f.blocks.fetch_add(c->run_blocks);
+    c->in_flight = c->run_blocks;
+    return true;
+}
+
+// Launches the run kernel with this context's share of the GPU.  end_flight once
+// the launch has ended.
 cudaError_t launch_share(cc_ctx* c, int limit, bool fresh, int budget)
 {
     end_flight(c);
@@ -397,7 +417,8 @@ cudaError_t launch_share(cc_ctx* c, int limit, bool fresh, int budget)
     if (c->device >= 0 && c->device < kMaxDevices) {
         RunsInFlight& f = g_in_flight[c->device];
         const int others = std::min(f.launches.fetch_add(1), kMostShares - 1);
-        grid = std::min(grid, std::max({1, c->run_blocks / (others + 1), c->run_blocks - f.blocks.load()}));
+        grid = std::min(grid, std::max({1, c->run_blocks / (others + 1), c->run_blocks - f.blocks.load(),
+                                        c->run_want / kWorkPerBlock}));
         f.blocks.fetch_add(grid);
         c->in_flight = grid;
     }
@@ -527,7 +548,13 @@ cc_status run(cc_ctx* c, int limit, int* done)
     c->ts_bodies = 0;
     DevState st;
     std::vector<JobState> js;
-    cc_status r = c->run_blocks > 0 ? run_kernel(c, limit, &st, js) : run_graphs(c, limit, &st, js);
+    cc_status r = CC_OK;
+    if (c->run_blocks > 0 && !graphs_beside_others(c)) {
+        r = run_kernel(c, limit, &st, js);
+    } else {
+        r = run_graphs(c, limit, &st, js);
+    }
+    end_flight(c);
     if (r != CC_OK) return r;
     r = check_device_error(c, st);
     if (r != CC_OK) return r;
@@ -1635,6 +1662,11 @@ int ctx_async_poll(cc_ctx* c, cc_status* st)
 cc_status ctx_async_continue(cc_ctx* c)
 {
     return launch_chunk(c);
+}
+
+void ctx_end_launch(cc_ctx* c)
+{
+    if (c->in_flight && cudaEventQuery(c->chunk_done) != cudaErrorNotReady) end_flight(c);
 }
 
 int ctx_async_poll_step(cc_ctx* c, cc_status* st)

@@ -165,6 +165,8 @@ int ctx_async_poll(cc_ctx* c, cc_status* st);
 // are final), and ctx_async_continue queues the next launch.
 int ctx_async_poll_step(cc_ctx* c, cc_status* st);
 cc_status ctx_async_continue(cc_ctx* c);
+// If the launch has ended, it no longer counts as one that shares the GPU.
+void ctx_end_launch(cc_ctx* c);
 
 // Whether a job of these sizes fits the place of job j (see ctx_load_job):
 // no more vertices, CSR entries, partitions, label rows or keys than the

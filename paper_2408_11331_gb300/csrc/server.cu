@@ -216,6 +216,9 @@ void harvest(cc_server* s, size_t idx)
 int poll_flights(cc_server* s)
 {
     int finished = 0;
+    // launches that have ended give up their share of the GPU before the first
+    // of the next ones is sized
+    for (Flight& f : s->flights) ctx_end_launch(f.ctx);
     for (size_t i = 0; i < s->flights.size();) {
         cc_status st = CC_OK;
         Flight& f = s->flights[i];

@@ -311,3 +311,38 @@ def test_noisy_labels(cc, n, k, classes, tight):
         batch.run_until_converged(20)
         assert [batch.history(j) for j in range(len(jobs))] == [r.stats for r in refs]
         np.testing.assert_array_equal(batch.cluster_ids(), np.concatenate([r.C for r in refs]))
+
+
+# Jobs that fill the GPU many times over (4 million CSR entries) run as graphs
+# while others are in flight; the same runs in turn, at once, and mixed with
+# small ones.
+def test_large_runs_in_threads(cc):
+    rng = np.random.default_rng(11)
+    n = 60011
+    u = rng.integers(0, n, 3_000_000)
+    v = np.where(rng.random(len(u)) < 0.5, u // 120 * 120 + rng.integers(0, 120, len(u)), rng.integers(0, n, len(u)))
+    large = csr_from_edges(n, u, np.minimum(v, n - 1))
+    labs = [np.where(rng.random((5, n)) < 0.3, rng.integers(0, n // 120, (5, n)), np.arange(n) // 120).astype(np.int32)
+            for _ in range(3)]
+    jobs = [(*large, lab) for lab in labs] + [_job(6007, 9), _job(20011, 12)]
+    refs = [oracle.sync_run(*j, 6) for j in jobs]
+    wrong = []
+
+    def work(i):
+        with cc.Consensus(*jobs[i]) as job:
+            for _ in range(8):
+                job.reset()
+                sweeps = job.run_until_converged(6)
+                ms, prop = job.last_run_timing()
+                if (sweeps, job.history()) != (refs[i].sweeps, refs[i].stats) or len(ms) != sweeps or \
+                        not np.array_equal(job.cluster_ids(), refs[i].C):
+                    wrong.append(i)
+
+    for i in range(len(jobs)):
+        work(i)
+    threads = [threading.Thread(target=work, args=(i,)) for i in range(len(jobs))]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not wrong
