@@ -313,15 +313,19 @@ def test_noisy_labels(cc, n, k, classes, tight):
         np.testing.assert_array_equal(batch.cluster_ids(), np.concatenate([r.C for r in refs]))
 
 
+def _large_graph(rng, n):
+    u = rng.integers(0, n, 50 * n)
+    v = np.where(rng.random(len(u)) < 0.5, u // 120 * 120 + rng.integers(0, 120, len(u)), rng.integers(0, n, len(u)))
+    return csr_from_edges(n, u, np.minimum(v, n - 1))
+
+
 # Jobs that fill the GPU many times over (4 million CSR entries) run as graphs
 # while others are in flight; the same runs in turn, at once, and mixed with
 # small ones.
 def test_large_runs_in_threads(cc):
     rng = np.random.default_rng(11)
     n = 60011
-    u = rng.integers(0, n, 3_000_000)
-    v = np.where(rng.random(len(u)) < 0.5, u // 120 * 120 + rng.integers(0, 120, len(u)), rng.integers(0, n, len(u)))
-    large = csr_from_edges(n, u, np.minimum(v, n - 1))
+    large = _large_graph(rng, n)
     labs = [np.where(rng.random((5, n)) < 0.3, rng.integers(0, n // 120, (5, n)), np.arange(n) // 120).astype(np.int32)
             for _ in range(3)]
     jobs = [(*large, lab) for lab in labs] + [_job(6007, 9), _job(20011, 12)]
@@ -346,3 +350,41 @@ def test_large_runs_in_threads(cc):
     for t in threads:
         t.join()
     assert not wrong
+
+
+# A small job's run is a chain of small kernels; beside another thread's large runs
+# it waits for their kernels, not for the end of a run with each of its own.
+def test_small_run_beside_large_ones(cc):
+    rng = np.random.default_rng(12)
+    n = 60011
+    lab = np.where(rng.random((12, n)) < 0.3, rng.integers(0, n // 120, (12, n)), np.arange(n) // 120).astype(np.int32)
+    small_job = _job(1000, 10)
+    ref = oracle.sync_run(*small_job, 20)
+    stop = threading.Event()
+
+    def runs(job):
+        while not stop.is_set():
+            job.reset()
+            job.run_until_converged(6)
+
+    def median(job, count):
+        times = []
+        for _ in range(count):
+            t0 = time.perf_counter()
+            job.reset()
+            assert job.run_until_converged(20) == ref.sweeps
+            times.append(time.perf_counter() - t0)
+            np.testing.assert_array_equal(job.cluster_ids(), ref.C)
+        return np.median(times)
+
+    with cc.Consensus(*_large_graph(rng, n), lab) as large, cc.Consensus(*small_job) as small:
+        large.run_until_converged(6)
+        alone = median(small, 20)
+        thread = threading.Thread(target=runs, args=(large,))
+        thread.start()
+        try:
+            beside = median(small, 20)
+        finally:
+            stop.set()
+            thread.join()
+    assert beside < 15 * alone, (beside, alone)  # about 100 where each kernel waits for a run
