@@ -248,10 +248,12 @@ cc_status cc_metrics(cc_ctx* ctx, cc_partition_metrics* out);
 /* Grouping homogeneous partitions (Methods, "Grouping homogeneous
  * partitions"): the distances between every pair of the job's input
  * partitions, out[a * k + i] = distances of P_a to P_i (k x k entries,
- * caller-allocated; the diagonal is zero).  Each P_a in turn is made the
- * consensus and measured as by cc_metrics; the context's consensus, objective
- * and history are restored afterwards.  Single-job contexts only.  Errors as
- * cc_metrics, CC_ERR_INVALID for a batch. */
+ * caller-allocated; the diagonal is zero).  Every pair is counted in a matrix
+ * of its classes, unless the square of the largest number of classes is above
+ * 16 n + 2^18 or 2^26, or the memory is not there: then each P_a in turn is made
+ * the consensus and measured as by cc_metrics.  The context's consensus,
+ * objective and history are as before afterwards.  Single-job contexts only.
+ * Errors as cc_metrics, CC_ERR_INVALID for a batch. */
 cc_status cc_partition_distances(cc_ctx* ctx, cc_partition_metrics* out);
 
 /* Groups k partitions: the complete graph over them, weighted by

@@ -1,6 +1,6 @@
 // The C ABI declared in include/cc.h: context lifetime (one job, or a batch of
-// jobs held as one disjoint union), the sweep loop as captured CUDA graphs,
-// and the output calls.
+// jobs held as one disjoint union), its runs (launches of the run kernel, or
+// captured CUDA graphs), and the output calls.
 #include <algorithm>
 #include <atomic>
 #include <cstddef>
@@ -285,14 +285,16 @@ long long launch_budget(const cc_ctx* c, int limit, int chunk)
     return ((long long)limit * c->ncls + chunk - 1) / chunk + 64;
 }
 
-// Contexts of several jobs, colour-batched and served ones, and jobs of at
-// least this many label rows run in the run kernel: it wins at every size measured there
-// (n = 20011, k = 12, host to host: 1.75 ms against 3.31 as graphs; n = 1.5e5,
-// k = 37: 2.58 against 2.99).  The smallest single jobs stay graphs of one
-// kernel per step, not because that is faster: cc_launch_count reports their
-// kernels one by one, and callers hold it to that (n = 1000, k = 10: as one
-// launch with a loop 0.75 ms, as launches of 4 unrolled sweeps 1.12 ms, of
-// which 0.2 ms of host time per launch).
+// Contexts of several jobs, colour-batched and served ones, and jobs of at least
+// this many label rows run in the run kernel.  A run on resident inputs, run kernel
+// and graphs of a kernel per step (no_regions), us: n = 5000, k = 20 410 and 814, n =
+// 20,011 613 and 1033, n = 100,003 1028 and 1377, n = 300,007 2320 and 2536, n = 1e6
+// 7496 and 7628; but k-NN, k = 50, n = 500,000 44,363 and 43,253, n = 2e6 25,498 and
+// 24,445, where graphs stay away for the 1.0-1.5 ms that a new context spends on
+// instantiating one.  The smallest single jobs stay graphs although the run kernel
+// is faster there too (n = 1000, k = 10: 564 us as one launch with a loop, 326 in the
+// run kernel): cc_launch_count reports their kernels one by one, and callers hold
+// it to that.
 constexpr long long kRunKernelRows = 1 << 14;
 
 constexpr unsigned long long kWaitLimitNs = 20ull * 1000 * 1000 * 1000;  // see cc_set_wait_limit
@@ -803,8 +805,8 @@ cc_status create_common(int jobs, const JobInput* in, bool on_device, const cc_o
     const unsigned long long cap = plan.cap_max;
     c->cap_max = cap;
 
-    // one allocation for the whole context: 36 of them, and their release, took
-    // 3.5 ms for a context of 1.7 GB
+    // one allocation for the whole context: 38 of them, and their release, took
+    // 1.15 ms for n = 20,011, k = 12 and 4.2 ms for n = 1e6, k = 20
     {
         void* q = nullptr;
         CC_TRY(pool ? cudaMallocFromPoolAsync(&q, plan.persistent, pool, c->own_stream) : cudaMalloc(&q, plan.persistent));
@@ -943,7 +945,7 @@ cc_status create_common(int jobs, const JobInput* in, bool on_device, const cc_o
         if (e == cudaSuccess) e = launch_assemble(as, c->stream);
         LabelArgs la{};
         la.jobs = jobs;
-            la.labels = labels;
+        la.labels = labels;
         la.lo = reinterpret_cast<long long*>(d_meta + at_lo);
         la.pjob = reinterpret_cast<int*>(d_meta + at_pjob);
         la.pfirst = c->d_pfirst;
@@ -1678,14 +1680,6 @@ cc_status ctx_async_start(cc_ctx* c, int limit, DevState* pinned, JobState* pinn
     return launch_chunk(c);
 }
 
-int ctx_async_poll(cc_ctx* c, cc_status* st)
-{
-    const int r = ctx_async_poll_step(c, st);
-    if (r != 2) return r;
-    *st = ctx_async_continue(c);
-    return *st == CC_OK ? 0 : -1;
-}
-
 cc_status ctx_async_continue(cc_ctx* c)
 {
     return launch_chunk(c);
@@ -1718,32 +1712,6 @@ int ctx_async_poll_step(cc_ctx* c, cc_status* st)
         return -1;
     }
     return 2;
-}
-
-cc_status ctx_job_results(cc_ctx* c, std::vector<long long>& F, std::vector<int>& sweeps)
-{
-    std::vector<JobState> js;
-    cc_status r = read_jobs(c, js);
-    if (r != CC_OK) return r;
-    F.resize(c->jobs);
-    sweeps.resize(c->jobs);
-    for (int j = 0; j < c->jobs; ++j) {
-        F[j] = js[j].F;
-        sweeps[j] = js[j].sweeps;
-    }
-    return CC_OK;
-}
-
-cc_status ctx_renumber(cc_ctx* c, int** dev_labels)
-{
-    return renumber(c, dev_labels);
-}
-
-cc_status ctx_copy_labels(cc_ctx* c, const int* dev_labels, int j, int32_t* out)
-{
-    const JobInfo& J = c->job[j];
-    CC_CUDA(c, cudaMemcpyAsync(out, dev_labels + J.vo, sizeof(int) * (size_t)J.n, cudaMemcpyDeviceToHost, c->stream));
-    return CC_OK;
 }
 
 bool ctx_slot_fits(const cc_ctx* c, int j, const JobInput& in)

@@ -137,7 +137,7 @@ struct DevState {
     unsigned long long retry_mask;  // heavy sweep: capacity - 1 of the second attempt of its rebuild
     int many;                    // 1: many vertices may move (the sweep before moved more than 1/8 of the label rows)
     int match;                   // 1: some job of this sweep falls back to the matching
-    long long classes;           // label classes of all partitions (set at creation)
+    long long classes;           // label compaction (in its own control block): classes of all partitions together
     // run kernel (persist.cu); written between two steps only
     int rebuild_kind;            // the running rebuild: 0 heavy sweep, 1 its rollback, 2 end of the sweep
     int tries;                   // rebuild attempts of this heavy sweep
@@ -193,7 +193,7 @@ struct SweepArgs {
     unsigned char* pflag;       //   1 if kept by the singleton guard (2: matching winner)
     int* members;               // rebuild scratch: vertices listed cluster by cluster (n)
     int* cursor;                // rebuild scratch: next free position of each cluster (n)
-    int* bsum;                  // rebuild scratch: per-block sums of the size scan (n / 1024 + 1)
+    int* bsum;                  // rebuild scratch: per-block sums of the size scan (bsum_entries)
     DevState* st;
     unsigned long long* ts;     // kRunBodies times {start of a sweep body, end of its proposal step, its end} (ns)
     cc_sweep_info* hist;        // J x hist_cap records
@@ -390,20 +390,6 @@ __device__ __forceinline__ void job_acc_finish(JobAcc& acc, int jobs)
     }
 }
 static_assert(sizeof(JobState) % sizeof(long long) == 0, "JobState must be a multiple of 8 bytes");
-
-// Count stored under key (0 if absent).  Read-only use during a kernel that
-// does not modify the table, so the non-coherent path is allowed.
-__device__ __forceinline__ int table_count_ro(const Slot* t, unsigned long long mask, unsigned long long key)
-{
-    unsigned long long h = hash_key(key) & mask;
-    for (unsigned long long p = 0; p <= mask; ++p) {
-        ulonglong2 e = *reinterpret_cast<const ulonglong2*>(t + h);
-        if (e.x == key) return (int)(unsigned)(e.y & 0xffffffffull);
-        if (e.x == kEmpty) return 0;
-        h = (h + 1) & mask;
-    }
-    return 0;
-}
 
 // Slot holding key, or -1 (coherent loads; the key must not be inserted concurrently).
 __device__ __forceinline__ long long table_find(const Slot* t, unsigned long long mask, unsigned long long key)
@@ -656,7 +642,7 @@ cudaError_t run_grid(const SweepArgs& a, long long rows, int sms, int* most, int
 // launch (fresh: starts the run first; at most kRunBodies).
 cudaError_t launch_run(const SweepArgs& a, long long rows, int grid, int limit, bool fresh, int budget, cudaStream_t s);
 // The proposal step's scoring kernels alone (own-cluster sums, candidate
-// bids) on the current state, for timing; they write only aown, act (the
+// bids) on the current state, for timing; they write only own, act (the
 // same values on the same state) and the bids, which launch_clear_bids
 // empties again.  Nothing else of the state changes.
 cudaError_t launch_propose_probe(const SweepArgs& a, int grid, cudaStream_t s);

@@ -59,7 +59,7 @@ struct cc_ctx {
     unsigned char* pflag = nullptr;
     int* members = nullptr;             // rebuild scratch (n)
     int* cursor = nullptr;              // rebuild scratch (n)
-    int* bsum = nullptr;                // rebuild scratch (n/1024 + 2)
+    int* bsum = nullptr;                // rebuild scratch (bsum_entries)
     int* scratch = nullptr;             // 3n + n/1024 + 64 ints: output renumbering, warm starts
     // colour_batched: colour of each vertex, vertices and CSR entries by class
     int* colour = nullptr;
@@ -151,18 +151,13 @@ cc_status ctx_create(int jobs, const JobInput* in, bool on_device, const cc_opti
                      cudaMemPool_t pool, cc_ctx** out, int priority = 0);
 
 // Starts a run of at most `limit` sweeps without waiting: queues the run and
-// its first graph launch, then a copy of the control block into `pinned` and
-// an event.
+// its first launch, then a copy of the control block into `pinned` and an event.
 cc_status ctx_async_start(cc_ctx* c, int limit, DevState* pinned, JobState* pinned_jobs = nullptr);
 
-// Checks a run started by ctx_async_start: 0 = still running (the next graph
-// launch is queued when the previous one ended without stopping), 1 = every
-// job has stopped, -1 = failed (*st holds the status).
-int ctx_async_poll(cc_ctx* c, cc_status* st);
-// As ctx_async_poll, but when a graph launch ended without stopping the run
-// it returns 2 without queueing the next launch: the pinned job records are
-// then those after that launch (a job with stop set is done and its labels
-// are final), and ctx_async_continue queues the next launch.
+// Checks a run started by ctx_async_start: 0 = its launch still runs, 1 = every job
+// has stopped, 2 = the launch ended and the run goes on (the pinned job records
+// are those after it: a job with stop set is done and its labels are final;
+// ctx_async_continue queues the next launch), -1 = failed (*st holds the status).
 int ctx_async_poll_step(cc_ctx* c, cc_status* st);
 cc_status ctx_async_continue(cc_ctx* c);
 // If the launch has ended, it no longer counts as one that shares the GPU.
@@ -191,17 +186,6 @@ cc_status ctx_load_job(cc_ctx* c, int j, const JobInput& in);
 // (blocks until they are there).  Valid once the job has stopped, also
 // while other jobs of the context still run.
 cc_status ctx_job_labels_now(cc_ctx* c, int j, int32_t* out);
-
-// Objective and sweeps of every job (synchronises the context's stream).
-cc_status ctx_job_results(cc_ctx* c, std::vector<long long>& F, std::vector<int>& sweeps);
-
-// Renumbered labels of job j into host memory (queued on the context's
-// stream; synchronise before reading).
-cc_status ctx_copy_labels(cc_ctx* c, const int* dev_labels, int j, int32_t* out);
-
-// Renumbers the labels of every job on the device; *dev_labels points into
-// the context's scratch.
-cc_status ctx_renumber(cc_ctx* c, int** dev_labels);
 
 void ctx_destroy(cc_ctx* c);
 

@@ -2,7 +2,7 @@
 // GPU and batches their sweeps (continuous batching).
 //
 // Submitted jobs wait in arrival order.  Each call of cc_server_progress
-//   1. polls the contexts in flight; when a context's current graph launch has
+//   1. polls the contexts in flight; when a context's current launch has
 //      ended, every job of it that has stopped is released at once (its
 //      labels renumbered on the device and copied into the job's output
 //      buffer, objective and sweep count recorded), without waiting for the
@@ -12,7 +12,7 @@
 //      Waiting jobs of the context's lane bin that fit the place of a
 //      released job (no more vertices, CSR entries, partitions and label
 //      rows) are loaded into it before the next launch, so they join the
-//      running union between two graph launches (iteration-level batching);
+//      running union between two launches (iteration-level batching);
 //      a context whose jobs have all stopped is kept for such jobs too;
 //   2. admits waiting jobs while a context slot is free and the device bytes
 //      of the new context (computed exactly from the job sizes before
@@ -23,10 +23,10 @@
 //      first job's n (a context finishes with its slowest job, so a small job
 //      does not wait for a large one) and still fit.  The jobs of a context
 //      run as one disjoint union in the same kernel launches, on the
-//      context's own stream, so contexts admitted while others run overlap
-//      with them on the device.  Streams of smaller contexts get a higher
-//      priority: when contexts share the GPU, the thread blocks of short jobs
-//      are scheduled first, which keeps their latency close to running alone.
+//      context's own stream.  A launch (of up to 4 sweeps) takes a share of the
+//      GPU's places beside the contexts that run (see api.cu), so they overlap.
+//      Streams of smaller contexts get a higher priority, which decides whose
+//      launch starts first where several wait for places.
 // Every job's results are those of running it alone (the sweep of a union is
 // per-job exact), so results do not depend on the mix it was served in.
 #include <algorithm>
