@@ -64,10 +64,10 @@ UNIT = "edge-partitions/s"
 # changed since).
 NOMINAL_HBM_GBS = 7900.0  # GB300 HBM3e, nominal (the roofline's peak is the measured copy rate)
 
-PROPOSAL_TRAFFIC = {"knn_n2000000_k50": 12.06e9, "lfr_n1000000_k20": 2.802e9}
+PROPOSAL_TRAFFIC = {"knn_n2000000_k50": 12.06e9, "lfr_n1000000_k20": 2.803e9}
 PROPOSAL_TRAFFIC_SOURCE = {
     "knn_n2000000_k50": "ncu dram__bytes_read.sum + dram__bytes_write.sum of k_own, k_edges, k_collect over one "
-                        "run at n=500000 (2.946 GB), scaled by nnz (x4.0921)",
+                        "run at n=500000 (2.948 GB), scaled by nnz (x4.0921)",
     "lfr_n1000000_k20": "ncu dram__bytes_read.sum + dram__bytes_write.sum of k_own, k_edges, k_collect over one "
                         "run at n=500000 (1.401 GB), scaled by nnz (x2.0002)"}
 
