@@ -228,7 +228,9 @@ cc_status start_state(cc_ctx* c)
 }
 
 // Graph of `bodies` sweeps with every step a plain node, or (bodies 0) of a
-// run: a WHILE node repeats the sweep, its optional parts behind IF nodes.
+// run: a WHILE node repeats the sweep, its optional parts behind IF nodes; or
+// (kOneSweep) of one sweep so.
+constexpr int kOneSweep = -1;
 cc_status ensure_graph(cc_ctx* c, int bodies, cudaGraphExec_t* out)
 {
     auto it = c->graphs.find(bodies);
@@ -240,6 +242,7 @@ cc_status ensure_graph(cc_ctx* c, int bodies, cudaGraphExec_t* out)
     CC_CUDA(c, cudaStreamBeginCapture(c->own_stream, cudaStreamCaptureModeThreadLocal));
     cudaError_t e = cudaSuccess;
     if (bodies == 0) e = capture_run_loop(c->args, c->rows, c->grid, c->own_stream, c->loop_stream, c->body_stream);
+    if (bodies == kOneSweep) e = launch_sweep(c->args, c->rows, c->grid, c->own_stream, c->body_stream);
     for (int s = 0; s < bodies && e == cudaSuccess; ++s)
         e = launch_sweep(c->args, c->rows, c->grid, c->own_stream, nullptr);
     for (cudaStream_t st : {c->body_stream, c->loop_stream}) {
@@ -490,12 +493,15 @@ cudaError_t size_run(cc_ctx* c)
     return run_grid(c->args, c->rows, stream_sms(c->stream, c->sms), &c->run_blocks, &c->run_want);
 }
 
+// Sweeps of a run that may be abandoned for lack of table space and retried.
+constexpr int kRetries = 64;
+
 // A run as launches of the run kernel: one unless the run is very long, or
 // the context's lanes are to be timed after its first sweep.
 cc_status run_kernel(cc_ctx* c, int limit, DevState* out, std::vector<JobState>& js)
 {
     DevState& st = *out;
-    long long left = (long long)limit * c->ncls + 64;  // 64: sweeps abandoned for lack of table space and retried
+    long long left = (long long)limit * c->ncls + kRetries;
     int before = 0;
     for (bool fresh = true; left > 0; fresh = false) {
         const int budget = !c->tuned ? 1 : (int)std::min<long long>(left, kRunBodies);
@@ -526,21 +532,24 @@ cc_status run_kernel(cc_ctx* c, int limit, DevState* out, std::vector<JobState>&
 // the sweep until the run stops, or, with no_regions, plain graphs of up to
 // kChunk sweeps, launched until the device says the run has stopped.  An
 // autotuned context runs its first sweep alone (a plain graph of one body: the
-// loop holds kLoopSweeps) and times its lanes on the state that left.
+// loop holds kLoopSweeps) and times its lanes on the state that left.  A run of
+// one sweep at most is a graph of one (three calls of cc_sweep at n = 200, k = 5:
+// 577 us so before the loop, 647 with it, @one@ so again).
 cc_status run_graphs(cc_ctx* c, int limit, DevState* out, std::vector<JobState>& js)
 {
     DevState& st = *out;
     const int chunk = chunk_bodies(c, limit);
-    long long left = (long long)limit * c->ncls + 64;  // 64: sweeps abandoned for lack of table space and retried
+    long long left = (long long)limit * c->ncls + kRetries;
     long long launches = launch_budget(c, limit, chunk);
     int before = 0;
     for (;;) {
-        const bool loop = c->tuned && !c->opt.no_regions;
-        const int bodies = !c->tuned ? 1 : loop ? (int)std::min<long long>(left, kRunBodies) : chunk;
+        const bool one = c->tuned && !c->opt.no_regions && before == 0 && left == 1 + kRetries;
+        const bool loop = c->tuned && !c->opt.no_regions && !one;
+        const int bodies = !c->tuned || one ? 1 : loop ? (int)std::min<long long>(left, kRunBodies) : chunk;
         if (before == 0) CC_CUDA(c, launch_run_begin(c->args, limit, bodies, c->stream));
         else if (loop) CC_CUDA(c, launch_run_more(c->args, before + bodies, c->stream));
         cudaGraphExec_t exec = nullptr;
-        cc_status r = ensure_graph(c, loop ? 0 : bodies, &exec);
+        cc_status r = ensure_graph(c, loop ? 0 : one ? kOneSweep : bodies, &exec);
         if (r != CC_OK) return r;
         if (before == 0 || loop) c->launches += 1;
         CC_CUDA(c, cudaGraphLaunch(exec, c->stream));
@@ -548,7 +557,9 @@ cc_status run_graphs(cc_ctx* c, int limit, DevState* out, std::vector<JobState>&
         if (r != CC_OK) return r;
         const int ran = st.run_bodies - before;
         const long long turns = (ran + kLoopSweeps - 1) / kLoopSweeps;
-        c->launches += loop ? turns * (kLoopSweeps * kKernelsOutsideRegions + 1) : (long long)bodies * kKernelsPerSweep;
+        c->launches += loop  ? turns * (kLoopSweeps * kKernelsOutsideRegions + 1)
+                       : one ? kKernelsOutsideRegions
+                             : (long long)bodies * kKernelsPerSweep;
         c->ts_from = before;
         c->ts_bodies = ran;
         before = st.run_bodies;

@@ -388,3 +388,24 @@ def test_small_run_beside_large_ones(cc):
             stop.set()
             thread.join()
     assert beside < 15 * alone, (beside, alone)  # about 100 where each kernel waits for a run
+
+
+# A small job's cc_sweep is a graph of one sweep: the kernels of one body outside
+# its regions, and none of a second.
+def test_single_sweeps_of_a_small_job(cc):
+    ro, col, lab = _job(1000, 10)
+    ref = oracle.sync_run(ro, col, lab, 20)
+    outside = 17  # begin, own, edges, collect, route, 6 gates, bid, match keys, commit, match reset, end jobs, end
+    with cc.Consensus(ro, col, lab) as job:
+        for rounds in range(2):
+            job.reset()
+            for s in range(ref.sweeps):
+                before = job.launch_count()
+                assert job.sweep() == ref.stats[s]
+                assert job.launch_count() - before >= 1 + outside
+                assert len(job.last_run_timing()[0]) == 1
+            assert job.launch_count() - before == 1 + outside  # the last one proposes nothing
+            np.testing.assert_array_equal(job.cluster_ids(), ref.C)
+            job.reset()
+            assert job.run_until_converged(20) == ref.sweeps
+            assert job.history() == ref.stats
