@@ -331,6 +331,9 @@ cc_status cc_sweep(cc_ctx* ctx, cc_sweep_info* info);
  * sweeps (one after the end of the run is skipped on the device).  With
  * no_regions, sweeps are submitted as plain graphs of up to 4, and the host
  * reads the stop flag after each.
+ * The run kernel holds its places on the GPU until it ends: kernels of the
+ * caller's on other streams run beside it if they are small, larger ones wait
+ * for the end of the run.  A stream of a green context keeps it to that part.
  * *sweeps_done (may be NULL) counts every sweep run, the final empty one
  * included.  Errors as cc_sweep. */
 cc_status cc_run_until_converged(cc_ctx* ctx, int32_t max_sweeps, int32_t* sweeps_done);

@@ -534,7 +534,7 @@ cc_status run_kernel(cc_ctx* c, int limit, DevState* out, std::vector<JobState>&
 // autotuned context runs its first sweep alone (a plain graph of one body: the
 // loop holds kLoopSweeps) and times its lanes on the state that left.  A run of
 // one sweep at most is a graph of one (three calls of cc_sweep at n = 200, k = 5:
-// 577 us so before the loop, 647 with it, @one@ so again).
+// 585 us before the loop, 592 with it, 523 so again).
 cc_status run_graphs(cc_ctx* c, int limit, DevState* out, std::vector<JobState>& js)
 {
     DevState& st = *out;

@@ -460,14 +460,15 @@ inline size_t run_smem(int jobs)
     return (2 * jobs <= kSmemJobs ? 2 : 1) * smem_jobs_bytes(jobs);
 }
 
-// Places for blocks that a run leaves free, so that the caller's kernels on
-// other streams find one: four blocks of a run take all registers of an SM, and
-// with every place taken a small kernel waited for the end of the run (n =
-// 300,007, k = 24: 1224 us, now 47).  Two of 608 cost the run nothing (n = 1e6,
-// k = 20: 6.96 ms both), eight cost it 1%.
+// A place for a block that a run leaves free, so that the caller's small kernels
+// on other streams find one: four blocks of a run take all registers of an SM,
+// and with every place taken such a kernel waited for the end of the run (beside n
+// = 300,007, k = 24: one block 1224 us, 48 so; 2^20 floats 1225 and 299; one that
+// fills the GPU waits all the same).  It costs a run 0-0.6% (two places 0-6%, where
+// a step's rounds of work come out uneven: n = 1e5 with 32 lanes; eight 1%).
 inline int spare_blocks(int resident)
 {
-    return std::min(2, resident / 64);
+    return std::min(1, resident / 64);
 }
 
 }  // namespace
