@@ -328,7 +328,8 @@ cc_status cc_sweep(cc_ctx* ctx, cc_sweep_info* info);
  * While other contexts run on the device it takes a share of it, or, for a job
  * that fills it many times over, runs as the graph below.
  * A smaller job's run is one launch of a CUDA graph whose loop holds two
- * sweeps (one after the end of the run is skipped on the device).  With
+ * sweeps (one after the end of the run is skipped on the device; one sweep if
+ * the run may take no more).  With
  * no_regions, sweeps are submitted as plain graphs of up to 4, and the host
  * reads the stop flag after each.
  * The run kernel holds its places on the GPU until it ends: kernels of the
