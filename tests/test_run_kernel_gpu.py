@@ -409,3 +409,48 @@ def test_single_sweeps_of_a_small_job(cc):
             job.reset()
             assert job.run_until_converged(20) == ref.sweeps
             assert job.history() == ref.stats
+
+
+# Batches and colour-batched jobs of that size beside another thread's runs: the
+# graph of a run with several jobs, and with colour classes.
+def test_large_batches_beside_runs(cc):
+    rng = np.random.default_rng(13)
+    n = 60011
+    lab = np.where(rng.random((4, n)) < 0.3, rng.integers(0, n // 120, (4, n)), np.arange(n) // 120).astype(np.int32)
+    large = (*_large_graph(rng, n), lab)
+    jobs = [_job(900, 12), large, _job(3001, 5)]
+    refs = [oracle.sync_run(*j, 5) for j in jobs]
+    colour = oracle.colour_run(*large, 2)
+    small_job = _job(1000, 10)
+    stop = threading.Event()
+
+    def runs():
+        with cc.Consensus(*small_job) as small:
+            while not stop.is_set():
+                small.reset()
+                small.run_until_converged(20)
+
+    thread = threading.Thread(target=runs)
+    thread.start()
+    graphs = 0
+    try:
+        with cc.ConsensusBatch(jobs) as batch, cc.Consensus(*large, _options(cc, colour_batched=1)) as coloured, \
+                cc.ConsensusBatch(jobs, _options(cc, active_set=1, debug_checks=1)) as active:
+            for _ in range(4):
+                for b in (batch, active):
+                    before = b.launch_count()
+                    b.reset()
+                    b.run_until_converged(5)
+                    graphs += b.launch_count() - before > 20
+                    np.testing.assert_array_equal(b.cluster_ids(), np.concatenate([r.C for r in refs]))
+                    assert [b.history(j)[-1] for j in range(3)] == [r.stats[-1] for r in refs]
+                before = coloured.launch_count()
+                coloured.reset()
+                coloured.run_until_converged(2)
+                graphs += coloured.launch_count() - before > 20
+                assert coloured.history() == colour.stats
+                np.testing.assert_array_equal(coloured.cluster_ids(), colour.C)
+    finally:
+        stop.set()
+        thread.join()
+    assert graphs > 0
